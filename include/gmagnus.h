@@ -253,10 +253,9 @@ int gm_plan_get_row_products(const gm_plan* plan, int64_t* ip_out_device, void* 
  * latency-critical section where an allocation (which may synchronise the whole device) is not
  * acceptable, or a host whose allocator is owned by another runtime.  For them this entry point
  * computes IP_i = sum over stored entries j of A[i,:] of nnz(B[A.col[j],:]) for every row of A and
- * allocates nothing: no cudaMalloc / cudaFree, no stream-ordered allocation, no allocator hook.
- * Its scratch (products per stored entry, their prefix sums, tile sums of the scan) lives in a
- * fixed array inside the library image: about 12.6 MB of device memory on every GPU that loads the
- * library, held until the process exits.
+ * allocates nothing: no cudaMalloc / cudaFree, no stream-ordered allocation, no allocator hook.  It needs no
+ * scratch memory either: a block adds up the rows that lie in its share of A's entries, and the few rows that
+ * blocks share are added up in ip_out_device itself.
  *   A, B           host structs with DEVICE pointers, as for gm_spgemm_plan; only row_ptr and col_idx are
  *                  read, so vals may be NULL and dtype is ignored.  Columns of A are not range-checked:
  *                  an entry of A.col_idx outside [0, B.n_rows) reads past B.row_ptr
@@ -264,11 +263,8 @@ int gm_plan_get_row_products(const gm_plan* plan, int64_t* ip_out_device, void* 
  *   cuda_stream    the work is enqueued there; the call does not synchronise
  * Limit: A->nnz <= GM_NOALLOC_MAX_NNZ_A (1,048,576); larger inputs are rejected with GM_ERR_CAPACITY
  * and nothing is launched.  Any number of rows.
- * The first call on each device looks up the address of the scratch array (one
- * cudaGetSymbolAddress with that device current); make that first call before starting any stream
- * capture.  Every call uses the same scratch array: everything in it is rewritten before it is
- * read, so nothing needs clearing, but two calls whose kernels can overlap on the GPU (different
- * streams, or concurrent host threads) race on it — serialise them. */
+ * The first call on each device queries it; make that first call before starting any stream capture.
+ * Calls may overlap on the GPU (different streams, concurrent host threads) as long as they write different arrays. */
 #define GM_NOALLOC_MAX_NNZ_A 1048576
 int gm_row_products_noalloc(const gm_csr* A, const gm_csr* B, int64_t* ip_out_device, void* cuda_stream);
 

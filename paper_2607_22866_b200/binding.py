@@ -107,6 +107,8 @@ def _torch_free(ptr, stream, user):
 def load_library(install_torch_allocator: bool = True):
     """Loads (building it first if needed) libgmagnus.so and declares the C signatures."""
     global _lib, _alloc_cb, _free_cb
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is not None:
             return _lib
@@ -200,8 +202,9 @@ def planner_batches(heavy_prefix: np.ndarray, stage_elems: int) -> list[int]:
 
 
 def _stream_ptr(stream) -> int:
-    s = torch.cuda.current_stream() if stream is None else stream
-    return int(s.cuda_stream)
+    if stream is None:  # (without building a Stream object: a few microseconds that a small product feels)
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+    return int(stream.cuda_stream)
 
 
 class Plan:
@@ -246,10 +249,10 @@ NOALLOC_MAX_NNZ_A = 1048576
 
 def row_products_noalloc(A: DeviceCSR, B: DeviceCSR, out: torch.Tensor, stream=None) -> torch.Tensor:
     """gm_row_products_noalloc: IP_i for every row of A, written into the caller's int64 device tensor
-    `out` (A.n_rows entries).  The library allocates nothing: its scratch is a fixed array in the library
-    image, so nnz(A) is limited to NOALLOC_MAX_NNZ_A and calls that overlap on the GPU race on it."""
+    `out` (A.n_rows entries).  The library allocates nothing; nnz(A) is limited to NOALLOC_MAX_NNZ_A."""
     assert out.dtype == torch.int64 and out.is_contiguous() and out.numel() >= A.n_rows
-    a, b = A._struct(), B._struct()
+    a = A._struct()
+    b = a if B is A else B._struct()
     _check(load_library().gm_row_products_noalloc(ctypes.byref(a), ctypes.byref(b), out.data_ptr(),
                                                   _stream_ptr(stream)), "gm_row_products_noalloc")
     return out
@@ -260,7 +263,8 @@ def spgemm_plan(A: DeviceCSR, B: DeviceCSR, smem_bytes: int = 232448, opts: Plan
     """gm_spgemm_plan_ex on the current (or given) torch stream."""
     lib = load_library()
     h = ctypes.c_void_p()
-    a, b = A._struct(), B._struct()
+    a = A._struct()
+    b = a if B is A else B._struct()
     _check(lib.gm_spgemm_plan_ex(ctypes.byref(a), ctypes.byref(b), smem_bytes,
                                  ctypes.byref(opts) if opts else None, _stream_ptr(stream), ctypes.byref(h)),
            "gm_spgemm_plan")
@@ -268,8 +272,8 @@ def spgemm_plan(A: DeviceCSR, B: DeviceCSR, smem_bytes: int = 232448, opts: Plan
 
 
 def _wrap(ptr: int, numel: int, dtype) -> torch.Tensor:
-    block = _live.pop(ptr)
-    return block.view(dtype)[:numel] if numel else block.view(dtype)[:0]
+    t = _live.pop(ptr).view(dtype)
+    return t if t.numel() == numel else t[:numel]
 
 
 def spgemm_execute(plan: Plan, stream=None) -> DeviceCSR:

@@ -6,12 +6,14 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <mutex>
 #include <string>
 #include <vector>
 
 #include "gm_common.cuh"
 #include "gm_k1_analysis.cuh"
 #include "gm_k3_light.cuh"
+#include "gm_k3_rows.cuh"
 #include "gm_k4_expand.cuh"
 #include "gm_k4_direct.cuh"
 #include "gm_k4_stream.cuh"
@@ -98,8 +100,94 @@ static void dev_free(void* p, cudaStream_t st) {
 struct Buf {
   void* p = nullptr;
   size_t bytes = 0;
-  template <typename T> T* as() const { return static_cast<T*>(p); }
 };
+
+// What the host needs to know about a device, looked up once (the memory query goes to the kernel driver: 0.2 to 2.6 ms a
+// call on a shared host, more than most products take).
+struct DeviceFacts {
+  bool known = false;
+  int num_sms = 0, smem_optin = 0;
+  size_t total_mem = 0;
+  cudaStream_t side_stream = nullptr;  // see execute_t
+};
+constexpr int kMaxDevices = 64;
+static std::mutex g_facts_mutex;
+static DeviceFacts g_facts[kMaxDevices];
+
+static int device_facts(DeviceFacts* out) {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) {
+    cudaGetLastError();
+    return fail(GM_ERR_CUDA, "no CUDA device: this library has no CPU path");
+  }
+  if (dev < 0 || dev >= kMaxDevices) return fail(GM_ERR_INVALID_ARG, "device index out of range");
+  std::lock_guard<std::mutex> lock(g_facts_mutex);
+  DeviceFacts& f = g_facts[dev];
+  if (!f.known) {
+    int n_dev = 0;
+    if (cudaGetDeviceCount(&n_dev) != cudaSuccess || n_dev == 0) {
+      cudaGetLastError();
+      return fail(GM_ERR_CUDA, "no CUDA device: this library has no CPU path");
+    }
+    size_t free_b = 0;
+    GM_CUDA(cudaDeviceGetAttribute(&f.num_sms, cudaDevAttrMultiProcessorCount, dev));
+    GM_CUDA(cudaDeviceGetAttribute(&f.smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+    GM_CUDA(cudaMemGetInfo(&free_b, &f.total_mem));
+    f.known = true;
+  }
+  *out = f;
+  return GM_OK;
+}
+
+// One second stream per device for the life of the process (creating and destroying a stream per plan cost more than the
+// overlap gained on millisecond products); executes that share it are ordered by their own events.  NULL: none.
+static cudaStream_t side_stream() {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return nullptr;
+  std::lock_guard<std::mutex> lock(g_facts_mutex);
+  cudaStream_t& st = g_facts[dev].side_stream;
+  if (!st && cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking) != cudaSuccess) {
+    cudaGetLastError();
+    st = nullptr;
+  }
+  return st;
+}
+
+// Page-locked host memory that kernels write to and the host reads after a synchronisation: a plan takes one slot and
+// gives it back when it is destroyed.  (Copies to ordinary host variables took 12 to 25 us of host time each.)
+struct HostSlot {
+  int err[4];            // [0] first device-side problem of an execute, [1] malformed input
+  u64 totals[kK1Words];  // K1Totals
+  i64 c_total;           // nnz(C)
+  i64 tail[16];          // copy of gm_plan::c_total
+};
+constexpr int kHostSlotBytes = 512;
+static_assert(sizeof(HostSlot) <= kHostSlotBytes, "one slot");
+static std::mutex g_slot_mutex;
+static std::vector<HostSlot*> g_free_slots;
+
+static HostSlot* take_slot() {
+  std::lock_guard<std::mutex> lock(g_slot_mutex);
+  if (g_free_slots.empty()) {
+    constexpr int kSlab = 64;
+    void* slab = nullptr;
+    if (cudaHostAlloc(&slab, kSlab * kHostSlotBytes, cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) {
+      cudaGetLastError();
+      return nullptr;
+    }
+    for (int i = kSlab - 1; i >= 0; --i)
+      g_free_slots.push_back(reinterpret_cast<HostSlot*>(static_cast<char*>(slab) + i * kHostSlotBytes));
+  }
+  HostSlot* s = g_free_slots.back();
+  g_free_slots.pop_back();
+  std::memset(s, 0, kHostSlotBytes);
+  return s;
+}
+static void give_slot(HostSlot* s) {
+  if (!s) return;
+  std::lock_guard<std::mutex> lock(g_slot_mutex);
+  g_free_slots.push_back(s);
+}
 
 // ------------------------------------------------------------------------------------------------
 // plan
@@ -155,15 +243,20 @@ struct gm_plan {
   gm_exec_stats stats{};
   int num_sms = 148;
   cudaStream_t plan_stream = nullptr;
-  gm::LightBins bins{};
+  gm::RowRules rules{};
+  gm::i64 class_rows[gm::kRowClasses]{};  // light rows per class (see gm_k1_analysis.cuh)
+  gm::i64 staged_light = 0;        // products of the light rows that are merged or sorted
+  int merge_lists = 0;             // most entries of A in a merged row
+  bool merge_only = false;         // every row of A is merged or empty
+  gm::LightBins bins{};            // hash rows by entry count, for their numeric pass
   int bin_slots[gm::kMaxLightBins]{};
+  gm::HostSlot* slot = nullptr;
   std::vector<gm::Batch> batches;
   std::vector<int32_t> x_heavy_host;
   int64_t max_batch_rows = 0;
   int64_t n_seg = 0;
   std::vector<gm::Buf> owned;
   // device arrays
-  int64_t* nz_off = nullptr;       // nnzA + 1
   int64_t* ip = nullptr;           // nA
   int32_t* heavy_flag = nullptr;   // nA
   int32_t* x_heavy = nullptr;      // nH
@@ -194,16 +287,18 @@ struct gm_plan {
   unsigned char* parent_tag = nullptr;  // per parent of the level that runs: != 0, not split
   std::vector<int64_t> heavy_nz_off_host;
   int64_t* heavy_nz_off = nullptr; // nH + 1
-  int32_t* sym_rows = nullptr;     // bins x nA
-  int* sym_fill = nullptr;         // 8
-  int32_t* num_rows = nullptr;     // bins x nA
+  int32_t* class_list = nullptr;   // classes x nA: light rows per class
+  int64_t* light_off = nullptr;    // nA: a row's place in the light staging area, -1: none
+  int32_t* light_col = nullptr;    // light staging area: finished rows, at the place of their products
+  void* light_val = nullptr;
+  int32_t* num_rows = nullptr;     // bins x nA: hash rows by entry count
   int* num_fill = nullptr;         // 8
   int32_t* row_nnz = nullptr;      // nA
   int64_t* scan_tmp = nullptr;
   int64_t* c_total = nullptr;      // [0] running nnz(C) (device carry), [1] heavy entries, [2] products and [3] entries of
                                    // small chunks, [4] products and [5] entries of mid-size chunks, [6] products and
                                    // [7] chunks that left the hierarchy early, [8] products the levels did not move
-  int* err = nullptr;
+  int* err = nullptr;              // in the host slot: kernels write it through the mapping
   // heavy workspace
   int32_t* stage_col[2]{};
   void* stage_val[2]{};
@@ -221,7 +316,7 @@ struct gm_plan {
   gm::PhaseTimes times;
   HostSink* sink = nullptr;        // set by gm_spgemm_host for the duration of one execute
   // light rows run next to the heavy path on a stream of the plan's own (Algorithm 3 keeps separate queues for them)
-  cudaStream_t light_stream = nullptr;
+  cudaStream_t light_stream = nullptr;  // (the device's, not owned)
   cudaEvent_t ev_fork = nullptr, ev_light = nullptr;
 };
 
@@ -240,6 +335,31 @@ static int plan_alloc(gm_plan* p, T** out, size_t n, cudaStream_t st) {
   p->info.workspace_bytes += static_cast<int64_t>(b.bytes);
   *out = static_cast<T*>(b.p);
   return GM_OK;
+}
+
+// Several device arrays in one allocation: the allocator hook of the Python binding costs a few microseconds a call.
+struct Arena {
+  struct Item { void** slot; size_t offset; };
+  std::vector<Item> items;
+  size_t bytes = 0;
+  template <typename T>
+  void add(T** slot, size_t n) {
+    items.push_back({reinterpret_cast<void**>(slot), bytes});
+    bytes += (n * sizeof(T) + 255) & ~size_t{255};
+  }
+  int commit(gm_plan* p, cudaStream_t st) {
+    unsigned char* base = nullptr;
+    GM_TRY(plan_alloc(p, &base, bytes, st));
+    for (const Item& it : items) *it.slot = base + it.offset;
+    return GM_OK;
+  }
+};
+
+// First segment of heavy row h (h = 0 .. rows_heavy); the offsets are on the host only when there are several batches.
+static i64 seg_begin(const gm_plan* p, i64 h) {
+  if (h == 0) return 0;
+  if (h == p->info.rows_heavy) return p->n_seg;
+  return p->heavy_nz_off_host[static_cast<size_t>(h)];
 }
 
 static unsigned grid_for(i64 n, int threads, int num_sms, int per_sm = 16) {
@@ -275,22 +395,31 @@ __global__ void k_validate_csr(const i64* __restrict__ row_ptr, const int32_t* _
   }
 }
 
+static int launch_row_analysis(gm_plan* p, K1Totals* totals, HeavyTile* tiles, u32* parts, cudaStream_t st) {
+  const gm_csr& A = p->A;
+  const int T = k1_tile_items(A.n_rows, A.nnz, p->num_sms);
+  const unsigned grid = static_cast<unsigned>(std::min<i64>((A.n_rows + A.nnz + T - 1) / T, static_cast<i64>(p->num_sms) * 6));
+  const bool wide = p->B.n_cols > (i64{1} << 24);
+  auto kern = T == kK1Small ? (wide ? k1_rows<kK1Small, i64> : k1_rows<kK1Small, u32>)
+                            : (wide ? k1_rows<kK1Large, i64> : k1_rows<kK1Large, u32>);
+  kern<<<grid, kK1Threads, 0, st>>>(A.row_ptr, A.col_idx, A.n_rows, A.nnz, p->B.row_ptr, p->rules, p->ip, parts, p->heavy_flag,
+                                    p->row_nnz, p->light_off, p->class_list, A.n_rows, tiles, totals, p->slot->totals);
+  GM_CUDA(cudaGetLastError());
+  return GM_OK;
+}
+
 static int build_plan(gm_plan* p, cudaStream_t st) {
   const gm_csr& A = p->A;
   const gm_csr& B = p->B;
-  const i64 nA = A.n_rows, nnzA = A.nnz;
+  const i64 nA = A.n_rows;
   gm_plan_info& info = p->info;
   info.n_rows = nA;
   info.n_cols_c = B.n_cols;
 
-  int dev = 0;
-  GM_CUDA(cudaGetDevice(&dev));
-  // (two attribute queries: cudaGetDeviceProperties fills in the whole structure and takes milliseconds)
-  int num_sms = 0, smem_optin = 0;
-  GM_CUDA(cudaDeviceGetAttribute(&num_sms, cudaDevAttrMultiProcessorCount, dev));
-  GM_CUDA(cudaDeviceGetAttribute(&smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-  p->num_sms = num_sms;
-  if (p->smem_bytes > static_cast<size_t>(smem_optin))
+  DeviceFacts facts;
+  GM_TRY(device_facts(&facts));
+  p->num_sms = facts.num_sms;
+  if (p->smem_bytes > static_cast<size_t>(facts.smem_optin))
     return fail(GM_ERR_UNSUPPORTED_SMEM, "smem_bytes exceeds the device's opt-in shared memory per block");
   {
     const int rc = planner_params(B.n_cols, A.dtype, p->smem_bytes, &p->opts, &info.params);
@@ -315,8 +444,9 @@ static int build_plan(gm_plan* p, cudaStream_t st) {
                   : std::min(o.early_exit ? o.early_exit : p->small_max, p->small_max);
   }
 
-  GM_TRY(plan_alloc(p, &p->err, 4, st));
-  GM_CUDA(cudaMemsetAsync(p->err, 0, 4 * sizeof(int), st));
+  p->slot = take_slot();
+  if (!p->slot) return fail(GM_ERR_OOM, "page-locked host memory for the plan's counters could not be had");
+  p->err = p->slot->err;
   if (p->opts.validate_inputs) {
     for (const gm_csr* M : {&A, &B}) {
       if (M->n_rows == 0) continue;
@@ -324,63 +454,60 @@ static int build_plan(gm_plan* p, cudaStream_t st) {
                                                                           M->n_cols, M->nnz, p->err + 1);
     }
     info.launches += 2;
-    int bad = 0;
-    GM_CUDA(cudaMemcpyAsync(&bad, p->err + 1, sizeof(int), cudaMemcpyDeviceToHost, st));
     GM_CUDA(cudaStreamSynchronize(st));
-    if (bad) return fail(GM_ERR_BAD_CSR, "row_ptr not monotone / columns out of range or not strictly ascending");
+    if (p->slot->err[1]) return fail(GM_ERR_BAD_CSR, "row_ptr not monotone / columns out of range or not strictly ascending");
   }
 
-  // ---- K1: products per stored entry, flattened product space, products per row
-  int32_t* nz_len = nullptr;
-  K1Totals* totals = nullptr;
-  int64_t* heavy_pos = nullptr;
-  GM_TRY(plan_alloc(p, &nz_len, static_cast<size_t>(nnzA) + 1, st));
-  GM_TRY(plan_alloc(p, &p->nz_off, static_cast<size_t>(nnzA) + 1, st));
-  GM_TRY(plan_alloc(p, &p->ip, static_cast<size_t>(nA) + 1, st));
-  GM_TRY(plan_alloc(p, &p->heavy_flag, static_cast<size_t>(nA) + 1, st));
-  GM_TRY(plan_alloc(p, &heavy_pos, static_cast<size_t>(nA) + 1, st));
-  GM_TRY(plan_alloc(p, &totals, 1, st));
-  GM_TRY(plan_alloc(p, &p->row_nnz, static_cast<size_t>(nA) + 1, st));
-  GM_TRY(plan_alloc(p, &p->c_total, 16, st));
-  GM_TRY(plan_alloc(p, &p->scan_tmp, static_cast<size_t>(scan_tmp_elems(std::max<i64>(std::max(nnzA, nA), 1))), st));
-  GM_CUDA(cudaMemsetAsync(totals, 0, sizeof(K1Totals), st));
-  if (nnzA > 0) k1_nz_len<<<grid_for(nnzA, 256, p->num_sms, 32), 256, 0, st>>>(A.col_idx, nnzA, B.row_ptr, nz_len);
-  exclusive_scan<int32_t, i64>(nz_len, p->nz_off, nnzA, p->scan_tmp, nullptr, nullptr, nullptr, st);
-  if (nA > 0) {
-    k1_row_products<<<grid_for(nA, 256, p->num_sms), 256, 0, st>>>(A.row_ptr, nA, p->nz_off, prm.tau, B.n_cols, p->ip,
-                                                                  p->heavy_flag, totals);
-  }
-  exclusive_scan<int32_t, i64>(p->heavy_flag, heavy_pos, nA, p->scan_tmp, nullptr, nullptr, nullptr, st);
-  info.launches += (nnzA > 0 ? 3 : 1) + (nA > 0 ? 3 : 1) + (nA > 0 ? 2 : 0) + 1;
-
-  // ---- light rows: bins by IP_i for the symbolic pass
+  // ---- K1: products per row, classes, totals
   {
+    // light rows: merged by a thread (when there are enough rows to fill the device with one thread each), sorted by a
+    // warp, or (above kSortMaxProducts: only with a tau that large) hashed
+    RowRules& r = p->rules;
+    r.tau = prm.tau;
+    r.c_cols = B.n_cols;
+    r.merge = nA >= kMergeMinRows ? 1 : 0;
+    r.sort_max = kSortMaxProducts;
+    r.n_hash = 0;
     const int top_cap = static_cast<int>(pow2_ceil(static_cast<uint64_t>(std::max<i64>(prm.tau, 16))));
-    const int std_caps[] = {16, 64, 256, 1024, 4096, 16384, 65536};
+    for (int c : {1024, 4096, 16384, 65536})
+      if (c < top_cap) r.hash_cap[r.n_hash++] = c;
+    r.hash_cap[r.n_hash++] = std::max(top_cap, 1024);
     int nb = 0;
-    for (int c : std_caps)
+    for (int c : {16, 64, 256, 1024, 4096, 16384, 65536})
       if (c < top_cap && nb < kMaxLightBins - 1) { p->bins.cap[nb] = c; p->bin_slots[nb] = 2 * c; ++nb; }
     p->bins.cap[nb] = top_cap;
     p->bin_slots[nb] = prm.light_slots;
     p->bins.n_bins = nb + 1;
   }
-  GM_TRY(plan_alloc(p, &p->sym_rows, static_cast<size_t>(p->bins.n_bins) * static_cast<size_t>(std::max<i64>(nA, 1)), st));
-  GM_TRY(plan_alloc(p, &p->num_rows, static_cast<size_t>(p->bins.n_bins) * static_cast<size_t>(std::max<i64>(nA, 1)), st));
-  GM_TRY(plan_alloc(p, &p->sym_fill, 8, st));
-  GM_TRY(plan_alloc(p, &p->num_fill, 8, st));
-  GM_CUDA(cudaMemsetAsync(p->sym_fill, 0, 8 * sizeof(int), st));
-  if (nA > 0) {
-    // tau may be below the top bin's capacity (forced tau): rows with tau < IP <= cap are heavy and skipped
-    k1_bin_rows<i64><<<static_cast<unsigned>((nA + 255) / 256), 256, 0, st>>>(p->ip, p->heavy_flag, nA, p->bins, nA,
-                                                                             p->sym_fill, p->sym_rows);
+  K1Totals* totals = nullptr;
+  HeavyTile* tiles = nullptr;
+  u32* parts = nullptr;
+  size_t zeroed = 0;
+  {
+    Arena ar;
+    const size_t n1 = static_cast<size_t>(nA) + 1;
+    ar.add(&totals, 1);
+    ar.add(&tiles, static_cast<size_t>((nA + kHeavyRows - 1) / kHeavyRows) + 1);
+    ar.add(&p->ip, n1);
+    ar.add(&parts, n1);
+    zeroed = ar.bytes;  // what the row analysis wants zeroed comes first
+    ar.add(&p->c_total, 16);
+    ar.add(&p->heavy_flag, n1);
+    ar.add(&p->row_nnz, n1);
+    ar.add(&p->light_off, n1);
+    ar.add(&p->class_list, static_cast<size_t>(kHashClass0 + p->rules.n_hash) * n1);
+    ar.add(&p->scan_tmp, static_cast<size_t>(scan_tmp_elems(std::max<i64>(nA, 1))));
+    GM_TRY(ar.commit(p, st));
   }
-
-  // ---- first host sync: totals
   K1Totals ht{};
-  int fill[8] = {0};
-  GM_CUDA(cudaMemcpyAsync(&ht, totals, sizeof(ht), cudaMemcpyDeviceToHost, st));
-  GM_CUDA(cudaMemcpyAsync(fill, p->sym_fill, sizeof(fill), cudaMemcpyDeviceToHost, st));
-  GM_CUDA(cudaStreamSynchronize(st));
+  if (nA > 0) {
+    GM_CUDA(cudaMemsetAsync(totals, 0, zeroed, st));
+    GM_TRY(launch_row_analysis(p, totals, tiles, parts, st));
+    info.launches += 1;
+    // ---- first host sync: totals
+    GM_CUDA(cudaStreamSynchronize(st));
+    std::memcpy(&ht, p->slot->totals, sizeof(ht));
+  }
   info.products_total = static_cast<int64_t>(ht.products_total);
   info.products_heavy = static_cast<int64_t>(ht.products_heavy);
   info.products_max_row = static_cast<int64_t>(ht.products_max_row);
@@ -389,40 +516,58 @@ static int build_plan(gm_plan* p, cudaStream_t st) {
   info.rows_empty = static_cast<int64_t>(ht.rows_empty);
   info.rows_light = nA - info.rows_heavy - info.rows_empty;
   info.nnz_a_heavy = static_cast<int64_t>(ht.nnz_a_heavy);
-  for (int b = 0; b < 8; ++b) info.light_bin_rows[b] = fill[b];
+  for (int c = 0; c < kRowClasses; ++c) {
+    p->class_rows[c] = static_cast<i64>(ht.class_rows[c]);
+    info.light_bin_rows[std::min(c, 7)] += p->class_rows[c];
+  }
+  p->staged_light = static_cast<i64>(ht.staged_light);
+  p->merge_lists = static_cast<int>(ht.merge_max_lists);
+  p->merge_only = p->class_rows[kMergeClass] > 0 && p->class_rows[kMergeClass] + info.rows_empty == nA;
   const i64 nH = info.rows_heavy;
   p->n_seg = info.nnz_a_heavy;
 
+  // ---- light rows: staging area (not when all rows are merged), bins of the hash rows
+  {
+    Arena ar;
+    unsigned char* lv = nullptr;
+    bool hash_rows = false;
+    for (int c = kHashClass0; c < kRowClasses; ++c) hash_rows |= p->class_rows[c] > 0;
+    if (p->staged_light > 0 && !p->merge_only) {
+      ar.add(&p->light_col, static_cast<size_t>(p->staged_light) + 8);
+      ar.add(&lv, (static_cast<size_t>(p->staged_light) + 8) * static_cast<size_t>(p->sv));
+    }
+    if (hash_rows) {
+      ar.add(&p->num_rows, static_cast<size_t>(p->bins.n_bins) * static_cast<size_t>(nA));
+      ar.add(&p->num_fill, 8);
+    }
+    if (ar.bytes) GM_TRY(ar.commit(p, st));
+    p->light_val = lv;
+  }
+
   // ---- heavy rows: lists, prefix sums, segment table
   if (nH > 0) {
-    int64_t *heavy_ip = nullptr, *heavy_nnz = nullptr;
-    GM_TRY(plan_alloc(p, &p->x_heavy, static_cast<size_t>(nH), st));
-    GM_TRY(plan_alloc(p, &heavy_ip, static_cast<size_t>(nH) + 1, st));
-    GM_TRY(plan_alloc(p, &heavy_nnz, static_cast<size_t>(nH) + 1, st));
-    GM_TRY(plan_alloc(p, &p->heavy_base, static_cast<size_t>(nH) + 1, st));
-    GM_TRY(plan_alloc(p, &p->heavy_nz_off, static_cast<size_t>(nH) + 1, st));
-    GM_TRY(plan_alloc(p, &p->seg_off, static_cast<size_t>(p->n_seg) + 1, st));
-    GM_TRY(plan_alloc(p, &p->seg_bstart, static_cast<size_t>(p->n_seg) + 1, st));
-    GM_TRY(plan_alloc(p, &p->seg_j, static_cast<size_t>(p->n_seg) + 1, st));
-    GM_TRY(plan_alloc(p, &p->seg_brow, static_cast<size_t>(p->n_seg) + 1, st));
-    GM_TRY(plan_alloc(p, &p->seg_hrow, static_cast<size_t>(p->n_seg) + 1, st));
-    k1_heavy_scatter<<<grid_for(nA, 256, p->num_sms), 256, 0, st>>>(p->heavy_flag, heavy_pos, p->ip, A.row_ptr, nA,
-                                                                   p->x_heavy, heavy_ip, heavy_nnz);
-    exclusive_scan<i64, i64>(heavy_ip, p->heavy_base, nH, p->scan_tmp, nullptr, nullptr, nullptr, st);
-    exclusive_scan<i64, i64>(heavy_nnz, p->heavy_nz_off, nH, p->scan_tmp, nullptr, nullptr, nullptr, st);
-    k1_heavy_segments<<<grid_for(p->n_seg + 1, 256, p->num_sms, 32), 256, 0, st>>>(
-        p->x_heavy, nH, p->heavy_nz_off, p->heavy_base, A.row_ptr, A.col_idx, p->nz_off, B.row_ptr, p->n_seg, p->seg_off,
-        p->seg_bstart, p->seg_j, p->seg_brow, p->seg_hrow);
-    info.launches += 8;
-    std::vector<int64_t> hb(static_cast<size_t>(nH) + 1);
-    p->x_heavy_host.resize(static_cast<size_t>(nH));
-    GM_CUDA(cudaMemcpyAsync(hb.data(), p->heavy_base, hb.size() * sizeof(int64_t), cudaMemcpyDeviceToHost, st));
-    GM_CUDA(cudaMemcpyAsync(p->x_heavy_host.data(), p->x_heavy, static_cast<size_t>(nH) * sizeof(int32_t),
-                            cudaMemcpyDeviceToHost, st));
-    p->heavy_nz_off_host.resize(static_cast<size_t>(nH) + 1);
-    GM_CUDA(cudaMemcpyAsync(p->heavy_nz_off_host.data(), p->heavy_nz_off, (static_cast<size_t>(nH) + 1) * sizeof(int64_t),
-                            cudaMemcpyDeviceToHost, st));
-    GM_CUDA(cudaStreamSynchronize(st));
+    i64* tmp2 = nullptr;
+    int32_t* seg_len = nullptr;
+    {
+      Arena ar;
+      ar.add(&p->x_heavy, static_cast<size_t>(nH));
+      ar.add(&p->heavy_base, static_cast<size_t>(nH) + 1);
+      ar.add(&p->heavy_nz_off, static_cast<size_t>(nH) + 1);
+      ar.add(&p->seg_off, static_cast<size_t>(p->n_seg) + 1);
+      ar.add(&p->seg_bstart, static_cast<size_t>(p->n_seg) + 1);
+      ar.add(&p->seg_j, static_cast<size_t>(p->n_seg) + 1);
+      ar.add(&p->seg_brow, static_cast<size_t>(p->n_seg) + 1);
+      ar.add(&p->seg_hrow, static_cast<size_t>(p->n_seg) + 1);
+      ar.add(&seg_len, static_cast<size_t>(p->n_seg) + 1);
+      ar.add(&tmp2, static_cast<size_t>(scan_tmp_elems(p->n_seg)));
+      GM_TRY(ar.commit(p, st));
+    }
+    k1_heavy_lists<<<static_cast<unsigned>((nA + kHeavyRows - 1) / kHeavyRows), kHeavyThreads, 0, st>>>(
+        p->ip, p->heavy_flag, A.row_ptr, nA, tiles, p->x_heavy, p->heavy_base, p->heavy_nz_off);
+    k1_heavy_segments<<<grid_for(p->n_seg, 256, p->num_sms, 32), 256, 0, st>>>(
+        p->x_heavy, nH, p->heavy_nz_off, A.row_ptr, A.col_idx, B.row_ptr, p->n_seg, seg_len, p->seg_bstart, p->seg_j,
+        p->seg_brow, p->seg_hrow);
+    info.launches += 2 + exclusive_scan<int32_t, i64>(seg_len, p->seg_off, p->n_seg, tmp2, nullptr, nullptr, nullptr, st);
 
     // The expansion writes the first level's children itself (see gm_k4_direct.cuh) unless asked to run that
     // level as separate histogram and multisplit passes.
@@ -452,9 +597,7 @@ static int build_plan(gm_plan* p, cudaStream_t st) {
     // 2^29 took 7 % off the step), at least 2^29 products, at most what 32-bit tile positions allow.
     i64 stage = p->opts.stage_elems;
     if (stage <= 0) {
-      size_t free_b = 0, total_b = 0;
-      GM_CUDA(cudaMemGetInfo(&free_b, &total_b));
-      stage = std::max<i64>(i64{1} << 29, static_cast<i64>(total_b / 5) / (static_cast<i64>(n_buf) * (4 + p->sv)));
+      stage = std::max<i64>(i64{1} << 29, static_cast<i64>(facts.total_mem / 5) / (static_cast<i64>(n_buf) * (4 + p->sv)));
       stage = std::max(stage, info.products_max_row);  // a row is never split
     }
     stage = std::min(stage, info.products_heavy);
@@ -463,7 +606,20 @@ static int build_plan(gm_plan* p, cudaStream_t st) {
     if (info.products_max_row > stage)
       return fail(GM_ERR_CAPACITY, "a heavy row has " + std::to_string(info.products_max_row) +
                                        " products, more than one staging half-buffer holds (" + std::to_string(stage) + ")");
-    if (!cut_batches(hb.data(), nH, stage, &p->batches)) return fail(GM_ERR_CAPACITY, "batch cutting failed");
+    if (stage >= info.products_heavy) {  // everything at once: nothing to cut, the lists stay on the device
+      p->batches.push_back(Batch{0, nH, 0, info.products_heavy});
+    } else {
+      std::vector<int64_t> hb(static_cast<size_t>(nH) + 1);
+      p->x_heavy_host.resize(static_cast<size_t>(nH));
+      p->heavy_nz_off_host.resize(static_cast<size_t>(nH) + 1);
+      GM_CUDA(cudaMemcpyAsync(hb.data(), p->heavy_base, hb.size() * sizeof(int64_t), cudaMemcpyDeviceToHost, st));
+      GM_CUDA(cudaMemcpyAsync(p->x_heavy_host.data(), p->x_heavy, static_cast<size_t>(nH) * sizeof(int32_t),
+                              cudaMemcpyDeviceToHost, st));
+      GM_CUDA(cudaMemcpyAsync(p->heavy_nz_off_host.data(), p->heavy_nz_off, (static_cast<size_t>(nH) + 1) * sizeof(int64_t),
+                              cudaMemcpyDeviceToHost, st));
+      GM_CUDA(cudaStreamSynchronize(st));
+      if (!cut_batches(hb.data(), nH, stage, &p->batches)) return fail(GM_ERR_CAPACITY, "batch cutting failed");
+    }
     info.n_batches = static_cast<int64_t>(p->batches.size());
     info.stage_elems = 0;
     for (const Batch& b : p->batches) {
@@ -479,61 +635,57 @@ static int build_plan(gm_plan* p, cudaStream_t st) {
       p->stage_val[i] = v;
     }
     const size_t n_chunks_max = static_cast<size_t>(p->max_batch_rows) * static_cast<size_t>(prm.chunks_required);
-    GM_TRY(plan_alloc(p, &p->level_off[0], n_chunks_max + 1, st));
+    Arena ar;
+    ar.add(&p->level_off[0], n_chunks_max + 1);
     if (prm.n_levels > 0) {
-      GM_TRY(plan_alloc(p, &p->counts, n_chunks_max + 1, st));
-      GM_TRY(plan_alloc(p, &p->cursor, n_chunks_max + 1, st));
-      GM_TRY(plan_alloc(p, &p->level_off[1], n_chunks_max + 1, st));
+      ar.add(&p->counts, n_chunks_max + 1);
+      ar.add(&p->cursor, n_chunks_max + 1);
+      ar.add(&p->level_off[1], n_chunks_max + 1);
     }
-    GM_TRY(plan_alloc(p, &p->chunk_nnz, n_chunks_max + 1, st));
-    GM_TRY(plan_alloc(p, &p->chunk_nnz_off, n_chunks_max + 1, st));
-    GM_TRY(plan_alloc(p, &p->chunk_base, n_chunks_max + 1, st));
-    GM_TRY(plan_alloc(p, &p->mid_list, n_chunks_max + 1, st));
-    GM_TRY(plan_alloc(p, &p->big_list, n_chunks_max + 1, st));
-    GM_TRY(plan_alloc(p, &p->acc_counters, 8, st));
+    ar.add(&p->chunk_nnz, n_chunks_max + 1);
+    ar.add(&p->chunk_nnz_off, n_chunks_max + 1);
+    ar.add(&p->chunk_base, n_chunks_max + 1);
+    ar.add(&p->mid_list, n_chunks_max + 1);
+    ar.add(&p->big_list, n_chunks_max + 1);
+    ar.add(&p->acc_counters, 8);
     if (p->exit_max >= 0) {
-      GM_TRY(plan_alloc(p, &p->exit_tag[0], n_chunks_max + 1, st));
-      GM_TRY(plan_alloc(p, &p->exit_tag[1], n_chunks_max + 1, st));
-      GM_TRY(plan_alloc(p, &p->parent_tag, n_chunks_max + 1, st));
+      ar.add(&p->exit_tag[0], n_chunks_max + 1);
+      ar.add(&p->exit_tag[1], n_chunks_max + 1);
+      ar.add(&p->parent_tag, n_chunks_max + 1);
     }
     const size_t n_tiles_max = static_cast<size_t>(info.stage_elems) / std::min({kExpandTile, kSplitTile, kGatherTile, kDirectTileSmall}) + 2;
-    GM_TRY(plan_alloc(p, &p->tile_meta, n_tiles_max, st));
-    GM_TRY(plan_alloc(p, &p->row_meta, n_tiles_max, st));
+    ar.add(&p->tile_meta, n_tiles_max);
+    ar.add(&p->row_meta, n_tiles_max);
+    i64 max_seg_b = 0;
+    for (const Batch& b : p->batches) max_seg_b = std::max(max_seg_b, seg_begin(p, b.h1) - seg_begin(p, b.h0));
     if (p->direct) {
-      const int F0 = prm.fanout[0];
-      i64 max_seg_b = 0;
-      for (const Batch& b : p->batches)
-        max_seg_b = std::max(max_seg_b, p->heavy_nz_off_host[static_cast<size_t>(b.h1)] - p->heavy_nz_off_host[static_cast<size_t>(b.h0)]);
-      GM_TRY(plan_alloc(p, &p->child_bound, static_cast<size_t>(B.n_rows) * static_cast<size_t>(F0 + 1) + 1, st));
-      GM_TRY(plan_alloc(p, &p->seg_prefix, (static_cast<size_t>(max_seg_b) + 1) * static_cast<size_t>(F0), st));
-      GM_TRY(plan_alloc(p, &p->seg_h, (static_cast<size_t>(max_seg_b) + 1) * static_cast<size_t>(F0), st));
-      GM_TRY(plan_alloc(p, &p->seg_tile_sums, (static_cast<size_t>(max_seg_b) / kGTile + 2) * static_cast<size_t>(F0), st));
-      if (p->stream)
-        GM_TRY(plan_alloc(p, &p->seg_rec, (static_cast<size_t>(max_seg_b) + 1) * static_cast<size_t>(stream_rec_words(F0)), st));
-      if (B.n_rows > 0) {
-        k_child_bounds<<<grid_for(B.n_rows * (F0 + 1), 256, p->num_sms, 32), 256, 0, st>>>(B.row_ptr, B.col_idx, B.n_rows, F0,
-                                                                                        prm.shift[0], p->child_bound);
-        ++info.launches;
-      }
+      const size_t F0 = static_cast<size_t>(prm.fanout[0]);
+      ar.add(&p->child_bound, static_cast<size_t>(B.n_rows) * (F0 + 1) + 1);
+      ar.add(&p->seg_prefix, (static_cast<size_t>(max_seg_b) + 1) * F0);
+      ar.add(&p->seg_h, (static_cast<size_t>(max_seg_b) + 1) * F0);
+      ar.add(&p->seg_tile_sums, (static_cast<size_t>(max_seg_b) / kGTile + 2) * F0);
+      if (p->stream) ar.add(&p->seg_rec, (static_cast<size_t>(max_seg_b) + 1) * static_cast<size_t>(stream_rec_words(prm.fanout[0])));
     }
     i64 csc_scan_len = 0;
     if (p->csc) {
-      i64 max_seg_b = 0;
-      for (const Batch& b : p->batches)
-        max_seg_b = std::max(max_seg_b, p->heavy_nz_off_host[static_cast<size_t>(b.h1)] - p->heavy_nz_off_host[static_cast<size_t>(b.h0)]);
-      GM_TRY(plan_alloc(p, &p->csc_cnt, static_cast<size_t>(B.n_rows) + 1, st));
-      GM_TRY(plan_alloc(p, &p->csc_ptr, static_cast<size_t>(B.n_rows) + 2, st));
-      GM_TRY(plan_alloc(p, &p->csc_cursor, static_cast<size_t>(B.n_rows) + 2, st));
-      GM_TRY(plan_alloc(p, &p->csc_perm, static_cast<size_t>(max_seg_b) + 1, st));
-      GM_TRY(plan_alloc(p, &p->csc_len, static_cast<size_t>(max_seg_b) + 1, st));
-      GM_TRY(plan_alloc(p, &p->csc_off, static_cast<size_t>(max_seg_b) + 2, st));
+      ar.add(&p->csc_cnt, static_cast<size_t>(B.n_rows) + 1);
+      ar.add(&p->csc_ptr, static_cast<size_t>(B.n_rows) + 2);
+      ar.add(&p->csc_cursor, static_cast<size_t>(B.n_rows) + 2);
+      ar.add(&p->csc_perm, static_cast<size_t>(max_seg_b) + 1);
+      ar.add(&p->csc_len, static_cast<size_t>(max_seg_b) + 1);
+      ar.add(&p->csc_off, static_cast<size_t>(max_seg_b) + 2);
       csc_scan_len = std::max<i64>(B.n_rows, max_seg_b);
     }
-    int64_t* tmp2 = nullptr;  // the per-batch scans can be longer than the ones above
-    GM_TRY(plan_alloc(p, &tmp2, static_cast<size_t>(scan_tmp_elems(std::max<i64>({static_cast<i64>(n_chunks_max), nnzA, nA, csc_scan_len, 1}))), st));
-    p->scan_tmp = tmp2;
+    // the per-batch scans can be longer than the ones above
+    ar.add(&p->scan_tmp, static_cast<size_t>(scan_tmp_elems(std::max<i64>({static_cast<i64>(n_chunks_max), nA, csc_scan_len, 1}))));
+    GM_TRY(ar.commit(p, st));
+    if (p->direct && B.n_rows > 0) {
+      k_child_bounds<<<grid_for(B.n_rows * (prm.fanout[0] + 1), 256, p->num_sms, 32), 256, 0, st>>>(
+          B.row_ptr, B.col_idx, B.n_rows, prm.fanout[0], prm.shift[0], p->child_bound);
+      ++info.launches;
+    }
+    GM_CUDA(cudaStreamSynchronize(st));
   }
-  GM_CUDA(cudaStreamSynchronize(st));
   return GM_OK;
 }
 
@@ -541,42 +693,140 @@ static int build_plan(gm_plan* p, cudaStream_t st) {
 // execute
 // ------------------------------------------------------------------------------------------------
 template <typename V, bool NUMERIC, int G, int LPN, int BT>
-static int launch_light_one(gm_plan* p, const int32_t* rows, const int* n_rows_dev, i64 n_rows_upper, int slots, int cap,
-                            const i64* c_row_ptr, int32_t* c_col, V* c_val, i64 c_capacity, cudaStream_t st) {
+static int launch_hash_one(gm_plan* p, const int32_t* rows, i64 n_rows, const int* n_rows_dev, int slots, int cap,
+                           const i64* c_row_ptr, int32_t* c_col, V* c_val, i64 c_capacity, cudaStream_t st) {
   constexpr int kGroups = BT / G;
   const size_t smem = kGroups * light_group_bytes<V, NUMERIC>(slots, cap, G);
   auto kern = k3_light_rows<V, G, LPN, BT, NUMERIC>;
   // (static shared memory counts towards the 48 KB that need no opt-in)
   if (smem > 32 * 1024) GM_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)));
-  const unsigned grid = grid_for(n_rows_upper, kGroups, p->num_sms, 2048 / BT * 4);
+  const unsigned grid = grid_for(n_rows, kGroups, p->num_sms, 2048 / BT * 4);
   kern<<<grid, BT, smem, st>>>(p->A.row_ptr, p->A.col_idx, static_cast<const V*>(p->A.vals), p->B.row_ptr, p->B.col_idx,
-                               static_cast<const V*>(p->B.vals), rows, n_rows_dev, slots, cap, p->row_nnz, c_row_ptr, c_col,
-                               c_val, c_capacity, p->err);
+                               static_cast<const V*>(p->B.vals), rows, static_cast<int>(n_rows), n_rows_dev, slots, cap, p->row_nnz,
+                               c_row_ptr, c_col, c_val, c_capacity, p->err);
   ++p->stats.launches;
   GM_CUDA(cudaGetLastError());
   return GM_OK;
 }
 
+// The hash accumulator's two passes (rows above kSortMaxProducts products).  Symbolic: the classes of the row analysis;
+// numeric: the same rows binned again by their entry counts (n_rows: an upper bound, n_rows_dev: the bin's fill).
 template <typename V, bool NUMERIC>
-static int launch_light(gm_plan* p, const int32_t* rows_all, const int* fill_dev, const i64* rows_upper,
-                        const i64* c_row_ptr, int32_t* c_col, V* c_val, i64 c_capacity, cudaStream_t st) {
-  const i64 stride = std::max<i64>(p->A.n_rows, 1);
-  for (int b = 0; b < p->bins.n_bins; ++b) {
-    if (rows_upper[b] <= 0) continue;
-    const int cap = p->bins.cap[b], slots = p->bin_slots[b];
-    const int32_t* rows = rows_all + static_cast<size_t>(b) * stride;
-    const int* nd = fill_dev + b;
-    const i64 up = rows_upper[b];
-#define GM_LIGHT(G, LPN, BT) launch_light_one<V, NUMERIC, G, LPN, BT>(p, rows, nd, up, slots, cap, c_row_ptr, c_col, c_val, c_capacity, st)
-    int rc;
-    if (cap <= 16) rc = GM_LIGHT(8, 1, 256);
-    else if (cap <= 64) rc = GM_LIGHT(32, 4, 256);
-    else if (cap <= 256) rc = GM_LIGHT(128, 8, 128);
-    else if (cap <= 1024) rc = GM_LIGHT(256, 16, 256);
-    else if (cap <= 4096) rc = GM_LIGHT(512, 32, 512);
-    else rc = GM_LIGHT(1024, 32, 1024);
+static int launch_hash(gm_plan* p, int cap, int slots, const int32_t* rows, i64 n_rows, const int* n_rows_dev,
+                       const i64* c_row_ptr, int32_t* c_col, V* c_val, i64 c_capacity, cudaStream_t st) {
+#define GM_LIGHT(G, LPN, BT) \
+  launch_hash_one<V, NUMERIC, G, LPN, BT>(p, rows, n_rows, n_rows_dev, slots, cap, c_row_ptr, c_col, c_val, c_capacity, st)
+  if (cap <= 16) return GM_LIGHT(8, 1, 256);
+  if (cap <= 64) return GM_LIGHT(32, 4, 256);
+  if (cap <= 256) return GM_LIGHT(128, 8, 128);
+  if (cap <= 1024) return GM_LIGHT(256, 16, 256);
+  if (cap <= 4096) return GM_LIGHT(512, 32, 512);
+  return GM_LIGHT(1024, 32, 1024);
 #undef GM_LIGHT
-    GM_TRY(rc);
+}
+
+// One thread per row: count, write to C, or write to the staging area.
+template <typename V, int MODE>
+static int launch_merge(gm_plan* p, const int32_t* rows, i64 n_rows, const i64* c_row_ptr, int32_t* out_col, V* out_val,
+                        cudaStream_t st) {
+  const unsigned grid = static_cast<unsigned>((n_rows + kMergeThreads - 1) / kMergeThreads);
+  // Entries for C are collected in shared memory, but the rows of B that neighbouring rows share want to stay in L1: with
+  // 60 % of it as shared memory the 1024^2 grid's numeric pass takes 95 us, with all of it (more blocks per SM) 127, with 30 % 108.
+#define GM_MERGE(NL)                                                                                                       \
+  do {                                                                                                                     \
+    auto kern = k3_merge_rows<V, NL, MODE>;                                                                                \
+    if (MODE == kMergeToC) GM_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 60));        \
+    kern<<<grid, kMergeThreads, 0, st>>>(p->A.row_ptr, p->A.col_idx, static_cast<const V*>(p->A.vals), p->B.row_ptr,       \
+                                         p->B.col_idx, static_cast<const V*>(p->B.vals), rows, n_rows, p->light_off,       \
+                                         p->row_nnz, c_row_ptr, out_col, out_val);                                         \
+  } while (0)
+  if (p->merge_lists <= 2) GM_MERGE(2);
+  else if (p->merge_lists <= 4) GM_MERGE(4);
+  else if (p->merge_lists <= 5) GM_MERGE(5);
+  else GM_MERGE(kMergeMaxLists);
+#undef GM_MERGE
+  ++p->stats.launches;
+  GM_CUDA(cudaGetLastError());
+  return GM_OK;
+}
+
+template <typename V, typename Key, int KMAX>
+static int launch_sort_one(gm_plan* p, const SortLists& lists, i64 n, cudaStream_t st) {
+  const unsigned grid = grid_for(n, kSortWarps, p->num_sms, KMAX > 4 ? 16 : 24);
+  k3_sort_rows<V, Key, KMAX><<<grid, kSortWarps * 32, 0, st>>>(
+      p->A.row_ptr, p->A.col_idx, static_cast<const V*>(p->A.vals), p->B.row_ptr, p->B.col_idx,
+      static_cast<const V*>(p->B.vals), lists, p->light_off, p->row_nnz, p->light_col, static_cast<V*>(p->light_val));
+  ++p->stats.launches;
+  GM_CUDA(cudaGetLastError());
+  return GM_OK;
+}
+
+// Light rows, everything that does not need C: merged and sorted rows go to the staging area (when every row is merged
+// they are only counted), hash rows are counted.
+template <typename V>
+static int light_front(gm_plan* p, cudaStream_t st) {
+  const i64 stride = p->A.n_rows;
+  auto list = [&](int c) { return p->class_list + static_cast<i64>(c) * stride; };
+  if (p->merge_only)
+    return launch_merge<V, kMergeCount>(p, nullptr, p->A.n_rows, nullptr, nullptr, nullptr, st);
+  if (p->class_rows[kMergeClass] > 0)
+    GM_TRY((launch_merge<V, kMergeToStage>(p, list(kMergeClass), p->class_rows[kMergeClass], nullptr, p->light_col,
+                                           static_cast<V*>(p->light_val), st)));
+  // a key packs a product's column with its position in the row: 32 bits unless the matrix is very wide
+  int col_bits = 1;
+  while (col_bits < 31 && (i64{1} << col_bits) < p->B.n_cols) ++col_bits;
+  {
+    SortLists l{};
+    i64 n = 0;
+    for (int i = 0; i < 2; ++i) { const int c = kSortClass0 + 4 - i; l.rows[i] = list(c); l.n[i] = p->class_rows[c]; n += l.n[i]; }
+    const int pos_bits = l.n[0] > 0 ? 9 : 8;
+    if (n > 0 && col_bits + pos_bits <= 32) GM_TRY((launch_sort_one<V, u32, 16>(p, l, n, st)));
+    else if (n > 0) GM_TRY((launch_sort_one<V, u64, 16>(p, l, n, st)));
+  }
+  {
+    SortLists l{};
+    i64 n = 0;
+    for (int i = 0; i < 3; ++i) { const int c = kSortClass0 + 2 - i; l.rows[i] = list(c); l.n[i] = p->class_rows[c]; n += l.n[i]; }
+    if (n > 0 && col_bits + 7 <= 32) GM_TRY((launch_sort_one<V, u32, 4>(p, l, n, st)));
+    else if (n > 0) GM_TRY((launch_sort_one<V, u64, 4>(p, l, n, st)));
+  }
+  for (int c = kHashClass0; c < kHashClass0 + p->rules.n_hash; ++c) {
+    if (p->class_rows[c] <= 0) continue;
+    const int cap = p->rules.hash_cap[c - kHashClass0];
+    const int slots = cap == p->bins.cap[p->bins.n_bins - 1] ? p->bin_slots[p->bins.n_bins - 1] : 2 * cap;
+    GM_TRY((launch_hash<V, false>(p, cap, slots, list(c), p->class_rows[c], nullptr, nullptr, nullptr, nullptr, 0, st)));
+  }
+  return GM_OK;
+}
+
+// Light rows [r0, r1) into C, once C.row_ptr covers them.
+template <typename V>
+static int light_back(gm_plan* p, i64 r0, i64 r1, const i64* c_row_ptr, int32_t* c_col, V* c_val, i64 capacity, cudaStream_t st) {
+  if (p->info.rows_light <= 0 || r1 <= r0) return GM_OK;
+  if (p->merge_only) return launch_merge<V, kMergeToC>(p, nullptr, p->A.n_rows, c_row_ptr, c_col, c_val, st);
+  if (p->staged_light > 0) {
+    i64 n_staged = 0;
+    for (int c = 0; c < kHashClass0; ++c) n_staged += p->class_rows[c];
+    const i64 avg = p->staged_light / n_staged;
+#define GM_COPY(LPR)                                                                                                     \
+  k3_copy_rows<V, LPR><<<static_cast<unsigned>(((r1 - r0) * LPR + 255) / 256), 256, 0, st>>>(                             \
+      p->light_col, static_cast<const V*>(p->light_val), p->light_off, r0, r1, c_row_ptr, c_col, c_val, capacity, p->err)
+    if (avg <= 16) GM_COPY(8);
+    else GM_COPY(32);
+#undef GM_COPY
+    ++p->stats.launches;
+    GM_CUDA(cudaGetLastError());
+  }
+  if (p->num_rows) {
+    GM_CUDA(cudaMemsetAsync(p->num_fill, 0, 8 * sizeof(int), st));
+    k1_bin_rows<<<static_cast<unsigned>((r1 - r0 + 255) / 256), 256, 0, st>>>(
+        p->row_nnz, p->heavy_flag, p->light_off, r0, r1 - r0, p->bins, p->A.n_rows, p->num_fill, p->num_rows);
+    ++p->stats.launches;
+    i64 upper = 0;  // a row's numeric bin is never above its class
+    for (int c = kHashClass0; c < kRowClasses; ++c) upper += p->class_rows[c];
+    for (int b = 0; b < p->bins.n_bins; ++b)
+      GM_TRY((launch_hash<V, true>(p, p->bins.cap[b], p->bin_slots[b], p->num_rows + static_cast<i64>(b) * p->A.n_rows, upper,
+                                   p->num_fill + b, c_row_ptr, c_col, c_val, capacity, st)));
   }
   return GM_OK;
 }
@@ -722,8 +972,8 @@ static int heavy_batch_front(gm_plan* p, const Batch& b, HeavyBatchState<V>* hs,
   if (p->direct) {
     // ---- run starts of every (segment, child) from counts alone, then the products straight into the children
     const int F = prm.fanout[0];
-    const i64 seg0 = p->heavy_nz_off_host[static_cast<size_t>(b.h0)];
-    const i64 n_seg_b = p->heavy_nz_off_host[static_cast<size_t>(b.h1)] - seg0;
+    const i64 seg0 = seg_begin(p, b.h0);
+    const i64 n_seg_b = seg_begin(p, b.h1) - seg0;
     const i64 n_gt = (n_seg_b + kGTile - 1) / kGTile;
     const i64 n_child = rows_b * F;
     const unsigned ggrid = static_cast<unsigned>((n_gt + (256 / F) - 1) / (256 / F));
@@ -736,12 +986,11 @@ static int heavy_batch_front(gm_plan* p, const Batch& b, HeavyBatchState<V>* hs,
     p->stats.launches += 4;
     tm.end(st);
     tm.begin(PhaseTimes::kScan, st);
-    exclusive_scan<u32, i64>(p->counts, off_nxt, n_child, p->scan_tmp, nullptr, nullptr, nullptr, st);
+    p->stats.launches += 1 + exclusive_scan<u32, i64>(p->counts, off_nxt, n_child, p->scan_tmp, nullptr, nullptr, nullptr, st);
     // (the cursor array of the multisplit is free in this mode: it holds R)
     u32* const row_base = reinterpret_cast<u32*>(p->cursor);
     k_g_row_base<<<grid_for(n_child, 256, p->num_sms, 32), 256, 0, st>>>(p->seg_prefix, p->heavy_nz_off + b.h0, seg0, rows_b, F,
                                                                         off_nxt, row_base);
-    p->stats.launches += 4;
     tm.end(st);
     tm.begin(PhaseTimes::kExpand, st);
     if (p->stream) {
@@ -790,8 +1039,8 @@ static int heavy_batch_front(gm_plan* p, const Batch& b, HeavyBatchState<V>* hs,
     // ---- outer-product order: masked CSR -> CSC of the batch's segments (counting sort by row of B), then the
     // expansion walks the product space in that order
     tm.begin(PhaseTimes::kExpand, st);
-    const i64 seg0 = p->heavy_nz_off_host[static_cast<size_t>(b.h0)];
-    const i64 n_seg_b = p->heavy_nz_off_host[static_cast<size_t>(b.h1)] - seg0;
+    const i64 seg0 = seg_begin(p, b.h0);
+    const i64 n_seg_b = seg_begin(p, b.h1) - seg0;
     const i64 nB = p->B.n_rows;
     GM_CUDA(cudaMemsetAsync(p->csc_cnt, 0, static_cast<size_t>(nB + 1) * sizeof(int32_t), st));
     k_csc_count<<<grid_for(n_seg_b, 256, p->num_sms, 16), 256, 0, st>>>(p->seg_brow, seg0, n_seg_b, p->csc_cnt);
@@ -880,8 +1129,8 @@ static int heavy_batch_front(gm_plan* p, const Batch& b, HeavyBatchState<V>* hs,
     }
     tm.end(st);
     tm.begin(PhaseTimes::kScan, st);
-    exclusive_scan<u32, i64>(p->counts, off_nxt, n_child, p->scan_tmp, nullptr, nullptr, reinterpret_cast<i64*>(p->cursor), st);
-    p->stats.launches += 3;
+    p->stats.launches +=
+        exclusive_scan<u32, i64>(p->counts, off_nxt, n_child, p->scan_tmp, nullptr, nullptr, reinterpret_cast<i64*>(p->cursor), st);
     tm.end(st);
     tm.begin(PhaseTimes::kSplit, st);
     // the counts of this level have been scanned: the array is free to receive the next level's
@@ -930,10 +1179,10 @@ static int heavy_batch_front(gm_plan* p, const Batch& b, HeavyBatchState<V>* hs,
 
   GM_TRY((launch_accumulate<V>(p, b, *hs, st)));  // (records its own two phases)
   tm.begin(PhaseTimes::kScan, st);
-  exclusive_scan<u32, i64>(p->chunk_nnz, p->chunk_nnz_off, hs->n_chunks, p->scan_tmp, nullptr, nullptr, nullptr, st);
+  p->stats.launches +=
+      1 + exclusive_scan<u32, i64>(p->chunk_nnz, p->chunk_nnz_off, hs->n_chunks, p->scan_tmp, nullptr, nullptr, nullptr, st);
   k_heavy_row_counts<<<grid_for(rows_b, 256, p->num_sms), 256, 0, st>>>(p->chunk_nnz_off, hs->log2_cpr, rows_b, p->x_heavy,
                                                                         b.h0, p->row_nnz, p->c_total + 1);
-  p->stats.launches += 4;
   tm.end(st);
   return GM_OK;
 }
@@ -961,9 +1210,10 @@ static int execute_t(gm_plan* p, cudaStream_t st, gm_csr* C) {
   cudaEvent_t ev_total0 = nullptr, ev_total1 = nullptr;
   if (tm.enabled) { ev_total0 = tm.get(); ev_total1 = tm.get(); cudaEventRecord(ev_total0, st); }
 
-  GM_CUDA(cudaMemsetAsync(p->err, 0, sizeof(int), st));
-  GM_CUDA(cudaMemsetAsync(p->row_nnz, 0, static_cast<size_t>(nA + 1) * sizeof(int32_t), st));
-  GM_CUDA(cudaMemsetAsync(p->c_total, 0, 16 * sizeof(int64_t), st));
+  HostSlot* const slot = p->slot;
+  slot->err[0] = 0;  // (nothing of this plan is in flight: every execute ends with a synchronisation)
+  slot->c_total = 0;
+  if (info.rows_heavy > 0) GM_CUDA(cudaMemsetAsync(p->c_total, 0, 16 * sizeof(int64_t), st));
 
   // ---- result row_ptr
   i64* c_row_ptr = static_cast<i64*>(dev_alloc(static_cast<size_t>(nA + 1) * sizeof(i64), st));
@@ -974,24 +1224,12 @@ static int execute_t(gm_plan* p, cudaStream_t st, gm_csr* C) {
   // stream, forked from and joined back into the caller's with events (never when single_stream is set)
   bool fork = !p->opts.single_stream && info.rows_light > 0 && info.rows_heavy > 0;
   if (fork && !p->light_stream) {
-    // one second stream per device for the life of the process (creating and destroying a stream per plan cost more
-    // than the overlap gained on millisecond products); executes that share it are ordered by their own events
-    static cudaStream_t side_streams[64] = {nullptr};
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) {
+    p->light_stream = side_stream();
+    if (!p->light_stream || cudaEventCreateWithFlags(&p->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
+        cudaEventCreateWithFlags(&p->ev_light, cudaEventDisableTiming) != cudaSuccess) {
+      cudaGetLastError();
+      p->light_stream = nullptr;
       fork = false;
-    } else {
-      if (!side_streams[dev] && cudaStreamCreateWithFlags(&side_streams[dev], cudaStreamNonBlocking) != cudaSuccess) {
-        cudaGetLastError();
-        side_streams[dev] = nullptr;
-      }
-      p->light_stream = side_streams[dev];
-      if (!p->light_stream || cudaEventCreateWithFlags(&p->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
-          cudaEventCreateWithFlags(&p->ev_light, cudaEventDisableTiming) != cudaSuccess) {
-        cudaGetLastError();
-        p->light_stream = nullptr;
-        fork = false;
-      }
     }
   }
   cudaStream_t lst = fork ? p->light_stream : st;
@@ -1006,38 +1244,22 @@ static int execute_t(gm_plan* p, cudaStream_t st, gm_csr* C) {
   };
 #define GM_TRY_C(expr) do { int rc2_ = (expr); if (rc2_ != GM_OK) { cudaStreamSynchronize(st); cleanup(); return rc2_; } } while (0)
 
-  // ---- light rows, symbolic (Algorithm 3: Symbolic(A[x_light,:], B))
+  // ---- light rows, all that does not need C (Algorithm 3: Symbolic(A[x_light,:], B), and for most rows the sums too)
   fork_light();
   tm.begin(PhaseTimes::kLightSym, lst);
-  GM_TRY_C((launch_light<V, false>(p, p->sym_rows, p->sym_fill, info.light_bin_rows, nullptr, nullptr, nullptr, 0, lst)));
+  GM_TRY_C(light_front<V>(p, lst));
   tm.end(lst);
   bool light_counted = !fork;  // the heavy path joins before the first prefix sum over the per-row counts
-
-  // a row's numeric bin is never above its symbolic bin
-  i64 num_upper[kMaxLightBins] = {0};
-  {
-    i64 run = 0;
-    for (int b = p->bins.n_bins - 1; b >= 0; --b) { run += info.light_bin_rows[b]; num_upper[b] = run; }
-  }
-  // numeric pass of the light rows in [r0, r1) (all of them by default)
-  auto light_numeric_range = [&](i64 capacity, i64 r0, i64 r1, cudaStream_t s2) -> int {
+  auto light_rows_to_c = [&](i64 cap, i64 r0, i64 r1, cudaStream_t s2) -> int {
     tm.begin(PhaseTimes::kLightNum, s2);
-    if (info.rows_light > 0 && r1 > r0) {
-      GM_CUDA(cudaMemsetAsync(p->num_fill, 0, 8 * sizeof(int), s2));
-      k1_bin_rows<int32_t><<<static_cast<unsigned>((r1 - r0 + 255) / 256), 256, 0, s2>>>(
-          p->row_nnz + r0, p->heavy_flag + r0, r1 - r0, p->bins, std::max<i64>(nA, 1), p->num_fill, p->num_rows, r0);
-      ++p->stats.launches;
-      GM_TRY((launch_light<V, true>(p, p->num_rows, p->num_fill, num_upper, c_row_ptr, c_col, c_val, capacity, s2)));
-    }
+    const int rc = light_back<V>(p, r0, r1, c_row_ptr, c_col, c_val, cap, s2);
     tm.end(s2);
-    return GM_OK;
+    return rc;
   };
-  auto light_numeric = [&](i64 capacity, cudaStream_t s2) -> int { return light_numeric_range(capacity, 0, nA, s2); };
 
   const size_t n_batches = p->batches.size();
   i64 capacity = 0;
   i64 total = 0;
-  i64 heavy_total = 0;
   int dev_err = 0;
   if (n_batches <= 1) {
     // ---- everything is resident at once: count, allocate C exactly, then fill
@@ -1046,26 +1268,26 @@ static int execute_t(gm_plan* p, cudaStream_t st, gm_csr* C) {
     join_light();
     light_counted = true;
     tm.begin(PhaseTimes::kScan, st);
-    exclusive_scan<int32_t, i64>(p->row_nnz, c_row_ptr, nA, p->scan_tmp, nullptr, p->c_total, nullptr, st);
-    p->stats.launches += 3;
+    p->stats.launches += exclusive_scan<int32_t, i64>(p->row_nnz, c_row_ptr, nA, p->scan_tmp, nullptr, nullptr, nullptr, st,
+                                                      reinterpret_cast<i64*>(&slot->c_total));
     tm.end(st);
-    if (cudaMemcpyAsync(&total, p->c_total, sizeof(i64), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-        cudaStreamSynchronize(st) != cudaSuccess) {
+    if (cudaStreamSynchronize(st) != cudaSuccess) {
       cleanup();
       return fail(GM_ERR_CUDA, std::string("symbolic phase failed: ") + cudaGetErrorString(cudaGetLastError()));
     }
+    total = *static_cast<volatile i64*>(&slot->c_total);
     capacity = total;
     c_col = static_cast<int32_t*>(dev_alloc(static_cast<size_t>(std::max<i64>(total, 1)) * sizeof(int32_t), st));
     c_val = static_cast<V*>(dev_alloc(static_cast<size_t>(std::max<i64>(total, 1)) * sizeof(V), st));
     if (!c_col || !c_val) { cleanup(); return fail(GM_ERR_OOM, "allocation of C (" + std::to_string(total) + " entries) failed"); }
-    // the gather of the heavy rows and the numeric pass of the light rows write different rows of C
+    // the heavy and the light rows write different rows of C
     fork_light();
     if (n_batches == 1) {
       tm.begin(PhaseTimes::kAccSym, st);
       GM_TRY_C((launch_gather<V>(p, p->batches[0], hs, c_row_ptr, c_col, c_val, capacity, st)));
       tm.end(st);
     }
-    GM_TRY_C(light_numeric(capacity, lst));
+    GM_TRY_C(light_rows_to_c(capacity, 0, nA, lst));
     join_light();
   } else {
     // ---- heavy rows in several staging-buffer fills: C is appended in row order into reserved room
@@ -1076,25 +1298,30 @@ static int execute_t(gm_plan* p, cudaStream_t st, gm_csr* C) {
     if (p->opts.c_capacity > 0) {
       tries.push_back(p->opts.c_capacity);
     } else {
-      size_t free_b = 0, total_b = 0;
-      GM_CUDA(cudaMemGetInfo(&free_b, &total_b));
+      DeviceFacts facts;
+      GM_TRY_C(device_facts(&facts));
       const i64 entry = static_cast<i64>(4 + sizeof(V));
       const i64 inputs = (A.nnz + (&A == &B ? 0 : B.nnz)) * entry + (A.n_rows + B.n_rows + 2) * 8;
-      const i64 by_total = (static_cast<i64>(total_b) - info.workspace_bytes - inputs - (nA + 1) * 8 - (i64{3} << 30)) / entry;
-      const i64 by_free = (static_cast<i64>(free_b) - (nA + 1) * 8 - (i64{1} << 30)) / entry;
-      const i64 hi = std::max<i64>(1, std::min<i64>(info.c_nnz_upper, std::max(by_total, by_free)));
-      const i64 lo = std::max<i64>(1, std::min<i64>(info.c_nnz_upper, by_free));
-      tries.push_back(hi);
-      for (int k = 1; k <= 8 && hi > lo; ++k) tries.push_back(hi - (hi - lo) * k / 8);
+      const i64 by_total = (static_cast<i64>(facts.total_mem) - info.workspace_bytes - inputs - (nA + 1) * 8 - (i64{3} << 30)) / entry;
+      tries.push_back(std::max<i64>(1, std::min<i64>(info.c_nnz_upper, by_total)));
     }
-    for (i64 cand : tries) {
-      capacity = cand;
+    for (size_t k = 0; k < tries.size(); ++k) {
+      capacity = tries[k];
       c_col = static_cast<int32_t*>(dev_alloc(static_cast<size_t>(capacity) * sizeof(int32_t), st));
       c_val = c_col ? static_cast<V*>(dev_alloc(static_cast<size_t>(capacity) * sizeof(V), st)) : nullptr;
       if (c_col && c_val) break;
       dev_free(c_col, st);
       c_col = nullptr;
       c_val = nullptr;
+      if (k == 0 && p->opts.c_capacity <= 0) {
+        // refused: go down in eight steps to what the device says is free
+        size_t free_b = 0, total_b = 0;
+        if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) { cudaGetLastError(); break; }
+        const i64 by_free = (static_cast<i64>(free_b) - (nA + 1) * 8 - (i64{1} << 30)) / static_cast<i64>(4 + sizeof(V));
+        const i64 hi = std::max(capacity, std::min<i64>(info.c_nnz_upper, by_free));
+        const i64 lo = std::max<i64>(1, std::min<i64>(info.c_nnz_upper, by_free));
+        for (int q = 1; q <= 8 && hi > lo; ++q) tries.push_back(hi - (hi - lo) * q / 8);
+      }
     }
     if (!c_col || !c_val) { cleanup(); return fail(GM_ERR_OOM, "allocation of C (room for " + std::to_string(capacity) + " entries) failed"); }
     for (size_t bi = 0; bi < n_batches; ++bi) {
@@ -1106,8 +1333,8 @@ static int execute_t(gm_plan* p, cudaStream_t st, gm_csr* C) {
       const i64 r0 = bi == 0 ? 0 : p->x_heavy_host[static_cast<size_t>(b.h0)];
       const i64 r1 = bi + 1 == n_batches ? nA : p->x_heavy_host[static_cast<size_t>(p->batches[bi + 1].h0)];
       tm.begin(PhaseTimes::kScan, st);
-      exclusive_scan<int32_t, i64>(p->row_nnz + r0, c_row_ptr + r0, r1 - r0, p->scan_tmp, p->c_total, p->c_total, nullptr, st);
-      p->stats.launches += 3;
+      p->stats.launches += exclusive_scan<int32_t, i64>(p->row_nnz + r0, c_row_ptr + r0, r1 - r0, p->scan_tmp, p->c_total,
+                                                        p->c_total, nullptr, st);
       tm.end(st);
       tm.begin(PhaseTimes::kAccSym, st);
       GM_TRY_C((launch_gather<V>(p, b, hs, c_row_ptr, c_col, c_val, capacity, st)));
@@ -1115,7 +1342,7 @@ static int execute_t(gm_plan* p, cudaStream_t st, gm_csr* C) {
       if (HostSink* sk = p->sink) {
         // The caller wants C on the host: finish rows [r0, r1) now (their light rows too), note how many entries
         // of C that makes, and send the previous batch's entries on their way while this batch computes.
-        GM_TRY_C(light_numeric_range(capacity, r0, r1, st));
+        GM_TRY_C(light_rows_to_c(capacity, r0, r1, st));
         if (sk->events.size() <= bi) {
           cudaEvent_t ev = nullptr;
           if (cudaEventCreateWithFlags(&ev, cudaEventDisableTiming) != cudaSuccess) { cleanup(); return fail(GM_ERR_CUDA, "event creation failed"); }
@@ -1139,23 +1366,19 @@ static int execute_t(gm_plan* p, cudaStream_t st, gm_csr* C) {
         if (bi + 1 == n_batches) send(bi);
       }
     }
-    if (!p->sink) GM_TRY_C(light_numeric(capacity, st));
-    if (cudaMemcpyAsync(&total, p->c_total, sizeof(i64), cudaMemcpyDeviceToHost, st) != cudaSuccess) {
-      cleanup();
-      return fail(GM_ERR_CUDA, "copy of nnz(C) failed");
-    }
+    if (!p->sink) GM_TRY_C(light_rows_to_c(capacity, 0, nA, st));
   }
   if (tm.enabled) cudaEventRecord(ev_total1, st);
-  // heavy entries; products and entries of small chunks; of mid-size chunks; products and chunks that left the
-  // hierarchy early; products the multisplit levels left in place
-  i64 tail_totals[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-  cudaMemcpyAsync(tail_totals, p->c_total + 1, 8 * sizeof(i64), cudaMemcpyDeviceToHost, st);
-  cudaError_t e1 = cudaMemcpyAsync(&dev_err, p->err, sizeof(int), cudaMemcpyDeviceToHost, st);
-  cudaError_t e2 = cudaStreamSynchronize(st);
-  if (e1 != cudaSuccess || e2 != cudaSuccess) {
+  // [0] nnz(C) so far (several batches), [1] heavy entries; products and entries of small chunks; of mid-size chunks;
+  // products and chunks that left the hierarchy early; products the multisplit levels left in place
+  if (n_batches > 0) cudaMemcpyAsync(slot->tail, p->c_total, 9 * sizeof(i64), cudaMemcpyDeviceToHost, st);
+  const cudaError_t e2 = cudaStreamSynchronize(st);
+  if (e2 != cudaSuccess) {
     cleanup();
-    return fail(GM_ERR_CUDA, std::string("execute failed: ") + cudaGetErrorString(e2 != cudaSuccess ? e2 : e1));
+    return fail(GM_ERR_CUDA, std::string("execute failed: ") + cudaGetErrorString(e2));
   }
+  if (n_batches > 1) total = slot->tail[0];
+  dev_err = *static_cast<volatile int*>(&slot->err[0]);
   if (dev_err != kDevOk || total > capacity) {
     cleanup();
     if (dev_err == kDevOk) dev_err = kDevCapacity;
@@ -1163,15 +1386,17 @@ static int execute_t(gm_plan* p, cudaStream_t st, gm_csr* C) {
   }
 #undef GM_TRY_C
   p->stats.c_nnz = total;
-  heavy_total = tail_totals[0];
-  p->stats.c_nnz_heavy = heavy_total;
-  p->stats.small_chunk_products = tail_totals[1];
-  p->stats.small_chunk_entries = tail_totals[2];
-  p->stats.mid_chunk_products = tail_totals[3];
-  p->stats.mid_chunk_entries = tail_totals[4];
-  p->stats.early_exit_products = tail_totals[5];
-  p->stats.early_exit_chunks = tail_totals[6];
-  p->stats.split_products -= tail_totals[7];
+  if (n_batches > 0) {
+    const i64* t = slot->tail;
+    p->stats.c_nnz_heavy = t[1];
+    p->stats.small_chunk_products = t[2];
+    p->stats.small_chunk_entries = t[3];
+    p->stats.mid_chunk_products = t[4];
+    p->stats.mid_chunk_entries = t[5];
+    p->stats.early_exit_products = t[6];
+    p->stats.early_exit_chunks = t[7];
+    p->stats.split_products -= t[8];
+  }
   p->stats.c_capacity = capacity;
   if (tm.enabled) {
     float ph[PhaseTimes::kCount];
@@ -1224,11 +1449,6 @@ int gm_spgemm_plan_ex(const gm_csr* A, const gm_csr* B, size_t smem_bytes, const
   GM_TRY(check_csr_arg(B, "B"));
   if (A->dtype != B->dtype) return fail(GM_ERR_DTYPE, "A and B have different value types");
   if (A->n_cols != B->n_rows) return fail(GM_ERR_DIM_MISMATCH, "A.n_cols != B.n_rows");
-  int n_dev = 0;
-  if (cudaGetDeviceCount(&n_dev) != cudaSuccess || n_dev == 0) {
-    cudaGetLastError();
-    return fail(GM_ERR_CUDA, "no CUDA device: this library has no CPU path");
-  }
   gm_plan* p = new gm_plan();
   p->A = *A;
   p->B = *B;
@@ -1299,6 +1519,7 @@ void gm_plan_destroy(gm_plan* plan) {
   if (plan->ev_fork) cudaEventDestroy(plan->ev_fork);
   if (plan->ev_light) cudaEventDestroy(plan->ev_light);
   for (auto& b : plan->owned) dev_free(b.p, plan->plan_stream);
+  give_slot(plan->slot);
   delete plan;
 }
 
@@ -1424,26 +1645,6 @@ namespace gm {
 
 constexpr i64 kNoAllocMaxNnz = GM_NOALLOC_MAX_NNZ_A;
 
-// Scratch of the no-allocation entry point, part of the library image on every device that loads it.
-// In host code this name is only a handle for cudaGetSymbolAddress, not a device address.
-struct NoAllocScratch {
-  i64 nz_off[kNoAllocMaxNnz + 8];                    // prefix sums of the products per stored entry of A
-  i64 scan_tmp[kNoAllocMaxNnz / kScanTile + 8];      // tile sums of the prefix sum
-  int32_t nz_len[kNoAllocMaxNnz + 8];                // products per stored entry of A
-};
-static __device__ __align__(256) NoAllocScratch g_noalloc_scratch;
-
-__global__ void k1_row_products_only(const i64* __restrict__ a_row_ptr, i64 n_rows, const i64* __restrict__ nz_off,
-                                     i64* __restrict__ ip) {
-  for (i64 i = static_cast<i64>(blockIdx.x) * blockDim.x + threadIdx.x; i < n_rows;
-       i += static_cast<i64>(gridDim.x) * blockDim.x)
-    ip[i] = nz_off[a_row_ptr[i + 1]] - nz_off[a_row_ptr[i]];
-}
-
-constexpr int kNoAllocMaxDevices = 64;
-static NoAllocScratch* g_noalloc_ptr[kNoAllocMaxDevices] = {nullptr};
-static int g_noalloc_sms[kNoAllocMaxDevices] = {0};
-
 }  // namespace gm
 
 extern "C" int gm_row_products_noalloc(const gm_csr* A, const gm_csr* B, int64_t* ip_out_device, void* cuda_stream) {
@@ -1453,30 +1654,18 @@ extern "C" int gm_row_products_noalloc(const gm_csr* A, const gm_csr* B, int64_t
   if (A->n_cols != B->n_rows) return fail(GM_ERR_DIM_MISMATCH, "A.n_cols != B.n_rows");
   if (A->nnz > kNoAllocMaxNnz)
     return fail(GM_ERR_CAPACITY, "gm_row_products_noalloc handles at most " + std::to_string(kNoAllocMaxNnz) +
-                                     " stored entries of A (got " + std::to_string(A->nnz) + "): its scratch is a fixed array");
-  int dev = 0;
-  GM_CUDA(cudaGetDevice(&dev));
-  if (dev < 0 || dev >= kNoAllocMaxDevices) return fail(GM_ERR_INVALID_ARG, "device index out of range");
-  if (!g_noalloc_ptr[dev]) {
-    // set-up, once per device, with that device current: the device address behind the symbol
-    void* ptr = nullptr;
-    GM_CUDA(cudaGetSymbolAddress(&ptr, g_noalloc_scratch));
-    int sms = 0;
-    GM_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    g_noalloc_sms[dev] = sms;
-    g_noalloc_ptr[dev] = static_cast<NoAllocScratch*>(ptr);
-  }
-  NoAllocScratch* sc = g_noalloc_ptr[dev];
-  const int sms = g_noalloc_sms[dev];
+                                     " stored entries of A (got " + std::to_string(A->nnz) + ")");
+  DeviceFacts facts;
+  GM_TRY(device_facts(&facts));
+  if (A->n_rows == 0) return GM_OK;
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-  // scratch members are addressed through the device pointer, never through the host-side symbol
-  int32_t* nz_len = reinterpret_cast<int32_t*>(reinterpret_cast<char*>(sc) + offsetof(NoAllocScratch, nz_len));
-  i64* nz_off = reinterpret_cast<i64*>(reinterpret_cast<char*>(sc) + offsetof(NoAllocScratch, nz_off));
-  i64* scan_tmp = reinterpret_cast<i64*>(reinterpret_cast<char*>(sc) + offsetof(NoAllocScratch, scan_tmp));
-  if (A->nnz > 0) k1_nz_len<<<grid_for(A->nnz, 256, sms, 32), 256, 0, st>>>(A->col_idx, A->nnz, B->row_ptr, nz_len);
-  exclusive_scan<int32_t, i64>(nz_len, nz_off, A->nnz, scan_tmp, nullptr, nullptr, nullptr, st);
-  if (A->n_rows > 0)
-    k1_row_products_only<<<grid_for(A->n_rows, 256, sms), 256, 0, st>>>(A->row_ptr, A->n_rows, nz_off, ip_out_device);
+  const int T = k1_tile_items(A->n_rows, A->nnz, facts.num_sms);
+  const unsigned grid = static_cast<unsigned>((A->n_rows + A->nnz + T - 1) / T);
+  const bool wide = B->n_cols > (i64{1} << 24);
+  auto kern = T == kK1Small ? (wide ? k1_row_products_only<kK1Small, i64> : k1_row_products_only<kK1Small, u32>)
+                            : (wide ? k1_row_products_only<kK1Large, i64> : k1_row_products_only<kK1Large, u32>);
+  GM_CUDA(cudaMemsetAsync(ip_out_device, 0, static_cast<size_t>(A->n_rows) * sizeof(int64_t), st));
+  kern<<<grid, kK1Threads, 0, st>>>(A->row_ptr, A->col_idx, A->n_rows, A->nnz, B->row_ptr, ip_out_device);
   GM_CUDA(cudaGetLastError());
   return GM_OK;
 }

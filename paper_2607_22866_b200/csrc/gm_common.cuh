@@ -20,7 +20,12 @@ enum DevError : int {
   kDevTimeout = 4,       // a bounded wait on an asynchronous copy gave up
 };
 
-__device__ __forceinline__ void dev_set_error(int* flag, int code) { atomicCAS(flag, 0, code); }
+// The flag lies in page-locked host memory (plain accesses only: atomics over PCIe are not a given); the first problem
+// stays, unless two blocks meet theirs at the same moment.
+__device__ __forceinline__ void dev_set_error(int* flag, int code) {
+  volatile int* f = flag;
+  if (*f == 0) *f = code;
+}
 
 __device__ __forceinline__ u32 lanemask_lt() {
   u32 m;

@@ -55,7 +55,8 @@ template <typename V, int G, int LPN, int BT, bool NUMERIC>
 __global__ void __launch_bounds__(BT) k3_light_rows(
     const i64* __restrict__ a_row_ptr, const int32_t* __restrict__ a_col, const V* __restrict__ a_val,
     const i64* __restrict__ b_row_ptr, const int32_t* __restrict__ b_col, const V* __restrict__ b_val,
-    const int32_t* __restrict__ rows, const int* __restrict__ n_rows_ptr, int slots, int cap,
+    const int32_t* __restrict__ rows, int n_rows_host, const int* __restrict__ n_rows_ptr,  // n_rows_ptr: when only the device knows
+    int slots, int cap,
     int32_t* __restrict__ row_nnz,                         // symbolic: out
     const i64* __restrict__ c_row_ptr, int32_t* __restrict__ c_col, V* __restrict__ c_val, i64 c_capacity,  // numeric
     int* __restrict__ err) {
@@ -69,7 +70,7 @@ __global__ void __launch_bounds__(BT) k3_light_rows(
   int32_t* keys = reinterpret_cast<int32_t*>(base + (NUMERIC ? static_cast<size_t>(cap) * 8 + static_cast<size_t>(slots) * sizeof(V) : 0));
   __shared__ int s_count[kGroups];
 
-  const int n_rows = *n_rows_ptr;
+  const int n_rows = n_rows_ptr ? *n_rows_ptr : n_rows_host;
   for (int ri = blockIdx.x * kGroups + gid; ri < n_rows; ri += gridDim.x * kGroups) {
     const int row = rows[ri];
     for (int s = t; s < slots; s += G) {

@@ -1,0 +1,298 @@
+// K3r — light rows of few products: merged by one thread or sorted by one warp (Algorithm 1 with a sorted accumulator
+// instead of a hash table; Section III-E sorts a row after hashing it).
+//
+//   k3_merge_rows  one thread per row of C: a merge of at most eight (sorted) rows of B.  The heads of the lists live in
+//                  registers, every step takes the smallest column and advances all lists that show it.  Nothing is
+//                  shared between lanes, so a step costs the instruction stream a few instructions per list for 32
+//                  rows at once.
+//   k3_sort_rows   one warp per row, up to 512 products: the products' (column, position) keys are sorted in registers
+//                  (see warp_sort_keys), runs of equal columns are added up in the original order.
+//
+// Both replace the hash accumulator for these sizes.  What bound that one was not memory: a group of lanes cleared a
+// table, inserted with compare-and-swap, compacted the table and sorted the entries with a barrier per step, and did the
+// first two twice (symbolic, numeric).
+//
+// Rows either go to the staging area of the light rows at light_off[row], from where k3_copy_rows moves them once
+// C.row_ptr is known (one pass over the products, and the entries are written twice), or, when every row of the matrix
+// is merged, they are counted first and then written to their place in C: a second merge is cheaper than the copy.
+#pragma once
+#include "gm_common.cuh"
+#include "gm_k1_analysis.cuh"
+#include "gm_sort.cuh"
+
+namespace gm {
+
+// ------------------------------------------------------------------------------------------------------------------
+// merge
+// ------------------------------------------------------------------------------------------------------------------
+constexpr int kMergeThreads = 128;
+constexpr int kMergeStageEntries = 2048;  // entries of C one block collects in shared memory before it writes them out
+
+enum MergeMode { kMergeCount = 0, kMergeToC = 1, kMergeToStage = 2 };
+
+// One row.  emit(i, column, sum) for the row's i-th entry; returns the number of entries.
+template <typename V, int NL, bool NUMERIC, typename Emit>
+__device__ __forceinline__ int merge_row(i64 s, i64 e, const int32_t* __restrict__ a_col, const V* __restrict__ a_val,
+                                         const i64* __restrict__ b_row_ptr, const int32_t* __restrict__ b_col,
+                                         const V* __restrict__ b_val, Emit emit) {
+  i64 base[NL];
+  int at[NL], len[NL];
+  int32_t head[NL];
+  V hv[NL], av[NL];  // (a head's value is loaded with its column: one latency per step, not two)
+#pragma unroll
+  for (int l = 0; l < NL; ++l) {
+    base[l] = 0; at[l] = 0; len[l] = 0; av[l] = V(0); hv[l] = V(0);
+    if (s + l < e) {
+      const int32_t k = a_col[s + l];
+      base[l] = b_row_ptr[k];
+      len[l] = static_cast<int>(b_row_ptr[k + 1] - base[l]);
+      if (NUMERIC) av[l] = a_val[s + l];
+    }
+  }
+#pragma unroll
+  for (int l = 0; l < NL; ++l) {
+    head[l] = INT_MAX;
+    if (len[l] > 0) {
+      head[l] = b_col[base[l]];
+      if (NUMERIC) hv[l] = b_val[base[l]];
+    }
+  }
+  int n = 0;
+  for (;;) {
+    int32_t m = head[0];
+#pragma unroll
+    for (int l = 1; l < NL; ++l) m = min(m, head[l]);
+    if (m == INT_MAX) break;  // (columns are below INT_MAX: n_cols <= INT_MAX)
+    V sum = V(0);
+#pragma unroll
+    for (int l = 0; l < NL; ++l) {
+      if (head[l] == m) {
+        if (NUMERIC) sum += av[l] * hv[l];
+        ++at[l];
+        head[l] = INT_MAX;
+        if (at[l] < len[l]) {
+          head[l] = b_col[base[l] + at[l]];
+          if (NUMERIC) hv[l] = b_val[base[l] + at[l]];
+        }
+      }
+    }
+    emit(n, m, sum);
+    ++n;
+  }
+  return n;
+}
+
+// MODE kMergeCount / kMergeToC: rows 0 .. n_rows - 1 in order; kMergeToStage: the rows of a list.
+template <typename V, int NL, int MODE>
+__global__ void __launch_bounds__(kMergeThreads) k3_merge_rows(
+    const i64* __restrict__ a_row_ptr, const int32_t* __restrict__ a_col, const V* __restrict__ a_val,
+    const i64* __restrict__ b_row_ptr, const int32_t* __restrict__ b_col, const V* __restrict__ b_val,
+    const int32_t* __restrict__ rows, i64 n_rows, const i64* __restrict__ light_off, int32_t* __restrict__ row_nnz,
+    const i64* __restrict__ c_row_ptr, int32_t* __restrict__ out_col, V* __restrict__ out_val) {
+  const i64 i = static_cast<i64>(blockIdx.x) * kMergeThreads + threadIdx.x;
+  if constexpr (MODE == kMergeToC) {
+    // the block's rows are consecutive, and so are their entries in C: collected in shared memory, written in one run
+    // (a thread writing its own entries would touch one sector per lane and store)
+    __shared__ int32_t s_col[kMergeStageEntries];
+    __shared__ V s_val[kMergeStageEntries];
+    const i64 r0 = static_cast<i64>(blockIdx.x) * kMergeThreads;
+    const i64 r1 = min(n_rows, r0 + kMergeThreads);
+    const i64 c0 = c_row_ptr[r0];
+    const i64 n_out = c_row_ptr[r1] - c0;
+    if (n_out <= kMergeStageEntries) {
+      if (i < n_rows) {
+        const int at = static_cast<int>(c_row_ptr[i] - c0);
+        merge_row<V, NL, true>(a_row_ptr[i], a_row_ptr[i + 1], a_col, a_val, b_row_ptr, b_col, b_val, [&](int q, int32_t c, V v) {
+          s_col[at + q] = c;
+          s_val[at + q] = v;
+        });
+      }
+      __syncthreads();
+      for (int q = threadIdx.x; q < static_cast<int>(n_out); q += kMergeThreads) {
+        out_col[c0 + q] = s_col[q];
+        out_val[c0 + q] = s_val[q];
+      }
+    } else if (i < n_rows) {
+      const i64 at = c_row_ptr[i];
+      merge_row<V, NL, true>(a_row_ptr[i], a_row_ptr[i + 1], a_col, a_val, b_row_ptr, b_col, b_val, [&](int q, int32_t c, V v) {
+        out_col[at + q] = c;
+        out_val[at + q] = v;
+      });
+    }
+  } else if (i < n_rows) {
+    const i64 row = MODE == kMergeToStage ? static_cast<i64>(rows[i]) : i;
+    const i64 at = MODE == kMergeToStage ? light_off[row] : 0;
+    const int n = merge_row<V, NL, MODE == kMergeToStage>(
+        a_row_ptr[row], a_row_ptr[row + 1], a_col, a_val, b_row_ptr, b_col, b_val, [&](int q, int32_t c, V v) {
+          if constexpr (MODE == kMergeToStage) {
+            out_col[at + q] = c;
+            out_val[at + q] = v;
+          }
+        });
+    row_nnz[row] = n;
+  }
+}
+
+// ------------------------------------------------------------------------------------------------------------------
+// sort
+// ------------------------------------------------------------------------------------------------------------------
+constexpr int kSortWarps = 4;
+
+// Lists of the classes one launch handles, longest rows first.
+struct SortLists {
+  const int32_t* rows[kSortClasses];
+  i64 n[kSortClasses];
+};
+
+template <typename V, typename Key, int KMAX>
+struct SortSmem {
+  i64 base[32];   // per (non-empty) row of B of the current 32 entries of A: its start minus its first product
+  V a[32];
+  V val[32 * KMAX];
+  Key key[32 * KMAX];
+};
+
+// The products of A[s..e) into sm.key / sm.val; returns how many.
+template <typename V, typename Key, int K, int KMAX>
+__device__ __forceinline__ int gather_row(i64 s, i64 e, const int32_t* __restrict__ a_col, const V* __restrict__ a_val,
+                                          const i64* __restrict__ b_row_ptr, const int32_t* __restrict__ b_col,
+                                          const V* __restrict__ b_val, SortSmem<V, Key, KMAX>& sm) {
+  constexpr int kPosBits = 5 + (K == 1 ? 0 : K == 2 ? 1 : K == 4 ? 2 : K == 8 ? 3 : 4);
+  constexpr int U = K >= 4 ? 4 : K;  // windows of 32 products in flight
+  const int lane = threadIdx.x & 31;
+  int done = 0;
+  for (i64 j0 = s; j0 < e; j0 += 32) {
+    const i64 j = j0 + lane;
+    i64 b0 = 0;
+    int len = 0;
+    V av = V(0);
+    if (j < e) {
+      const int32_t k = a_col[j];
+      av = a_val[j];
+      b0 = b_row_ptr[k];
+      len = static_cast<int>(b_row_ptr[k + 1] - b0);
+    }
+    const u32 some = __ballot_sync(0xffffffffu, len > 0);
+    const int inc = warp_inclusive_scan(len);
+    const int ex = inc - len;
+    const int total = __shfl_sync(0xffffffffu, inc, 31);
+    if (len > 0) {
+      const int p = __popc(some & lanemask_lt());
+      sm.base[p] = b0 - ex;
+      sm.a[p] = av;
+    }
+    __syncwarp();
+    int started = 0;  // rows of B that start before the window
+    for (int f0 = 0; f0 < total; f0 += 32 * U) {
+      int32_t c[U];
+      V v[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        // which row of B a product belongs to: the rows that start inside the window, as a bit mask over its positions
+        const int w = ex - (f0 + u * 32);
+        const u32 heads = __reduce_or_sync(0xffffffffu, (len > 0 && w >= 0 && w < 32) ? 1u << w : 0u);
+        const int f = f0 + u * 32 + lane;
+        if (f < total) {
+          const int q = started + __popc(heads & (lanemask_lt() | (1u << lane))) - 1;
+          const i64 src = sm.base[q] + f;
+          c[u] = b_col[src];
+          v[u] = b_val[src] * sm.a[q];
+        }
+        started += __popc(heads);
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int f = f0 + u * 32 + lane;
+        if (f < total) {
+          sm.key[done + f] = (static_cast<Key>(static_cast<u32>(c[u])) << kPosBits) | static_cast<Key>(done + f);
+          sm.val[done + f] = v[u];
+        }
+      }
+    }
+    done += total;
+    __syncwarp();
+  }
+  return done;
+}
+
+template <typename V, typename Key, int K, int KMAX>
+__device__ __forceinline__ void sort_row(i64 row, const i64* __restrict__ a_row_ptr, const int32_t* __restrict__ a_col,
+                                         const V* __restrict__ a_val, const i64* __restrict__ b_row_ptr,
+                                         const int32_t* __restrict__ b_col, const V* __restrict__ b_val,
+                                         const i64* __restrict__ light_off, int32_t* __restrict__ row_nnz,
+                                         int32_t* __restrict__ out_col, V* __restrict__ out_val, SortSmem<V, Key, KMAX>& sm) {
+  constexpr int kPosBits = 5 + (K == 1 ? 0 : K == 2 ? 1 : K == 4 ? 2 : K == 8 ? 3 : 4);
+  const int lane = threadIdx.x & 31;
+  const i64 at = light_off[row];
+  const int n = gather_row<V, Key, K, KMAX>(a_row_ptr[row], a_row_ptr[row + 1], a_col, a_val, b_row_ptr, b_col, b_val, sm);
+  Key key[K];
+#pragma unroll
+  for (int r = 0; r < K; ++r) {
+    const int q = r * 32 + lane;
+    key[r] = q < n ? sm.key[q] : ~Key(0);  // padding sorts to the end
+  }
+  __syncwarp();
+  warp_sort_keys<Key, K>(key, lane);
+  const int m = warp_sum_runs<V, Key, K, kPosBits>(key, n, sm.key, sm.val, 0u, out_col + at, out_val + at);
+  if (lane == 0) row_nnz[row] = m;
+  __syncwarp();  // the warp's shared memory is reused by its next row
+}
+
+// Warps take rows in list order; SortLists holds the classes K = KMAX, KMAX / 2, ... (n = 0: no such rows).
+template <typename V, typename Key, int KMAX>
+__global__ void __launch_bounds__(kSortWarps * 32, KMAX > 4 ? 8 : 12) k3_sort_rows(
+    const i64* __restrict__ a_row_ptr, const int32_t* __restrict__ a_col, const V* __restrict__ a_val,
+    const i64* __restrict__ b_row_ptr, const int32_t* __restrict__ b_col, const V* __restrict__ b_val, SortLists lists,
+    const i64* __restrict__ light_off, int32_t* __restrict__ row_nnz, int32_t* __restrict__ out_col, V* __restrict__ out_val) {
+  __shared__ SortSmem<V, Key, KMAX> s_sm[kSortWarps];
+  SortSmem<V, Key, KMAX>& sm = s_sm[threadIdx.x >> 5];
+  const i64 n_warps = static_cast<i64>(gridDim.x) * kSortWarps;
+  const i64 w0 = static_cast<i64>(blockIdx.x) * kSortWarps + (threadIdx.x >> 5);
+  i64 before = 0;
+#define GM_SORT_CLASS(I, K)                                                                                                   \
+  if constexpr (K <= KMAX) {                                                                                                  \
+    /* the warps go on round-robin from one class to the next */                                                              \
+    for (i64 q = ((w0 - before) % n_warps + n_warps) % n_warps; q < lists.n[I]; q += n_warps)                                  \
+      sort_row<V, Key, K, KMAX>(lists.rows[I][q], a_row_ptr, a_col, a_val, b_row_ptr, b_col, b_val, light_off, row_nnz, out_col, \
+                                out_val, sm);                                                                                 \
+    before += lists.n[I];                                                                                                     \
+  }
+  if constexpr (KMAX > 4) {
+    GM_SORT_CLASS(0, 16)
+    GM_SORT_CLASS(1, 8)
+  } else {
+    GM_SORT_CLASS(0, 4)
+    GM_SORT_CLASS(1, 2)
+    GM_SORT_CLASS(2, 1)
+  }
+#undef GM_SORT_CLASS
+}
+
+// ------------------------------------------------------------------------------------------------------------------
+// staged rows -> C
+// ------------------------------------------------------------------------------------------------------------------
+// LPR lanes per row of [r0, r1).
+template <typename V, int LPR>
+__global__ void __launch_bounds__(256) k3_copy_rows(const int32_t* __restrict__ s_col, const V* __restrict__ s_val,
+                                                    const i64* __restrict__ light_off, i64 r0, i64 r1,
+                                                    const i64* __restrict__ c_row_ptr, int32_t* __restrict__ c_col,
+                                                    V* __restrict__ c_val, i64 c_capacity, int* __restrict__ err) {
+  const i64 row = r0 + (static_cast<i64>(blockIdx.x) * 256 + threadIdx.x) / LPR;
+  const int l = threadIdx.x % LPR;
+  if (row >= r1) return;
+  const i64 src = light_off[row];
+  if (src < 0) return;
+  const i64 dst = c_row_ptr[row];
+  const int n = static_cast<int>(c_row_ptr[row + 1] - dst);
+  if (dst + n > c_capacity) {
+    if (l == 0) dev_set_error(err, kDevCapacity);
+    return;
+  }
+#pragma unroll 4
+  for (int q = l; q < n; q += LPR) {
+    c_col[dst + q] = s_col[src + q];
+    c_val[dst + q] = s_val[src + q];
+  }
+}
+
+}  // namespace gm

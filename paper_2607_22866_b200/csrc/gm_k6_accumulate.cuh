@@ -28,6 +28,7 @@
 // small one shares the chunk table out statically; nothing waits on anything but block-wide barriers.
 #pragma once
 #include "gm_common.cuh"
+#include "gm_sort.cuh"
 
 namespace gm {
 
@@ -145,57 +146,6 @@ constexpr int kSmallWarps = 4;            // warps per block of the small-chunk 
 // 44.0 / 43.6 / 41.6.
 constexpr int kSmallBlocksPerSm = 8;
 
-// Sorts 32 * K packed keys, K per lane, element e = r * 32 + lane in key[r]; ascending in e afterwards.
-// Steps whose partner sits in another lane are the same instruction sequence for every step width, so they run
-// as loops over the width; only the steps that pair registers are unrolled.  (Fully unrolled, the networks of
-// all K together did not fit the instruction cache, and the warps of a block run different K.)
-template <int K>
-__device__ __forceinline__ void warp_sort_keys(u32 (&key)[K], int lane) {
-  auto lane_step = [&](int mask, bool lower) {  // partner: same register, lane ^ mask; the lower lane keeps the smaller key
-#pragma unroll
-    for (int r = 0; r < K; ++r) {
-      const u32 o = __shfl_xor_sync(0xffffffffu, key[r], mask);
-      key[r] = lower ? min(key[r], o) : max(key[r], o);
-    }
-  };
-  // merges inside one register row (k = 2 .. 32): first step partner e ^ (k - 1), then e ^ j for j = k/4 .. 1
-#pragma unroll 1
-  for (int k = 2; k <= 32; k <<= 1) {
-    lane_step(k - 1, (lane & (k >> 1)) == 0);
-#pragma unroll 1
-    for (int j = k >> 2; j > 0; j >>= 1) lane_step(j, (lane & j) == 0);
-  }
-  // merges across register rows (k = 64 .. 32 K)
-#pragma unroll
-  for (int k = 64; k <= 32 * K; k <<= 1) {
-    const int rm = k / 32 - 1;  // first step: partner register r ^ rm, partner lane lane ^ 31
-#pragma unroll
-    for (int r = 0; r < K; ++r) {
-      if ((r ^ rm) > r) {
-        const u32 a = key[r], b = key[r ^ rm];
-        const u32 oa = __shfl_xor_sync(0xffffffffu, b, 31);
-        const u32 ob = __shfl_xor_sync(0xffffffffu, a, 31);
-        key[r] = min(a, oa);
-        key[r ^ rm] = max(b, ob);
-      }
-    }
-#pragma unroll
-    for (int j = k >> 2; j >= 32; j >>= 1) {  // partner in the same lane
-      const int rj = j / 32;
-#pragma unroll
-      for (int r = 0; r < K; ++r) {
-        if ((r & rj) == 0) {
-          const u32 a = key[r], b = key[r | rj];
-          key[r] = min(a, b);
-          key[r | rj] = max(a, b);
-        }
-      }
-    }
-#pragma unroll 1
-    for (int j = 16; j > 0; j >>= 1) lane_step(j, (lane & j) == 0);
-  }
-}
-
 // One small chunk by one warp.  s_key / s_val: 32 * K entries of this warp's shared memory.
 template <typename V, int K>
 __device__ __forceinline__ int small_chunk(int32_t* col, V* val, int n, u32 wmask, u32* s_key, V* s_val,
@@ -215,33 +165,8 @@ __device__ __forceinline__ int small_chunk(int32_t* col, V* val, int n, u32 wmas
     }
   }
   const u32 col_base = static_cast<u32>(__shfl_sync(0xffffffffu, c_first, 0)) & ~wmask;
-  warp_sort_keys<K>(key, lane);
-#pragma unroll
-  for (int r = 0; r < K; ++r) s_key[r * 32 + lane] = key[r];
-  __syncwarp();
-  // runs of equal columns: the lane that owns a run's first element adds the run up and writes it
-  int base = 0;
-#pragma unroll
-  for (int r = 0; r < K; ++r) {
-    if (r * 32 < n) {  // warp-uniform
-      const int e = r * 32 + lane;
-      const u32 c = key[r] >> kSmallIdxBits;
-      const bool head = e < n && (e == 0 || (s_key[e - 1] >> kSmallIdxBits) != c);
-      const u32 heads = __ballot_sync(0xffffffffu, head);
-      if (head) {
-        V sum = s_val[key[r] & ((1u << kSmallIdxBits) - 1u)];
-        for (int q = e + 1; q < n; ++q) {
-          const u32 kq = s_key[q];
-          if ((kq >> kSmallIdxBits) != c) break;
-          sum += s_val[kq & ((1u << kSmallIdxBits) - 1u)];
-        }
-        const int p = base + __popc(heads & lanemask_lt());
-        col[p] = static_cast<int32_t>(col_base | c);
-        val[p] = sum;
-      }
-      base += __popc(heads);
-    }
-  }
+  warp_sort_keys<u32, K>(key, lane);
+  const int base = warp_sum_runs<V, u32, K, kSmallIdxBits>(key, n, s_key, s_val, col_base, col, val);
   if (lane == 0) *nnz_out = static_cast<u32>(base);
   __syncwarp();  // the warp's shared memory is reused by its next chunk
   return base;

@@ -1,0 +1,67 @@
+"""Row analysis and light rows at the sizes where their kernels change hands: tiles of entries and rows, widths of the
+one-warp sort, the merge of few short rows.  Against the oracle, with its tolerance (tau * sum|a*b|)."""
+import numpy as np
+import pytest
+import torch
+
+import gen
+import oracle
+from helpers import random_csr
+from parity import check_product
+
+pytestmark = pytest.mark.gpu
+
+
+def _csr(row_lists, n_cols, rng, dtype):
+    rp = np.zeros(len(row_lists) + 1, np.int64)
+    np.cumsum([len(r) for r in row_lists], out=rp[1:])
+    col = np.concatenate([np.sort(np.asarray(r, np.int32)) for r in row_lists] + [np.zeros(0, np.int32)]).astype(np.int32)
+    return gen.CSR(len(row_lists), n_cols, rp, col, rng.uniform(-1, 1, col.size).astype(dtype))
+
+
+@pytest.mark.parametrize("dtype", [np.float32, np.float64])
+@pytest.mark.parametrize("n_cols", [700, 1 << 21, (1 << 23) + 5, (1 << 27) + 1])  # 32-bit and 64-bit sort keys
+def test_sorted_rows_around_every_width(dtype, n_cols):
+    # row r of B has 2**r entries from some 600 columns, so that columns repeat; rows of A spell their product counts in binary
+    rng = np.random.default_rng(n_cols % 1000)
+    pool = np.unique(np.concatenate([[0, n_cols - 1], rng.choice(n_cols, 600, replace=False) if n_cols < 1000 else rng.integers(0, n_cols, 600)]))
+    B = _csr([rng.choice(pool, 1 << r, replace=False) for r in range(10)] + [[]], n_cols, rng, dtype)
+    sizes = [0, 1, 2, 31, 32, 33, 63, 64, 65, 127, 128, 129, 255, 256, 257, 511, 512, 513, 800, 1023]
+    A = _csr([[r for r in range(10) if n >> r & 1] + [10] for n in sizes] * 3, 11, rng, dtype)
+    C, info, stats = check_product(A, B, tau=700)  # sort, hash and heavy rows
+    assert info.rows_heavy == 6
+    check_product(A, B, tau=8)
+
+
+@pytest.mark.parametrize("dtype", [np.float32, np.float64])
+@pytest.mark.parametrize("lists", [1, 2, 4, 5, 8])
+def test_merged_rows(dtype, lists):
+    # enough rows for one thread each; alone in the matrix (counted, then written to C) and next to longer rows (staged)
+    rng = np.random.default_rng(lists)
+    n, m = (1 << 16) + 77, 5000
+    B = _csr([rng.choice(40 + 7 * i % 4000, int(rng.integers(0, 9)), replace=False) for i in range(3000)], m, rng, dtype)
+    rows = [rng.choice(3000, int(k), replace=False) for k in rng.integers(0, lists + 1, n)]
+    A = _csr(rows, 3000, rng, dtype)
+    C, info, stats = check_product(A, B)
+    assert info.rows_heavy == 0
+    rows[5], rows[n - 1] = np.arange(40), np.arange(300)
+    check_product(_csr(rows, 3000, rng, dtype), B, tau=400)
+
+
+def test_rows_of_every_length_across_tiles():
+    # a hub row over many tiles, runs of empty rows longer than a tile, rows that end exactly at a tile's edge
+    import paper_2607_22866_b200 as gm
+    rng = np.random.default_rng(4)
+    B = random_csr(rng, 6000, 900, 0.01, np.float32)
+    for lengths in ([6000, 0, 0, 5000, 1], [0] * 5000 + [1] + [0] * 5000, [511, 1, 0, 512, 1023, 0] * 40, [3] * 400 + [2045, 2048, 2047] * 90):
+        A = _csr([rng.choice(6000, k, replace=False) for k in lengths], 6000, rng, np.float32)
+        dA, dB = gm.DeviceCSR.from_host(A), gm.DeviceCSR.from_host(B)
+        ref = oracle.row_products(A, B)
+        plan = gm.spgemm_plan(dA, dB)
+        assert np.array_equal(plan.row_products().cpu().numpy(), ref)
+        info = plan.info()
+        assert info.products_total == ref.sum() and info.rows_empty == int((ref == 0).sum()) and info.rows_heavy == int((ref > info.params.tau).sum())
+        assert info.nnz_a_heavy == int(np.asarray(lengths)[ref > info.params.tau].sum())
+        out = torch.full((A.n_rows,), -1, dtype=torch.int64, device="cuda")
+        assert np.array_equal(gm.row_products_noalloc(dA, dB, out).cpu().numpy(), ref)
+    check_product(A, B)
