@@ -20,6 +20,7 @@
 #include "gm_k4_csc.cuh"
 #include "gm_k5_multisplit.cuh"
 #include "gm_k6_accumulate.cuh"
+#include "gm_k6_tasks.cuh"
 #include "gm_k7_gather.cuh"
 #include "gm_planner.h"
 #include "gm_scan.cuh"
@@ -159,6 +160,7 @@ struct HostSlot {
   int err[4];            // [0] first device-side problem of an execute, [1] malformed input
   u64 totals[kK1Words];  // K1Totals
   i64 c_total;           // nnz(C)
+  i64 n_tasks;           // tasks of the heavy rows
   i64 tail[16];          // copy of gm_plan::c_total
 };
 constexpr int kHostSlotBytes = 512;
@@ -313,6 +315,22 @@ struct gm_plan {
   int* acc_counters = nullptr;     // list lengths and tickets (see k6_classify)
   gm::TileMeta* row_meta = nullptr;   // per tile of the expansion kernel: heavy rows it touches (fused histogram)
   gm::TileMeta* tile_meta = nullptr;  // per tile of the expansion / multisplit kernels: groups it touches
+  // heavy rows as tasks (see gm_k6_tasks.cuh): no staged products, no levels
+  bool use_tasks = false;
+  gm::TaskRules task_rules{};
+  int acc_width = 0, acc_threads = 0;
+  gm::u32* piece_bound = nullptr;  // n_rows(B) x (granules + 1)
+  gm::u64* longest_row = nullptr;
+  gm::u32* part_cols = nullptr;    // granules x (kMaxParts + 1)
+  gm::u32* granule_counts = nullptr;
+  gm::u32* row_tasks = nullptr;    // nH
+  int64_t* row_task_off = nullptr; // nH + 1
+  std::vector<int64_t> task_begin; // per batch (and the end): first task
+  gm::HeavyTask* tasks = nullptr;
+  int64_t* task_off = nullptr;     // place of a task in the staging area
+  int32_t* task_list[3]{};         // small, mid, big
+  int* task_counters = nullptr;    // 8 per batch
+  int* task_tickets = nullptr;     // 4 per batch
   gm::PhaseTimes times;
   HostSink* sink = nullptr;        // set by gm_spgemm_host for the duration of one execute
   // light rows run next to the heavy path on a stream of the plan's own (Algorithm 3 keeps separate queues for them)
@@ -320,6 +338,9 @@ struct gm_plan {
   cudaEvent_t ev_fork = nullptr, ev_light = nullptr;
 };
 
+#ifndef GM_MID_MIN_TASK_BLOCKS
+#define GM_MID_MIN_TASK_BLOCKS 5
+#endif
 #ifndef GM_MID_MIN_BLOCKS
 #define GM_MID_MIN_BLOCKS 7
 #endif
@@ -404,6 +425,116 @@ static int launch_row_analysis(gm_plan* p, K1Totals* totals, HeavyTile* tiles, u
                             : (wide ? k1_rows<kK1Large, i64> : k1_rows<kK1Large, u32>);
   kern<<<grid, kK1Threads, 0, st>>>(A.row_ptr, A.col_idx, A.n_rows, A.nnz, p->B.row_ptr, p->rules, p->ip, parts, p->heavy_flag,
                                     p->row_nnz, p->light_off, p->class_list, A.n_rows, tiles, totals, p->slot->totals);
+  GM_CUDA(cudaGetLastError());
+  return GM_OK;
+}
+
+// Sizes of the heavy rows' tasks; false: they do not fit (then the rows go through the staged products).
+static bool plan_task_rules(gm_plan* p) {
+  const gm_params& prm = p->info.params;
+  const gm_plan_opts& o = p->opts;
+  if (p->B.nnz >= (i64{1} << 32) || p->B.n_rows == 0) return false;  // piece boundaries are 32-bit positions in B's arrays
+  // two accumulators per SM unless another number was asked for: one block's flush overlaps the other's sums (measured
+  // with staged products, R-MAT scale 20: 41.0 against 59.5 ms for the same chunks)
+  const int ctas = prm.acc_ctas_per_sm == 1 ? 2 : prm.acc_ctas_per_sm;
+  const int bt = 1024 / ctas;
+  const size_t budget = p->smem_bytes / static_cast<size_t>(ctas) - 1024;
+  i64 w = prm.chunk_width;
+  auto smem = [&](i64 width) { return p->sv == 4 ? big_task_smem_bytes<float>(static_cast<int>(width), bt) : big_task_smem_bytes<double>(static_cast<int>(width), bt); };
+  while (w > 32 && smem(w) > budget) w /= 2;
+  if (smem(w) > budget) return false;
+  const i64 granules = (prm.chunk_width / w) * prm.chunks_required;
+  if (granules > 512) return false;
+  p->acc_width = static_cast<int>(w);
+  p->acc_threads = bt;
+  TaskRules& r = p->task_rules;
+  r.granules = static_cast<int>(granules);
+  r.log2_g = ilog2_floor(static_cast<uint64_t>(w));
+  r.small_max = p->small_max;
+  r.small_width = 1u << 22;  // a sort key packs the column inside the task with a position of at most nine bits
+  const i64 span = static_cast<i64>(pow2_ceil(static_cast<uint64_t>(std::max<i64>(p->B.n_cols, 32))));
+  r.mid_width = static_cast<u32>(std::max<i64>(w, std::min<i64>(32768, span)));
+  int mid = o.mid_chunk_max < 0 ? 0 : (o.mid_chunk_max ? o.mid_chunk_max : (p->sv == 4 ? 4096 : 2048));
+  const size_t fixed = (p->sv == 4 ? sizeof(Pieces<float, kMidThreads * kMidPerThread>) : sizeof(Pieces<double, kMidThreads * kMidPerThread>)) + 2048;
+  while (mid > r.small_max && mid_task_smem_bytes(static_cast<int>(r.mid_width), p->sv, mid) + fixed > p->smem_bytes / GM_MID_MIN_TASK_BLOCKS) mid /= 2;
+  r.mid_max = std::max(mid, r.small_max);
+  // A hub row's granule is cut when it would keep a block busy for longer than an eighth of its even share of the whole.
+  r.split_above = static_cast<u32>(std::min<i64>(1u << 30, std::max<i64>(std::max<i64>(1 << 15, w), p->info.products_heavy / (static_cast<i64>(p->num_sms) * ctas * 8))));
+  r.max_parts = kMaxParts;
+  return true;
+}
+
+// Tasks of the heavy rows: piece boundaries of B, products per row and granule, ranges, lists.
+static int plan_tasks(gm_plan* p, cudaStream_t st) {
+  const gm_csr& A = p->A;
+  const gm_csr& B = p->B;
+  const TaskRules& r = p->task_rules;
+  const i64 nH = p->info.rows_heavy;
+  const size_t n_batches = p->batches.size();
+  u32* n_long = nullptr;
+  int32_t* long_rows = nullptr;
+  i64* tmp = nullptr;
+  {
+    Arena ar;
+    ar.add(&p->longest_row, 1);
+    ar.add(&n_long, 1);
+    ar.add(&p->task_counters, 8 * n_batches);
+    const size_t zeroed = ar.bytes;
+    ar.add(&p->task_tickets, 4 * n_batches);
+    ar.add(&p->piece_bound, static_cast<size_t>(B.n_rows) * static_cast<size_t>(r.granules + 1));
+    ar.add(&p->part_cols, static_cast<size_t>(r.granules) * (kMaxParts + 1));
+    ar.add(&p->row_tasks, static_cast<size_t>(nH));
+    ar.add(&p->row_task_off, static_cast<size_t>(nH) + 1);
+    ar.add(&tmp, static_cast<size_t>(scan_tmp_elems(nH)));
+    if (r.granules > 1) {
+      ar.add(&p->granule_counts, static_cast<size_t>(nH) * static_cast<size_t>(r.granules));
+      ar.add(&long_rows, static_cast<size_t>(nH));
+    }
+    GM_TRY(ar.commit(p, st));
+    GM_CUDA(cudaMemsetAsync(p->longest_row, 0, zeroed, st));
+  }
+  k_piece_bounds<<<grid_for(B.n_rows * (r.granules + 1), 256, p->num_sms, 32), 256, 0, st>>>(B.row_ptr, B.col_idx, B.n_rows, r.granules,
+                                                                                           r.log2_g, p->piece_bound, p->longest_row);
+  k_granule_parts<<<static_cast<unsigned>(r.granules), 32, 0, st>>>(B.col_idx, p->piece_bound, p->longest_row, r.granules, r.log2_g,
+                                                                  p->part_cols);
+  p->info.launches += 2;
+  if (r.granules > 1) {
+    k_granule_counts<<<grid_for(nH, 8, p->num_sms, 8), 256, 0, st>>>(p->x_heavy, nH, A.row_ptr, A.col_idx, p->piece_bound, r.granules,
+                                                                   p->granule_counts, long_rows, n_long);
+    k_granule_counts_long<<<static_cast<unsigned>(p->num_sms * 4), 256, 0, st>>>(p->x_heavy, A.row_ptr, A.col_idx, p->piece_bound, r.granules,
+                                                                               p->granule_counts, long_rows, n_long);
+    p->info.launches += 2;
+  }
+  k_task_count<<<static_cast<unsigned>((nH + 127) / 128), 128, 0, st>>>(p->granule_counts, p->heavy_base, nH, r, p->row_tasks);
+  p->info.launches += 1 + exclusive_scan<u32, i64>(p->row_tasks, p->row_task_off, nH, tmp, nullptr, nullptr, nullptr, st,
+                                                  reinterpret_cast<i64*>(&p->slot->n_tasks));
+  p->task_begin.assign(n_batches + 1, 0);
+  for (size_t i = 1; i < n_batches; ++i)
+    GM_CUDA(cudaMemcpyAsync(&p->task_begin[i], p->row_task_off + p->batches[i].h0, sizeof(i64), cudaMemcpyDeviceToHost, st));
+  GM_CUDA(cudaStreamSynchronize(st));
+  p->task_begin[n_batches] = p->slot->n_tasks;
+  i64 max_tasks = 0;
+  for (size_t i = 0; i < n_batches; ++i) max_tasks = std::max(max_tasks, p->task_begin[i + 1] - p->task_begin[i]);
+  {
+    const size_t n = static_cast<size_t>(p->slot->n_tasks), m = static_cast<size_t>(max_tasks);
+    Arena ar;
+    ar.add(&p->tasks, n);
+    ar.add(&p->task_off, n + 1);
+    for (auto& l : p->task_list) ar.add(&l, n);
+    ar.add(&p->chunk_nnz, m + 1);
+    ar.add(&p->chunk_nnz_off, m + 1);
+    ar.add(&p->chunk_base, m + 1);
+    ar.add(&p->tile_meta, static_cast<size_t>(p->info.stage_elems) / kGatherTile + 2);
+    ar.add(&p->scan_tmp, static_cast<size_t>(scan_tmp_elems(std::max<i64>(max_tasks, A.n_rows))));
+    GM_TRY(ar.commit(p, st));
+  }
+  for (size_t i = 0; i < n_batches; ++i) {
+    const Batch& b = p->batches[i];
+    k_task_emit<<<static_cast<unsigned>((b.h1 - b.h0 + 127) / 128), 128, 0, st>>>(
+        p->granule_counts, p->heavy_base, b.h0, b.h1, b.elem0, r, p->row_task_off, p->x_heavy, A.row_ptr, p->part_cols, p->tasks,
+        p->task_off, p->task_list[0], p->task_list[1], p->task_list[2], p->task_counters + 8 * i);
+    ++p->info.launches;
+  }
   GM_CUDA(cudaGetLastError());
   return GM_OK;
 }
@@ -544,30 +675,18 @@ static int build_plan(gm_plan* p, cudaStream_t st) {
     p->light_val = lv;
   }
 
-  // ---- heavy rows: lists, prefix sums, segment table
+  // ---- heavy rows
   if (nH > 0) {
-    i64* tmp2 = nullptr;
-    int32_t* seg_len = nullptr;
     {
       Arena ar;
       ar.add(&p->x_heavy, static_cast<size_t>(nH));
       ar.add(&p->heavy_base, static_cast<size_t>(nH) + 1);
       ar.add(&p->heavy_nz_off, static_cast<size_t>(nH) + 1);
-      ar.add(&p->seg_off, static_cast<size_t>(p->n_seg) + 1);
-      ar.add(&p->seg_bstart, static_cast<size_t>(p->n_seg) + 1);
-      ar.add(&p->seg_j, static_cast<size_t>(p->n_seg) + 1);
-      ar.add(&p->seg_brow, static_cast<size_t>(p->n_seg) + 1);
-      ar.add(&p->seg_hrow, static_cast<size_t>(p->n_seg) + 1);
-      ar.add(&seg_len, static_cast<size_t>(p->n_seg) + 1);
-      ar.add(&tmp2, static_cast<size_t>(scan_tmp_elems(p->n_seg)));
       GM_TRY(ar.commit(p, st));
     }
     k1_heavy_lists<<<static_cast<unsigned>((nA + kHeavyRows - 1) / kHeavyRows), kHeavyThreads, 0, st>>>(
         p->ip, p->heavy_flag, A.row_ptr, nA, tiles, p->x_heavy, p->heavy_base, p->heavy_nz_off);
-    k1_heavy_segments<<<grid_for(p->n_seg, 256, p->num_sms, 32), 256, 0, st>>>(
-        p->x_heavy, nH, p->heavy_nz_off, A.row_ptr, A.col_idx, B.row_ptr, p->n_seg, seg_len, p->seg_bstart, p->seg_j,
-        p->seg_brow, p->seg_hrow);
-    info.launches += 2 + exclusive_scan<int32_t, i64>(seg_len, p->seg_off, p->n_seg, tmp2, nullptr, nullptr, nullptr, st);
+    ++info.launches;
 
     // The expansion writes the first level's children itself (see gm_k4_direct.cuh) unless asked to run that
     // level as separate histogram and multisplit passes.
@@ -589,6 +708,7 @@ static int build_plan(gm_plan* p, cudaStream_t st) {
       p->stream = p->direct && p->opts.expand_staging == 1 && reinterpret_cast<uintptr_t>(B.col_idx) % 16 == 0 &&
                   reinterpret_cast<uintptr_t>(B.vals) % 16 == 0 && p->smem_bytes >= kStreamWarps * warp_smem + 1024;
     }
+    p->use_tasks = !p->csc && !p->stream && (prm.n_levels == 0 || (prm.n_levels == 1 && p->direct)) && plan_task_rules(p);
     // one staging buffer is enough when no multisplit pass runs (no levels, or one level done by the expansion)
     const int n_buf = prm.n_levels > (p->direct ? 1 : 0) ? 2 : 1;
 
@@ -633,6 +753,29 @@ static int build_plan(gm_plan* p, cudaStream_t st) {
       unsigned char* v = nullptr;
       GM_TRY(plan_alloc(p, &v, se * static_cast<size_t>(p->sv), st));
       p->stage_val[i] = v;
+    }
+    if (p->use_tasks) {
+      GM_TRY(plan_tasks(p, st));
+      GM_CUDA(cudaStreamSynchronize(st));
+      return GM_OK;
+    }
+    // ---- segment table: one segment per stored entry of a heavy row
+    {
+      i64* tmp2 = nullptr;
+      int32_t* seg_len = nullptr;
+      Arena ar;
+      ar.add(&p->seg_off, static_cast<size_t>(p->n_seg) + 1);
+      ar.add(&p->seg_bstart, static_cast<size_t>(p->n_seg) + 1);
+      ar.add(&p->seg_j, static_cast<size_t>(p->n_seg) + 1);
+      ar.add(&p->seg_brow, static_cast<size_t>(p->n_seg) + 1);
+      ar.add(&p->seg_hrow, static_cast<size_t>(p->n_seg) + 1);
+      ar.add(&seg_len, static_cast<size_t>(p->n_seg) + 1);
+      ar.add(&tmp2, static_cast<size_t>(scan_tmp_elems(p->n_seg)));
+      GM_TRY(ar.commit(p, st));
+      k1_heavy_segments<<<grid_for(p->n_seg, 256, p->num_sms, 32), 256, 0, st>>>(
+          p->x_heavy, nH, p->heavy_nz_off, A.row_ptr, A.col_idx, B.row_ptr, p->n_seg, seg_len, p->seg_bstart, p->seg_j,
+          p->seg_brow, p->seg_hrow);
+      info.launches += 1 + exclusive_scan<int32_t, i64>(seg_len, p->seg_off, p->n_seg, tmp2, nullptr, nullptr, nullptr, st);
     }
     const size_t n_chunks_max = static_cast<size_t>(p->max_batch_rows) * static_cast<size_t>(prm.chunks_required);
     Arena ar;
@@ -1187,6 +1330,101 @@ static int heavy_batch_front(gm_plan* p, const Batch& b, HeavyBatchState<V>* hs,
   return GM_OK;
 }
 
+// The tasks of one batch: sums into the staging area.  BIG: the dense accumulator's tasks, else the other classes (on the
+// second stream: their blocks fill the SMs as the last big tasks run out).
+template <typename V, bool BIG>
+static int task_batch_sums(gm_plan* p, size_t bi, cudaStream_t st) {
+  const Batch& b = p->batches[bi];
+  const TaskRules& r = p->task_rules;
+  const i64 t0 = p->task_begin[bi], n = p->task_begin[bi + 1] - t0;
+  const HeavyTask* tasks = p->tasks + t0;
+  const int* counters = p->task_counters + 8 * bi;
+  int* tickets = p->task_tickets + 4 * bi;
+  int32_t* out_col = p->stage_col[0];
+  V* out_val = static_cast<V*>(p->stage_val[0]);
+  const TaskInput<V> in{p->A.col_idx, static_cast<const V*>(p->A.vals), p->B.row_ptr, p->B.col_idx, static_cast<const V*>(p->B.vals),
+                        p->piece_bound, r.granules, r.log2_g};
+  PhaseTimes& tm = p->times;
+  if constexpr (BIG) {
+    tm.begin(PhaseTimes::kAccNum, st);
+    const size_t smem = big_task_smem_bytes<V>(p->acc_width, p->acc_threads);
+    const int per_sm = 1024 / p->acc_threads;
+    const unsigned grid = static_cast<unsigned>(std::min<i64>(n, static_cast<i64>(p->num_sms) * per_sm));
+#define GM_BIG(BT)                                                                                                        \
+  do {                                                                                                                    \
+    auto kern = k6_big_tasks<V, BT>;                                                                                      \
+    GM_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)));            \
+    kern<<<grid, BT, smem, st>>>(in, tasks, n, p->task_list[2] + t0, counters, tickets, out_col, out_val, p->chunk_nnz);  \
+  } while (0)
+    if (p->acc_threads == 512) GM_BIG(512);
+    else if (p->acc_threads == 256) GM_BIG(256);
+    else GM_BIG(128);
+#undef GM_BIG
+    ++p->stats.launches;
+    tm.end(st);
+    GM_CUDA(cudaGetLastError());
+    return GM_OK;
+  }
+  if (r.mid_max > r.small_max) {
+    tm.begin(PhaseTimes::kAccMid, st);
+    const size_t smem = mid_task_smem_bytes(static_cast<int>(r.mid_width), sizeof(V), r.mid_max);
+    auto kern = k6_mid_tasks<V>;
+    GM_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)));
+    int per_sm = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kMidThreads, smem) != cudaSuccess || per_sm < 1) per_sm = 1;
+    kern<<<static_cast<unsigned>(std::min<i64>(n, static_cast<i64>(p->num_sms) * per_sm)), kMidThreads, smem, st>>>(
+        in, tasks, p->task_list[1] + t0, counters + 1, tickets + 1, static_cast<int>(r.mid_width), r.mid_max, out_col, out_val, p->chunk_nnz,
+        reinterpret_cast<u64*>(p->c_total + 4));
+    ++p->stats.launches;
+    tm.end(st);
+  }
+  if (r.small_max > 0) {
+    tm.begin(PhaseTimes::kAccSmall, st);
+    const unsigned grid = static_cast<unsigned>(std::min<i64>((n + kSmallWarps - 1) / kSmallWarps, static_cast<i64>(p->num_sms) * (r.small_max > 128 ? 8 : 10)));
+    if (r.small_max > 128)
+      k6_small_tasks<V, 16><<<grid, kSmallWarps * 32, 0, st>>>(in, tasks, p->task_list[0] + t0, counters, out_col, out_val, p->chunk_nnz,
+                                                             reinterpret_cast<u64*>(p->c_total + 2));
+    else
+      k6_small_tasks<V, 4><<<grid, kSmallWarps * 32, 0, st>>>(in, tasks, p->task_list[0] + t0, counters, out_col, out_val, p->chunk_nnz,
+                                                            reinterpret_cast<u64*>(p->c_total + 2));
+    ++p->stats.launches;
+    tm.end(st);
+  }
+  GM_CUDA(cudaGetLastError());
+  return GM_OK;
+}
+
+// Prefix sums of the batch's entry counts, entries per heavy row.
+static int task_batch_counts(gm_plan* p, size_t bi, cudaStream_t st) {
+  const Batch& b = p->batches[bi];
+  const i64 n = p->task_begin[bi + 1] - p->task_begin[bi];
+  PhaseTimes& tm = p->times;
+  tm.begin(PhaseTimes::kScan, st);
+  p->stats.launches += 1 + exclusive_scan<u32, i64>(p->chunk_nnz, p->chunk_nnz_off, n, p->scan_tmp, nullptr, nullptr, nullptr, st);
+  k_task_row_counts<<<grid_for(b.h1 - b.h0, 256, p->num_sms), 256, 0, st>>>(p->chunk_nnz_off, p->row_task_off, b.h0, b.h1, p->x_heavy,
+                                                                          p->row_nnz, p->c_total + 1);
+  tm.end(st);
+  p->stats.final_chunks += (b.h1 - b.h0) * p->info.params.chunks_required;
+  p->stats.staged_products += b.elems;
+  return GM_OK;
+}
+
+template <typename V>
+static int task_batch_gather(gm_plan* p, size_t bi, const i64* c_row_ptr, int32_t* c_col, V* c_val, i64 c_capacity, cudaStream_t st) {
+  const Batch& b = p->batches[bi];
+  const i64 t0 = p->task_begin[bi], n = p->task_begin[bi + 1] - t0;
+  k_task_bases<<<grid_for(b.h1 - b.h0, 256, p->num_sms), 256, 0, st>>>(p->chunk_nnz_off, p->row_task_off, b.h0, b.h1, p->x_heavy, c_row_ptr,
+                                                                     p->chunk_base);
+  // the batch's entry count is only known on the device: it is at most the batch's product count
+  const unsigned grid = static_cast<unsigned>((b.elems + kGatherTile - 1) / kGatherTile);
+  k_tile_bounds<<<grid_for(grid, 256, p->num_sms), 256, 0, st>>>(p->chunk_nnz_off, n, 0, 0, kGatherTile, p->tile_meta, p->chunk_nnz_off + n);
+  k7_gather<V><<<grid, kGatherThreads, 0, st>>>(p->stage_col[0], static_cast<const V*>(p->stage_val[0]), p->task_off + t0, p->chunk_nnz_off,
+                                                p->chunk_base, n, p->tile_meta, c_col, c_val, c_capacity, p->err);
+  p->stats.launches += 3;
+  GM_CUDA(cudaGetLastError());
+  return GM_OK;
+}
+
 static int dev_error_to_status(int code) {
   switch (code) {
     case kDevOk: return GM_OK;
@@ -1214,6 +1452,7 @@ static int execute_t(gm_plan* p, cudaStream_t st, gm_csr* C) {
   slot->err[0] = 0;  // (nothing of this plan is in flight: every execute ends with a synchronisation)
   slot->c_total = 0;
   if (info.rows_heavy > 0) GM_CUDA(cudaMemsetAsync(p->c_total, 0, 16 * sizeof(int64_t), st));
+  if (p->use_tasks) GM_CUDA(cudaMemsetAsync(p->task_tickets, 0, 4 * p->batches.size() * sizeof(int), st));
 
   // ---- result row_ptr
   i64* c_row_ptr = static_cast<i64*>(dev_alloc(static_cast<size_t>(nA + 1) * sizeof(i64), st));
@@ -1222,7 +1461,7 @@ static int execute_t(gm_plan* p, cudaStream_t st, gm_csr* C) {
   V* c_val = nullptr;
   // ---- light and heavy rows are independent until C.row_ptr is formed: the light rows' kernels go to a second
   // stream, forked from and joined back into the caller's with events (never when single_stream is set)
-  bool fork = !p->opts.single_stream && info.rows_light > 0 && info.rows_heavy > 0;
+  bool fork = !p->opts.single_stream && info.rows_heavy > 0 && (info.rows_light > 0 || p->use_tasks);
   if (fork && !p->light_stream) {
     p->light_stream = side_stream();
     if (!p->light_stream || cudaEventCreateWithFlags(&p->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
@@ -1246,9 +1485,11 @@ static int execute_t(gm_plan* p, cudaStream_t st, gm_csr* C) {
 
   // ---- light rows, all that does not need C (Algorithm 3: Symbolic(A[x_light,:], B), and for most rows the sums too)
   fork_light();
+  if (p->use_tasks) GM_TRY_C((task_batch_sums<V, true>(p, 0, st)));  // the longest tasks first
   tm.begin(PhaseTimes::kLightSym, lst);
   GM_TRY_C(light_front<V>(p, lst));
   tm.end(lst);
+  if (p->use_tasks) GM_TRY_C((task_batch_sums<V, false>(p, 0, lst)));
   bool light_counted = !fork;  // the heavy path joins before the first prefix sum over the per-row counts
   auto light_rows_to_c = [&](i64 cap, i64 r0, i64 r1, cudaStream_t s2) -> int {
     tm.begin(PhaseTimes::kLightNum, s2);
@@ -1264,9 +1505,10 @@ static int execute_t(gm_plan* p, cudaStream_t st, gm_csr* C) {
   if (n_batches <= 1) {
     // ---- everything is resident at once: count, allocate C exactly, then fill
     HeavyBatchState<V> hs;
-    if (n_batches == 1) GM_TRY_C(heavy_batch_front<V>(p, p->batches[0], &hs, st));
+    if (n_batches == 1 && !p->use_tasks) GM_TRY_C(heavy_batch_front<V>(p, p->batches[0], &hs, st));
     join_light();
     light_counted = true;
+    if (p->use_tasks) GM_TRY_C(task_batch_counts(p, 0, st));
     tm.begin(PhaseTimes::kScan, st);
     p->stats.launches += exclusive_scan<int32_t, i64>(p->row_nnz, c_row_ptr, nA, p->scan_tmp, nullptr, nullptr, nullptr, st,
                                                       reinterpret_cast<i64*>(&slot->c_total));
@@ -1284,7 +1526,8 @@ static int execute_t(gm_plan* p, cudaStream_t st, gm_csr* C) {
     fork_light();
     if (n_batches == 1) {
       tm.begin(PhaseTimes::kAccSym, st);
-      GM_TRY_C((launch_gather<V>(p, p->batches[0], hs, c_row_ptr, c_col, c_val, capacity, st)));
+      if (p->use_tasks) GM_TRY_C(task_batch_gather<V>(p, 0, c_row_ptr, c_col, c_val, capacity, st));
+      else GM_TRY_C((launch_gather<V>(p, p->batches[0], hs, c_row_ptr, c_col, c_val, capacity, st)));
       tm.end(st);
     }
     GM_TRY_C(light_rows_to_c(capacity, 0, nA, lst));
@@ -1327,7 +1570,18 @@ static int execute_t(gm_plan* p, cudaStream_t st, gm_csr* C) {
     for (size_t bi = 0; bi < n_batches; ++bi) {
       const Batch& b = p->batches[bi];
       HeavyBatchState<V> hs;
-      GM_TRY_C(heavy_batch_front<V>(p, b, &hs, st));
+      if (p->use_tasks) {
+        if (bi > 0) {  // (the first batch's are already on their way)
+          fork_light();
+          GM_TRY_C((task_batch_sums<V, true>(p, bi, st)));
+          GM_TRY_C((task_batch_sums<V, false>(p, bi, lst)));
+        }
+        join_light();
+        light_counted = true;
+        GM_TRY_C(task_batch_counts(p, bi, st));
+      } else {
+        GM_TRY_C(heavy_batch_front<V>(p, b, &hs, st));
+      }
       if (!light_counted) { join_light(); light_counted = true; }
       // rows [r0, r1) of C get their offsets now: every light row in the range was counted up front
       const i64 r0 = bi == 0 ? 0 : p->x_heavy_host[static_cast<size_t>(b.h0)];
@@ -1337,7 +1591,8 @@ static int execute_t(gm_plan* p, cudaStream_t st, gm_csr* C) {
                                                         p->c_total, nullptr, st);
       tm.end(st);
       tm.begin(PhaseTimes::kAccSym, st);
-      GM_TRY_C((launch_gather<V>(p, b, hs, c_row_ptr, c_col, c_val, capacity, st)));
+      if (p->use_tasks) GM_TRY_C(task_batch_gather<V>(p, bi, c_row_ptr, c_col, c_val, capacity, st));
+      else GM_TRY_C((launch_gather<V>(p, b, hs, c_row_ptr, c_col, c_val, capacity, st)));
       tm.end(st);
       if (HostSink* sk = p->sink) {
         // The caller wants C on the host: finish rows [r0, r1) now (their light rows too), note how many entries

@@ -81,7 +81,7 @@ __device__ __forceinline__ int warp_sum_runs(const Key (&key)[K], int n, Key* s_
           sum += s_val[static_cast<u32>(kq) & ((1u << BITS) - 1u)];
         }
         const int p = base + __popc(heads & lanemask_lt());
-        col[p] = static_cast<int32_t>(col_base | static_cast<u32>(c));
+        col[p] = static_cast<int32_t>(col_base + static_cast<u32>(c));
         val[p] = sum;
       }
       base += __popc(heads);
