@@ -358,6 +358,12 @@ static int plan_alloc(gm_plan* p, T** out, size_t n, cudaStream_t st) {
   return GM_OK;
 }
 
+// Bytes a plan sets aside for the light rows' staging area before it knows their products.
+constexpr size_t kLightRoom = size_t{4} << 20;
+// C is allocated before its size is known, with room for every product, when that takes at most this much: the call then
+// does not wait in the middle for nnz(C), and the allocation overlaps the kernels.
+constexpr i64 kCRoomBytes = i64{64} << 20;
+
 // Several device arrays in one allocation: the allocator hook of the Python binding costs a few microseconds a call.
 struct Arena {
   struct Item { void** slot; size_t offset; };
@@ -614,6 +620,7 @@ static int build_plan(gm_plan* p, cudaStream_t st) {
   HeavyTile* tiles = nullptr;
   u32* parts = nullptr;
   size_t zeroed = 0;
+  unsigned char* light_room = nullptr;
   {
     Arena ar;
     const size_t n1 = static_cast<size_t>(nA) + 1;
@@ -628,6 +635,7 @@ static int build_plan(gm_plan* p, cudaStream_t st) {
     ar.add(&p->light_off, n1);
     ar.add(&p->class_list, static_cast<size_t>(kHashClass0 + p->rules.n_hash) * n1);
     ar.add(&p->scan_tmp, static_cast<size_t>(scan_tmp_elems(std::max<i64>(nA, 1))));
+    ar.add(&light_room, kLightRoom);  // the light rows' staging area, if it turns out to fit: an allocation less
     GM_TRY(ar.commit(p, st));
   }
   K1Totals ht{};
@@ -663,7 +671,11 @@ static int build_plan(gm_plan* p, cudaStream_t st) {
     unsigned char* lv = nullptr;
     bool hash_rows = false;
     for (int c = kHashClass0; c < kRowClasses; ++c) hash_rows |= p->class_rows[c] > 0;
-    if (p->staged_light > 0 && !p->merge_only) {
+    const size_t n_staged = static_cast<size_t>(p->staged_light) + 64;
+    if (p->staged_light > 0 && !p->merge_only && n_staged * static_cast<size_t>(4 + p->sv) <= kLightRoom) {
+      lv = light_room;
+      p->light_col = reinterpret_cast<int32_t*>(light_room + n_staged * static_cast<size_t>(p->sv));
+    } else if (p->staged_light > 0 && !p->merge_only) {
       ar.add(&p->light_col, static_cast<size_t>(p->staged_light) + 8);
       ar.add(&lv, (static_cast<size_t>(p->staged_light) + 8) * static_cast<size_t>(p->sv));
     }
@@ -772,7 +784,7 @@ static int build_plan(gm_plan* p, cudaStream_t st) {
       ar.add(&seg_len, static_cast<size_t>(p->n_seg) + 1);
       ar.add(&tmp2, static_cast<size_t>(scan_tmp_elems(p->n_seg)));
       GM_TRY(ar.commit(p, st));
-      k1_heavy_segments<<<grid_for(p->n_seg, 256, p->num_sms, 32), 256, 0, st>>>(
+      k1_heavy_segments<<<static_cast<unsigned>((p->n_seg + 8 * kSegRun - 1) / (8 * kSegRun)), 256, 0, st>>>(
           p->x_heavy, nH, p->heavy_nz_off, A.row_ptr, A.col_idx, B.row_ptr, p->n_seg, seg_len, p->seg_bstart, p->seg_j,
           p->seg_brow, p->seg_hrow);
       info.launches += 1 + exclusive_scan<int32_t, i64>(seg_len, p->seg_off, p->n_seg, tmp2, nullptr, nullptr, nullptr, st);
@@ -895,8 +907,8 @@ static int launch_merge(gm_plan* p, const int32_t* rows, i64 n_rows, const i64* 
 
 template <typename V, typename Key, int KMAX>
 static int launch_sort_one(gm_plan* p, const SortLists& lists, i64 n, cudaStream_t st) {
-  const unsigned grid = grid_for(n, kSortWarps, p->num_sms, KMAX > 4 ? 16 : 24);
-  k3_sort_rows<V, Key, KMAX><<<grid, kSortWarps * 32, 0, st>>>(
+  const unsigned grid = grid_for(n, kSortWarpsOf<KMAX>, p->num_sms, KMAX > 4 ? 16 : 24);
+  k3_sort_rows<V, Key, KMAX><<<grid, kSortWarpsOf<KMAX> * 32, 0, st>>>(
       p->A.row_ptr, p->A.col_idx, static_cast<const V*>(p->A.vals), p->B.row_ptr, p->B.col_idx,
       static_cast<const V*>(p->B.vals), lists, p->light_off, p->row_nnz, p->light_col, static_cast<V*>(p->light_val));
   ++p->stats.launches;
@@ -918,13 +930,21 @@ static int light_front(gm_plan* p, cudaStream_t st) {
   // a key packs a product's column with its position in the row: 32 bits unless the matrix is very wide
   int col_bits = 1;
   while (col_bits < 31 && (i64{1} << col_bits) < p->B.n_cols) ++col_bits;
+  if (const i64 n = p->class_rows[kSortClass0 + 5]; n > 0) {
+    SortLists l{};
+    l.rows[0] = list(kSortClass0 + 5);
+    l.n[0] = n;
+    if (col_bits + 10 <= 32) GM_TRY((launch_sort_one<V, u32, 32>(p, l, n, st)));
+    else GM_TRY((launch_sort_one<V, u64, 32>(p, l, n, st)));
+  }
   {
     SortLists l{};
-    i64 n = 0;
-    for (int i = 0; i < 2; ++i) { const int c = kSortClass0 + 4 - i; l.rows[i] = list(c); l.n[i] = p->class_rows[c]; n += l.n[i]; }
-    const int pos_bits = l.n[0] > 0 ? 9 : 8;
-    if (n > 0 && col_bits + pos_bits <= 32) GM_TRY((launch_sort_one<V, u32, 16>(p, l, n, st)));
-    else if (n > 0) GM_TRY((launch_sort_one<V, u64, 16>(p, l, n, st)));
+    for (int i = 0; i < 2; ++i) { const int c = kSortClass0 + 4 - i; l.rows[i] = list(c); l.n[i] = p->class_rows[c]; }
+    SortLists wide{};  // rows whose keys take 64 bits
+    for (int i = 0; i < 2; ++i)
+      if (col_bits + 9 - i > 32) { wide.rows[i] = l.rows[i]; wide.n[i] = l.n[i]; l.n[i] = 0; }
+    if (wide.n[0] + wide.n[1] > 0) GM_TRY((launch_sort_one<V, u64, 16>(p, wide, wide.n[0] + wide.n[1], st)));
+    if (l.n[0] + l.n[1] > 0) GM_TRY((launch_sort_one<V, u32, 16>(p, l, l.n[0] + l.n[1], st)));
   }
   {
     SortLists l{};
@@ -1032,7 +1052,8 @@ static int launch_accumulate(gm_plan* p, const Batch& b, const HeavyBatchState<V
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k6_small_chunks<V>, kSmallWarps * 32, 0) != cudaSuccess || per_sm < 1)
       per_sm = 4;
     k6_small_chunks<V><<<static_cast<unsigned>(p->num_sms * per_sm), kSmallWarps * 32, 0, st>>>(
-        hs.fin_col, hs.fin_val, hs.chunk_off, hs.n_chunks, W, small_max, p->chunk_nnz,
+        hs.fin_col, hs.fin_val, hs.chunk_off, hs.n_chunks,
+        std::max(0, std::min(hs.log2_cpr, 32 - kSmallIdxBits - ilog2_floor(static_cast<uint64_t>(W)))), small_max, p->chunk_nnz,
         reinterpret_cast<u64*>(p->c_total + 2), hs.tags, hs.alt_col, hs.alt_val, hs.xt);
     ++p->stats.launches;
     p->times.end(st);
@@ -1513,15 +1534,19 @@ static int execute_t(gm_plan* p, cudaStream_t st, gm_csr* C) {
     p->stats.launches += exclusive_scan<int32_t, i64>(p->row_nnz, c_row_ptr, nA, p->scan_tmp, nullptr, nullptr, nullptr, st,
                                                       reinterpret_cast<i64*>(&slot->c_total));
     tm.end(st);
-    if (cudaStreamSynchronize(st) != cudaSuccess) {
-      cleanup();
-      return fail(GM_ERR_CUDA, std::string("symbolic phase failed: ") + cudaGetErrorString(cudaGetLastError()));
+    const bool early_c = info.c_nnz_upper * static_cast<i64>(4 + sizeof(V)) <= kCRoomBytes;
+    if (early_c) {
+      capacity = info.c_nnz_upper;
+    } else {
+      if (cudaStreamSynchronize(st) != cudaSuccess) {
+        cleanup();
+        return fail(GM_ERR_CUDA, std::string("symbolic phase failed: ") + cudaGetErrorString(cudaGetLastError()));
+      }
+      capacity = total = *static_cast<volatile i64*>(&slot->c_total);
     }
-    total = *static_cast<volatile i64*>(&slot->c_total);
-    capacity = total;
-    c_col = static_cast<int32_t*>(dev_alloc(static_cast<size_t>(std::max<i64>(total, 1)) * sizeof(int32_t), st));
-    c_val = static_cast<V*>(dev_alloc(static_cast<size_t>(std::max<i64>(total, 1)) * sizeof(V), st));
-    if (!c_col || !c_val) { cleanup(); return fail(GM_ERR_OOM, "allocation of C (" + std::to_string(total) + " entries) failed"); }
+    c_col = static_cast<int32_t*>(dev_alloc(static_cast<size_t>(std::max<i64>(capacity, 1)) * sizeof(int32_t), st));
+    c_val = static_cast<V*>(dev_alloc(static_cast<size_t>(std::max<i64>(capacity, 1)) * sizeof(V), st));
+    if (!c_col || !c_val) { cleanup(); return fail(GM_ERR_OOM, "allocation of C (" + std::to_string(capacity) + " entries) failed"); }
     // the heavy and the light rows write different rows of C
     fork_light();
     if (n_batches == 1) {
@@ -1632,7 +1657,7 @@ static int execute_t(gm_plan* p, cudaStream_t st, gm_csr* C) {
     cleanup();
     return fail(GM_ERR_CUDA, std::string("execute failed: ") + cudaGetErrorString(e2));
   }
-  if (n_batches > 1) total = slot->tail[0];
+  total = n_batches > 1 ? slot->tail[0] : *static_cast<volatile i64*>(&slot->c_total);
   dev_err = *static_cast<volatile int*>(&slot->err[0]);
   if (dev_err != kDevOk || total > capacity) {
     cleanup();

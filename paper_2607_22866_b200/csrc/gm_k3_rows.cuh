@@ -5,7 +5,7 @@
 //                  registers, every step takes the smallest column and advances all lists that show it.  Nothing is
 //                  shared between lanes, so a step costs the instruction stream a few instructions per list for 32
 //                  rows at once.
-//   k3_sort_rows   one warp per row, up to 512 products: the products' (column, position) keys are sorted in registers
+//   k3_sort_rows   one warp per row, up to 1024 products: the products' (column, position) keys are sorted in registers
 //                  (see warp_sort_keys), runs of equal columns are added up in the original order.
 //
 // Both replace the hash accumulator for these sizes.  What bound that one was not memory: a group of lanes cleared a
@@ -136,7 +136,9 @@ __global__ void __launch_bounds__(kMergeThreads) k3_merge_rows(
 // ------------------------------------------------------------------------------------------------------------------
 // sort
 // ------------------------------------------------------------------------------------------------------------------
-constexpr int kSortWarps = 4;
+// warps per block: what 48 KB of shared memory hold
+template <int KMAX> constexpr int kSortWarpsOf = KMAX > 16 ? 2 : 4;
+template <int K> constexpr int kSortPosBits = 5 + (K == 1 ? 0 : K == 2 ? 1 : K == 4 ? 2 : K == 8 ? 3 : K == 16 ? 4 : 5);
 
 // Lists of the classes one launch handles, longest rows first.
 struct SortLists {
@@ -157,7 +159,7 @@ template <typename V, typename Key, int K, int KMAX>
 __device__ __forceinline__ int gather_row(i64 s, i64 e, const int32_t* __restrict__ a_col, const V* __restrict__ a_val,
                                           const i64* __restrict__ b_row_ptr, const int32_t* __restrict__ b_col,
                                           const V* __restrict__ b_val, SortSmem<V, Key, KMAX>& sm) {
-  constexpr int kPosBits = 5 + (K == 1 ? 0 : K == 2 ? 1 : K == 4 ? 2 : K == 8 ? 3 : 4);
+  constexpr int kPosBits = kSortPosBits<K>;
   constexpr int U = K >= 4 ? 4 : K;  // windows of 32 products in flight
   const int lane = threadIdx.x & 31;
   int done = 0;
@@ -221,7 +223,7 @@ __device__ __forceinline__ void sort_row(i64 row, const i64* __restrict__ a_row_
                                          const int32_t* __restrict__ b_col, const V* __restrict__ b_val,
                                          const i64* __restrict__ light_off, int32_t* __restrict__ row_nnz,
                                          int32_t* __restrict__ out_col, V* __restrict__ out_val, SortSmem<V, Key, KMAX>& sm) {
-  constexpr int kPosBits = 5 + (K == 1 ? 0 : K == 2 ? 1 : K == 4 ? 2 : K == 8 ? 3 : 4);
+  constexpr int kPosBits = kSortPosBits<K>;
   const int lane = threadIdx.x & 31;
   const i64 at = light_off[row];
   const int n = gather_row<V, Key, K, KMAX>(a_row_ptr[row], a_row_ptr[row + 1], a_col, a_val, b_row_ptr, b_col, b_val, sm);
@@ -240,10 +242,11 @@ __device__ __forceinline__ void sort_row(i64 row, const i64* __restrict__ a_row_
 
 // Warps take rows in list order; SortLists holds the classes K = KMAX, KMAX / 2, ... (n = 0: no such rows).
 template <typename V, typename Key, int KMAX>
-__global__ void __launch_bounds__(kSortWarps * 32, KMAX > 4 ? 8 : 12) k3_sort_rows(
+__global__ void __launch_bounds__(kSortWarpsOf<KMAX> * 32, KMAX > 4 ? 8 : 12) k3_sort_rows(
     const i64* __restrict__ a_row_ptr, const int32_t* __restrict__ a_col, const V* __restrict__ a_val,
     const i64* __restrict__ b_row_ptr, const int32_t* __restrict__ b_col, const V* __restrict__ b_val, SortLists lists,
     const i64* __restrict__ light_off, int32_t* __restrict__ row_nnz, int32_t* __restrict__ out_col, V* __restrict__ out_val) {
+  constexpr int kSortWarps = kSortWarpsOf<KMAX>;
   __shared__ SortSmem<V, Key, KMAX> s_sm[kSortWarps];
   SortSmem<V, Key, KMAX>& sm = s_sm[threadIdx.x >> 5];
   const i64 n_warps = static_cast<i64>(gridDim.x) * kSortWarps;
@@ -257,7 +260,9 @@ __global__ void __launch_bounds__(kSortWarps * 32, KMAX > 4 ? 8 : 12) k3_sort_ro
                                 out_val, sm);                                                                                 \
     before += lists.n[I];                                                                                                     \
   }
-  if constexpr (KMAX > 4) {
+  if constexpr (KMAX > 16) {
+    GM_SORT_CLASS(0, 32)
+  } else if constexpr (KMAX > 4) {
     GM_SORT_CLASS(0, 16)
     GM_SORT_CLASS(1, 8)
   } else {

@@ -174,15 +174,14 @@ __device__ __forceinline__ int small_chunk(int32_t* col, V* val, int n, u32 wmas
 
 template <typename V>
 __global__ void __launch_bounds__(kSmallWarps * 32, kSmallBlocksPerSm) k6_small_chunks(
-    int32_t* x_col, V* x_val, const i64* __restrict__ chunk_off, i64 n_chunks, int W, int small_max,
-    u32* __restrict__ chunk_nnz,
+    int32_t* x_col, V* x_val, const i64* __restrict__ chunk_off, i64 n_chunks, int join_bits, int small_max,
+    u32* __restrict__ chunk_nnz,  // (join_bits: chunks whose numbers agree above it may be sorted together)
     u64* __restrict__ totals,  // [0] += products, [1] += entries of the chunks handled here (statistics)
     const unsigned char* __restrict__ tags,  // per chunk, or NULL: != 0 for chunks that left the hierarchy early
     int32_t* x_col_alt, V* x_val_alt, ExitTags xt) {
   __shared__ u32 s_key[kSmallWarps][32 * kSmallMaxPerLane];
   __shared__ V s_val[kSmallWarps][32 * kSmallMaxPerLane];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const u32 wmask = static_cast<u32>(W - 1);
   const i64 n_groups = (n_chunks + 31) >> 5;
   __shared__ u64 s_sum[kSmallWarps][2];  // statistics, kept out of the registers of the sort
   if (lane == 0) { s_sum[w][0] = 0; s_sum[w][1] = 0; }
@@ -201,15 +200,28 @@ __global__ void __launch_bounds__(kSmallWarps * 32, kSmallBlocksPerSm) k6_small_
     // registers, and the extra live state spilled in the fp64 kernel, 42 -> 60 ms on R-MAT scale 21.)
     while (todo) {
       const int src = __ffs(todo) - 1;
-      todo &= todo - 1;
       const i64 s0 = __shfl_sync(0xffffffffu, cs, src);
-      const int n = __shfl_sync(0xffffffffu, cn, src);
+      int n = __shfl_sync(0xffffffffu, cn, src);
       const int tag = __shfl_sync(0xffffffffu, ctag, src);
-      // an early chunk lies in the buffer it was left in and is sorted over all the columns it spans
+      int last = src;
+      if (n < kAccSmallDefault) {
+        // Neighbouring chunks lie next to each other in the buffer and their columns ascend, so the next few are sorted
+        // with this one and counted to it (they get no entries of their own): a chunk costs a warp a chain of memory
+        // latencies and a sort of 32 keys at least, however little it holds.  Clipped-Zipf pair, a few dozen products a
+        // chunk: one chunk at a time took 1.64 ms.
+        const bool joins = k < n_chunks && (cn == 0 || (cn <= small_max && ctag == tag)) && (k >> join_bits) == (((g << 5) + src) >> join_bits);
+        const u32 stop = __ballot_sync(0xffffffffu, !joins && lane > src);
+        const int end = stop ? __ffs(stop) - 1 : 32;
+        const u32 fits = __ballot_sync(0xffffffffu, lane >= src && lane < end && cn > 0 && cs + cn - s0 <= kAccSmallDefault);
+        last = 31 - __clz(fits);
+        n = static_cast<int>(__shfl_sync(0xffffffffu, cs + cn, last) - s0);
+      }
+      todo &= ~((2u << last) - 1u);
+      // an early chunk lies in the buffer it was left in
       const bool alt = tag && xt.alt(tag);
       int32_t* col = (alt ? x_col_alt : x_col) + s0;
       V* val = (alt ? x_val_alt : x_val) + s0;
-      const u32 wm = tag ? (1u << xt.span_bits(tag)) - 1u : wmask;
+      const u32 wm = (1u << (32 - kSmallIdxBits)) - 1u;  // chunks sorted together agree on the column bits above
       u32* out = &chunk_nnz[(g << 5) + src];
       int m;
       if (n <= 32) m = small_chunk<V, 1>(col, val, n, wm, s_key[w], s_val[w], out);
