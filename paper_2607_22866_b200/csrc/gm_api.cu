@@ -318,7 +318,7 @@ struct gm_plan {
   // heavy rows as tasks (see gm_k6_tasks.cuh): no staged products, no levels
   bool use_tasks = false;
   gm::TaskRules task_rules{};
-  int acc_width = 0, acc_threads = 0;
+  int acc_width = 0, acc_threads = 0, acc_blocks = 0;
   gm::u32* piece_bound = nullptr;  // n_rows(B) x (granules + 1)
   gm::u64* longest_row = nullptr;
   gm::u32* part_cols = nullptr;    // granules x (kMaxParts + 1)
@@ -440,10 +440,9 @@ static bool plan_task_rules(gm_plan* p) {
   const gm_params& prm = p->info.params;
   const gm_plan_opts& o = p->opts;
   if (p->B.nnz >= (i64{1} << 32) || p->B.n_rows == 0) return false;  // piece boundaries are 32-bit positions in B's arrays
-  // two accumulators per SM unless another number was asked for: one block's flush overlaps the other's sums (measured
-  // with staged products, R-MAT scale 20: 41.0 against 59.5 ms for the same chunks)
-  const int ctas = prm.acc_ctas_per_sm == 1 ? 2 : prm.acc_ctas_per_sm;
-  const int bt = 1024 / ctas;
+  // kBigBlocks accumulators per SM unless another number was asked for
+  const int ctas = prm.acc_ctas_per_sm == 1 ? kBigBlocks : prm.acc_ctas_per_sm;
+  const int bt = prm.acc_ctas_per_sm == 1 ? kBigThreads : 1024 / ctas;
   const size_t budget = p->smem_bytes / static_cast<size_t>(ctas) - 1024;
   i64 w = prm.chunk_width;
   auto smem = [&](i64 width) { return p->sv == 4 ? big_task_smem_bytes<float>(static_cast<int>(width), bt) : big_task_smem_bytes<double>(static_cast<int>(width), bt); };
@@ -453,6 +452,7 @@ static bool plan_task_rules(gm_plan* p) {
   if (granules > 512) return false;
   p->acc_width = static_cast<int>(w);
   p->acc_threads = bt;
+  p->acc_blocks = ctas;
   TaskRules& r = p->task_rules;
   r.granules = static_cast<int>(granules);
   r.log2_g = ilog2_floor(static_cast<uint64_t>(w));
@@ -464,8 +464,10 @@ static bool plan_task_rules(gm_plan* p) {
   const size_t fixed = (p->sv == 4 ? sizeof(Pieces<float, kMidThreads * kMidPerThread>) : sizeof(Pieces<double, kMidThreads * kMidPerThread>)) + 2048;
   while (mid > r.small_max && mid_task_smem_bytes(static_cast<int>(r.mid_width), p->sv, mid) + fixed > p->smem_bytes / GM_MID_MIN_TASK_BLOCKS) mid /= 2;
   r.mid_max = std::max(mid, r.small_max);
-  // A hub row's granule is cut when it would keep a block busy for longer than an eighth of its even share of the whole.
-  r.split_above = static_cast<u32>(std::min<i64>(1u << 30, std::max<i64>(std::max<i64>(1 << 15, w), p->info.products_heavy / (static_cast<i64>(p->num_sms) * ctas * 8))));
+  // A hub row's granule is cut when it would keep a block busy for longer than an eighth of its even share of the whole (but
+  // not below 8192 products, where the pieces of the sub-ranges get short: R-MAT scale 12 took 312 us with a floor of 32768,
+  // 295 with 8192; and only with more products than columns, which is what the sub-ranges' places in the staging area take).
+  r.split_above = static_cast<u32>(std::min<i64>(1u << 30, std::max<i64>(std::max<i64>(1 << 13, w), p->info.products_heavy / (static_cast<i64>(p->num_sms) * ctas * 8))));
   r.max_parts = kMaxParts;
   return true;
 }
@@ -1369,17 +1371,17 @@ static int task_batch_sums(gm_plan* p, size_t bi, cudaStream_t st) {
   if constexpr (BIG) {
     tm.begin(PhaseTimes::kAccNum, st);
     const size_t smem = big_task_smem_bytes<V>(p->acc_width, p->acc_threads);
-    const int per_sm = 1024 / p->acc_threads;
-    const unsigned grid = static_cast<unsigned>(std::min<i64>(n, static_cast<i64>(p->num_sms) * per_sm));
-#define GM_BIG(BT)                                                                                                        \
+    const unsigned grid = static_cast<unsigned>(std::min<i64>(n, static_cast<i64>(p->num_sms) * p->acc_blocks));
+#define GM_BIG(BT, BLOCKS)                                                                                                        \
   do {                                                                                                                    \
-    auto kern = k6_big_tasks<V, BT>;                                                                                      \
+    auto kern = k6_big_tasks<V, BT, BLOCKS>;                                                                                      \
     GM_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)));            \
     kern<<<grid, BT, smem, st>>>(in, tasks, n, p->task_list[2] + t0, counters, tickets, out_col, out_val, p->chunk_nnz);  \
   } while (0)
-    if (p->acc_threads == 512) GM_BIG(512);
-    else if (p->acc_threads == 256) GM_BIG(256);
-    else GM_BIG(128);
+    if (p->acc_blocks == kBigBlocks && p->acc_threads == kBigThreads) GM_BIG(kBigThreads, kBigBlocks);
+    else if (p->acc_blocks == 2) GM_BIG(512, 2);
+    else if (p->acc_blocks == 4) GM_BIG(256, 4);
+    else GM_BIG(128, 8);
 #undef GM_BIG
     ++p->stats.launches;
     tm.end(st);

@@ -11,8 +11,8 @@
 // one team can sum together.
 //   small  at most small_max products, any width: sorted by one warp
 //   mid    at most mid_max products, at most mid_width columns: a 128-thread block, symbolic then numeric pass
-//   big    one granule, or part of one: dense accumulator; two blocks per SM, so that one block's flush runs next to the
-//          other's sums
+//   big    one granule, or part of one: dense accumulator; three blocks per SM, so that one block's flush runs next to the
+//          others' sums
 // A granule with very many products (a hub row's) is cut further into sub-ranges with about equally many products, so that
 // no block is left alone with it at the end; the boundaries inside a row of B are then found by binary search.
 // Results go to the staging area at the place of the task's products (sub-ranges: at the distance of their first column,
@@ -564,7 +564,7 @@ struct TaskFeed {
 constexpr int kMidPerThread = 2;    // rows of B per thread and round
 // Windows of 32 products a warp has in flight (fp64: with four the registers spill, 1.35 against 1.19 ms for the big tasks
 // of R-MAT scale 17, 1.89 against 1.67 for the mid ones).
-template <typename V> constexpr int kTaskUnroll = 16 / sizeof(V);
+template <typename V> constexpr int kMidUnroll = 16 / sizeof(V);
 
 inline size_t mid_task_smem_bytes(int width, int val_bytes, int entries) {
   const size_t n_words = static_cast<size_t>(width) / 32;
@@ -577,7 +577,7 @@ __global__ void __launch_bounds__(kMidThreads, 6) k6_mid_tasks(
     int width, int entries, int32_t* __restrict__ out_col, V* __restrict__ out_val, u32* __restrict__ task_nnz,
     u64* __restrict__ totals) {  // [0] += products, [1] += entries (statistics)
   extern __shared__ __align__(16) unsigned char smem_mid_raw[];
-  constexpr int T = kMidThreads, PER = kMidPerThread, U = kTaskUnroll<V>;
+  constexpr int T = kMidThreads, PER = kMidPerThread, U = kMidUnroll<V>;
   constexpr int kWarps = T / 32;
   constexpr int CAP = T * PER;
   const int n_words = width >> 5;
@@ -740,6 +740,13 @@ __global__ void __launch_bounds__(kMidThreads, 6) k6_mid_tasks(
 // Bank spreading: the low bits of a power-law matrix's columns are mostly zero; the slot of a column inside its group of
 // 32 is exclusive-ored with bits of the group's number (16-byte words stay whole: the flush reads them).
 constexpr int kBigPerThread = 1;
+template <typename V> constexpr int kBigUnroll = 8 / sizeof(V);  // windows of 32 products a warp has in flight
+// Default: three blocks of 384 threads per SM, so that two blocks sum while one looks for its pieces or flushes.  R-MAT
+// scale 19 fp32 / block-dense fp32, ms of this kernel: 2 x 512 threads 24.1 / 8.0, 3 x 512 24.0 / 7.6, 3 x 256 23.9 / 8.6,
+// 3 x 384 with four windows in flight 24.3 / 8.0, with two 22.9 / 7.2.  What binds it is the shared-memory pipe (70 % busy;
+// the compare-and-swap of an add takes about eleven of its cycles per 32 products).
+constexpr int kBigThreads = 384, kBigBlocks = 3;
+
 
 template <typename V>
 inline size_t big_task_smem_bytes(int W, int threads) {
@@ -764,12 +771,12 @@ __device__ __forceinline__ u32 touched_in(const int4& x, double) {
   return (x.x != 0 || x.y != kIdle) + (x.z != 0 || x.w != kIdle);
 }
 
-template <typename V, int BT>
-__global__ void __launch_bounds__(BT, 1024 / BT) k6_big_tasks(
+template <typename V, int BT, int BLOCKS>
+__global__ void __launch_bounds__(BT, BLOCKS) k6_big_tasks(
     TaskInput<V> in, const HeavyTask* __restrict__ tasks, i64 n_tasks, const int32_t* __restrict__ list, const int* __restrict__ counters,
     int* ticket, int32_t* __restrict__ out_col, V* __restrict__ out_val, u32* __restrict__ task_nnz) {
   extern __shared__ __align__(128) unsigned char smem_acc_raw[];
-  constexpr int CAP = BT * kBigPerThread, PER = kBigPerThread, U = kTaskUnroll<V>;
+  constexpr int CAP = BT * kBigPerThread, PER = kBigPerThread, U = kBigUnroll<V>;
   constexpr int kWarps = BT / 32;
   const int W = 1 << in.log2_g;
   const u32 mask = static_cast<u32>(W - 1);
