@@ -43,8 +43,7 @@ DEFAULT_CONFIG = 2  # R-MAT scale 20, edge factor 16, fp32: the largest fp32 pow
 # (R-MAT scale 17: one batch holds the whole product, 1.09 G products, about 9 GB staged).  Traffic grows in
 # proportion to the products processed, so a full-size launch is its algorithmic figure times this ratio.  A kernel
 # that has changed since its capture must lose its entry (traffic is then reported as null).
-TRAFFIC_RATIO = {"k4_expand": 1.03, "k5a_histogram": 1.00, "k5b_multisplit": 1.00, "k6_small_chunks": 0.63,
-                 "k6_mid_chunks": 0.99, "k6_accumulate": 1.00, "k7_gather": 1.00}
+TRAFFIC_RATIO = {"k4_expand": 1.03, "k5a_histogram": 1.00, "k5b_multisplit": 1.00, "k7_gather": 1.00}
 TRAFFIC_SOURCE = ("single-kernel, single-launch ncu DRAM-counter captures on the same recipe 2**3 smaller (R-MAT scale 17, "
                   "one batch holds the whole product), scaled by products")
 
@@ -243,19 +242,23 @@ def kernel_table(info, stats_avg, sv, nnz_b, n_light_entries_a):
     moved = stats_avg["split_products"]
     split = (2 * se * moved + 4 * ((L - l0) * e - moved)
              + sum(8 * (parents[l] + 1) + 8 * parents[l + 1] for l in range(l0, L)))
+    # heavy rows summed where their products are generated: nothing staged, B read (each kernel once, at least), entries
+    # written; the expansion's time is then zero
+    staged = stats_avg["ms_expand"] > 0
+    in_small, in_mid, in_big = (e_small, e_mid, e - e_small - e_mid) if staged else (nnz_b, nnz_b, nnz_b)
     seg_tables = (12 * p.fanout[0] * info.nnz_a_heavy + 4 * parents[1]) if l0 else 0
     tbl = {
         "k3_light_symbolic": (4 * n_light_entries_a + 8 * info.rows_light + 4 * nnz_b, stats_avg["ms_light_symbolic"]),
         "k3_light_numeric": (se * n_light_entries_a + se * nnz_b + se * (nnz_c - nnz_ch), stats_avg["ms_light_numeric"]),
-        "k4_expand": (se * e + se * nnz_b + 24 * info.nnz_a_heavy + (4 * p.fanout[0] * info.nnz_a_heavy if l0 else 0),
+        "k4_expand": ((se * e + se * nnz_b + 24 * info.nnz_a_heavy + (4 * p.fanout[0] * info.nnz_a_heavy if l0 else 0)) if staged else 0,
                       stats_avg["ms_expand"]),
-        "k5a_histogram": (hist + seg_tables, stats_avg["ms_histogram"]),
+        "k5a_histogram": (hist + seg_tables if staged else 0, stats_avg["ms_histogram"]),
         "k5b_multisplit": (split, stats_avg["ms_multisplit"]),
         # chunks of few products are sorted by one warp each, mid-size ones take a small block each (its second pass
         # re-reads the chunk from L2: not counted), the dense-accumulator kernel owes the rest
-        "k6_small_chunks": (se * e_small + se * nnz_small + 12 * chunks, stats_avg["ms_small_chunks"]),
-        "k6_mid_chunks": (se * e_mid + se * nnz_mid, stats_avg["ms_mid_chunks"]),
-        "k6_accumulate": (se * (e - e_small - e_mid) + se * (nnz_ch - nnz_small - nnz_mid) + 12 * chunks,
+        "k6_small_chunks": (se * in_small + se * nnz_small + (12 * chunks if staged else 0), stats_avg["ms_small_chunks"]),
+        "k6_mid_chunks": (se * in_mid + se * nnz_mid, stats_avg["ms_mid_chunks"]),
+        "k6_accumulate": (se * in_big + se * (nnz_ch - nnz_small - nnz_mid) + (12 * chunks if staged else 0),
                           stats_avg["ms_accumulate"]),
         "k7_gather": (2 * se * nnz_ch + 24 * chunks, stats_avg["ms_gather"]),
     }

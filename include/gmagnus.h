@@ -74,7 +74,7 @@ typedef struct gm_plan_opts {
   int32_t separate_histogram; /* 1: always run the stand-alone histogram kernel per level (otherwise a
                               first level that runs as separate passes is counted by the expansion) */
   int32_t validate_inputs; /* 1: debug mode.  row_ptr / col_idx of A and B are checked on the device first
-                              (GM_ERR_BAD_CSR), and before every chunk accumulation a pass over the staging buffer
+                              (GM_ERR_BAD_CSR), and where products are staged, before every chunk accumulation a pass
                               checks that each product lies in the columns its chunk owns (GM_ERR_INTERNAL)     */
   int32_t single_stream;   /* 1: every kernel of a call runs on the caller's stream.  0 (default): the light rows'
                               kernels run on a second stream of the plan's, forked from and joined back into the
@@ -200,14 +200,18 @@ int64_t gm_planner_batches(const int64_t* heavy_prefix, int64_t n_heavy, int64_t
  *   smem_bytes  shared memory per block the kernels may use (s_LM); at most the device's opt-in
  *               maximum (232448 on B200), at least 16384
  *   plan_out    receives the plan; release it with gm_plan_destroy
- * Runs on `cuda_stream` (gm_spgemm_plan: the legacy default stream) and synchronises it before
- * returning, because the planner needs counts on the host.  The plan borrows A's and B's arrays. */
+ * Runs on `cuda_stream` (gm_spgemm_plan: the legacy default stream) and synchronises it on the way,
+ * because the planner needs counts on the host; kernels that fill the plan's own tables may still run
+ * when it returns (gm_spgemm_execute and gm_plan_destroy wait for them where they have to).  The plan
+ * borrows A's and B's arrays. */
 int gm_spgemm_plan(const gm_csr* A, const gm_csr* B, size_t smem_bytes, gm_plan** plan_out);
 int gm_spgemm_plan_ex(const gm_csr* A, const gm_csr* B, size_t smem_bytes,
                       const gm_plan_opts* opts, void* cuda_stream, gm_plan** plan_out);
 
 /* The rest of Algorithm 3: light rows by Gustavson's method with a shared-memory hash accumulator
- * (symbolic, then numeric); heavy rows, batch by batch, through the expansion (outer-product)
+ * (rows of few products: one sort or merge); heavy rows, batch by batch, either cut into ranges of columns whose
+ * products are summed where they are generated, without being staged (column spaces that one split covers, rows of
+ * B long enough for it), or through the expansion (outer-product)
  * kernel (Algorithm 4), one histogram + multisplit (Algorithm 5) per level (by default the first
  * level is done by the expansion kernel itself, see gm_plan_opts.level0_multisplit), the
  * chunk-accumulate kernels (the chunks are binned by size as in Section III-E: small ones by a one-warp

@@ -154,6 +154,34 @@ static cudaStream_t side_stream() {
   return st;
 }
 
+// Streams of the host entry point: taken for a call, given back after it, at most kKeptStreams kept per device.
+constexpr size_t kKeptStreams = 4;
+static std::vector<cudaStream_t> g_free_streams[kMaxDevices];
+
+static cudaStream_t take_stream() {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) { cudaGetLastError(); return nullptr; }
+  {
+    std::lock_guard<std::mutex> lock(g_facts_mutex);
+    if (!g_free_streams[dev].empty()) {
+      cudaStream_t st = g_free_streams[dev].back();
+      g_free_streams[dev].pop_back();
+      return st;
+    }
+  }
+  cudaStream_t st = nullptr;
+  if (cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking) != cudaSuccess) { cudaGetLastError(); return nullptr; }
+  return st;
+}
+static void give_stream(cudaStream_t st) {  // (the caller has waited for it)
+  int dev = 0;
+  if (cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < kMaxDevices) {
+    std::lock_guard<std::mutex> lock(g_facts_mutex);
+    if (g_free_streams[dev].size() < kKeptStreams) { g_free_streams[dev].push_back(st); return; }
+  }
+  cudaStreamDestroy(st);
+}
+
 // Page-locked host memory that kernels write to and the host reads after a synchronisation: a plan takes one slot and
 // gives it back when it is destroyed.  (Copies to ordinary host variables took 12 to 25 us of host time each.)
 struct HostSlot {
@@ -253,6 +281,7 @@ struct gm_plan {
   gm::LightBins bins{};            // hash rows by entry count, for their numeric pass
   int bin_slots[gm::kMaxLightBins]{};
   gm::HostSlot* slot = nullptr;
+  bool pending = false;            // kernels of the plan may still run on plan_stream
   std::vector<gm::Batch> batches;
   std::vector<int32_t> x_heavy_host;
   int64_t max_batch_rows = 0;
@@ -769,8 +798,8 @@ static int build_plan(gm_plan* p, cudaStream_t st) {
       p->stage_val[i] = v;
     }
     if (p->use_tasks) {
+      p->pending = true;  // (the lists' kernels may still run when the call returns: see gm_spgemm_execute)
       GM_TRY(plan_tasks(p, st));
-      GM_CUDA(cudaStreamSynchronize(st));
       return GM_OK;
     }
     // ---- segment table: one segment per stored entry of a heavy row
@@ -841,7 +870,7 @@ static int build_plan(gm_plan* p, cudaStream_t st) {
           B.row_ptr, B.col_idx, B.n_rows, prm.fanout[0], prm.shift[0], p->child_bound);
       ++info.launches;
     }
-    GM_CUDA(cudaStreamSynchronize(st));
+    p->pending = true;
   }
   return GM_OK;
 }
@@ -1758,6 +1787,10 @@ int gm_spgemm_execute(gm_plan* plan, void* cuda_stream, gm_csr* C_out) {
   if (!plan || !C_out) return fail(GM_ERR_INVALID_ARG, "plan or C_out is null");
   std::memset(C_out, 0, sizeof(*C_out));
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
+  if (plan->pending) {
+    if (st != plan->plan_stream) GM_CUDA(cudaStreamSynchronize(plan->plan_stream));
+    plan->pending = false;  // (an execute ends with a synchronisation of its stream)
+  }
   return plan->A.dtype == GM_F32 ? execute_t<float>(plan, st, C_out) : execute_t<double>(plan, st, C_out);
 }
 
@@ -1798,6 +1831,7 @@ void gm_csr_free(gm_csr* C) {
 
 void gm_plan_destroy(gm_plan* plan) {
   if (!plan) return;
+  if (plan->pending) cudaStreamSynchronize(plan->plan_stream);
   if (plan->ev_fork) cudaEventDestroy(plan->ev_fork);
   if (plan->ev_light) cudaEventDestroy(plan->ev_light);
   for (auto& b : plan->owned) dev_free(b.p, plan->plan_stream);
@@ -1812,32 +1846,38 @@ int gm_spgemm_host(const gm_csr* A_host, const gm_csr* B_host, size_t smem_bytes
   if (!C_host || !C_host->row_ptr || c_capacity < 0) return fail(GM_ERR_INVALID_ARG, "C_host needs caller-owned buffers");
   if (A_host->dtype != B_host->dtype) return fail(GM_ERR_DTYPE, "A and B have different value types");
   const size_t sv = static_cast<size_t>(value_bytes(A_host->dtype));
-  cudaStream_t st = nullptr;
-  GM_CUDA(cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking));
+  cudaStream_t st = take_stream();
+  if (!st) return fail(GM_ERR_CUDA, "stream creation failed");
   gm_csr dev[2];
   std::vector<void*> tmp;
   int rc = GM_OK;
   auto upload = [&](const gm_csr* H, gm_csr* D) -> int {
     *D = *H;
-    void* rp = dev_alloc(static_cast<size_t>(H->n_rows + 1) * 8, st);
-    void* ci = dev_alloc(static_cast<size_t>(H->nnz) * 4, st);
-    void* va = dev_alloc(static_cast<size_t>(H->nnz) * sv, st);
-    tmp.push_back(rp); tmp.push_back(ci); tmp.push_back(va);
-    if (!rp || !ci || !va) return fail(GM_ERR_OOM, "device allocation for an input failed");
+    const size_t rp_bytes = (static_cast<size_t>(H->n_rows + 1) * 8 + 255) & ~size_t{255};
+    const size_t ci_bytes = (static_cast<size_t>(H->nnz) * 4 + 255) & ~size_t{255};
+    char* rp = static_cast<char*>(dev_alloc(rp_bytes + ci_bytes + static_cast<size_t>(H->nnz) * sv, st));
+    if (!rp) return fail(GM_ERR_OOM, "device allocation for an input failed");
+    tmp.push_back(rp);
+    char* ci = rp + rp_bytes;
+    char* va = ci + ci_bytes;
     GM_CUDA(cudaMemcpyAsync(rp, H->row_ptr, static_cast<size_t>(H->n_rows + 1) * 8, cudaMemcpyHostToDevice, st));
     if (H->nnz > 0) {
       GM_CUDA(cudaMemcpyAsync(ci, H->col_idx, static_cast<size_t>(H->nnz) * 4, cudaMemcpyHostToDevice, st));
       GM_CUDA(cudaMemcpyAsync(va, H->vals, static_cast<size_t>(H->nnz) * sv, cudaMemcpyHostToDevice, st));
     }
-    D->row_ptr = static_cast<const int64_t*>(rp);
-    D->col_idx = static_cast<const int32_t*>(ci);
+    D->row_ptr = reinterpret_cast<const int64_t*>(rp);
+    D->col_idx = reinterpret_cast<const int32_t*>(ci);
     D->vals = va;
     return GM_OK;
   };
   gm_plan* plan = nullptr;
   gm_csr C{};
   rc = upload(A_host, &dev[0]);
-  if (rc == GM_OK) rc = upload(B_host, &dev[1]);
+  // a matrix multiplied with itself is sent once
+  const bool same = A_host->n_rows == B_host->n_rows && A_host->n_cols == B_host->n_cols && A_host->nnz == B_host->nnz &&
+                    A_host->row_ptr == B_host->row_ptr && A_host->col_idx == B_host->col_idx && A_host->vals == B_host->vals;
+  if (rc == GM_OK && same) dev[1] = dev[0];
+  else if (rc == GM_OK) rc = upload(B_host, &dev[1]);
   if (rc == GM_OK) rc = gm_spgemm_plan_ex(&dev[0], &dev[1], smem_bytes, opts, st, &plan);
   // With several batches, C's entries travel to the host batch by batch while later batches compute.
   HostSink sink;
@@ -1895,7 +1935,7 @@ int gm_spgemm_host(const gm_csr* A_host, const gm_csr* B_host, size_t smem_bytes
   }
   for (cudaEvent_t ev : sink.events) cudaEventDestroy(ev);
   if (sink.h_totals) cudaFreeHost(sink.h_totals);
-  cudaStreamDestroy(st);
+  give_stream(st);
   return rc;
 }
 
