@@ -464,6 +464,7 @@ static int launch_row_analysis(gm_plan* p, K1Totals* totals, HeavyTile* tiles, u
   return GM_OK;
 }
 
+constexpr i64 kMinPieceProducts = 5;
 // Sizes of the heavy rows' tasks; false: they do not fit (then the rows go through the staged products).
 static bool plan_task_rules(gm_plan* p) {
   const gm_params& prm = p->info.params;
@@ -751,7 +752,12 @@ static int build_plan(gm_plan* p, cudaStream_t st) {
       p->stream = p->direct && p->opts.expand_staging == 1 && reinterpret_cast<uintptr_t>(B.col_idx) % 16 == 0 &&
                   reinterpret_cast<uintptr_t>(B.vals) % 16 == 0 && p->smem_bytes >= kStreamWarps * warp_smem + 1024;
     }
-    p->use_tasks = !p->csc && !p->stream && (prm.n_levels == 0 || (prm.n_levels == 1 && p->direct)) && plan_task_rules(p);
+    // Products are summed where they are generated unless the pieces of B's rows get too short: a task looks every row of B up
+    // in the boundary table, so that costs per (segment, granule) and not per product.  Products per (segment, granule) and time
+    // per call, tasks against staged products: R-MAT scale 18 fp64 with 4 edges a vertex about 9, 4.2 against 5.4 ms; R-MAT scale 20
+    // fp32 20, 188 against 198 ms; R-MAT scale 21 fp64 3.7, 291 against 278 ms.
+    p->use_tasks = !p->csc && !p->stream && (prm.n_levels == 0 || (prm.n_levels == 1 && p->direct)) && plan_task_rules(p) &&
+                   (prm.n_levels == 0 || info.products_heavy >= kMinPieceProducts * p->n_seg * p->task_rules.granules);
     // one staging buffer is enough when no multisplit pass runs (no levels, or one level done by the expansion)
     const int n_buf = prm.n_levels > (p->direct ? 1 : 0) ? 2 : 1;
 
@@ -839,7 +845,7 @@ static int build_plan(gm_plan* p, cudaStream_t st) {
       ar.add(&p->exit_tag[1], n_chunks_max + 1);
       ar.add(&p->parent_tag, n_chunks_max + 1);
     }
-    const size_t n_tiles_max = static_cast<size_t>(info.stage_elems) / std::min({kExpandTile, kSplitTile, kGatherTile, kDirectTileSmall}) + 2;
+    const size_t n_tiles_max = static_cast<size_t>(info.stage_elems) / std::min({kExpandTileShort, kSplitTile, kGatherTileMin, kDirectTileSmall}) + 2;
     ar.add(&p->tile_meta, n_tiles_max);
     ar.add(&p->row_meta, n_tiles_max);
     i64 max_seg_b = 0;
@@ -1133,16 +1139,16 @@ static int launch_gather(gm_plan* p, const Batch& b, const HeavyBatchState<V>& h
   k6_chunk_bases<<<grid_for(hs.n_chunks, 256, p->num_sms), 256, 0, st>>>(p->chunk_nnz_off, hs.n_chunks, hs.log2_cpr,
                                                                          p->x_heavy, b.h0, c_row_ptr, p->chunk_base);
   // the batch's heavy entry count is only known on the device: it is at most the batch's product count
-  const unsigned grid = static_cast<unsigned>((b.elems + kGatherTile - 1) / kGatherTile);
-  k_tile_bounds<<<grid_for(grid, 256, p->num_sms), 256, 0, st>>>(p->chunk_nnz_off, hs.n_chunks, 0, 0, kGatherTile,
-                                                               p->tile_meta, p->chunk_nnz_off + hs.n_chunks);
-  if (hs.tags && hs.xt.alt_bits)
-    k7_gather<V, true><<<grid, kGatherThreads, 0, st>>>(hs.fin_col, hs.fin_val, hs.chunk_off, p->chunk_nnz_off, p->chunk_base,
-                                                        hs.n_chunks, p->tile_meta, c_col, c_val, c_capacity, p->err,
-                                                        hs.alt_col, hs.alt_val, hs.tags, hs.xt.alt_bits);
-  else
-    k7_gather<V><<<grid, kGatherThreads, 0, st>>>(hs.fin_col, hs.fin_val, hs.chunk_off, p->chunk_nnz_off, p->chunk_base,
-                                                  hs.n_chunks, p->tile_meta, c_col, c_val, c_capacity, p->err);
+  const int tile = gather_tile(hs.n_chunks, b.elems);
+  const unsigned grid = static_cast<unsigned>((b.elems + tile - 1) / tile);
+  k_tile_bounds<<<grid_for(grid, 256, p->num_sms), 256, 0, st>>>(p->chunk_nnz_off, hs.n_chunks, 0, 0, tile, p->tile_meta,
+                                                               p->chunk_nnz_off + hs.n_chunks);
+  const bool alt = hs.tags && hs.xt.alt_bits;
+  auto kern = alt ? (tile == kGatherTile ? k7_gather<V, kGatherTile, true> : tile == 4096 ? k7_gather<V, 4096, true> : k7_gather<V, 2048, true>)
+                  : (tile == kGatherTile ? k7_gather<V, kGatherTile> : tile == 4096 ? k7_gather<V, 4096> : k7_gather<V, 2048>);
+  kern<<<grid, kGatherThreads, 0, st>>>(hs.fin_col, hs.fin_val, hs.chunk_off, p->chunk_nnz_off, p->chunk_base, hs.n_chunks,
+                                        p->tile_meta, c_col, c_val, c_capacity, p->err, alt ? hs.alt_col : nullptr,
+                                        alt ? hs.alt_val : nullptr, alt ? hs.tags : nullptr, alt ? hs.xt.alt_bits : 0);
   p->stats.launches += 3;
   GM_CUDA(cudaGetLastError());
   return GM_OK;
@@ -1255,17 +1261,18 @@ static int heavy_batch_front(gm_plan* p, const Batch& b, HeavyBatchState<V>* hs,
   } else if (!p->direct) {
   tm.begin(PhaseTimes::kExpand, st);
   {
-    static_assert(kExpandTile == kSplitTile, "the fused histogram shares the multisplit's tiles");
-    const unsigned grid = static_cast<unsigned>((b.elems + kExpandTile - 1) / kExpandTile);
-    k_tile_bounds<<<grid_for(grid, 256, p->num_sms), 256, 0, st>>>(p->seg_off, p->n_seg, b.elem0, b.elems, kExpandTile,
-                                                                 p->tile_meta);
+    const bool short_segments = p->info.products_heavy < kExpandShortSegment * p->n_seg;
+    const int tile = short_segments ? kExpandTileShort : kExpandTile;
+    const unsigned grid = static_cast<unsigned>((b.elems + tile - 1) / tile);
+    k_tile_bounds<<<grid_for(grid, 256, p->num_sms), 256, 0, st>>>(p->seg_off, p->n_seg, b.elem0, b.elems, tile, p->tile_meta);
     ++p->stats.launches;
     if (fuse_hist) {
       GM_CUDA(cudaMemsetAsync(p->counts, 0, static_cast<size_t>(rows_b) * prm.fanout[0] * sizeof(u32), st));
-      k_tile_bounds<<<grid_for(grid, 256, p->num_sms), 256, 0, st>>>(off_cur, rows_b, 0, b.elems, kExpandTile, p->row_meta);
+      k_tile_bounds<<<grid_for(grid, 256, p->num_sms), 256, 0, st>>>(off_cur, rows_b, 0, b.elems, tile, p->row_meta);
       ++p->stats.launches;
     }
-    k4_expand<V><<<grid, kExpandThreads, 0, st>>>(p->seg_off, p->seg_bstart, p->seg_j, p->tile_meta,
+    auto kern = short_segments ? k4_expand<V, kExpandTileShort> : k4_expand<V, kExpandTile>;
+    kern<<<grid, kExpandThreads, 0, st>>>(p->seg_off, p->seg_bstart, p->seg_j, p->tile_meta,
                                                   static_cast<const V*>(p->A.vals), p->B.col_idx,
                                                   static_cast<const V*>(p->B.vals), b.elem0, b.elems, p->stage_col[0],
                                                   static_cast<V*>(p->stage_val[0]), p->row_meta, off_cur,
@@ -1470,8 +1477,9 @@ static int task_batch_gather(gm_plan* p, size_t bi, const i64* c_row_ptr, int32_
   // the batch's entry count is only known on the device: it is at most the batch's product count
   const unsigned grid = static_cast<unsigned>((b.elems + kGatherTile - 1) / kGatherTile);
   k_tile_bounds<<<grid_for(grid, 256, p->num_sms), 256, 0, st>>>(p->chunk_nnz_off, n, 0, 0, kGatherTile, p->tile_meta, p->chunk_nnz_off + n);
-  k7_gather<V><<<grid, kGatherThreads, 0, st>>>(p->stage_col[0], static_cast<const V*>(p->stage_val[0]), p->task_off + t0, p->chunk_nnz_off,
-                                                p->chunk_base, n, p->tile_meta, c_col, c_val, c_capacity, p->err);
+  k7_gather<V, kGatherTile><<<grid, kGatherThreads, 0, st>>>(
+      p->stage_col[0], static_cast<const V*>(p->stage_val[0]), p->task_off + t0, p->chunk_nnz_off, p->chunk_base, n, p->tile_meta, c_col,
+      c_val, c_capacity, p->err, nullptr, nullptr, nullptr, 0);
   p->stats.launches += 3;
   GM_CUDA(cudaGetLastError());
   return GM_OK;

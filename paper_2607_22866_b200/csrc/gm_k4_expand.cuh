@@ -24,7 +24,11 @@ constexpr int kExpandUnroll = 4;
 constexpr int kExpandHistCap = 2048;      // (row, child) bins of the fused histogram kept in shared memory
 constexpr int kExpandHistParents = 256;
 
-template <typename V>
+// Short rows of B: half the tile, so that its segments still fit the shared table (a tile with more searches the segment
+// table for every product: the clipped-Zipf pair, 5.6 products a segment, took 0.90 ms that way).
+constexpr int kExpandTileShort = 4096;
+constexpr int kExpandShortSegment = 9;  // mean products per segment below which the short tile is taken
+template <typename V, int TILE>
 __global__ void __launch_bounds__(kExpandThreads) k4_expand(
     const i64* __restrict__ seg_off, const i64* __restrict__ seg_bstart, const i64* __restrict__ seg_j,
     const TileMeta* __restrict__ tile_meta,  // per tile: first segment and number of segments
@@ -40,8 +44,8 @@ __global__ void __launch_bounds__(kExpandThreads) k4_expand(
   __shared__ i64 s_bstart[kExpandSegCap];
   __shared__ V s_aval[kExpandSegCap];
 
-  const i64 t0 = static_cast<i64>(blockIdx.x) * kExpandTile;
-  const int tn = static_cast<int>(min(static_cast<i64>(kExpandTile), n_elems - t0));
+  const i64 t0 = static_cast<i64>(blockIdx.x) * TILE;
+  const int tn = static_cast<int>(min(static_cast<i64>(TILE), n_elems - t0));
   const i64 p0 = elem0 + t0;  // global product index of the tile's first element
   const TileMeta tm = tile_meta[blockIdx.x];
   const i64 s_lo = tm.first;
@@ -87,7 +91,7 @@ __global__ void __launch_bounds__(kExpandThreads) k4_expand(
   auto count_product = [&](int q, int32_t c) {
     if (hist_mode != 0) count_in(find_par(q), c);
   };
-  constexpr int kPerWarp = kExpandTile / (kExpandThreads / 32);
+  constexpr int kPerWarp = TILE / (kExpandThreads / 32);
   const int w0 = warp * kPerWarp;
   const int w1 = min(tn, w0 + kPerWarp);
 

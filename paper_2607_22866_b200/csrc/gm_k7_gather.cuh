@@ -27,7 +27,16 @@ template <typename V> struct Pair;
 template <> struct Pair<float> { using type = float2; };
 template <> struct Pair<double> { using type = double2; };
 
-template <typename V, bool ALT = false>
+// Tiles with more chunks than the shared table search for every entry's chunk: the tile is halved (twice at most) until
+// its chunks, empty ones included, fit on average.  Clipped-Zipf pair, 512 chunks to a row of a few thousand entries: 0.57 ms with
+// tiles of 8192.
+constexpr int kGatherTileMin = 2048;
+inline int gather_tile(i64 n_chunks, i64 n_elems) {
+  int t = kGatherTile;
+  while (t > kGatherTileMin && n_chunks * t > n_elems * (kGatherChunkCap * 3 / 4)) t /= 2;
+  return t;
+}
+template <typename V, int TILE, bool ALT = false>
 __global__ void __launch_bounds__(kGatherThreads) k7_gather(
     const int32_t* __restrict__ s_col_in, const V* __restrict__ s_val_in,  // staging buffer (compacted chunks)
     const i64* __restrict__ chunk_off, const i64* __restrict__ chunk_nnz_off, const i64* __restrict__ chunk_base,
@@ -39,9 +48,9 @@ __global__ void __launch_bounds__(kGatherThreads) k7_gather(
   __shared__ i64 s_src[kGatherChunkCap];
   __shared__ i64 s_dst[kGatherChunkCap];
   const i64 n_out = chunk_nnz_off[n_chunks];
-  const i64 t0 = static_cast<i64>(blockIdx.x) * kGatherTile;
+  const i64 t0 = static_cast<i64>(blockIdx.x) * TILE;
   if (t0 >= n_out) return;
-  const int tn = static_cast<int>(min(static_cast<i64>(kGatherTile), n_out - t0));
+  const int tn = static_cast<int>(min(static_cast<i64>(TILE), n_out - t0));
   const TileMeta tm = tile_meta[blockIdx.x];
   const i64 k_lo = tm.first;
   const int n_k = tm.n;
