@@ -346,6 +346,7 @@ struct gm_plan {
   gm::TileMeta* tile_meta = nullptr;  // per tile of the expansion / multisplit kernels: groups it touches
   // heavy rows as tasks (see gm_k6_tasks.cuh): no staged products, no levels
   bool use_tasks = false;
+  bool finish = false;             // small product: one block does the counting between the kernels (see k_finish_small)
   gm::TaskRules task_rules{};
   int acc_width = 0, acc_threads = 0, acc_blocks = 0;
   gm::u32* piece_bound = nullptr;  // n_rows(B) x (granules + 1)
@@ -490,7 +491,12 @@ static bool plan_task_rules(gm_plan* p) {
   r.small_width = 1u << 22;  // a sort key packs the column inside the task with a position of at most nine bits
   const i64 span = static_cast<i64>(pow2_ceil(static_cast<uint64_t>(std::max<i64>(p->B.n_cols, 32))));
   r.mid_width = static_cast<u32>(std::max<i64>(w, std::min<i64>(32768, span)));
-  int mid = o.mid_chunk_max < 0 ? 0 : (o.mid_chunk_max ? o.mid_chunk_max : (p->sv == 4 ? 4096 : 2048));
+  // Hand-over to the dense accumulator: its flush goes with the columns of a granule, the two passes of the mid-size block with the
+  // products.  A quarter of the columns (R-MAT scale 19 fp32, 1024 / 2048 / 4096 products: 77 / 67 / 65 ms); an eighth for
+  // products that leave most of the device idle, where one block's time counts (scale 10 fp32: 130 us against 149 with all
+  // of the columns, scale 12 181 against 195).
+  const int mid_default = static_cast<int>(std::max<i64>(256, std::min<i64>(p->sv == 4 ? 4096 : 2048, w / (p->info.products_heavy < (i64{1} << 24) ? 8 : 4))));
+  int mid = o.mid_chunk_max < 0 ? 0 : (o.mid_chunk_max ? o.mid_chunk_max : mid_default);
   const size_t fixed = (p->sv == 4 ? sizeof(Pieces<float, kMidThreads * kMidPerThread>) : sizeof(Pieces<double, kMidThreads * kMidPerThread>)) + 2048;
   while (mid > r.small_max && mid_task_smem_bytes(static_cast<int>(r.mid_width), p->sv, mid) + fixed > p->smem_bytes / GM_MID_MIN_TASK_BLOCKS) mid /= 2;
   r.mid_max = std::max(mid, r.small_max);
@@ -512,12 +518,28 @@ static int plan_tasks(gm_plan* p, cudaStream_t st) {
   u32* n_long = nullptr;
   int32_t* long_rows = nullptr;
   i64* tmp = nullptr;
+  // Small products: the tables take their upper bound (a granule of n products gives fewer than 2 n / split_above
+  // sub-ranges), so that nothing waits for the number of tasks.
+  const i64 bound = nH * r.granules + 2 * (p->info.products_heavy / r.split_above) + 64;
+  p->finish = n_batches == 1 && bound <= kFinishMax && A.n_rows <= kFinishMax;
+  auto add_tables = [&](Arena& ar, i64 n_tasks, i64 max_tasks) {
+    const size_t n = static_cast<size_t>(n_tasks), m = static_cast<size_t>(max_tasks);
+    ar.add(&p->tasks, n);
+    ar.add(&p->task_off, n + 1);
+    for (auto& l : p->task_list) ar.add(&l, n);
+    ar.add(&p->chunk_nnz, m + 1);
+    ar.add(&p->chunk_nnz_off, m + 1);
+    ar.add(&p->chunk_base, m + 1);
+    ar.add(&p->tile_meta, static_cast<size_t>(p->info.stage_elems) / kGatherTile + 2);
+    ar.add(&p->scan_tmp, static_cast<size_t>(scan_tmp_elems(std::max<i64>(max_tasks, A.n_rows))));
+  };
   {
     Arena ar;
     ar.add(&p->longest_row, 1);
     ar.add(&n_long, 1);
     ar.add(&p->task_counters, 8 * n_batches);
     const size_t zeroed = ar.bytes;
+    ar.add(&p->c_total, 16);  // (next to the tickets: one clear for both, see execute_t)
     ar.add(&p->task_tickets, 4 * n_batches);
     ar.add(&p->piece_bound, static_cast<size_t>(B.n_rows) * static_cast<size_t>(r.granules + 1));
     ar.add(&p->part_cols, static_cast<size_t>(r.granules) * (kMaxParts + 1));
@@ -528,6 +550,7 @@ static int plan_tasks(gm_plan* p, cudaStream_t st) {
       ar.add(&p->granule_counts, static_cast<size_t>(nH) * static_cast<size_t>(r.granules));
       ar.add(&long_rows, static_cast<size_t>(nH));
     }
+    if (p->finish) add_tables(ar, bound, bound);
     GM_TRY(ar.commit(p, st));
     GM_CUDA(cudaMemsetAsync(p->longest_row, 0, zeroed, st));
   }
@@ -543,10 +566,19 @@ static int plan_tasks(gm_plan* p, cudaStream_t st) {
                                                                                p->granule_counts, long_rows, n_long);
     p->info.launches += 2;
   }
+  p->task_begin.assign(n_batches + 1, 0);
+  if (p->finish) {
+    p->task_begin[1] = bound;
+    const TaskTables tt{p->tasks, p->task_off, {p->task_list[0], p->task_list[1], p->task_list[2]}, p->task_counters, 0, bound};
+    k_plan_small<<<1, kFinishThreads, 0, st>>>(p->granule_counts, p->heavy_base, nH, r, p->row_tasks, p->row_task_off, p->x_heavy, A.row_ptr,
+                                              p->part_cols, tt);
+    ++p->info.launches;
+    GM_CUDA(cudaGetLastError());
+    return GM_OK;
+  }
   k_task_count<<<static_cast<unsigned>((nH + 127) / 128), 128, 0, st>>>(p->granule_counts, p->heavy_base, nH, r, p->row_tasks);
   p->info.launches += 1 + exclusive_scan<u32, i64>(p->row_tasks, p->row_task_off, nH, tmp, nullptr, nullptr, nullptr, st,
                                                   reinterpret_cast<i64*>(&p->slot->n_tasks));
-  p->task_begin.assign(n_batches + 1, 0);
   for (size_t i = 1; i < n_batches; ++i)
     GM_CUDA(cudaMemcpyAsync(&p->task_begin[i], p->row_task_off + p->batches[i].h0, sizeof(i64), cudaMemcpyDeviceToHost, st));
   GM_CUDA(cudaStreamSynchronize(st));
@@ -554,23 +586,16 @@ static int plan_tasks(gm_plan* p, cudaStream_t st) {
   i64 max_tasks = 0;
   for (size_t i = 0; i < n_batches; ++i) max_tasks = std::max(max_tasks, p->task_begin[i + 1] - p->task_begin[i]);
   {
-    const size_t n = static_cast<size_t>(p->slot->n_tasks), m = static_cast<size_t>(max_tasks);
     Arena ar;
-    ar.add(&p->tasks, n);
-    ar.add(&p->task_off, n + 1);
-    for (auto& l : p->task_list) ar.add(&l, n);
-    ar.add(&p->chunk_nnz, m + 1);
-    ar.add(&p->chunk_nnz_off, m + 1);
-    ar.add(&p->chunk_base, m + 1);
-    ar.add(&p->tile_meta, static_cast<size_t>(p->info.stage_elems) / kGatherTile + 2);
-    ar.add(&p->scan_tmp, static_cast<size_t>(scan_tmp_elems(std::max<i64>(max_tasks, A.n_rows))));
+    add_tables(ar, p->slot->n_tasks, max_tasks);
     GM_TRY(ar.commit(p, st));
   }
   for (size_t i = 0; i < n_batches; ++i) {
     const Batch& b = p->batches[i];
-    k_task_emit<<<static_cast<unsigned>((b.h1 - b.h0 + 127) / 128), 128, 0, st>>>(
-        p->granule_counts, p->heavy_base, b.h0, b.h1, b.elem0, r, p->row_task_off, p->x_heavy, A.row_ptr, p->part_cols, p->tasks,
-        p->task_off, p->task_list[0], p->task_list[1], p->task_list[2], p->task_counters + 8 * i);
+    const TaskTables tt{p->tasks, p->task_off, {p->task_list[0], p->task_list[1], p->task_list[2]}, p->task_counters + 8 * i,
+                        p->task_begin[i], p->task_begin[i + 1]};
+    k_task_emit<<<static_cast<unsigned>((b.h1 - b.h0 + 127) / 128), 128, 0, st>>>(p->granule_counts, p->heavy_base, b.h0, b.h1, b.elem0, r,
+                                                                                p->row_task_off, p->x_heavy, A.row_ptr, p->part_cols, tt);
     ++p->info.launches;
   }
   GM_CUDA(cudaGetLastError());
@@ -757,7 +782,7 @@ static int build_plan(gm_plan* p, cudaStream_t st) {
     // per call, tasks against staged products: R-MAT scale 18 fp64 with 4 edges a vertex about 9, 4.2 against 5.4 ms; R-MAT scale 20
     // fp32 20, 188 against 198 ms; R-MAT scale 21 fp64 3.7, 291 against 278 ms.
     p->use_tasks = !p->csc && !p->stream && (prm.n_levels == 0 || (prm.n_levels == 1 && p->direct)) && plan_task_rules(p) &&
-                   (prm.n_levels == 0 || info.products_heavy >= kMinPieceProducts * p->n_seg * p->task_rules.granules);
+                   (p->task_rules.granules <= 8 || info.products_heavy >= kMinPieceProducts * p->n_seg * p->task_rules.granules);
     // one staging buffer is enough when no multisplit pass runs (no levels, or one level done by the expansion)
     const int n_buf = prm.n_levels > (p->direct ? 1 : 0) ? 2 : 1;
 
@@ -1469,18 +1494,21 @@ static int task_batch_counts(gm_plan* p, size_t bi, cudaStream_t st) {
 }
 
 template <typename V>
-static int task_batch_gather(gm_plan* p, size_t bi, const i64* c_row_ptr, int32_t* c_col, V* c_val, i64 c_capacity, cudaStream_t st) {
+static int task_batch_gather(gm_plan* p, size_t bi, bool bases, const i64* c_row_ptr, int32_t* c_col, V* c_val, i64 c_capacity, cudaStream_t st) {
   const Batch& b = p->batches[bi];
   const i64 t0 = p->task_begin[bi], n = p->task_begin[bi + 1] - t0;
-  k_task_bases<<<grid_for(b.h1 - b.h0, 256, p->num_sms), 256, 0, st>>>(p->chunk_nnz_off, p->row_task_off, b.h0, b.h1, p->x_heavy, c_row_ptr,
-                                                                     p->chunk_base);
   // the batch's entry count is only known on the device: it is at most the batch's product count
   const unsigned grid = static_cast<unsigned>((b.elems + kGatherTile - 1) / kGatherTile);
-  k_tile_bounds<<<grid_for(grid, 256, p->num_sms), 256, 0, st>>>(p->chunk_nnz_off, n, 0, 0, kGatherTile, p->tile_meta, p->chunk_nnz_off + n);
+  if (bases) {
+    k_task_bases<<<grid_for(b.h1 - b.h0, 256, p->num_sms), 256, 0, st>>>(p->chunk_nnz_off, p->row_task_off, b.h0, b.h1, p->x_heavy, c_row_ptr,
+                                                                       p->chunk_base);
+    k_tile_bounds<<<grid_for(grid, 256, p->num_sms), 256, 0, st>>>(p->chunk_nnz_off, n, 0, 0, kGatherTile, p->tile_meta, p->chunk_nnz_off + n);
+    p->stats.launches += 2;
+  }
   k7_gather<V, kGatherTile><<<grid, kGatherThreads, 0, st>>>(
       p->stage_col[0], static_cast<const V*>(p->stage_val[0]), p->task_off + t0, p->chunk_nnz_off, p->chunk_base, n, p->tile_meta, c_col,
       c_val, c_capacity, p->err, nullptr, nullptr, nullptr, 0);
-  p->stats.launches += 3;
+  p->stats.launches += 1;
   GM_CUDA(cudaGetLastError());
   return GM_OK;
 }
@@ -1511,8 +1539,10 @@ static int execute_t(gm_plan* p, cudaStream_t st, gm_csr* C) {
   HostSlot* const slot = p->slot;
   slot->err[0] = 0;  // (nothing of this plan is in flight: every execute ends with a synchronisation)
   slot->c_total = 0;
-  if (info.rows_heavy > 0) GM_CUDA(cudaMemsetAsync(p->c_total, 0, 16 * sizeof(int64_t), st));
-  if (p->use_tasks) GM_CUDA(cudaMemsetAsync(p->task_tickets, 0, 4 * p->batches.size() * sizeof(int), st));
+  if (p->use_tasks)
+    GM_CUDA(cudaMemsetAsync(p->c_total, 0, reinterpret_cast<char*>(p->task_tickets + 4 * p->batches.size()) - reinterpret_cast<char*>(p->c_total), st));
+  else if (info.rows_heavy > 0)
+    GM_CUDA(cudaMemsetAsync(p->c_total, 0, 16 * sizeof(int64_t), st));
 
   // ---- result row_ptr
   i64* c_row_ptr = static_cast<i64*>(dev_alloc(static_cast<size_t>(nA + 1) * sizeof(i64), st));
@@ -1562,16 +1592,27 @@ static int execute_t(gm_plan* p, cudaStream_t st, gm_csr* C) {
   i64 capacity = 0;
   i64 total = 0;
   int dev_err = 0;
+  bool finished = false;  // small products: counts, C.row_ptr and the totals came from one launch
   if (n_batches <= 1) {
     // ---- everything is resident at once: count, allocate C exactly, then fill
     HeavyBatchState<V> hs;
     if (n_batches == 1 && !p->use_tasks) GM_TRY_C(heavy_batch_front<V>(p, p->batches[0], &hs, st));
     join_light();
     light_counted = true;
-    if (p->use_tasks) GM_TRY_C(task_batch_counts(p, 0, st));
+    finished = p->finish;
+    if (p->use_tasks && !finished) GM_TRY_C(task_batch_counts(p, 0, st));
     tm.begin(PhaseTimes::kScan, st);
-    p->stats.launches += exclusive_scan<int32_t, i64>(p->row_nnz, c_row_ptr, nA, p->scan_tmp, nullptr, nullptr, nullptr, st,
-                                                      reinterpret_cast<i64*>(&slot->c_total));
+    if (finished) {
+      k_finish_small<<<1, kFinishThreads, 0, st>>>(p->chunk_nnz, p->task_begin[1], p->chunk_nnz_off, p->row_task_off, info.rows_heavy, p->x_heavy,
+                                                   p->row_nnz, nA, c_row_ptr, &slot->c_total, p->chunk_base, kGatherTile, p->tile_meta,
+                                                   p->c_total, slot->tail);
+      p->stats.launches += 1;
+      p->stats.final_chunks += info.rows_heavy * info.params.chunks_required;
+      p->stats.staged_products += info.products_heavy;
+    } else {
+      p->stats.launches += exclusive_scan<int32_t, i64>(p->row_nnz, c_row_ptr, nA, p->scan_tmp, nullptr, nullptr, nullptr, st,
+                                                        reinterpret_cast<i64*>(&slot->c_total));
+    }
     tm.end(st);
     const bool early_c = info.c_nnz_upper * static_cast<i64>(4 + sizeof(V)) <= kCRoomBytes;
     if (early_c) {
@@ -1590,7 +1631,7 @@ static int execute_t(gm_plan* p, cudaStream_t st, gm_csr* C) {
     fork_light();
     if (n_batches == 1) {
       tm.begin(PhaseTimes::kAccSym, st);
-      if (p->use_tasks) GM_TRY_C(task_batch_gather<V>(p, 0, c_row_ptr, c_col, c_val, capacity, st));
+      if (p->use_tasks) GM_TRY_C(task_batch_gather<V>(p, 0, !finished, c_row_ptr, c_col, c_val, capacity, st));
       else GM_TRY_C((launch_gather<V>(p, p->batches[0], hs, c_row_ptr, c_col, c_val, capacity, st)));
       tm.end(st);
     }
@@ -1655,7 +1696,7 @@ static int execute_t(gm_plan* p, cudaStream_t st, gm_csr* C) {
                                                         p->c_total, nullptr, st);
       tm.end(st);
       tm.begin(PhaseTimes::kAccSym, st);
-      if (p->use_tasks) GM_TRY_C(task_batch_gather<V>(p, bi, c_row_ptr, c_col, c_val, capacity, st));
+      if (p->use_tasks) GM_TRY_C(task_batch_gather<V>(p, bi, true, c_row_ptr, c_col, c_val, capacity, st));
       else GM_TRY_C((launch_gather<V>(p, b, hs, c_row_ptr, c_col, c_val, capacity, st)));
       tm.end(st);
       if (HostSink* sk = p->sink) {
@@ -1690,7 +1731,7 @@ static int execute_t(gm_plan* p, cudaStream_t st, gm_csr* C) {
   if (tm.enabled) cudaEventRecord(ev_total1, st);
   // [0] nnz(C) so far (several batches), [1] heavy entries; products and entries of small chunks; of mid-size chunks;
   // products and chunks that left the hierarchy early; products the multisplit levels left in place
-  if (n_batches > 0) cudaMemcpyAsync(slot->tail, p->c_total, 9 * sizeof(i64), cudaMemcpyDeviceToHost, st);
+  if (n_batches > 0 && !finished) cudaMemcpyAsync(slot->tail, p->c_total, 9 * sizeof(i64), cudaMemcpyDeviceToHost, st);
   const cudaError_t e2 = cudaStreamSynchronize(st);
   if (e2 != cudaSuccess) {
     cleanup();

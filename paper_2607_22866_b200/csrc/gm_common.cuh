@@ -130,6 +130,18 @@ struct __align__(16) TileMeta {
   int off1;   // start of group first + 1 relative to the tile (tile + 1 if n == 1)
 };
 
+__device__ __forceinline__ TileMeta tile_bounds(const i64* off, i64 n_off, i64 bias, i64 n_elems, int tile, i64 t) {
+  const i64 p0 = bias + t * tile;
+  const i64 p1 = bias + min(n_elems, (t + 1) * tile) - 1;
+  const i64 f = last_le(off, 0, n_off - 1, p0);
+  const i64 l = last_le(off, f, n_off - 1, p1);
+  TileMeta m;
+  m.first = f;
+  m.n = static_cast<int>(min(l - f + 1, static_cast<i64>(INT_MAX)));
+  m.off1 = m.n >= 2 ? clamp_rel(off[f + 1] - p0, -1, tile + 1) : tile + 1;
+  return m;
+}
+
 // For every tile of `tile` consecutive elements (positions bias + t*tile ... of a flattened space whose
 // groups start at off[0..n_off)): the TileMeta above.  Run as its own small launch so that the searches of
 // all tiles overlap; a block that searched for its own tile would keep all its threads waiting through ~20
@@ -140,15 +152,7 @@ __global__ void k_tile_bounds(const i64* __restrict__ off, i64 n_off, i64 bias, 
   const i64 n_tiles = (n_elems + tile - 1) / tile;
   for (i64 t = static_cast<i64>(blockIdx.x) * blockDim.x + threadIdx.x; t < n_tiles;
        t += static_cast<i64>(gridDim.x) * blockDim.x) {
-    const i64 p0 = bias + t * tile;
-    const i64 p1 = bias + min(n_elems, (t + 1) * tile) - 1;
-    const i64 f = last_le(off, 0, n_off - 1, p0);
-    const i64 l = last_le(off, f, n_off - 1, p1);
-    TileMeta m;
-    m.first = f;
-    m.n = static_cast<int>(min(l - f + 1, static_cast<i64>(INT_MAX)));
-    m.off1 = m.n >= 2 ? clamp_rel(off[f + 1] - p0, -1, tile + 1) : tile + 1;
-    meta[t] = m;
+    meta[t] = tile_bounds(off, n_off, bias, n_elems, tile, t);
   }
 }
 

@@ -184,32 +184,32 @@ __global__ void __launch_bounds__(128) k_task_count(const u32* __restrict__ coun
   row_tasks[h] = cut_row(counts + h * r.granules, static_cast<u32>(heavy_base[h + 1] - heavy_base[h]), r, [](int, int, u32, u32) {});
 }
 
-// row_task_off: exclusive prefix sums of row_tasks.  Also sorts the tasks into the kernels' lists: list[0..2] (small, mid,
-// big; the huge ones of the big class from the front of its list, the others from the back of the batch's part).
-// Rows h0 .. h1 - 1 (a batch): counters[0] small, [1] mid, [2] huge, [3] other big.
-__global__ void __launch_bounds__(128) k_task_emit(const u32* __restrict__ counts, const i64* __restrict__ heavy_base, i64 h0, i64 h1,
-                                                   i64 elem0, TaskRules r, const i64* __restrict__ row_task_off,
-                                                   const int32_t* __restrict__ x_heavy, const i64* __restrict__ a_row_ptr,
-                                                   const u32* __restrict__ parts_tab, HeavyTask* __restrict__ tasks,
-                                                   i64* __restrict__ task_off, int32_t* __restrict__ small_list,
-                                                   int32_t* __restrict__ mid_list, int32_t* __restrict__ big_list, int* __restrict__ counters) {
-  const i64 h = h0 + static_cast<i64>(blockIdx.x) * blockDim.x + threadIdx.x;
-  const i64 t_first = row_task_off[h0], t_end = row_task_off[h1];  // the batch's tasks
-  if (h >= h1) return;
+// Where the tasks of a batch go.  lists: [0] small, [1] mid, [2] big (the huge ones from the front of the batch's part of the
+// list, the others from its back); counters: [0] small, [1] mid, [2] huge, [3] other big.
+struct TaskTables {
+  HeavyTask* tasks;
+  i64* task_off;
+  int32_t* list[3];
+  int* counters;
+  i64 first, end;  // the batch's part of the tables
+};
+
+// Writes the tasks of heavy row h, the first of them at position id.
+__device__ __forceinline__ void emit_row(const u32* __restrict__ counts, const i64* __restrict__ heavy_base, i64 h, i64 elem0,
+                                         const TaskRules& r, i64 id, const int32_t* __restrict__ x_heavy,
+                                         const i64* __restrict__ a_row_ptr, const u32* __restrict__ parts_tab, const TaskTables& tt) {
   const i64 row = x_heavy[h];
   HeavyTask t;
   t.a0 = a_row_ptr[row];
   t.n_a = static_cast<u32>(a_row_ptr[row + 1] - t.a0);
   i64 off = heavy_base[h] - elem0;
-  i64 id = row_task_off[h];
   auto put = [&](int cls, bool front) {
-    const int b = static_cast<int>(id - t_first);  // lists hold batch-relative ids
-    if (cls == 0) small_list[t_first + atomicAdd(&counters[0], 1)] = b;
-    else if (cls == 1) mid_list[t_first + atomicAdd(&counters[1], 1)] = b;
-    else if (front) big_list[t_first + atomicAdd(&counters[2], 1)] = b;
-    else big_list[t_end - 1 - atomicAdd(&counters[3], 1)] = b;
-    tasks[id] = t;
-    task_off[id] = t.off;
+    const int b = static_cast<int>(id - tt.first);  // lists hold batch-relative ids
+    if (cls < 2) tt.list[cls][tt.first + atomicAdd(&tt.counters[cls], 1)] = b;
+    else if (front) tt.list[2][tt.first + atomicAdd(&tt.counters[2], 1)] = b;
+    else tt.list[2][tt.end - 1 - atomicAdd(&tt.counters[3], 1)] = b;
+    tt.tasks[id] = t;
+    tt.task_off[id] = t.off;
     ++id;
   };
   cut_row(counts + h * r.granules, static_cast<u32>(heavy_base[h + 1] - heavy_base[h]), r, [&](int g, int w, u32 n, u32 parts) {
@@ -234,6 +234,15 @@ __global__ void __launch_bounds__(128) k_task_emit(const u32* __restrict__ count
     }
     off += n;
   });
+}
+
+// Rows h0 .. h1 - 1 (a batch).  row_task_off: exclusive prefix sums of row_tasks.
+__global__ void __launch_bounds__(128) k_task_emit(const u32* __restrict__ counts, const i64* __restrict__ heavy_base, i64 h0, i64 h1,
+                                                   i64 elem0, TaskRules r, const i64* __restrict__ row_task_off,
+                                                   const int32_t* __restrict__ x_heavy, const i64* __restrict__ a_row_ptr,
+                                                   const u32* __restrict__ parts_tab, TaskTables tt) {
+  const i64 h = h0 + static_cast<i64>(blockIdx.x) * blockDim.x + threadIdx.x;
+  if (h < h1) emit_row(counts, heavy_base, h, elem0, r, row_task_off[h], x_heavy, a_row_ptr, parts_tab, tt);
 }
 
 // ---------------------------------------------------------------------------------------------------------------------
@@ -914,6 +923,72 @@ __global__ void k_task_bases(const i64* __restrict__ nnz_off, const i64* __restr
     const i64 shift = c_row_ptr[x_heavy[h]] - nnz_off[a];
     for (i64 t = a; t < b; ++t) base[t] = nnz_off[t] + shift;
   }
+}
+
+// Everything between the sums and the gather in one launch of one block, for small products: prefix sums of the tasks'
+// entries, entries per heavy row, C.rowPtr, position in C of every task's first entry, the gather's tile records, and the
+// totals for the host.  (Five launches and a copy otherwise, each of which costs more than its work: 55 us from the last
+// sum to the end of the call for R-MAT scales 10 to 12, of 130 to 260.)
+constexpr i64 kFinishMax = 16384;  // tasks, and rows of A: above, one block takes as long as the launches
+constexpr int kFinishThreads = 1024;
+// out[0 .. n) = exclusive prefix sums of in (values from position n_valid on count as zero); returns the total (every thread).
+// Ends with a barrier.
+__device__ __forceinline__ i64 finish_scan(const u32* in, i64 n_valid, i64 n, i64* out, i64* tmp) {
+  i64 run = 0;
+  for (i64 i0 = 0; i0 < n; i0 += 4 * kFinishThreads) {
+    const i64 i = i0 + threadIdx.x * 4;
+    i64 v[4], sum = 0;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      v[k] = i + k < n_valid ? static_cast<i64>(in[i + k]) : 0;
+      sum += v[k];
+    }
+    __syncthreads();
+    i64 total;
+    i64 ex = run + block_exclusive_scan(sum, tmp, &total);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      if (i + k < n) out[i + k] = ex;
+      ex += v[k];
+    }
+    run += total;
+  }
+  if (threadIdx.x == 0) out[n] = run;
+  __syncthreads();
+  return run;
+}
+__global__ void __launch_bounds__(kFinishThreads) k_finish_small(const u32* task_nnz, i64 n_tasks, i64* nnz_off, const i64* row_task_off,
+                                                                 i64 n_heavy, const int32_t* x_heavy, int32_t* row_nnz, i64 n_rows,
+                                                                 i64* c_row_ptr, i64* host_total, i64* base, int tile, TileMeta* meta,
+                                                                 i64* totals, i64* host_totals) {
+  __shared__ i64 tmp[33];
+  const i64 heavy = finish_scan(task_nnz, row_task_off[n_heavy], n_tasks, nnz_off, tmp);  // (n_tasks: an upper bound)
+  for (i64 h = threadIdx.x; h < n_heavy; h += kFinishThreads)
+    row_nnz[x_heavy[h]] = static_cast<int32_t>(nnz_off[row_task_off[h + 1]] - nnz_off[row_task_off[h]]);
+  __syncthreads();
+  const i64 all = finish_scan(reinterpret_cast<const u32*>(row_nnz), n_rows, n_rows, c_row_ptr, tmp);
+  for (i64 h = threadIdx.x; h < n_heavy; h += kFinishThreads) {
+    const i64 a = row_task_off[h], b = row_task_off[h + 1];
+    const i64 shift = c_row_ptr[x_heavy[h]] - nnz_off[a];
+    for (i64 t = a; t < b; ++t) base[t] = nnz_off[t] + shift;
+  }
+  for (i64 t = threadIdx.x; t * tile < heavy; t += kFinishThreads) meta[t] = tile_bounds(nnz_off, n_tasks, 0, heavy, tile, t);
+  if (threadIdx.x < 9) host_totals[threadIdx.x] = threadIdx.x == 1 ? heavy : totals[threadIdx.x];
+  if (threadIdx.x == 0) *host_total = all;  // (the host reads after a synchronisation)
+}
+
+// The plan's side of small products: tasks per row, their prefix sums and the tasks themselves in one launch of one block.
+// The tables have room for an upper bound, so the host does not wait for the number of tasks.
+__global__ void __launch_bounds__(kFinishThreads) k_plan_small(const u32* counts, const i64* heavy_base, i64 n_heavy, TaskRules r,
+                                                               u32* row_tasks, i64* row_task_off, const int32_t* x_heavy,
+                                                               const i64* a_row_ptr, const u32* parts_tab, TaskTables tt) {
+  __shared__ i64 tmp[33];
+  for (i64 h = threadIdx.x; h < n_heavy; h += kFinishThreads)
+    row_tasks[h] = cut_row(counts + h * r.granules, static_cast<u32>(heavy_base[h + 1] - heavy_base[h]), r, [](int, int, u32, u32) {});
+  __syncthreads();
+  finish_scan(row_tasks, n_heavy, n_heavy, row_task_off, tmp);
+  for (i64 h = threadIdx.x; h < n_heavy; h += kFinishThreads)
+    emit_row(counts, heavy_base, h, 0, r, row_task_off[h], x_heavy, a_row_ptr, parts_tab, tt);
 }
 
 }  // namespace gm
