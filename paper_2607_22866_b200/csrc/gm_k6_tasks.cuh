@@ -298,10 +298,12 @@ struct RoundSize {
 // The products of a round that fall to warp `warp` of `n_warps`: a contiguous, equal share, 32 at a time and U times that in
 // flight: load(u, position in B, a) for the valid lanes of U windows, then use(u, valid) for each.  `load` only requests;
 // arithmetic on what it loads would wait there, window after window.
-// Most windows lie inside one piece; then the piece's data are in registers.  Otherwise every lane finds its piece from the
-// ones that start inside the window.  (Windows that end with their piece, the remaining lanes idle, took fewer instructions
-// per window and more time: with pieces of a few dozen products a warp has no more than one or two windows in flight.
-// R-MAT scale 19: 37.7 and 33.1 ms for the mid and the big tasks, against 26.9 and 23.6.)
+// Every lane finds its piece from the ones that start inside the windows, all U windows at once: the chain from one round of U
+// windows to the next is one look at the piece starts and a population count.  (Window after window, with a way of its own for
+// windows inside one piece, the chain of four dependent shared-memory loads per window bound the mid-size tasks: R-MAT scale 19
+// fp32 27.0 ms against 23.1, scale 17 fp64 1.66 against 1.52, block-dense fp32 0.65 against 0.51.  A second set of windows
+// requested before the first is used: 27.9, the registers cost more.  Windows that end with their piece, the remaining
+// lanes idle: 37.7.)
 template <typename V, int CAP, int U, typename Load, typename Use>
 __device__ __forceinline__ void walk_products(const Pieces<V, CAP>& pc, const RoundSize& rs, int warp, int n_warps, Load load, Use use) {
   int f = static_cast<int>((static_cast<i64>(rs.products) * warp) / n_warps);
@@ -314,35 +316,28 @@ __device__ __forceinline__ void walk_products(const Pieces<V, CAP>& pc, const Ro
     const int mid = (cur + hi + 1) >> 1;
     if (pc.ex[mid] <= f) cur = mid; else hi = mid - 1;
   }
-  int next = pc.ex[cur + 1];                                  // first product of the piece after the current one
-  u32 base = pc.base[cur] + static_cast<u32>(lane);
-  V a = pc.a[cur];
-  for (; f < f1; ) {
-    const int f_use = f;
+  for (; f < f1; f += U * 32) {
+    // pieces that start inside the U windows, as masks over the windows' positions
+    u32 heads[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) heads[u] = 0u;
+    for (int i = cur + 1 + lane;; i += 32) {
+      const u32 d = static_cast<u32>(pc.ex[i] - f);
+      if (U <= 2 && !__any_sync(0xffffffffu, d < U * 32u)) break;  // (inside one piece; four windows seldom are)
+#pragma unroll
+      for (int u = 0; u < U; ++u) heads[u] |= __reduce_or_sync(0xffffffffu, d - u * 32 < 32u ? 1u << (d & 31) : 0u);
+      if (!__all_sync(0xffffffffu, d < U * 32u)) break;  // (usually at once; ex is sorted)
+    }
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      if (f < f1) {  // (uniform)
-        if (f + 32 < next) {  // (uniform)
-          if (f + lane < f1) load(u, base + static_cast<u32>(f), a);
-        } else {
-          // pieces that start inside the window (after its first product), as a mask over its positions
-          const int d = pc.ex[cur + 1 + lane] - f;
-          const u32 heads = __reduce_or_sync(0xffffffffu, d < 32 ? 1u << d : 0u);
-          const int q = cur + __popc(heads & upto);
-          if (f + lane < f1) load(u, pc.base[q] + static_cast<u32>(f + lane), pc.a[q]);
-          // the window after this one starts in the piece of this one's last product, or in the next
-          cur += __popc(heads);
-          if (pc.ex[cur + 1] <= f + 32) ++cur;
-          next = pc.ex[cur + 1];
-          base = pc.base[cur < CAP ? cur : 0] + static_cast<u32>(lane);
-          a = pc.a[cur < CAP ? cur : 0];
-        }
-        f += 32;
-      }
+      const int q = cur + __popc(heads[u] & upto);
+      const int g = f + u * 32 + lane;
+      if (g < f1) load(u, pc.base[q] + static_cast<u32>(g), pc.a[q]);
+      cur += __popc(heads[u]);
     }
 #pragma unroll
     for (int u = 0; u < U; ++u)
-      if (f_use + u * 32 < f1) use(u, f_use + u * 32 + lane < f1);
+      if (f + u * 32 < f1) use(u, f + u * 32 + lane < f1);
   }
 }
 
