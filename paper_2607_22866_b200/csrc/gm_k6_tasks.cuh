@@ -974,6 +974,7 @@ __global__ void __launch_bounds__(kFinishThreads) k_finish_small(const u32* task
 
 // The plan's side of small products: tasks per row, their prefix sums and the tasks themselves in one launch of one block.
 // The tables have room for an upper bound, so the host does not wait for the number of tasks.
+// (Zipf-like, 4096 rows: 319 us with a count, a wait and an allocation in between, 284 with this.)
 __global__ void __launch_bounds__(kFinishThreads) k_plan_small(const u32* counts, const i64* heavy_base, i64 n_heavy, TaskRules r,
                                                                u32* row_tasks, i64* row_task_off, const int32_t* x_heavy,
                                                                const i64* a_row_ptr, const u32* parts_tab, TaskTables tt) {

@@ -4,7 +4,8 @@ import numpy as np
 import pytest
 
 import gen
-from parity import check_product
+import paper_2607_22866_b200 as gm
+from parity import check_product, make_opts
 
 pytestmark = pytest.mark.gpu
 
@@ -53,3 +54,36 @@ def test_products_that_cancel_keep_their_entry(dtype):
     A = gen.CSR(2, 2, np.array([0, 2, 3]), np.array([0, 1, 1], np.int32), np.array([2, 2, -1], dtype))
     C, info, stats = check_product(A, B, tau=16)
     assert C.nnz == 2 * cols.size and not C.val[:cols.size].any()
+
+
+@pytest.mark.parametrize("n_rows", [1, 2, 1023, 1024, 1025, 4095, 4096, 4097, 16383, 16384, 16385])
+def test_small_products_counted_by_one_block(n_rows):
+    # the one-block launches around the sums: one heavy row, and 16384 rows of A and one more (separate launches); heavy
+    # rows first, last and between empty and light ones; a kept plan executed again gives the same structure
+    rng = np.random.default_rng(n_rows)
+    m, n_cols = 500, 40000
+    B = _csr([_row(rng, n_cols, int(k), 2000) for k in rng.integers(20, 60, m)], n_cols, rng, np.float32)
+    heavy = {0, n_rows - 1, n_rows // 2, n_rows // 3}
+    rows = [rng.choice(m, 40 + i % 3 * 100, replace=False) if i in heavy else rng.choice(m, i % 3, replace=False) for i in range(n_rows)]
+    A = _csr(rows, m, rng, np.float32)
+    C, info, stats = check_product(A, B, tau=512)
+    assert info.rows_heavy == len(heavy)
+    dA, dB = gm.DeviceCSR.from_host(A), gm.DeviceCSR.from_host(B)
+    plan = gm.spgemm_plan(dA, dB, opts=make_opts(tau=512))
+    for _ in range(2):
+        D = gm.spgemm_execute(plan)
+        assert D.row_ptr.equal(C.row_ptr) and D.col.equal(C.col)
+
+
+@pytest.mark.parametrize("dtype", [np.float32, np.float64])
+@pytest.mark.parametrize("lengths", [(1,), (1, 2, 3), (31, 32, 33), (63, 64, 65), (1, 127, 128, 129), (1, 500)])
+def test_pieces_shorter_and_longer_than_the_windows(dtype, lengths):
+    # rows of B of the lengths at which a round of windows starts, ends or holds many of them: up to 128 pieces in one
+    # round, a piece that starts at the first product of a window or of the next round, pieces longer than a round
+    rng = np.random.default_rng(sum(lengths))
+    m, n_cols = 1500, 30000
+    B = _csr([_row(rng, n_cols, lengths[i % len(lengths)], 900) for i in range(m)], n_cols, rng, dtype)
+    rows = [rng.choice(m, k, replace=False) for k in (64, 65, 127, 128, 129, 255, 256, 257, 384, 385, 700, 1499)] + [np.arange(m)]
+    A = _csr(rows, m, rng, dtype)
+    C, info, stats = check_product(A, B, tau=16)
+    assert info.rows_heavy == len(rows)
