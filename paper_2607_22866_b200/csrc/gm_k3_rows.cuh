@@ -151,7 +151,7 @@ struct SortSmem {
   i64 base[32];   // per (non-empty) row of B of the current 32 entries of A: its start minus its first product
   V a[32];
   V val[32 * KMAX];
-  Key key[32 * KMAX];
+  alignas(16) Key key[32 * KMAX];
 };
 
 // The products of A[s..e) into sm.key / sm.val; returns how many.

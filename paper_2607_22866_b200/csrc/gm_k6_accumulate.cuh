@@ -179,7 +179,7 @@ __global__ void __launch_bounds__(kSmallWarps * 32, kSmallBlocksPerSm) k6_small_
     u64* __restrict__ totals,  // [0] += products, [1] += entries of the chunks handled here (statistics)
     const unsigned char* __restrict__ tags,  // per chunk, or NULL: != 0 for chunks that left the hierarchy early
     int32_t* x_col_alt, V* x_val_alt, ExitTags xt) {
-  __shared__ u32 s_key[kSmallWarps][32 * kSmallMaxPerLane];
+  __shared__ __align__(16) u32 s_key[kSmallWarps][32 * kSmallMaxPerLane];
   __shared__ V s_val[kSmallWarps][32 * kSmallMaxPerLane];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const i64 n_groups = (n_chunks + 31) >> 5;

@@ -421,7 +421,7 @@ __global__ void __launch_bounds__(kSmallWarps * 32, KMAX > 4 ? 8 : 10) k6_small_
     u64* __restrict__ totals) {  // [0] += products, [1] += entries (statistics)
   __shared__ u32 s_base[kSmallWarps][32];
   __shared__ V s_a[kSmallWarps][32];
-  __shared__ u32 s_key[kSmallWarps][32 * KMAX];
+  __shared__ __align__(16) u32 s_key[kSmallWarps][32 * KMAX];
   __shared__ V s_val[kSmallWarps][32 * KMAX];
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int n_list = counters[0];

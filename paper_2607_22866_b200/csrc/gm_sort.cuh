@@ -5,76 +5,96 @@
 
 namespace gm {
 
-// Sorts 32 * K packed keys, K per lane, element e = r * 32 + lane in key[r]; ascending in e afterwards.
-// Steps whose partner sits in another lane are the same instruction sequence for every step width, so they run
-// as loops over the width; only the steps that pair registers are unrolled.  (Fully unrolled, the networks of
-// all K together did not fit the instruction cache, and the warps of a block run different K.)
+// Sorts 32 * K packed keys, K per lane, ascending; element e = lane * K + r ends in key[r] (a bitonic network whose merges
+// begin with the mirrored partner, so that every run is ascending).
+// A lane's elements are neighbours, so that the short strides, which every merge ends with, stay inside the lane: 15 of the 36
+// steps for 256 keys exchange with another lane, against 33 with element r * 32 + lane in key[r], and an exchange takes a
+// shuffle per key, of which an SM does one at a time.  (ER, 30011 rows of 144 products fp64:
+// 75 -> 62 us; the sorts of the Zipf pair with 64-bit keys, rows up to 1024 products: the whole product 5.42 -> 4.95 ms.)
+// The merges across lanes are the same instruction sequence for every width and run as a loop; only the steps inside a lane
+// are unrolled.  (Fully unrolled, the networks of all K together did not fit the instruction cache, and the warps of a block
+// run different K.)
 template <typename Key, int K>
 __device__ __forceinline__ void warp_sort_keys(Key (&key)[K], int lane) {
-  auto lane_step = [&](int mask, bool lower) {  // partner: same register, lane ^ mask; the lower lane keeps the smaller key
+  auto order = [](Key& a, Key& b) {
+    const Key lo = min(a, b);
+    b = max(a, b);
+    a = lo;
+  };
+  auto strides_in_lane = [&](int from) {  // partner e ^ j for j = from .. 1
 #pragma unroll
-    for (int r = 0; r < K; ++r) {
-      const Key o = __shfl_xor_sync(0xffffffffu, key[r], mask);
-      key[r] = lower ? min(key[r], o) : max(key[r], o);
+    for (int j = K / 2; j > 0; j >>= 1) {
+      if (j > from) continue;
+#pragma unroll
+      for (int r = 0; r < K; ++r)
+        if ((r & j) == 0) order(key[r], key[r | j]);
     }
   };
-  // merges inside one register row (k = 2 .. 32): first step partner e ^ (k - 1), then e ^ j for j = k/4 .. 1
-#pragma unroll 1
-  for (int k = 2; k <= 32; k <<= 1) {
-    lane_step(k - 1, (lane & (k >> 1)) == 0);
-#pragma unroll 1
-    for (int j = k >> 2; j > 0; j >>= 1) lane_step(j, (lane & j) == 0);
+  // runs of K in every lane
+#pragma unroll
+  for (int k = 2; k <= K; k <<= 1) {
+#pragma unroll
+    for (int r = 0; r < K; ++r)
+      if ((r ^ (k - 1)) > r) order(key[r], key[r ^ (k - 1)]);
+    strides_in_lane(k / 4);
   }
-  // merges across register rows (k = 64 .. 32 K)
+  // merges of the runs of w lanes with their neighbours'; the lower lane of a pair keeps the smaller keys
+#pragma unroll 1
+  for (int w = 1; w < 32; w <<= 1) {
+    const bool lower = (lane & w) == 0;
+    const int mask = 2 * w - 1;
 #pragma unroll
-  for (int k = 64; k <= 32 * K; k <<= 1) {
-    const int rm = k / 32 - 1;  // first step: partner register r ^ rm, partner lane lane ^ 31
-#pragma unroll
-    for (int r = 0; r < K; ++r) {
-      if ((r ^ rm) > r) {
-        const Key a = key[r], b = key[r ^ rm];
-        const Key oa = __shfl_xor_sync(0xffffffffu, b, 31);
-        const Key ob = __shfl_xor_sync(0xffffffffu, a, 31);
-        key[r] = min(a, oa);
-        key[r ^ rm] = max(b, ob);
+    for (int r = 0; r < (K + 1) / 2; ++r) {  // mirrored: register K - 1 - r of lane ^ mask
+      const Key a = key[r], b = key[K - 1 - r];
+      const Key oa = __shfl_xor_sync(0xffffffffu, b, mask);
+      key[r] = lower ? min(a, oa) : max(a, oa);
+      if (K > 1) {
+        const Key ob = __shfl_xor_sync(0xffffffffu, a, mask);
+        key[K - 1 - r] = lower ? min(b, ob) : max(b, ob);
       }
     }
-#pragma unroll
-    for (int j = k >> 2; j >= 32; j >>= 1) {  // partner in the same lane
-      const int rj = j / 32;
+#pragma unroll 1
+    for (int j = w >> 1; j > 0; j >>= 1) {
+      const bool first = (lane & j) == 0;
 #pragma unroll
       for (int r = 0; r < K; ++r) {
-        if ((r & rj) == 0) {
-          const Key a = key[r], b = key[r | rj];
-          key[r] = min(a, b);
-          key[r | rj] = max(a, b);
-        }
+        const Key o = __shfl_xor_sync(0xffffffffu, key[r], j);
+        key[r] = first ? min(key[r], o) : max(key[r], o);
       }
     }
-#pragma unroll 1
-    for (int j = 16; j > 0; j >>= 1) lane_step(j, (lane & j) == 0);
+    strides_in_lane(K / 2);
   }
 }
 
 // Sorted keys (n valid ones) -> entries: the lane that owns a run's first element adds the run up in the order of the
 // positions (the low BITS bits of a key, indices into s_val) and writes it; returns the number of runs.
-// s_key: 32 * K entries of this warp's shared memory.
+// s_key: 32 * K entries of this warp's shared memory, 16-byte aligned.
 template <typename V, typename Key, int K, int BITS>
 __device__ __forceinline__ int warp_sum_runs(const Key (&key)[K], int n, Key* s_key, const V* s_val, u32 col_base, int32_t* col, V* val) {
   const int lane = threadIdx.x & 31;
+  constexpr int kVec = 16 / sizeof(Key);
+  if constexpr (K % kVec == 0) {
 #pragma unroll
-  for (int r = 0; r < K; ++r) s_key[r * 32 + lane] = key[r];
+    for (int r = 0; r < K; r += kVec) {
+      if constexpr (sizeof(Key) == 4) *reinterpret_cast<uint4*>(s_key + lane * K + r) = make_uint4(key[r], key[r + 1], key[r + 2], key[r + 3]);
+      else *reinterpret_cast<ulonglong2*>(s_key + lane * K + r) = make_ulonglong2(key[r], key[r + 1]);
+    }
+  } else {
+#pragma unroll
+    for (int r = 0; r < K; ++r) s_key[lane * K + r] = key[r];
+  }
   __syncwarp();
   int base = 0;
 #pragma unroll
   for (int r = 0; r < K; ++r) {
     if (r * 32 < n) {  // warp-uniform
       const int e = r * 32 + lane;
-      const Key c = key[r] >> BITS;
+      const Key k = s_key[e];
+      const Key c = k >> BITS;
       const bool head = e < n && (e == 0 || (s_key[e - 1] >> BITS) != c);
       const u32 heads = __ballot_sync(0xffffffffu, head);
       if (head) {
-        V sum = s_val[static_cast<u32>(key[r]) & ((1u << BITS) - 1u)];
+        V sum = s_val[static_cast<u32>(k) & ((1u << BITS) - 1u)];
         for (int q = e + 1; q < n; ++q) {
           const Key kq = s_key[q];
           if ((kq >> BITS) != c) break;
