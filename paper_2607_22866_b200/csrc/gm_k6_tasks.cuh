@@ -736,9 +736,10 @@ __global__ void __launch_bounds__(kMidThreads, 6) k6_mid_tasks(
 // ---------------------------------------------------------------------------------------------------------------------
 // big tasks: the dense accumulator
 // ---------------------------------------------------------------------------------------------------------------------
-// One value per column of the granule.  An idle slot holds -0.0, the identity of the addition, and a product is formed as
-// fma(a, b, +0.0), so that a slot that received anything is never -0.0 again: which columns have an entry is read off the
-// values, and a product costs one shared-memory add and nothing else.  The flush goes over the granule twice: every warp
+// One value per column of the granule.  An idle slot holds -0.0, the identity of the addition, and a product that is a zero
+// of either sign is added as +0.0, so that a slot that received anything is never -0.0 again: which columns have an entry
+// is read off the values, and a product costs one shared-memory add and nothing else.  (Rounded to the product first, then
+// +0.0 added: fma(a, b, +0.0) is -0.0 where a negative product underflows, and the column would have no entry.)  The flush goes over the granule twice: every warp
 // counts the entries of its share, the block adds the counts up, and the warp writes its share, a 16-byte word per lane at a
 // time (128 columns in fp32; 32 columns at a time took 36 instructions for each 32).
 // Bank spreading: the low bits of a power-law matrix's columns are mostly zero; the slot of a column inside its group of
@@ -762,8 +763,8 @@ template <typename V>
 __device__ __forceinline__ u32 group_xor(u32 group) { return (group ^ (group >> 5)) & (32u - 16u / sizeof(V)); }
 template <typename V>
 __device__ __forceinline__ u32 big_slot(u32 c, u32 mask) { return (c & mask) ^ group_xor<V>(c >> 5); }
-__device__ __forceinline__ float product(float a, float b) { return __fmaf_rn(a, b, 0.0f); }
-__device__ __forceinline__ double product(double a, double b) { return __fma_rn(a, b, 0.0); }
+__device__ __forceinline__ float product(float a, float b) { return plus_zero(__fmul_rn(a, b)); }
+__device__ __forceinline__ double product(double a, double b) { return plus_zero(__dmul_rn(a, b)); }
 
 // slots of a 16-byte word of the accumulator that received something
 __device__ __forceinline__ u32 touched_in(const int4& x, float) {

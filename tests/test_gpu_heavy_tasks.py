@@ -4,8 +4,9 @@ import numpy as np
 import pytest
 
 import gen
+import oracle
 import paper_2607_22866_b200 as gm
-from parity import check_product, make_opts
+from parity import check_product, make_opts, run_gpu
 
 pytestmark = pytest.mark.gpu
 
@@ -54,6 +55,27 @@ def test_products_that_cancel_keep_their_entry(dtype):
     A = gen.CSR(2, 2, np.array([0, 2, 3]), np.array([0, 1, 1], np.int32), np.array([2, 2, -1], dtype))
     C, info, stats = check_product(A, B, tau=16)
     assert C.nnz == 2 * cols.size and not C.val[:cols.size].any()
+
+
+@pytest.mark.parametrize("mid", [0, 16])  # hand-over to the dense accumulator: default, and nearly everything
+@pytest.mark.parametrize("dtype", [np.float32, np.float64])
+def test_products_that_underflow_keep_their_entry(dtype, mid):
+    # products of either sign that round to zero, or to a subnormal, alone in their column and next to others.  The bound:
+    # each of at most four products is off by half the smallest subnormal, sums of subnormals are exact, and the oracle's
+    # result is rounded once.
+    rng = np.random.default_rng(11)
+    n_cols, info = 20000, np.finfo(dtype)
+    tiny = dtype(1e-30) if dtype == np.float32 else dtype(1e-200)  # (its square underflows)
+    B = _csr([rng.choice(n_cols, 6000, replace=False) for _ in range(4)], n_cols, rng, dtype)
+    B.val[:] = np.where(B.val < 0, -tiny, tiny)
+    sub = info.smallest_subnormal / tiny * 8  # times tiny: a few subnormals
+    A = gen.CSR(4, 4, np.array([0, 1, 2, 4, 8]), np.array([0, 1, 2, 3, 0, 1, 2, 3], np.int32),
+                np.array([-tiny, tiny, tiny, -tiny, -sub, tiny, -tiny, sub], dtype))
+    C, plan, _ = run_gpu(A, B, tau=16, mid_chunk_max=mid, small_chunk_max=mid, validate_inputs=1)
+    ref = oracle.spgemm(A, B)
+    assert plan.rows_heavy == 4
+    assert np.array_equal(C.row_ptr.cpu().numpy(), ref.row_ptr) and np.array_equal(C.col.cpu().numpy(), ref.col)
+    assert np.all(np.abs(C.val.cpu().numpy().astype(np.longdouble) - ref.val) <= 4 * info.smallest_subnormal)
 
 
 @pytest.mark.parametrize("n_rows", [1, 2, 1023, 1024, 1025, 4095, 4096, 4097, 16383, 16384, 16385])
