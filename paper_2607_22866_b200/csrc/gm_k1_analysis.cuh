@@ -87,7 +87,8 @@ __device__ __forceinline__ i64 find_row(const i64* __restrict__ row_ptr, i64 n_r
   return lo;
 }
 
-// P: type of a warp's prefix sums.  A warp has T / 8 entries of the tile, so 32 bits do when B has at most 2^24 columns.
+// P: type of a warp's prefix sums.  A warp has T / 8 entries of the tile, at most 256, so 32 bits do for what is before
+// each of them when B has at most 2^24 columns; the warp's total, which can be 2^32 then, is kept in 64.
 template <int T, typename P>
 struct K1Tile {
   i64 r0, r1;  // row of the first item, and of the first item after the tile
@@ -132,14 +133,14 @@ __device__ __forceinline__ void k1_load_tile(K1Tile<T, P>& s, const i64* __restr
     }
   }
   for (int i = tid; i <= nr; i += kK1Threads) s.off[i] = static_cast<int>(max(a_row_ptr[r0 + i] - e0, i64{0}));
-  P run = 0;
+  i64 run = 0;
 #pragma unroll
   for (int k = 0; k < kPer; ++k) {
     const P inc = warp_inclusive_scan(static_cast<P>(len[k]));
-    s.pre[q0 + k * 32] = run + inc - static_cast<P>(len[k]);
-    run += __shfl_sync(0xffffffffu, inc, 31);
+    s.pre[q0 + k * 32] = static_cast<P>(run) + inc - static_cast<P>(len[k]);
+    run += static_cast<i64>(__shfl_sync(0xffffffffu, inc, 31));
   }
-  if (lane == 0) s.sum[warp] = static_cast<i64>(run);
+  if (lane == 0) s.sum[warp] = run;
   __syncthreads();
   if (tid <= kK1Threads / 32) {
     i64 base = 0;

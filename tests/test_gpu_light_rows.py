@@ -65,3 +65,17 @@ def test_rows_of_every_length_across_tiles():
         out = torch.full((A.n_rows,), -1, dtype=torch.int64, device="cuda")
         assert np.array_equal(gm.row_products_noalloc(dA, dB, out).cpu().numpy(), ref)
     check_product(A, B)
+
+
+@pytest.mark.parametrize("n_cols", [1 << 24, (1 << 24) + 1])  # 32-bit prefix sums, and the first width with 64-bit ones
+@pytest.mark.parametrize("n_rows", [40000, 80000])  # small and large tiles
+def test_row_products_of_full_rows(n_rows, n_cols):
+    # every entry of A meets a full row of B: a warp of a large tile adds up 256 of them, 2^32 products at 2^24 columns
+    import paper_2607_22866_b200 as gm
+    A = gm.DeviceCSR(n_rows, 1, torch.arange(n_rows + 1, device="cuda"), torch.zeros(n_rows, dtype=torch.int32, device="cuda"),
+                     torch.ones(n_rows, device="cuda"))
+    B = gm.DeviceCSR(1, n_cols, torch.tensor([0, n_cols], device="cuda"), torch.arange(n_cols, dtype=torch.int32, device="cuda"),
+                     torch.ones(n_cols, device="cuda"))
+    out = torch.full((n_rows,), -1, dtype=torch.int64, device="cuda")
+    gm.row_products_noalloc(A, B, out)
+    assert bool((out == n_cols).all())
