@@ -1540,16 +1540,11 @@ static int execute_t(gm_plan* p, cudaStream_t st, gm_csr* C) {
   if (tm.enabled) { ev_total0 = tm.get(); ev_total1 = tm.get(); cudaEventRecord(ev_total0, st); }
 
   HostSlot* const slot = p->slot;
-  slot->err[0] = 0;  // (nothing of this plan is in flight: every execute ends with a synchronisation)
+  slot->err[0] = 0;  // (nothing of this plan is in flight: every return of an execute has waited for its streams)
   slot->c_total = 0;
-  if (p->use_tasks)
-    GM_CUDA(cudaMemsetAsync(p->c_total, 0, reinterpret_cast<char*>(p->task_tickets + 4 * p->batches.size()) - reinterpret_cast<char*>(p->c_total), st));
-  else if (info.rows_heavy > 0)
-    GM_CUDA(cudaMemsetAsync(p->c_total, 0, 16 * sizeof(int64_t), st));
 
   // ---- result row_ptr
   i64* c_row_ptr = static_cast<i64*>(dev_alloc(static_cast<size_t>(nA + 1) * sizeof(i64), st));
-  if (!c_row_ptr) return fail(GM_ERR_OOM, "allocation of C.row_ptr failed");
   int32_t* c_col = nullptr;
   V* c_val = nullptr;
   // ---- light and heavy rows are independent until C.row_ptr is formed: the light rows' kernels go to a second
@@ -1567,14 +1562,24 @@ static int execute_t(gm_plan* p, cudaStream_t st, gm_csr* C) {
   cudaStream_t lst = fork ? p->light_stream : st;
   auto fork_light = [&]() { if (fork) { cudaEventRecord(p->ev_fork, st); cudaStreamWaitEvent(lst, p->ev_fork, 0); } };
   auto join_light = [&]() { if (fork) { cudaEventRecord(p->ev_light, lst); cudaStreamWaitEvent(st, p->ev_light, 0); } };
-  auto cleanup = [&]() {
+  auto cleanup = [&]() {  // waits for all that is queued: the caller may free or reuse what it reads and writes
+    cudaStreamSynchronize(st);
     if (fork) cudaStreamSynchronize(lst);
     if (p->sink && p->sink->copy_stream) cudaStreamSynchronize(p->sink->copy_stream);  // copies out of C in flight
     dev_free(c_row_ptr, st);
     dev_free(c_col, st);
     dev_free(c_val, st);
   };
-#define GM_TRY_C(expr) do { int rc2_ = (expr); if (rc2_ != GM_OK) { cudaStreamSynchronize(st); cleanup(); return rc2_; } } while (0)
+#define GM_TRY_C(expr) do { int rc2_ = (expr); if (rc2_ != GM_OK) { cleanup(); return rc2_; } } while (0)
+
+  if (!c_row_ptr) { cleanup(); return fail(GM_ERR_OOM, "allocation of C.row_ptr failed"); }
+  if (info.rows_heavy > 0) {
+    char* const end = p->use_tasks ? reinterpret_cast<char*>(p->task_tickets + 4 * p->batches.size()) : reinterpret_cast<char*>(p->c_total + 16);
+    if (cudaMemsetAsync(p->c_total, 0, end - reinterpret_cast<char*>(p->c_total), st) != cudaSuccess) {
+      cleanup();
+      return fail(GM_ERR_CUDA, std::string("clearing the counters failed: ") + cudaGetErrorString(cudaGetLastError()));
+    }
+  }
 
   // ---- light rows, all that does not need C (Algorithm 3: Symbolic(A[x_light,:], B), and for most rows the sums too)
   fork_light();
@@ -1839,11 +1844,10 @@ int gm_spgemm_execute(gm_plan* plan, void* cuda_stream, gm_csr* C_out) {
   if (!plan || !C_out) return fail(GM_ERR_INVALID_ARG, "plan or C_out is null");
   std::memset(C_out, 0, sizeof(*C_out));
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-  if (plan->pending) {
-    if (st != plan->plan_stream) GM_CUDA(cudaStreamSynchronize(plan->plan_stream));
-    plan->pending = false;  // (an execute ends with a synchronisation of its stream)
-  }
-  return plan->A.dtype == GM_F32 ? execute_t<float>(plan, st, C_out) : execute_t<double>(plan, st, C_out);
+  if (plan->pending && st != plan->plan_stream) GM_CUDA(cudaStreamSynchronize(plan->plan_stream));
+  const int rc = plan->A.dtype == GM_F32 ? execute_t<float>(plan, st, C_out) : execute_t<double>(plan, st, C_out);
+  plan->pending = false;  // (whatever the result, the execute has waited for its stream)
+  return rc;
 }
 
 int gm_plan_get_info(const gm_plan* plan, gm_plan_info* out) {
