@@ -81,8 +81,9 @@ typedef struct gm_plan_opts {
                               caller's stream with events, next to the heavy rows' kernels (Algorithm 3)      */
   int32_t level0_multisplit; /* first multisplit level: 1 = separate histogram and multisplit passes over
                               the staging buffer (Algorithm 5 as printed); 2 = the expansion kernel writes
-                              the first level's children itself; 0 (default) = the latter when the heavy
-                              rows' segments are long compared with the fan-out, else the former        */
+                              the first level's children itself; 0 (default) = no level at all where the heavy
+                              rows are summed without staged products (see gm_plan_info.heavy_tasks), else 2 when
+                              their segments are long compared with the fan-out, else 1                 */
   int32_t small_chunk_max; /* final chunks of at most this many products are sorted by one warp each (Section
                               III-A's branch for light chunks); 0 = default (128; 256 for rows that
                               are summed without staged products), -1 = none, at most 512                       */
@@ -138,6 +139,8 @@ typedef struct gm_plan_info {
   int64_t light_bin_rows[8]; /* light rows per size class of the symbolic pass                 */
   int64_t launches;        /* kernels launched while planning                                  */
   int64_t level0_direct;   /* 1: the expansion kernel writes the first level's children itself  */
+  int64_t heavy_tasks;     /* 1: the heavy rows' products are summed where they are generated, in ranges of columns;
+                              nothing is expanded, staged or split.  Only with level0_multisplit and expand_order 0 */
 } gm_plan_info;
 
 /* Filled by the most recent gm_spgemm_execute on the plan.  Times are CUDA-event milliseconds on

@@ -774,18 +774,19 @@ static int build_plan(gm_plan* p, cudaStream_t st) {
     p->csc = p->opts.expand_order == 1;
     p->direct = prm.n_levels > 0 && prm.fanout[0] <= 256 && !p->csc &&
                 (p->opts.level0_multisplit == 2 || (p->opts.level0_multisplit == 0 && long_segments && bounds_fit));
-    info.level0_direct = p->direct ? 1 : 0;
     {
       const size_t warp_smem = stream_warp_smem_bytes(prm.n_levels > 0 ? prm.fanout[0] : 2, p->sv);
       p->stream = p->direct && p->opts.expand_staging == 1 && reinterpret_cast<uintptr_t>(B.col_idx) % 16 == 0 &&
                   reinterpret_cast<uintptr_t>(B.vals) % 16 == 0 && p->smem_bytes >= kStreamWarps * warp_smem + 1024;
     }
-    // Products are summed where they are generated unless the pieces of B's rows get too short: a task looks every row of B up
+    // Products are summed where they are generated, unless a first level is asked for or the pieces of B's rows get too short: a task looks every row of B up
     // in the boundary table, so that costs per (segment, granule) and not per product.  Products per (segment, granule) and time
     // per call, tasks against staged products: R-MAT scale 18 fp64 with 4 edges a vertex about 9, 4.2 against 5.4 ms; R-MAT scale 20
     // fp32 20, 188 against 198 ms; R-MAT scale 21 fp64 3.7, 291 against 278 ms.
-    p->use_tasks = !p->csc && !p->stream && (prm.n_levels == 0 || (prm.n_levels == 1 && p->direct)) && plan_task_rules(p) &&
+    p->use_tasks = p->opts.level0_multisplit == 0 && !p->csc && !p->stream && (prm.n_levels == 0 || (prm.n_levels == 1 && p->direct)) && plan_task_rules(p) &&
                    (p->task_rules.granules <= 8 || info.products_heavy >= kMinPieceProducts * p->n_seg * p->task_rules.granules);
+    info.heavy_tasks = p->use_tasks ? 1 : 0;
+    info.level0_direct = p->direct && !p->use_tasks ? 1 : 0;
     // one staging buffer is enough when no multisplit pass runs (no levels, or one level done by the expansion)
     const int n_buf = prm.n_levels > (p->direct ? 1 : 0) ? 2 : 1;
 

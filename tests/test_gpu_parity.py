@@ -319,7 +319,7 @@ def test_config2_rmat20_full_size_sampled_rows():
     A, B, _ = gen.config_inputs(2)
     info, stats = _check_sampled_rows(A, B, whole_row_ptr=True)
     assert info.n_batches >= 8 and info.params.levels() == [32] and stats.c_capacity >= stats.c_nnz
-    assert info.level0_direct == 1
+    assert info.heavy_tasks == 1 and info.level0_direct == 0
 
 
 def test_config3_rmat21_fp64_full_size_default_plan():
@@ -327,7 +327,7 @@ def test_config3_rmat21_fp64_full_size_default_plan():
     # children written by the expansion kernel, several batches, a result of more than 100 GB
     A, B, _ = gen.config_inputs(3)
     info, stats = _check_sampled_rows(A, B, n_random=150, n_heavy=50)
-    assert info.params.levels() == [128] and info.level0_direct == 1 and info.n_batches > 1
+    assert info.params.levels() == [128] and info.level0_direct == 1 and info.heavy_tasks == 0 and info.n_batches > 1
 
 
 def test_config4_zipf_pair_full_size_default_plan():
@@ -416,13 +416,27 @@ def test_fused_and_stand_alone_histogram_agree(separate):
 
 @pytest.mark.parametrize("dtype,fanout,width", [(np.float32, 4, 512), (np.float64, 32, 256), (np.float32, 256, 32)])
 def test_expansion_straight_into_the_first_level(dtype, fanout, width):
-    # default path: the expansion kernel places every product in its level-0 child from counts alone.
+    # asked for: the expansion kernel places every product in its level-0 child from counts alone.
     # Several batches, one to three levels, and (narrow chunks with fan-out 256) tiles with more
     # (segment, child) pairs than the per-tile table of run starts holds.
     A = gen.rmat(13, 16, seed=11, dtype=dtype)
     C, info, stats = check_product(A, A, tau=256, chunk_width=width, max_fanout=fanout, stage_elems=1 << 20,
                                    level0_multisplit=2)
-    assert info.level0_direct == 1 and info.n_batches > 1 and info.params.n_levels >= 1
+    assert info.level0_direct == 1 and info.heavy_tasks == 0 and info.n_batches > 1 and info.params.n_levels >= 1
+
+
+@pytest.mark.parametrize("level0", [1, 2])
+@pytest.mark.parametrize("width", [16384, 2048])  # no level, one level
+@pytest.mark.parametrize("dtype", [np.float32, np.float64])
+def test_staged_products_where_tasks_are_the_default(dtype, width, level0):
+    # a first level asked for by number is what runs: the same product as tasks and with staged products
+    A = gen.rmat(14, 16, seed=13, dtype=dtype)
+    kw = dict(tau=512, chunk_width=width, stage_elems=1 << 22)
+    C0, info0, _ = check_product(A, A, **kw)
+    assert info0.heavy_tasks == 1 and info0.level0_direct == 0
+    C1, info1, _ = check_product(A, A, level0_multisplit=level0, **kw)
+    assert info1.heavy_tasks == 0 and info1.level0_direct == (1 if level0 == 2 and width == 2048 else 0)
+    assert torch.equal(C0.row_ptr, C1.row_ptr) and torch.equal(C0.col, C1.col)
 
 
 @pytest.mark.parametrize("dtype,fanout,width", [(np.float32, 32, 512), (np.float64, 128, 128), (np.float32, 2, 8192)])
@@ -436,6 +450,7 @@ def test_bulk_copy_expansion_and_plain_loads_agree(dtype, fanout, width):
     C1, info, _ = check_product(A, A, expand_staging=1, **kw)
     assert info.level0_direct == 1 and info.n_batches > 1 and info.params.levels()[0] == fanout
     C2, info2, _ = check_product(A, A, **kw)
+    assert info2.level0_direct == 1 and info2.heavy_tasks == 0
     assert torch.equal(C1.row_ptr, C2.row_ptr) and torch.equal(C1.col, C2.col)
 
 
