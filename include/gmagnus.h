@@ -74,8 +74,8 @@ typedef struct gm_plan_opts {
   int32_t separate_histogram; /* 1: always run the stand-alone histogram kernel per level (otherwise a
                               first level that runs as separate passes is counted by the expansion) */
   int32_t validate_inputs; /* 1: debug mode.  row_ptr / col_idx of A and B are checked on the device first
-                              (GM_ERR_BAD_CSR), and where products are staged, before every chunk accumulation a pass
-                              checks that each product lies in the columns its chunk owns (GM_ERR_INTERNAL)     */
+                              (GM_ERR_BAD_CSR), and before the heavy rows' products are summed a pass checks that each
+                              lies in the columns its chunk or task owns (GM_ERR_INTERNAL)                      */
   int32_t single_stream;   /* 1: every kernel of a call runs on the caller's stream.  0 (default): the light rows'
                               kernels run on a second stream of the plan's, forked from and joined back into the
                               caller's stream with events, next to the heavy rows' kernels (Algorithm 3)      */

@@ -1418,6 +1418,34 @@ static int heavy_batch_front(gm_plan* p, const Batch& b, HeavyBatchState<V>* hs,
   return GM_OK;
 }
 
+static int dev_error_to_status(int code) {
+  switch (code) {
+    case kDevOk: return GM_OK;
+    case kDevCapacity: return fail(GM_ERR_CAPACITY, "C did not fit the room reserved for it (raise c_capacity or stage fewer products)");
+    case kDevTableFull: return fail(GM_ERR_INTERNAL, "a light-row hash table overflowed");
+    case kDevBadChunk: return fail(GM_ERR_INTERNAL, "an intermediate product reached a chunk that does not own its column");
+    case kDevTimeout: return fail(GM_ERR_TIMEOUT, "a bounded wait on an asynchronous copy gave up");
+    default: return fail(GM_ERR_INTERNAL, "unknown device error code");
+  }
+}
+
+template <typename V>
+static TaskInput<V> task_input(const gm_plan* p) {
+  return TaskInput<V>{p->A.col_idx, static_cast<const V*>(p->A.vals), p->B.row_ptr, p->B.col_idx, static_cast<const V*>(p->B.vals),
+                      p->piece_bound, p->task_rules.granules, p->task_rules.log2_g};
+}
+
+// Debug mode: nothing is summed when a product is not in the columns of its task (the sums keep a task's columns in shared memory).
+template <typename V>
+static int validate_tasks(gm_plan* p, cudaStream_t st) {
+  k_validate_tasks<V><<<grid_for(p->info.rows_heavy, 1, p->num_sms, 8), 256, 0, st>>>(task_input<V>(p), p->tasks, p->row_task_off, p->heavy_base,
+                                                                                    p->info.rows_heavy, p->B.n_cols, p->err);
+  ++p->stats.launches;
+  GM_CUDA(cudaGetLastError());
+  GM_CUDA(cudaStreamSynchronize(st));
+  return dev_error_to_status(*static_cast<volatile int*>(&p->slot->err[0]));
+}
+
 // The tasks of one batch: sums into the staging area.  BIG: the dense accumulator's tasks, else the other classes (on the
 // second stream: their blocks fill the SMs as the last big tasks run out).
 template <typename V, bool BIG>
@@ -1430,8 +1458,7 @@ static int task_batch_sums(gm_plan* p, size_t bi, cudaStream_t st) {
   int* tickets = p->task_tickets + 4 * bi;
   int32_t* out_col = p->stage_col[0];
   V* out_val = static_cast<V*>(p->stage_val[0]);
-  const TaskInput<V> in{p->A.col_idx, static_cast<const V*>(p->A.vals), p->B.row_ptr, p->B.col_idx, static_cast<const V*>(p->B.vals),
-                        p->piece_bound, r.granules, r.log2_g};
+  const TaskInput<V> in = task_input<V>(p);
   PhaseTimes& tm = p->times;
   if constexpr (BIG) {
     tm.begin(PhaseTimes::kAccNum, st);
@@ -1517,17 +1544,6 @@ static int task_batch_gather(gm_plan* p, size_t bi, bool bases, const i64* c_row
   return GM_OK;
 }
 
-static int dev_error_to_status(int code) {
-  switch (code) {
-    case kDevOk: return GM_OK;
-    case kDevCapacity: return fail(GM_ERR_CAPACITY, "C did not fit the room reserved for it (raise c_capacity or stage fewer products)");
-    case kDevTableFull: return fail(GM_ERR_INTERNAL, "a light-row hash table overflowed");
-    case kDevBadChunk: return fail(GM_ERR_INTERNAL, "an intermediate product reached a chunk that does not own its column");
-    case kDevTimeout: return fail(GM_ERR_TIMEOUT, "a bounded wait on an asynchronous copy gave up");
-    default: return fail(GM_ERR_INTERNAL, "unknown device error code");
-  }
-}
-
 template <typename V>
 static int execute_t(gm_plan* p, cudaStream_t st, gm_csr* C) {
   const gm_csr& A = p->A;
@@ -1581,6 +1597,8 @@ static int execute_t(gm_plan* p, cudaStream_t st, gm_csr* C) {
       return fail(GM_ERR_CUDA, std::string("clearing the counters failed: ") + cudaGetErrorString(cudaGetLastError()));
     }
   }
+
+  if (p->use_tasks && p->opts.validate_inputs) GM_TRY_C(validate_tasks<V>(p, st));
 
   // ---- light rows, all that does not need C (Algorithm 3: Symbolic(A[x_light,:], B), and for most rows the sums too)
   fork_light();

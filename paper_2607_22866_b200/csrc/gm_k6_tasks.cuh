@@ -283,6 +283,42 @@ __device__ __forceinline__ void find_piece(const TaskInput<V>& in, int32_t k, u3
   }
 }
 
+// Debug mode: every product of heavy row h (a block each) lies in the columns of exactly one task.  The tasks' ranges ascend
+// and do not overlap, the entries of every piece lie in its task's columns, and the pieces hold the row's products.
+template <typename V>
+__global__ void __launch_bounds__(256) k_validate_tasks(TaskInput<V> in, const HeavyTask* __restrict__ tasks, const i64* __restrict__ row_task_off,
+                                                        const i64* __restrict__ heavy_base, i64 n_heavy, i64 n_cols, int* __restrict__ err) {
+  __shared__ i64 s_sum[33];
+  for (i64 h = blockIdx.x; h < n_heavy; h += gridDim.x) {
+    i64 sum = 0;
+    bool bad = false;
+    u32 from = 0;
+    for (i64 id = row_task_off[h]; id < row_task_off[h + 1]; ++id) {
+      const HeavyTask t = tasks[id];
+      bad |= t.lo < from || t.hi <= t.lo;
+      from = t.hi;
+      const i64 before = sum;
+      for (u32 j = threadIdx.x; j < t.n_a; j += 256) {
+        u32 a, b;
+        find_piece(in, in.a_col[t.a0 + j], t.lo, t.hi, a, b);
+        for (u32 q = a; q < b; ++q) {
+          const i64 c = in.b_col[q];
+          bad |= c < static_cast<i64>(t.lo) || c >= static_cast<i64>(t.hi) || c >= n_cols;
+        }
+        sum += static_cast<i64>(b) - static_cast<i64>(a);
+      }
+      i64 n;
+      block_exclusive_scan(sum - before, s_sum, &n);
+      __syncthreads();
+      bad |= t.n != 0 && n != static_cast<i64>(t.n);  // (0: a sub-range, not counted)
+    }
+    i64 n;
+    block_exclusive_scan(sum, s_sum, &n);
+    __syncthreads();
+    if (bad || n != heavy_base[h + 1] - heavy_base[h]) dev_set_error(err, kDevBadChunk);
+  }
+}
+
 // The non-empty pieces of a round of rows of B, in shared memory: piece q holds the products [ex[q], ex[q + 1]) of the
 // round, and product f of it is the entry at position base[q] + f of B, times a[q].
 template <typename V, int CAP>

@@ -2,11 +2,12 @@
 of columns, granules cut into sub-ranges.  Against the oracle, with its tolerance (tau * sum|a*b|)."""
 import numpy as np
 import pytest
+import torch
 
 import gen
 import oracle
 import paper_2607_22866_b200 as gm
-from parity import check_product, make_opts, run_gpu
+from parity import check_product, compare_rows, make_opts, run_gpu
 
 pytestmark = pytest.mark.gpu
 
@@ -109,3 +110,22 @@ def test_pieces_shorter_and_longer_than_the_windows(dtype, lengths):
     A = _csr(rows, m, rng, dtype)
     C, info, stats = check_product(A, B, tau=16)
     assert info.rows_heavy == len(rows)
+
+
+@pytest.mark.parametrize("dtype", [np.float32, np.float64])
+@pytest.mark.parametrize("stage", [0, 1 << 20])  # one batch, several
+def test_debug_mode_finds_products_outside_their_task(dtype, stage):
+    # columns of B that change behind the plan's back: debug mode reports it before anything is summed, and with the columns
+    # of the plan the same plan computes the product
+    A = gen.rmat(12, 16, seed=8, dtype=dtype)
+    dA, dB = gm.DeviceCSR.from_host(A), gm.DeviceCSR.from_host(A)
+    plan = gm.spgemm_plan(dA, dB, opts=make_opts(tau=256, chunk_width=512, validate_inputs=1, stage_elems=stage))
+    assert plan.info().heavy_tasks == 1 and (plan.info().n_batches > 1) == (stage > 0)
+    col = dB.col.clone()
+    for bad in (torch.full_like(col, 5), A.n_cols - 1 - col):
+        dB.col.copy_(bad)
+        with pytest.raises(gm.GmError) as ei:
+            gm.spgemm_execute(plan)
+        assert ei.value.status == -10
+    dB.col.copy_(col)
+    compare_rows(gm.spgemm_execute(plan), oracle.spgemm(A, A), dtype)
