@@ -68,7 +68,7 @@ typedef struct gm_plan_opts {
   int64_t tau;             /* heavy-row threshold: row i is heavy iff IP_i > tau               */
   int32_t chunk_width;     /* W: columns per final chunk (power of two)                        */
   int32_t max_fanout;      /* n_chunksMax: most children one multisplit level may produce (pow2) */
-  int32_t acc_ctas_per_sm; /* 1, 2, 4 or 8: how many chunk accumulators share one SM (sets W)  */
+  int32_t acc_ctas_per_sm; /* 1, 2, 4 or 8: how many dense accumulators share one SM (sets W)  */
   int64_t stage_elems;     /* capacity, in intermediate products, of each staging half-buffer  */
   int64_t c_capacity;      /* room, in entries, reserved for C when heavy rows need > 1 batch  */
   int32_t separate_histogram; /* 1: always run the stand-alone histogram kernel per level (otherwise a
@@ -120,8 +120,8 @@ typedef struct gm_params {
   int32_t n_levels;          /* number of multisplit levels (0 when one chunk covers C.m)      */
   int32_t fanout[GM_MAX_LEVELS]; /* v_chunks: children per parent at each level                */
   int32_t shift[GM_MAX_LEVELS];  /* child at level l = (col >> shift[l]) & (fanout[l] - 1)     */
-  int32_t acc_ctas_per_sm;
-  int32_t acc_block_threads; /* threads of one accumulate block                                  */
+  int32_t acc_ctas_per_sm;   /* chunk accumulators per SM (tasks: gm_plan_info.task_ctas_per_sm) */
+  int32_t acc_block_threads; /* threads of one of them                                           */
 } gm_params;
 
 typedef struct gm_plan_info {
@@ -141,6 +141,8 @@ typedef struct gm_plan_info {
   int64_t level0_direct;   /* 1: the expansion kernel writes the first level's children itself  */
   int64_t heavy_tasks;     /* 1: the heavy rows' products are summed where they are generated, in ranges of columns;
                               nothing is expanded, staged or split.  Only with level0_multisplit and expand_order 0 */
+  int64_t task_ctas_per_sm; /* dense accumulators of the tasks that share one SM (0: no tasks): acc_ctas_per_sm if
+                              that was given, else three                                       */
 } gm_plan_info;
 
 /* Filled by the most recent gm_spgemm_execute on the plan.  Times are CUDA-event milliseconds on

@@ -65,7 +65,8 @@ class PlanInfo(ctypes.Structure):
                 ("rows_light", ctypes.c_int64), ("rows_empty", ctypes.c_int64), ("nnz_a_heavy", ctypes.c_int64),
                 ("c_nnz_upper", ctypes.c_int64), ("n_batches", ctypes.c_int64), ("stage_elems", ctypes.c_int64),
                 ("workspace_bytes", ctypes.c_int64), ("light_bin_rows", ctypes.c_int64 * 8),
-                ("launches", ctypes.c_int64), ("level0_direct", ctypes.c_int64), ("heavy_tasks", ctypes.c_int64)]
+                ("launches", ctypes.c_int64), ("level0_direct", ctypes.c_int64), ("heavy_tasks", ctypes.c_int64),
+                ("task_ctas_per_sm", ctypes.c_int64)]
 
 
 class ExecStats(ctypes.Structure):

@@ -472,8 +472,8 @@ static bool plan_task_rules(gm_plan* p) {
   const gm_plan_opts& o = p->opts;
   if (p->B.nnz >= (i64{1} << 32) || p->B.n_rows == 0) return false;  // piece boundaries are 32-bit positions in B's arrays
   // kBigBlocks accumulators per SM unless another number was asked for
-  const int ctas = prm.acc_ctas_per_sm == 1 ? kBigBlocks : prm.acc_ctas_per_sm;
-  const int bt = prm.acc_ctas_per_sm == 1 ? kBigThreads : 1024 / ctas;
+  const int ctas = o.acc_ctas_per_sm == 0 ? kBigBlocks : o.acc_ctas_per_sm;
+  const int bt = o.acc_ctas_per_sm == 0 ? kBigThreads : 1024 / ctas;
   const size_t budget = p->smem_bytes / static_cast<size_t>(ctas) - 1024;
   i64 w = prm.chunk_width;
   auto smem = [&](i64 width) { return p->sv == 4 ? big_task_smem_bytes<float>(static_cast<int>(width), bt) : big_task_smem_bytes<double>(static_cast<int>(width), bt); };
@@ -786,6 +786,7 @@ static int build_plan(gm_plan* p, cudaStream_t st) {
     p->use_tasks = p->opts.level0_multisplit == 0 && !p->csc && !p->stream && (prm.n_levels == 0 || (prm.n_levels == 1 && p->direct)) && plan_task_rules(p) &&
                    (p->task_rules.granules <= 8 || info.products_heavy >= kMinPieceProducts * p->n_seg * p->task_rules.granules);
     info.heavy_tasks = p->use_tasks ? 1 : 0;
+    info.task_ctas_per_sm = p->use_tasks ? p->acc_blocks : 0;
     info.level0_direct = p->direct && !p->use_tasks ? 1 : 0;
     // one staging buffer is enough when no multisplit pass runs (no levels, or one level done by the expansion)
     const int n_buf = prm.n_levels > (p->direct ? 1 : 0) ? 2 : 1;
@@ -1471,6 +1472,7 @@ static int task_batch_sums(gm_plan* p, size_t bi, cudaStream_t st) {
     kern<<<grid, BT, smem, st>>>(in, tasks, n, p->task_list[2] + t0, counters, tickets, out_col, out_val, p->chunk_nnz);  \
   } while (0)
     if (p->acc_blocks == kBigBlocks && p->acc_threads == kBigThreads) GM_BIG(kBigThreads, kBigBlocks);
+    else if (p->acc_blocks == 1) GM_BIG(1024, 1);
     else if (p->acc_blocks == 2) GM_BIG(512, 2);
     else if (p->acc_blocks == 4) GM_BIG(256, 4);
     else GM_BIG(128, 8);

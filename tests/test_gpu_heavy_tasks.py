@@ -129,3 +129,12 @@ def test_debug_mode_finds_products_outside_their_task(dtype, stage):
         assert ei.value.status == -10
     dB.col.copy_(col)
     compare_rows(gm.spgemm_execute(plan), oracle.spgemm(A, A), dtype)
+
+
+@pytest.mark.parametrize("dtype", [np.float32, np.float64])
+@pytest.mark.parametrize("ctas", [0, 1, 2, 4, 8])
+def test_accumulators_per_sm_as_asked(dtype, ctas):
+    # few products to a hand-over, so that the dense accumulator takes most tasks; several batches
+    A = gen.rmat(13, 16, seed=8, dtype=dtype)
+    C, info, _ = check_product(A, A, tau=256, acc_ctas_per_sm=ctas, small_chunk_max=32, mid_chunk_max=64, stage_elems=1 << 22)
+    assert info.heavy_tasks == 1 and info.task_ctas_per_sm == (ctas or 3)
