@@ -466,6 +466,13 @@ static int launch_row_analysis(gm_plan* p, K1Totals* totals, HeavyTile* tiles, u
 }
 
 constexpr i64 kMinPieceProducts = 5;
+
+// Most bytes a table per row of B (boundaries of children or of granules) may take: 1 GB, or what a staging buffer of the
+// default size takes.
+static i64 table_room(const gm_plan* p) {
+  return std::max<i64>(i64{1} << 30, std::min<i64>(p->info.products_heavy, i64{1} << 29) * (4 + p->sv));
+}
+
 // Sizes of the heavy rows' tasks; false: they do not fit (then the rows go through the staged products).
 static bool plan_task_rules(gm_plan* p) {
   const gm_params& prm = p->info.params;
@@ -481,6 +488,7 @@ static bool plan_task_rules(gm_plan* p) {
   if (smem(w) > budget) return false;
   const i64 granules = (prm.chunk_width / w) * prm.chunks_required;
   if (granules > 512) return false;
+  if ((p->B.n_rows * (granules + 1) + (granules > 1 ? p->info.rows_heavy * granules : 0)) * 4 > table_room(p)) return false;
   p->acc_width = static_cast<int>(w);
   p->acc_threads = bt;
   p->acc_blocks = ctas;
@@ -767,10 +775,9 @@ static int build_plan(gm_plan* p, cudaStream_t st) {
     // with F0 = 256 and ~60 products per segment measured 3x slower that way).
     const bool long_segments = prm.n_levels > 0 &&
                                info.products_heavy >= 2 * static_cast<i64>(prm.fanout[0]) * std::max<i64>(info.nnz_a_heavy, 1);
-    // ... and a table of F0 + 1 boundaries per row of B, which must stay small (at most 1 GB, or what a staging
-    // buffer of the default size takes)
+    // ... and a table of F0 + 1 boundaries per row of B, which must stay small
     const i64 bound_bytes = prm.n_levels > 0 ? B.n_rows * static_cast<i64>(prm.fanout[0] + 1) * 4 : 0;
-    const bool bounds_fit = bound_bytes <= std::max<i64>(i64{1} << 30, std::min<i64>(info.products_heavy, i64{1} << 29) * (4 + p->sv));
+    const bool bounds_fit = bound_bytes <= table_room(p);
     p->csc = p->opts.expand_order == 1;
     p->direct = prm.n_levels > 0 && prm.fanout[0] <= 256 && !p->csc &&
                 (p->opts.level0_multisplit == 2 || (p->opts.level0_multisplit == 0 && long_segments && bounds_fit));

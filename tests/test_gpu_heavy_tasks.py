@@ -138,3 +138,20 @@ def test_accumulators_per_sm_as_asked(dtype, ctas):
     A = gen.rmat(13, 16, seed=8, dtype=dtype)
     C, info, _ = check_product(A, A, tau=256, acc_ctas_per_sm=ctas, small_chunk_max=32, mid_chunk_max=64, stage_elems=1 << 22)
     assert info.heavy_tasks == 1 and info.task_ctas_per_sm == (ctas or 3)
+
+
+@pytest.mark.parametrize("n_rows_b,tasks", [(1000, 1), (30_000_000, 0)])
+def test_tables_per_row_of_b_stay_small(n_rows_b, tasks):
+    # boundaries of eight granules for 30 M rows of B are more than a gigabyte, for products that take a megabyte: staged
+    rng = np.random.default_rng(6)
+    n_cols = 131072
+    B = _csr([_row(rng, n_cols, 300, 5000) for _ in range(1000)], n_cols, rng, np.float32)
+    A = _csr([rng.choice(1000, k, replace=False) for k in (3, 40, 200, 1000)], n_rows_b, rng, np.float32)
+    rp = torch.full((n_rows_b + 1,), int(B.nnz), dtype=torch.int64, device="cuda")
+    rp[:1001] = torch.from_numpy(B.row_ptr).cuda()
+    dA = gm.DeviceCSR.from_host(A)
+    dB = gm.DeviceCSR(n_rows_b, n_cols, rp, torch.from_numpy(B.col).cuda(), torch.from_numpy(B.val).cuda())
+    C, info, _ = gm.spgemm(dA, dB)
+    assert info.rows_heavy == 4 and info.heavy_tasks == tasks
+    assert info.workspace_bytes < 3 << 29
+    compare_rows(C, oracle.spgemm(gen.CSR(4, 1000, A.row_ptr, A.col, A.val), B), np.float32)
