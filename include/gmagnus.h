@@ -69,7 +69,9 @@ typedef struct gm_plan_opts {
   int32_t chunk_width;     /* W: columns per final chunk (power of two)                        */
   int32_t max_fanout;      /* n_chunksMax: most children one multisplit level may produce (pow2) */
   int32_t acc_ctas_per_sm; /* 1, 2, 4 or 8: how many dense accumulators share one SM (sets W)  */
-  int64_t stage_elems;     /* capacity, in intermediate products, of each staging half-buffer  */
+  int64_t stage_elems;     /* capacity, in intermediate products, of each staging half-buffer, and of the
+                              area in which light rows wait for their place in C (when they have more products,
+                              or the area is refused, light rows take the hash accumulator)         */
   int64_t c_capacity;      /* room, in entries, reserved for C when heavy rows need > 1 batch  */
   int32_t separate_histogram; /* 1: always run the stand-alone histogram kernel per level (otherwise a
                               first level that runs as separate passes is counted by the expansion) */

@@ -276,6 +276,8 @@ struct gm_plan {
   gm::RowRules rules{};
   gm::i64 class_rows[gm::kRowClasses]{};  // light rows per class (see gm_k1_analysis.cuh)
   gm::i64 staged_light = 0;        // products of the light rows that are merged or sorted
+  void* light_stage = nullptr;     // the area, if it is an allocation of its own
+  bool light_relist = false;       // the area is gone, the rows have to be listed for the hash accumulator first
   int merge_lists = 0;             // most entries of A in a merged row
   bool merge_only = false;         // every row of A is merged or empty
   gm::LightBins bins{};            // hash rows by entry count, for their numeric pass
@@ -388,6 +390,16 @@ static int plan_alloc(gm_plan* p, T** out, size_t n, cudaStream_t st) {
   return GM_OK;
 }
 
+static void plan_free(gm_plan* p, void* q, cudaStream_t st) {
+  for (size_t i = 0; q && i < p->owned.size(); ++i) {
+    if (p->owned[i].p != q) continue;
+    p->info.workspace_bytes -= static_cast<int64_t>(p->owned[i].bytes);
+    p->owned.erase(p->owned.begin() + static_cast<std::ptrdiff_t>(i));
+    dev_free(q, st);
+    return;
+  }
+}
+
 // Bytes a plan sets aside for the light rows' staging area before it knows their products.
 constexpr size_t kLightRoom = size_t{4} << 20;
 // C is allocated before its size is known, with room for every product, when that takes at most this much: the call then
@@ -452,16 +464,85 @@ __global__ void k_validate_csr(const i64* __restrict__ row_ptr, const int32_t* _
   }
 }
 
-static int launch_row_analysis(gm_plan* p, K1Totals* totals, HeavyTile* tiles, u32* parts, cudaStream_t st) {
+// What the row analysis wants zeroed, at the front of an arena.
+struct K1Zeroed {
+  K1Totals* totals = nullptr;
+  HeavyTile* tiles = nullptr;
+  i64* ip = nullptr;
+  u32* parts = nullptr;
+  size_t bytes = 0;
+  void add_to(Arena& ar, i64 n_rows) {
+    ar.add(&totals, 1);
+    ar.add(&tiles, static_cast<size_t>((n_rows + kHeavyRows - 1) / kHeavyRows) + 1);
+    ar.add(&ip, static_cast<size_t>(n_rows) + 1);
+    ar.add(&parts, static_cast<size_t>(n_rows) + 1);
+    bytes = ar.bytes;
+  }
+};
+
+// Row analysis: products per row, classes, totals (waits for them).
+static int analyse_rows(gm_plan* p, const K1Zeroed& z, cudaStream_t st) {
   const gm_csr& A = p->A;
-  const int T = k1_tile_items(A.n_rows, A.nnz, p->num_sms);
-  const unsigned grid = static_cast<unsigned>(std::min<i64>((A.n_rows + A.nnz + T - 1) / T, static_cast<i64>(p->num_sms) * 6));
-  const bool wide = p->B.n_cols > (i64{1} << 24);
-  auto kern = T == kK1Small ? (wide ? k1_rows<kK1Small, i64> : k1_rows<kK1Small, u32>)
-                            : (wide ? k1_rows<kK1Large, i64> : k1_rows<kK1Large, u32>);
-  kern<<<grid, kK1Threads, 0, st>>>(A.row_ptr, A.col_idx, A.n_rows, A.nnz, p->B.row_ptr, p->rules, p->ip, parts, p->heavy_flag,
-                                    p->row_nnz, p->light_off, p->class_list, A.n_rows, tiles, totals, p->slot->totals);
-  GM_CUDA(cudaGetLastError());
+  K1Totals ht{};
+  if (A.n_rows > 0) {
+    GM_CUDA(cudaMemsetAsync(z.totals, 0, z.bytes, st));
+    const int T = k1_tile_items(A.n_rows, A.nnz, p->num_sms);
+    const unsigned grid = static_cast<unsigned>(std::min<i64>((A.n_rows + A.nnz + T - 1) / T, static_cast<i64>(p->num_sms) * 6));
+    const bool wide = p->B.n_cols > (i64{1} << 24);
+    auto kern = T == kK1Small ? (wide ? k1_rows<kK1Small, i64> : k1_rows<kK1Small, u32>)
+                              : (wide ? k1_rows<kK1Large, i64> : k1_rows<kK1Large, u32>);
+    kern<<<grid, kK1Threads, 0, st>>>(A.row_ptr, A.col_idx, A.n_rows, A.nnz, p->B.row_ptr, p->rules, z.ip, z.parts, p->heavy_flag,
+                                      p->row_nnz, p->light_off, p->class_list, A.n_rows, z.tiles, z.totals, p->slot->totals);
+    ++p->info.launches;
+    GM_CUDA(cudaGetLastError());
+    GM_CUDA(cudaStreamSynchronize(st));
+    std::memcpy(&ht, p->slot->totals, sizeof(ht));
+  }
+  gm_plan_info& info = p->info;
+  info.products_total = static_cast<int64_t>(ht.products_total);
+  info.products_heavy = static_cast<int64_t>(ht.products_heavy);
+  info.products_max_row = static_cast<int64_t>(ht.products_max_row);
+  info.c_nnz_upper = static_cast<int64_t>(ht.c_nnz_upper);
+  info.rows_heavy = static_cast<int64_t>(ht.rows_heavy);
+  info.rows_empty = static_cast<int64_t>(ht.rows_empty);
+  info.rows_light = A.n_rows - info.rows_heavy - info.rows_empty;
+  info.nnz_a_heavy = static_cast<int64_t>(ht.nnz_a_heavy);
+  std::memset(info.light_bin_rows, 0, sizeof(info.light_bin_rows));
+  for (int c = 0; c < kRowClasses; ++c) {
+    p->class_rows[c] = static_cast<i64>(ht.class_rows[c]);
+    info.light_bin_rows[std::min(c, 7)] += p->class_rows[c];
+  }
+  p->staged_light = static_cast<i64>(ht.staged_light);
+  p->merge_lists = static_cast<int>(ht.merge_max_lists);
+  p->merge_only = p->class_rows[kMergeClass] > 0 && p->class_rows[kMergeClass] + info.rows_empty == A.n_rows;
+  return GM_OK;
+}
+
+// Lists the light rows for the hash accumulator, which needs no staging area, and gives that area back if there is one: for
+// products whose area is refused, larger than asked for, or in the way of C.
+static int light_rows_by_hash(gm_plan* p, cudaStream_t st) {
+  const i64 nA = p->A.n_rows;
+  p->light_relist = true;
+  plan_free(p, p->light_stage, st);
+  p->light_stage = nullptr;
+  p->light_col = nullptr;
+  p->light_val = nullptr;
+  RowRules& r = p->rules;
+  r.merge = 0;
+  r.sort_max = 0;
+  r.n_hash = p->bins.n_bins;
+  for (int b = 0; b < p->bins.n_bins; ++b) r.hash_cap[b] = p->bins.cap[b];
+  Arena ar;
+  K1Zeroed z;  // (its own: a copy of the plan's products per row may be under way)
+  z.add_to(ar, nA);
+  int32_t* lists = nullptr;
+  ar.add(&lists, static_cast<size_t>(kHashClass0 + r.n_hash) * static_cast<size_t>(nA));
+  ar.add(&p->num_rows, static_cast<size_t>(p->bins.n_bins) * static_cast<size_t>(nA));
+  ar.add(&p->num_fill, 8);
+  GM_TRY(ar.commit(p, st));
+  p->class_list = lists;
+  GM_TRY(analyse_rows(p, z, st));
+  p->light_relist = false;
   return GM_OK;
 }
 
@@ -684,19 +765,12 @@ static int build_plan(gm_plan* p, cudaStream_t st) {
     p->bin_slots[nb] = prm.light_slots;
     p->bins.n_bins = nb + 1;
   }
-  K1Totals* totals = nullptr;
-  HeavyTile* tiles = nullptr;
-  u32* parts = nullptr;
-  size_t zeroed = 0;
   unsigned char* light_room = nullptr;
+  K1Zeroed z;
   {
     Arena ar;
     const size_t n1 = static_cast<size_t>(nA) + 1;
-    ar.add(&totals, 1);
-    ar.add(&tiles, static_cast<size_t>((nA + kHeavyRows - 1) / kHeavyRows) + 1);
-    ar.add(&p->ip, n1);
-    ar.add(&parts, n1);
-    zeroed = ar.bytes;  // what the row analysis wants zeroed comes first
+    z.add_to(ar, nA);
     ar.add(&p->c_total, 16);
     ar.add(&p->heavy_flag, n1);
     ar.add(&p->row_nnz, n1);
@@ -706,53 +780,38 @@ static int build_plan(gm_plan* p, cudaStream_t st) {
     ar.add(&light_room, kLightRoom);  // the light rows' staging area, if it turns out to fit: an allocation less
     GM_TRY(ar.commit(p, st));
   }
-  K1Totals ht{};
-  if (nA > 0) {
-    GM_CUDA(cudaMemsetAsync(totals, 0, zeroed, st));
-    GM_TRY(launch_row_analysis(p, totals, tiles, parts, st));
-    info.launches += 1;
-    // ---- first host sync: totals
-    GM_CUDA(cudaStreamSynchronize(st));
-    std::memcpy(&ht, p->slot->totals, sizeof(ht));
-  }
-  info.products_total = static_cast<int64_t>(ht.products_total);
-  info.products_heavy = static_cast<int64_t>(ht.products_heavy);
-  info.products_max_row = static_cast<int64_t>(ht.products_max_row);
-  info.c_nnz_upper = static_cast<int64_t>(ht.c_nnz_upper);
-  info.rows_heavy = static_cast<int64_t>(ht.rows_heavy);
-  info.rows_empty = static_cast<int64_t>(ht.rows_empty);
-  info.rows_light = nA - info.rows_heavy - info.rows_empty;
-  info.nnz_a_heavy = static_cast<int64_t>(ht.nnz_a_heavy);
-  for (int c = 0; c < kRowClasses; ++c) {
-    p->class_rows[c] = static_cast<i64>(ht.class_rows[c]);
-    info.light_bin_rows[std::min(c, 7)] += p->class_rows[c];
-  }
-  p->staged_light = static_cast<i64>(ht.staged_light);
-  p->merge_lists = static_cast<int>(ht.merge_max_lists);
-  p->merge_only = p->class_rows[kMergeClass] > 0 && p->class_rows[kMergeClass] + info.rows_empty == nA;
+  p->ip = z.ip;
+  GM_TRY(analyse_rows(p, z, st));  // ---- first host sync: totals
   const i64 nH = info.rows_heavy;
   p->n_seg = info.nnz_a_heavy;
 
   // ---- light rows: staging area (not when all rows are merged), bins of the hash rows
-  {
+  bool hash_all = false;
+  if (p->staged_light > 0 && !p->merge_only) {
+    // at most what a staging buffer of the heavy rows may hold (see below): the area takes room for every product, where C
+    // may have one entry for many, and the hash accumulator takes none
+    const i64 most = p->opts.stage_elems > 0 ? p->opts.stage_elems : std::max<i64>(i64{1} << 29, static_cast<i64>(facts.total_mem / 5) / (4 + p->sv));
+    const size_t n_staged = static_cast<size_t>(p->staged_light) + 64, bytes = n_staged * static_cast<size_t>(4 + p->sv);
+    unsigned char* area = light_room;
+    if (p->staged_light > most) hash_all = true;
+    else if (bytes > kLightRoom) hash_all = plan_alloc(p, &area, bytes, st) != GM_OK;
+    if (!hash_all) {
+      p->light_stage = area == light_room ? nullptr : area;
+      p->light_val = area;
+      p->light_col = reinterpret_cast<int32_t*>(area + n_staged * static_cast<size_t>(p->sv));
+    }
+  }
+  if (hash_all) {
+    GM_TRY(light_rows_by_hash(p, st));
+  } else {
     Arena ar;
-    unsigned char* lv = nullptr;
     bool hash_rows = false;
     for (int c = kHashClass0; c < kRowClasses; ++c) hash_rows |= p->class_rows[c] > 0;
-    const size_t n_staged = static_cast<size_t>(p->staged_light) + 64;
-    if (p->staged_light > 0 && !p->merge_only && n_staged * static_cast<size_t>(4 + p->sv) <= kLightRoom) {
-      lv = light_room;
-      p->light_col = reinterpret_cast<int32_t*>(light_room + n_staged * static_cast<size_t>(p->sv));
-    } else if (p->staged_light > 0 && !p->merge_only) {
-      ar.add(&p->light_col, static_cast<size_t>(p->staged_light) + 8);
-      ar.add(&lv, (static_cast<size_t>(p->staged_light) + 8) * static_cast<size_t>(p->sv));
-    }
     if (hash_rows) {
       ar.add(&p->num_rows, static_cast<size_t>(p->bins.n_bins) * static_cast<size_t>(nA));
       ar.add(&p->num_fill, 8);
+      GM_TRY(ar.commit(p, st));
     }
-    if (ar.bytes) GM_TRY(ar.commit(p, st));
-    p->light_val = lv;
   }
 
   // ---- heavy rows
@@ -765,7 +824,7 @@ static int build_plan(gm_plan* p, cudaStream_t st) {
       GM_TRY(ar.commit(p, st));
     }
     k1_heavy_lists<<<static_cast<unsigned>((nA + kHeavyRows - 1) / kHeavyRows), kHeavyThreads, 0, st>>>(
-        p->ip, p->heavy_flag, A.row_ptr, nA, tiles, p->x_heavy, p->heavy_base, p->heavy_nz_off);
+        p->ip, p->heavy_flag, A.row_ptr, nA, z.tiles, p->x_heavy, p->heavy_base, p->heavy_nz_off);
     ++info.launches;
 
     // The expansion writes the first level's children itself (see gm_k4_direct.cuh) unless asked to run that
@@ -1562,6 +1621,7 @@ static int execute_t(gm_plan* p, cudaStream_t st, gm_csr* C) {
   PhaseTimes& tm = p->times;
   p->stats = gm_exec_stats{};
   tm.reset();
+  if (p->sink) p->sink->copied = 0;
   cudaEvent_t ev_total0 = nullptr, ev_total1 = nullptr;
   if (tm.enabled) { ev_total0 = tm.get(); ev_total1 = tm.get(); cudaEventRecord(ev_total0, st); }
 
@@ -1873,8 +1933,15 @@ int gm_spgemm_execute(gm_plan* plan, void* cuda_stream, gm_csr* C_out) {
   std::memset(C_out, 0, sizeof(*C_out));
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
   if (plan->pending && st != plan->plan_stream) GM_CUDA(cudaStreamSynchronize(plan->plan_stream));
-  const int rc = plan->A.dtype == GM_F32 ? execute_t<float>(plan, st, C_out) : execute_t<double>(plan, st, C_out);
+  auto run = [&]() { return plan->A.dtype == GM_F32 ? execute_t<float>(plan, st, C_out) : execute_t<double>(plan, st, C_out); };
+  if (plan->light_relist) GM_TRY(light_rows_by_hash(plan, st));  // (an execute before this one had no room for the lists)
+  int rc = run();
   plan->pending = false;  // (whatever the result, the execute has waited for its stream)
+  if (plan->light_stage && (rc == GM_ERR_OOM || (rc == GM_ERR_CAPACITY && plan->opts.c_capacity <= 0))) {
+    // C does not fit beside the light rows' staging area: once more without it
+    GM_TRY(light_rows_by_hash(plan, st));
+    rc = run();
+  }
   return rc;
 }
 

@@ -23,7 +23,7 @@ constexpr int kMergeClass = 0;
 constexpr int kSortClass0 = 1;
 constexpr int kSortClasses = 6;
 constexpr int kHashClass0 = kSortClass0 + kSortClasses;
-constexpr int kMaxHashClasses = 5;
+constexpr int kMaxHashClasses = 8;
 constexpr int kRowClasses = kHashClass0 + kMaxHashClasses;
 constexpr int kMergeMaxLists = 8;      // a merged row has at most this many entries in A ...
 constexpr int kMergeMaxProducts = 64;  // ... and at most this many products
@@ -33,7 +33,7 @@ constexpr i64 kMergeMinRows = 1 << 16;  // below this many rows one thread per r
 struct RowRules {
   i64 tau, c_cols;
   int merge;                      // 1: rows that fit the merge kernel go there
-  int sort_max;                   // rows of at most this many products are sorted by one warp
+  int sort_max;                   // rows of at most this many products are sorted by one warp (0: none)
   int n_hash;
   int hash_cap[kMaxHashClasses];
 };
@@ -443,6 +443,7 @@ __global__ void k1_heavy_segments(const int32_t* __restrict__ x_heavy, i64 n_hea
 // rows with cap[b - 1] < entries <= cap[b].  Rows that are not in a hash class (light_off >= 0: staged; heavy; empty)
 // are left out.
 constexpr int kMaxLightBins = 8;
+static_assert(kMaxLightBins <= kMaxHashClasses, "the bins serve as classes when every light row is hashed");
 struct LightBins {
   int n_bins;
   int cap[kMaxLightBins];

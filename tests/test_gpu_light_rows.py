@@ -28,9 +28,27 @@ def test_sorted_rows_around_every_width(dtype, n_cols):
     B = _csr([rng.choice(pool, 1 << r, replace=False) for r in range(10)] + [[]], n_cols, rng, dtype)
     sizes = [0, 1, 2, 31, 32, 33, 63, 64, 65, 127, 128, 129, 255, 256, 257, 511, 512, 513, 800, 1023]
     A = _csr([[r for r in range(10) if n >> r & 1] + [10] for n in sizes] * 3, 11, rng, dtype)
-    C, info, stats = check_product(A, B, tau=700)  # sort, hash and heavy rows
+    C, info, stats = check_product(A, B, tau=700)  # sorted and heavy rows
     assert info.rows_heavy == 6
     check_product(A, B, tau=8)
+
+
+@pytest.mark.parametrize("dtype", [np.float32, np.float64])
+@pytest.mark.parametrize("n_cols", [3000, (1 << 23) + 5])
+def test_hashed_rows_around_every_class(dtype, n_cols):
+    # rows above what one warp sorts, next to sorted and heavy ones; few and many entries for their products
+    rng = np.random.default_rng(n_cols % 1000)
+    pool = rng.choice(n_cols, 2500, replace=False)
+    B = _csr([rng.choice(pool if r % 2 else pool[: (1 << r) + 3], 1 << r, replace=False) for r in range(12)] + [[]], n_cols, rng, dtype)
+    sizes = [1, 700, 1023, 1024, 1025, 1100, 2047, 2048, 2049, 4000, 4095]
+    A = _csr([[r for r in range(12) if n >> r & 1] for n in sizes] * 3, 13, rng, dtype)
+    B2 = _csr([rng.choice(pool, 600, replace=False) for _ in range(14)], n_cols, rng, dtype)
+    A2 = _csr([rng.choice(14, k, replace=False) for k in (1, 2, 6, 7, 13, 14)], 14, rng, dtype)
+    for X, Y in ((A, B), (A2, B2)):
+        ip = oracle.row_products(X, Y)
+        for tau in (1500, 4095, 8192):
+            C, info, stats = check_product(X, Y, tau=tau)
+            assert info.light_bin_rows[7] == int(((ip > 1024) & (ip <= tau)).sum()) > 0
 
 
 @pytest.mark.parametrize("dtype", [np.float32, np.float64])

@@ -14,17 +14,26 @@ pytestmark = pytest.mark.gpu
 
 @pytest.fixture
 def allocator():
-    """The torch allocator behind a predicate: allocator.refuse(bytes) -> True refuses the request."""
+    """The torch allocator behind a predicate: allocator.refuse(bytes) -> True refuses the request.  allocator.held: what is
+    handed out and not given back (results too)."""
     lib = binding.load_library()
 
     class Hook:
         refuse = staticmethod(lambda n: False)
+        held = {}  # bytes by address
 
     def alloc(n, stream, user):
-        return None if Hook.refuse(n) else binding._torch_alloc(n, stream, user)
+        p = None if Hook.refuse(n) else binding._torch_alloc(n, stream, user)
+        if p:
+            Hook.held[p] = n
+        return p
 
-    cb = binding._ALLOC_FN(alloc)
-    lib.gm_set_allocator(cb, binding._free_cb, None)
+    def free(p, stream, user):
+        Hook.held.pop(p, None)
+        binding._torch_free(p, stream, user)
+
+    cbs = binding._ALLOC_FN(alloc), binding._FREE_FN(free)
+    lib.gm_set_allocator(*cbs, None)
     yield Hook
     lib.gm_set_allocator(binding._alloc_cb, binding._free_cb, None)
 
@@ -59,3 +68,78 @@ def test_a_refused_c_leaves_nothing_running(allocator, opts, granted):
     allocator.refuse = staticmethod(lambda n: False)
     C, _, _ = gm.spgemm(dA, dA)
     compare_rows(C, oracle.spgemm(A, A), np.float32)
+
+
+def _light_matrix(dtype):
+    """30011 rows of 144 products and some of none, one, a thousand: no heavy row with tau = 1024."""
+    A = gen.erdos_renyi_k(30011, 12, seed=5, dtype=dtype)
+    rows = np.split(A.col, A.row_ptr[1:-1])
+    rng = np.random.default_rng(5)
+    for i, k in ((0, 0), (7, 1), (8, 85), (30010, 84), (12345, 20), (12346, 0)):
+        rows[i] = np.sort(rng.choice(A.n_rows, k, replace=False)).astype(np.int32)
+    rp = np.zeros(A.n_rows + 1, np.int64)
+    np.cumsum([len(r) for r in rows], out=rp[1:])
+    return gen.CSR(A.n_rows, A.n_cols, rp, np.concatenate(rows).astype(np.int32), rng.uniform(-1, 1, rp[-1]).astype(dtype))
+
+
+@pytest.mark.parametrize("dtype", [np.float32, np.float64])
+@pytest.mark.parametrize("how", ["more products than asked for", "area refused", "C refused beside it", "C refused beside it, from the host"])
+def test_light_rows_without_room_for_their_products(allocator, how, dtype):
+    A = _light_matrix(dtype)
+    ref = oracle.spgemm(A, A)
+    ip = oracle.row_products(A, A)
+    area = int(ip.sum()) * (4 + np.dtype(dtype).itemsize)
+    assert ip.max() <= 1024 and area > 1 << 25
+    opts = make_opts(tau=1024, stage_elems=1 << 20 if how == "more products than asked for" else 0)
+    dA = gm.DeviceCSR.from_host(A)
+    if how == "area refused":
+        allocator.refuse = staticmethod(lambda n: n > area)
+    elif how.startswith("C refused"):
+        allocator.refuse = staticmethod(lambda n: sum(allocator.held.values()) + n > 3 * area // 2 + (20 << 20))
+    if how.endswith("host"):
+        rp, col, val = np.empty(A.n_rows + 1, np.int64), np.empty(ref.nnz, np.int32), np.empty(ref.nnz, dtype)
+        assert gm.spgemm_host(A, A, rp, col, val, opts=opts) == ref.nnz
+        assert np.array_equal(rp, ref.row_ptr) and np.array_equal(col, ref.col)
+        return
+    plan = gm.spgemm_plan(dA, dA, opts=opts)
+    hashed = how != "C refused beside it"
+    assert plan.info().light_bin_rows[7] == (plan.info().rows_light if hashed else 0)
+    for _ in range(2):
+        compare_rows(gm.spgemm_execute(plan), ref, dtype)
+        info = plan.info()
+        assert info.light_bin_rows[7] == info.rows_light == int((ip > 0).sum()) and info.workspace_bytes < area
+        assert np.array_equal(plan.row_products().cpu().numpy(), ip)
+
+
+def test_merged_rows_beside_a_long_one_without_room_for_their_products(allocator):
+    A, _, _ = gen.config_inputs(1, shrink=2)  # 5-point stencil
+    rows = np.split(A.col, A.row_ptr[1:-1])
+    rows[77] = np.arange(0, A.n_cols, A.n_cols // 700, dtype=np.int32)
+    rp = np.zeros(A.n_rows + 1, np.int64)
+    np.cumsum([len(r) for r in rows], out=rp[1:])
+    A = gen.CSR(A.n_rows, A.n_cols, rp, np.concatenate(rows), np.random.default_rng(1).uniform(-1, 1, rp[-1]))
+    dA = gm.DeviceCSR.from_host(A)
+    C, info, _ = gm.spgemm(dA, dA)
+    assert info.rows_heavy > 0 and info.light_bin_rows[0] > 0
+    allocator.refuse = staticmethod(lambda n: n > 12 * info.products_total * 3 // 4)
+    D, info, _ = gm.spgemm(dA, dA)
+    assert info.light_bin_rows[7] == info.rows_light
+    ref = oracle.spgemm(A, A)
+    compare_rows(C, ref, np.float64)
+    compare_rows(D, ref, np.float64)
+
+
+def test_no_room_for_the_lists_of_the_hash_accumulator(allocator):
+    # C refused, and then what hashing the light rows takes: an error, and the plan can still be executed later
+    A = _light_matrix(np.float32)
+    ref = oracle.spgemm(A, A)
+    dA = gm.DeviceCSR.from_host(A)
+    plan = gm.spgemm_plan(dA, dA, opts=make_opts(tau=1024))
+    for granted in (0, 0, 1, 2):  # C.row_ptr and the lists; the lists again; C.row_ptr; C.val
+        allocator.refuse = staticmethod(_after(granted))
+        with pytest.raises(gm.GmError) as ei:
+            gm.spgemm_execute(plan)
+        assert ei.value.status == -5
+    allocator.refuse = staticmethod(lambda n: False)
+    for _ in range(2):
+        compare_rows(gm.spgemm_execute(plan), ref, np.float32)
