@@ -365,6 +365,7 @@ struct gm_plan {
   int* task_tickets = nullptr;     // 4 per batch
   gm::PhaseTimes times;
   HostSink* sink = nullptr;        // set by gm_spgemm_host for the duration of one execute
+  bool c_is_passing = false;       // C is copied out and freed at once: what it takes more than its entries does not matter
   // light rows run next to the heavy path on a stream of the plan's own (Algorithm 3 keeps separate queues for them)
   cudaStream_t light_stream = nullptr;  // (the device's, not owned)
   cudaEvent_t ev_fork = nullptr, ev_light = nullptr;
@@ -405,6 +406,9 @@ constexpr size_t kLightRoom = size_t{4} << 20;
 // C is allocated before its size is known, with room for every product, when that takes at most this much: the call then
 // does not wait in the middle for nnz(C), and the allocation overlaps the kernels.
 constexpr i64 kCRoomBytes = i64{64} << 20;
+// ... and what the caller then holds for nothing is at most this much, or as much again as C itself takes: with more C is
+// moved to arrays of its size.
+constexpr i64 kCSpareBytes = i64{4} << 20;
 
 // Several device arrays in one allocation: the allocator hook of the Python binding costs a few microseconds a call.
 struct Arena {
@@ -1612,6 +1616,18 @@ static int task_batch_gather(gm_plan* p, size_t bi, bool bases, const i64* c_row
   return GM_OK;
 }
 
+// Arrays of C with room for `entries`; both or none.
+template <typename V>
+static bool alloc_c(i64 entries, int32_t** col, V** val, cudaStream_t st) {
+  const size_t n = static_cast<size_t>(std::max<i64>(entries, 1));
+  *col = static_cast<int32_t*>(dev_alloc(n * sizeof(int32_t), st));
+  *val = *col ? static_cast<V*>(dev_alloc(n * sizeof(V), st)) : nullptr;
+  if (*val) return true;
+  dev_free(*col, st);
+  *col = nullptr;
+  return false;
+}
+
 template <typename V>
 static int execute_t(gm_plan* p, cudaStream_t st, gm_csr* C) {
   const gm_csr& A = p->A;
@@ -1690,7 +1706,7 @@ static int execute_t(gm_plan* p, cudaStream_t st, gm_csr* C) {
   int dev_err = 0;
   bool finished = false;  // small products: counts, C.row_ptr and the totals came from one launch
   if (n_batches <= 1) {
-    // ---- everything is resident at once: count, allocate C exactly, then fill
+    // ---- everything is resident at once: count, allocate C, then fill
     HeavyBatchState<V> hs;
     if (n_batches == 1 && !p->use_tasks) GM_TRY_C(heavy_batch_front<V>(p, p->batches[0], &hs, st));
     join_light();
@@ -1710,8 +1726,7 @@ static int execute_t(gm_plan* p, cudaStream_t st, gm_csr* C) {
                                                         reinterpret_cast<i64*>(&slot->c_total));
     }
     tm.end(st);
-    const bool early_c = info.c_nnz_upper * static_cast<i64>(4 + sizeof(V)) <= kCRoomBytes;
-    if (early_c) {
+    if (info.c_nnz_upper * static_cast<i64>(4 + sizeof(V)) <= kCRoomBytes && alloc_c(info.c_nnz_upper, &c_col, &c_val, st)) {
       capacity = info.c_nnz_upper;
     } else {
       if (cudaStreamSynchronize(st) != cudaSuccess) {
@@ -1719,9 +1734,8 @@ static int execute_t(gm_plan* p, cudaStream_t st, gm_csr* C) {
         return fail(GM_ERR_CUDA, std::string("symbolic phase failed: ") + cudaGetErrorString(cudaGetLastError()));
       }
       capacity = total = *static_cast<volatile i64*>(&slot->c_total);
+      alloc_c(capacity, &c_col, &c_val, st);
     }
-    c_col = static_cast<int32_t*>(dev_alloc(static_cast<size_t>(std::max<i64>(capacity, 1)) * sizeof(int32_t), st));
-    c_val = static_cast<V*>(dev_alloc(static_cast<size_t>(std::max<i64>(capacity, 1)) * sizeof(V), st));
     if (!c_col || !c_val) { cleanup(); return fail(GM_ERR_OOM, "allocation of C (" + std::to_string(capacity) + " entries) failed"); }
     // the heavy and the light rows write different rows of C
     fork_light();
@@ -1751,12 +1765,7 @@ static int execute_t(gm_plan* p, cudaStream_t st, gm_csr* C) {
     }
     for (size_t k = 0; k < tries.size(); ++k) {
       capacity = tries[k];
-      c_col = static_cast<int32_t*>(dev_alloc(static_cast<size_t>(capacity) * sizeof(int32_t), st));
-      c_val = c_col ? static_cast<V*>(dev_alloc(static_cast<size_t>(capacity) * sizeof(V), st)) : nullptr;
-      if (c_col && c_val) break;
-      dev_free(c_col, st);
-      c_col = nullptr;
-      c_val = nullptr;
+      if (alloc_c(capacity, &c_col, &c_val, st)) break;
       if (k == 0 && p->opts.c_capacity <= 0) {
         // refused: go down in eight steps to what the device says is free
         size_t free_b = 0, total_b = 0;
@@ -1841,6 +1850,25 @@ static int execute_t(gm_plan* p, cudaStream_t st, gm_csr* C) {
     return dev_error_to_status(dev_err);
   }
 #undef GM_TRY_C
+  if (const i64 entry = static_cast<i64>(4 + sizeof(V));
+      n_batches <= 1 && !p->c_is_passing && (capacity - total) * entry > std::max(kCSpareBytes, total * entry)) {
+    int32_t* col = nullptr;
+    V* val = nullptr;
+    if (alloc_c(total, &col, &val, st)) {
+      cudaMemcpyAsync(col, c_col, static_cast<size_t>(total) * sizeof(int32_t), cudaMemcpyDeviceToDevice, st);
+      cudaMemcpyAsync(val, c_val, static_cast<size_t>(total) * sizeof(V), cudaMemcpyDeviceToDevice, st);
+      const cudaError_t e3 = cudaStreamSynchronize(st);
+      dev_free(c_col, st);
+      dev_free(c_val, st);
+      c_col = col;
+      c_val = val;
+      capacity = total;
+      if (e3 != cudaSuccess) {
+        cleanup();
+        return fail(GM_ERR_CUDA, std::string("moving C failed: ") + cudaGetErrorString(e3));
+      }
+    }
+  }
   p->stats.c_nnz = total;
   if (n_batches > 0) {
     const i64* t = slot->tail;
@@ -2041,6 +2069,7 @@ int gm_spgemm_host(const gm_csr* A_host, const gm_csr* B_host, size_t smem_bytes
                cudaMallocHost(reinterpret_cast<void**>(&sink.h_totals), plan->batches.size() * sizeof(int64_t)) == cudaSuccess;
     if (use_sink) plan->sink = &sink;
   }
+  if (plan) plan->c_is_passing = true;
   if (rc == GM_OK) rc = gm_spgemm_execute(plan, st, &C);
   if (plan) plan->sink = nullptr;
   if (rc == GM_OK) {
