@@ -79,8 +79,9 @@ typedef struct gm_plan_opts {
                               (GM_ERR_BAD_CSR), and before the heavy rows' products are summed a pass checks that each
                               lies in the columns its chunk or task owns (GM_ERR_INTERNAL)                      */
   int32_t single_stream;   /* 1: every kernel of a call runs on the caller's stream.  0 (default): the light rows'
-                              kernels run on a second stream of the plan's, forked from and joined back into the
-                              caller's stream with events, next to the heavy rows' kernels (Algorithm 3)      */
+                              kernels, and those of the heavy rows' smaller tasks, run on a second stream that the
+                              call has for itself, forked from and joined back into the caller's stream with
+                              events, next to the heavy rows' other kernels (Algorithm 3)                    */
   int32_t level0_multisplit; /* first multisplit level: 1 = separate histogram and multisplit passes over
                               the staging buffer (Algorithm 5 as printed); 2 = the expansion kernel writes
                               the first level's children itself; 0 (default) = no level at all where the heavy
@@ -232,7 +233,8 @@ int gm_spgemm_plan_ex(const gm_csr* A, const gm_csr* B, size_t smem_bytes,
  * unless single_stream is set); the call returns after synchronising that stream, because nnz(C) is needed
  * on the host.
  * A plan can be executed any number of times (values of A and B may change in between, their
- * structure may not).  Two executes of the same plan must not overlap.
+ * structure may not).  Two executes of the same plan must not overlap;
+ * executes of different plans may (streams, host threads).
  * Errors: GM_ERR_CAPACITY (C did not fit the reserved room; only possible when the heavy rows
  * need more than one batch), GM_ERR_OOM, GM_ERR_CUDA, GM_ERR_INTERNAL. */
 int gm_spgemm_execute(gm_plan* plan, void* cuda_stream, gm_csr* C_out);

@@ -109,7 +109,6 @@ struct DeviceFacts {
   bool known = false;
   int num_sms = 0, smem_optin = 0;
   size_t total_mem = 0;
-  cudaStream_t side_stream = nullptr;  // see execute_t
 };
 constexpr int kMaxDevices = 64;
 static std::mutex g_facts_mutex;
@@ -140,22 +139,10 @@ static int device_facts(DeviceFacts* out) {
   return GM_OK;
 }
 
-// One second stream per device for the life of the process (creating and destroying a stream per plan cost more than the
-// overlap gained on millisecond products); executes that share it are ordered by their own events.  NULL: none.
-static cudaStream_t side_stream() {
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return nullptr;
-  std::lock_guard<std::mutex> lock(g_facts_mutex);
-  cudaStream_t& st = g_facts[dev].side_stream;
-  if (!st && cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking) != cudaSuccess) {
-    cudaGetLastError();
-    st = nullptr;
-  }
-  return st;
-}
-
-// Streams of the host entry point: taken for a call, given back after it, at most kKeptStreams kept per device.
-constexpr size_t kKeptStreams = 4;
+// Streams that the library needs besides the caller's: taken for a call, given back after it, at most kKeptStreams kept per
+// device (creating and destroying one per plan cost more than the overlap gained on millisecond products).  Calls that run at
+// the same time have different ones: with one for the device, an execute waited for whatever another's stream was busy with.
+constexpr size_t kKeptStreams = 8;
 static std::vector<cudaStream_t> g_free_streams[kMaxDevices];
 
 static cudaStream_t take_stream() {
@@ -181,6 +168,11 @@ static void give_stream(cudaStream_t st) {  // (the caller has waited for it)
   }
   cudaStreamDestroy(st);
 }
+
+struct SideStream {
+  cudaStream_t st = nullptr;
+  ~SideStream() { if (st) give_stream(st); }
+};
 
 // Page-locked host memory that kernels write to and the host reads after a synchronisation: a plan takes one slot and
 // gives it back when it is destroyed.  (Copies to ordinary host variables took 12 to 25 us of host time each.)
@@ -366,8 +358,7 @@ struct gm_plan {
   gm::PhaseTimes times;
   HostSink* sink = nullptr;        // set by gm_spgemm_host for the duration of one execute
   bool c_is_passing = false;       // C is copied out and freed at once: what it takes more than its entries does not matter
-  // light rows run next to the heavy path on a stream of the plan's own (Algorithm 3 keeps separate queues for them)
-  cudaStream_t light_stream = nullptr;  // (the device's, not owned)
+  // light rows run next to the heavy path on a second stream (Algorithm 3 keeps separate queues for them)
   cudaEvent_t ev_fork = nullptr, ev_light = nullptr;
 };
 
@@ -1652,16 +1643,16 @@ static int execute_t(gm_plan* p, cudaStream_t st, gm_csr* C) {
   // ---- light and heavy rows are independent until C.row_ptr is formed: the light rows' kernels go to a second
   // stream, forked from and joined back into the caller's with events (never when single_stream is set)
   bool fork = !p->opts.single_stream && info.rows_heavy > 0 && (info.rows_light > 0 || p->use_tasks);
-  if (fork && !p->light_stream) {
-    p->light_stream = side_stream();
-    if (!p->light_stream || cudaEventCreateWithFlags(&p->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
-        cudaEventCreateWithFlags(&p->ev_light, cudaEventDisableTiming) != cudaSuccess) {
+  SideStream side;
+  if (fork) {
+    side.st = take_stream();
+    if (!side.st || (!p->ev_fork && cudaEventCreateWithFlags(&p->ev_fork, cudaEventDisableTiming) != cudaSuccess) ||
+        (!p->ev_light && cudaEventCreateWithFlags(&p->ev_light, cudaEventDisableTiming) != cudaSuccess)) {
       cudaGetLastError();
-      p->light_stream = nullptr;
       fork = false;
     }
   }
-  cudaStream_t lst = fork ? p->light_stream : st;
+  cudaStream_t lst = fork ? side.st : st;
   auto fork_light = [&]() { if (fork) { cudaEventRecord(p->ev_fork, st); cudaStreamWaitEvent(lst, p->ev_fork, 0); } };
   auto join_light = [&]() { if (fork) { cudaEventRecord(p->ev_light, lst); cudaStreamWaitEvent(st, p->ev_light, 0); } };
   auto cleanup = [&]() {  // waits for all that is queued: the caller may free or reuse what it reads and writes

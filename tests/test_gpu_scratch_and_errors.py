@@ -1,4 +1,7 @@
 """Refused allocations and error returns: what a call leaves behind, and what it still computes."""
+import threading
+import time
+
 import numpy as np
 import pytest
 import torch
@@ -170,3 +173,25 @@ def test_c_takes_little_more_than_its_entries(allocator, kind, dtype, refused):
     compare_rows(C, ref, dtype)
     held = C.col.untyped_storage().nbytes() + C.val.untyped_storage().nbytes()
     assert held == stats.c_capacity * entry <= (1 if refused else 2) * ref.nnz * entry + (0 if refused else 4 << 20)
+
+
+def test_an_execute_does_not_wait_for_another_ones_stream():
+    # one thread's stream is busy for half a second before its product: a product on another stream is done long before
+    A = gen.rmat(12, 16, seed=4, dtype=np.float32)
+    dA = gm.DeviceCSR.from_host(A)
+    plans, streams = [gm.spgemm_plan(dA, dA) for _ in range(2)], [torch.cuda.Stream() for _ in range(2)]
+    assert plans[0].info().rows_light > 0 and plans[0].info().rows_heavy > 0
+    results = [gm.spgemm_execute(p, stream=s) for p, s in zip(plans, streams)]
+    torch.cuda.synchronize()
+    with torch.cuda.stream(streams[0]):
+        torch.cuda._sleep(1_000_000_000)
+    busy = threading.Thread(target=lambda: results.append(gm.spgemm_execute(plans[0], stream=streams[0])))
+    busy.start()
+    time.sleep(0.1)
+    results.append(gm.spgemm_execute(plans[1], stream=streams[1]))
+    assert not streams[0].query()
+    busy.join()
+    assert len(results) == 4
+    ref = oracle.spgemm(A, A)
+    for C in results:
+        compare_rows(C, ref, np.float32)
