@@ -211,8 +211,9 @@ int64_t gm_planner_batches(const int64_t* heavy_prefix, int64_t n_heavy, int64_t
  *   plan_out    receives the plan; release it with gm_plan_destroy
  * Runs on `cuda_stream` (gm_spgemm_plan: the legacy default stream) and synchronises it on the way,
  * because the planner needs counts on the host; kernels that fill the plan's own tables may still run
- * when it returns (gm_spgemm_execute and gm_plan_destroy wait for them where they have to).  The plan
- * borrows A's and B's arrays. */
+ * when it returns (gm_spgemm_execute and gm_plan_destroy wait for them where they have to, also if the
+ * stream has been destroyed by then; the workspace is handed to the allocator's free with that stream).
+ * The plan borrows A's and B's arrays. */
 int gm_spgemm_plan(const gm_csr* A, const gm_csr* B, size_t smem_bytes, gm_plan** plan_out);
 int gm_spgemm_plan_ex(const gm_csr* A, const gm_csr* B, size_t smem_bytes,
                       const gm_plan_opts* opts, void* cuda_stream, gm_plan** plan_out);

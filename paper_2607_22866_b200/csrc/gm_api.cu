@@ -275,7 +275,8 @@ struct gm_plan {
   gm::LightBins bins{};            // hash rows by entry count, for their numeric pass
   int bin_slots[gm::kMaxLightBins]{};
   gm::HostSlot* slot = nullptr;
-  bool pending = false;            // kernels of the plan may still run on plan_stream
+  bool pending = false;            // kernels of the plan may still run on plan_stream; ev_fork is recorded behind them
+  unsigned long long plan_stream_id = 0;  // (the stream may be gone by the time the plan is used)
   std::vector<gm::Batch> batches;
   std::vector<int32_t> x_heavy_host;
   int64_t max_batch_rows = 0;
@@ -1939,6 +1940,13 @@ int gm_spgemm_plan_ex(const gm_csr* A, const gm_csr* B, size_t smem_bytes, const
     gm_plan_destroy(p);
     return rc;
   }
+  if (p->pending && (cudaEventCreateWithFlags(&p->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
+                     cudaStreamGetId(p->plan_stream, &p->plan_stream_id) != cudaSuccess ||
+                     cudaEventRecord(p->ev_fork, p->plan_stream) != cudaSuccess)) {
+    cudaStreamSynchronize(p->plan_stream);
+    gm_plan_destroy(p);
+    return fail(GM_ERR_CUDA, std::string("end of planning: ") + cudaGetErrorString(cudaGetLastError()));
+  }
   *plan_out = p;
   return GM_OK;
 }
@@ -1951,7 +1959,11 @@ int gm_spgemm_execute(gm_plan* plan, void* cuda_stream, gm_csr* C_out) {
   if (!plan || !C_out) return fail(GM_ERR_INVALID_ARG, "plan or C_out is null");
   std::memset(C_out, 0, sizeof(*C_out));
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-  if (plan->pending && st != plan->plan_stream) GM_CUDA(cudaStreamSynchronize(plan->plan_stream));
+  if (plan->pending) {
+    unsigned long long id = 0;
+    GM_CUDA(cudaStreamGetId(st, &id));
+    if (id != plan->plan_stream_id) GM_CUDA(cudaStreamWaitEvent(st, plan->ev_fork, 0));
+  }
   auto run = [&]() { return plan->A.dtype == GM_F32 ? execute_t<float>(plan, st, C_out) : execute_t<double>(plan, st, C_out); };
   if (plan->light_relist) GM_TRY(light_rows_by_hash(plan, st));  // (an execute before this one had no room for the lists)
   int rc = run();
@@ -2001,7 +2013,7 @@ void gm_csr_free(gm_csr* C) {
 
 void gm_plan_destroy(gm_plan* plan) {
   if (!plan) return;
-  if (plan->pending) cudaStreamSynchronize(plan->plan_stream);
+  if (plan->pending && plan->ev_fork) cudaEventSynchronize(plan->ev_fork);
   if (plan->ev_fork) cudaEventDestroy(plan->ev_fork);
   if (plan->ev_light) cudaEventDestroy(plan->ev_light);
   for (auto& b : plan->owned) dev_free(b.p, plan->plan_stream);

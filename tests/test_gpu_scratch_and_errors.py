@@ -1,6 +1,8 @@
 """Refused allocations and error returns: what a call leaves behind, and what it still computes."""
+import ctypes
 import threading
 import time
+from types import SimpleNamespace
 
 import numpy as np
 import pytest
@@ -195,3 +197,24 @@ def test_an_execute_does_not_wait_for_another_ones_stream():
     ref = oracle.spgemm(A, A)
     for C in results:
         compare_rows(C, ref, np.float32)
+
+
+@pytest.mark.parametrize("execute_on", ["default", "other", "none"])
+def test_a_plan_outlives_its_stream(execute_on):
+    # kernels that fill the plan's tables may still run when planning returns; the stream they run on is destroyed then
+    A = gen.rmat(15, 16, seed=4, dtype=np.float32)
+    dA = gm.DeviceCSR.from_host(A)
+    gm.spgemm_plan(dA, dA).destroy()
+    torch.cuda.synchronize()
+    rt, handle = torch.cuda.cudart(), ctypes.c_void_p()
+    assert int(rt.cudaStreamCreate(ctypes.addressof(handle))) == 0
+    plan = gm.spgemm_plan(dA, dA, stream=SimpleNamespace(cuda_stream=handle.value))
+    assert int(rt.cudaStreamDestroy(handle.value)) == 0
+    if execute_on != "none":
+        stream = torch.cuda.Stream() if execute_on == "other" else torch.cuda.current_stream()
+        with torch.cuda.stream(stream):
+            for _ in range(2):
+                compare_rows(gm.spgemm_execute(plan), oracle.spgemm(A, A, 0, 500), np.float32)
+    plan.destroy()
+    C, _, _ = gm.spgemm(dA, dA)
+    compare_rows(C, oracle.spgemm(A, A, 0, 500), np.float32)
