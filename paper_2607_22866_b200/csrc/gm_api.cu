@@ -1,6 +1,7 @@
 // C ABI of the library (see include/gmagnus.h): plan = setup phase of Algorithm 3, execute = the
 // light and heavy paths, batching of the heavy rows and assembly of C.
 #include <algorithm>
+#include <atomic>
 #include <climits>
 #include <cstddef>
 #include <cstdio>
@@ -263,7 +264,7 @@ struct gm_plan {
   gm_plan_opts opts{};
   gm_plan_info info{};
   gm_exec_stats stats{};
-  int num_sms = 148;
+  int num_sms = 148, smem_optin = 0;
   cudaStream_t plan_stream = nullptr;
   gm::RowRules rules{};
   gm::i64 class_rows[gm::kRowClasses]{};  // light rows per class (see gm_k1_analysis.cuh)
@@ -370,6 +371,22 @@ struct gm_plan {
 #define GM_MID_MIN_BLOCKS 7
 #endif
 namespace gm {
+
+// Lets a kernel take all the dynamic shared memory there is.  (The limit belongs to the kernel and not to a launch: set to what
+// one launch needs, it failed the launch of another host thread whose plan has a larger budget.)
+template <auto Kern>
+static int allow_smem(const gm_plan* p) {
+  static std::atomic<int> fixed{-1};  // static shared memory, known once the kernel is loaded
+  int n = fixed.load(std::memory_order_relaxed);
+  if (n < 0) {
+    cudaFuncAttributes a{};
+    GM_CUDA(cudaFuncGetAttributes(&a, Kern));
+    n = static_cast<int>(a.sharedSizeBytes);
+    fixed.store(n, std::memory_order_relaxed);
+  }
+  GM_CUDA(cudaFuncSetAttribute(Kern, cudaFuncAttributeMaxDynamicSharedMemorySize, p->smem_optin - n));
+  return GM_OK;
+}
 
 template <typename T>
 static int plan_alloc(gm_plan* p, T** out, size_t n, cudaStream_t st) {
@@ -701,6 +718,7 @@ static int build_plan(gm_plan* p, cudaStream_t st) {
   DeviceFacts facts;
   GM_TRY(device_facts(&facts));
   p->num_sms = facts.num_sms;
+  p->smem_optin = facts.smem_optin;
   if (p->smem_bytes > static_cast<size_t>(facts.smem_optin))
     return fail(GM_ERR_UNSUPPORTED_SMEM, "smem_bytes exceeds the device's opt-in shared memory per block");
   {
@@ -981,9 +999,9 @@ static int launch_hash_one(gm_plan* p, const int32_t* rows, i64 n_rows, const in
                            const i64* c_row_ptr, int32_t* c_col, V* c_val, i64 c_capacity, cudaStream_t st) {
   constexpr int kGroups = BT / G;
   const size_t smem = kGroups * light_group_bytes<V, NUMERIC>(slots, cap, G);
-  auto kern = k3_light_rows<V, G, LPN, BT, NUMERIC>;
+  constexpr auto kern = k3_light_rows<V, G, LPN, BT, NUMERIC>;
   // (static shared memory counts towards the 48 KB that need no opt-in)
-  if (smem > 32 * 1024) GM_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)));
+  if (smem > 32 * 1024) GM_TRY(allow_smem<kern>(p));
   const unsigned grid = grid_for(n_rows, kGroups, p->num_sms, 2048 / BT * 4);
   kern<<<grid, BT, smem, st>>>(p->A.row_ptr, p->A.col_idx, static_cast<const V*>(p->A.vals), p->B.row_ptr, p->B.col_idx,
                                static_cast<const V*>(p->B.vals), rows, static_cast<int>(n_rows), n_rows_dev, slots, cap, p->row_nnz,
@@ -1190,8 +1208,8 @@ static int launch_accumulate(gm_plan* p, const Batch& b, const HeavyBatchState<V
   if (mid_max > small_max) {
     p->times.begin(PhaseTimes::kAccMid, st);
     const size_t smem = mid_smem_bytes(W, sizeof(V), mid_max);
-    auto kern = k6_mid_chunks<V>;
-    if (smem > 32 * 1024) GM_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)));
+    constexpr auto kern = k6_mid_chunks<V>;
+    if (smem > 32 * 1024) GM_TRY(allow_smem<kern>(p));
     const int per_sm = std::max<int>(1, std::min<int>(2048 / kMidThreads, static_cast<int>((p->smem_bytes - 1024) / (smem + 1024))));
     const unsigned grid = static_cast<unsigned>(std::min<i64>(hs.n_chunks, static_cast<i64>(p->num_sms) * per_sm));
     kern<<<grid, kMidThreads, smem, st>>>(hs.fin_col, hs.fin_val, hs.chunk_off, p->mid_list, p->acc_counters, hs.log2_cpr, W,
@@ -1206,9 +1224,8 @@ static int launch_accumulate(gm_plan* p, const Batch& b, const HeavyBatchState<V
     const unsigned grid = static_cast<unsigned>(std::min<i64>(hs.n_chunks, static_cast<i64>(p->num_sms) * per_sm));
 #define GM_ACC(BT)                                                                                                   \
   do {                                                                                                               \
-    auto kern = k6_accumulate<V, BT>;                                                                                \
-    if (smem > 32 * 1024)                                                                                            \
-      GM_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)));     \
+    constexpr auto kern = k6_accumulate<V, BT>;                                                                      \
+    if (smem > 32 * 1024) GM_TRY(allow_smem<kern>(p));                                                               \
     kern<<<grid, BT, smem, st>>>(hs.fin_col, hs.fin_val, hs.chunk_off, hs.n_chunks, p->big_list, p->acc_counters,    \
                                  hs.log2_cpr, W, p->chunk_nnz);                                                      \
   } while (0)
@@ -1298,8 +1315,8 @@ static int heavy_batch_front(gm_plan* p, const Batch& b, HeavyBatchState<V>* hs,
           p->seg_h, row_base, p->seg_hrow, p->seg_j, static_cast<const V*>(p->A.vals), seg0, n_seg_b, b.h0, F, p->seg_rec);
       k_tile_bounds<<<grid_for(n_ranges, 256, p->num_sms), 256, 0, st>>>(p->seg_off, p->n_seg, b.elem0, b.elems,
                                                                        static_cast<int>(per_warp), p->tile_meta);
-      auto kern = k4_expand_stream<V>;
-      GM_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)));
+      constexpr auto kern = k4_expand_stream<V>;
+      GM_TRY(allow_smem<kern>(p));
       const int spin = p->opts.debug_spin_limit != 0 ? p->opts.debug_spin_limit : kCopySpinLimit;
       kern<<<grid, kStreamWarps * 32, smem, st>>>(p->seg_off, p->seg_bstart, p->n_seg, p->tile_meta, p->B.col_idx,
                                                   static_cast<const V*>(p->B.vals), p->B.nnz, b.elem0, b.elems, per_warp, seg0,
@@ -1529,8 +1546,8 @@ static int task_batch_sums(gm_plan* p, size_t bi, cudaStream_t st) {
     const unsigned grid = static_cast<unsigned>(std::min<i64>(n, static_cast<i64>(p->num_sms) * p->acc_blocks));
 #define GM_BIG(BT, BLOCKS)                                                                                                        \
   do {                                                                                                                    \
-    auto kern = k6_big_tasks<V, BT, BLOCKS>;                                                                                      \
-    GM_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)));            \
+    constexpr auto kern = k6_big_tasks<V, BT, BLOCKS>;                                                                    \
+    GM_TRY(allow_smem<kern>(p));                                                                                          \
     kern<<<grid, BT, smem, st>>>(in, tasks, n, p->task_list[2] + t0, counters, tickets, out_col, out_val, p->chunk_nnz);  \
   } while (0)
     if (p->acc_blocks == kBigBlocks && p->acc_threads == kBigThreads) GM_BIG(kBigThreads, kBigBlocks);
@@ -1547,8 +1564,8 @@ static int task_batch_sums(gm_plan* p, size_t bi, cudaStream_t st) {
   if (r.mid_max > r.small_max) {
     tm.begin(PhaseTimes::kAccMid, st);
     const size_t smem = mid_task_smem_bytes(static_cast<int>(r.mid_width), sizeof(V), r.mid_max);
-    auto kern = k6_mid_tasks<V>;
-    GM_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)));
+    constexpr auto kern = k6_mid_tasks<V>;
+    GM_TRY(allow_smem<kern>(p));
     int per_sm = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kMidThreads, smem) != cudaSuccess || per_sm < 1) per_sm = 1;
     kern<<<static_cast<unsigned>(std::min<i64>(n, static_cast<i64>(p->num_sms) * per_sm)), kMidThreads, smem, st>>>(

@@ -218,3 +218,32 @@ def test_a_plan_outlives_its_stream(execute_on):
     plan.destroy()
     C, _, _ = gm.spgemm(dA, dA)
     compare_rows(C, oracle.spgemm(A, A, 0, 500), np.float32)
+
+
+@pytest.mark.parametrize("opts", [dict(), dict(level0_multisplit=2)])  # tasks, chunks
+def test_budgets_of_shared_memory_in_several_threads(opts):
+    # the kernels' limits of dynamic shared memory belong to the process: one thread's small budget must not cut another's
+    # (which takes a launch right between the two, hence the many short calls)
+    rng = np.random.default_rng(9)
+    A, B = random_csr(rng, 64, 500, 0.5, np.float32), random_csr(rng, 500, 20000, 0.01, np.float32)
+    dA, dB = gm.DeviceCSR.from_host(A), gm.DeviceCSR.from_host(B)
+    ref, failed = oracle.spgemm(A, B), []
+
+    def work(smem):
+        try:
+            with torch.cuda.stream(torch.cuda.Stream()):
+                plan = gm.spgemm_plan(dA, dB, smem, make_opts(**opts))
+                for i in range(1000):
+                    C = gm.spgemm_execute(plan)
+                    if i % 250 == 0:
+                        compare_rows(C, ref, np.float32)
+        except Exception as e:  # (a thread's exception does not reach the test)
+            failed.append(e)
+
+    torch.cuda.synchronize()
+    threads = [threading.Thread(target=work, args=(smem,)) for smem in (232448, 101376, 232448, 65536)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not failed
