@@ -220,48 +220,63 @@ def oracle_timed(A, B, budget_s: float = 15.0):
 
 
 def kernel_table(info, stats_avg, sv, nnz_b, n_light_entries_a):
-    """Algorithmic (minimum) bytes per step for every kernel of the path, with its measured time."""
+    """Algorithmic (minimum) bytes per step for every part of the path that runs, with its measured time."""
     se = 4 + sv
     e = info.products_heavy
     p = info.params
     rows_h = info.rows_heavy
     L = p.n_levels
     nnz_c, nnz_ch = stats_avg["c_nnz"], stats_avg["c_nnz_heavy"]
-    chunks = stats_avg["final_chunks"]
+    nnz_cl = nnz_c - nnz_ch
     e_small, nnz_small = stats_avg["small_chunk_products"], stats_avg["small_chunk_entries"]
     e_mid, nnz_mid = stats_avg["mid_chunk_products"], stats_avg["mid_chunk_entries"]
-    parents = [rows_h]
-    for l in range(L):
-        parents.append(parents[-1] * p.fanout[l])
-    # the expansion writes the first level's children itself (level0_direct): no pass over the staging buffer for
-    # that level, only per-segment run starts (read two child-boundary rows of B, write one row of prefixes)
-    l0 = 1 if (L > 0 and info.level0_direct) else 0
-    hist = sum(4 * e + 8 * (parents[l] + 1) + 4 * parents[l + 1] for l in range(l0, L))
-    # a multisplit pass reads every column of the batch and moves (reads the value of, writes) only the products of
-    # chunks that have not left the hierarchy early
-    moved = stats_avg["split_products"]
-    split = (2 * se * moved + 4 * ((L - l0) * e - moved)
-             + sum(8 * (parents[l] + 1) + 8 * parents[l + 1] for l in range(l0, L)))
-    # heavy rows summed where their products are generated: nothing staged, B read (each kernel once, at least), entries
-    # written; the expansion's time is then zero
-    staged = stats_avg["ms_expand"] > 0
-    in_small, in_mid, in_big = (e_small, e_mid, e - e_small - e_mid) if staged else (nnz_b, nnz_b, nnz_b)
-    seg_tables = (12 * p.fanout[0] * info.nnz_a_heavy + 4 * parents[1]) if l0 else 0
-    tbl = {
-        "k3_light_symbolic": (4 * n_light_entries_a + 8 * info.rows_light + 4 * nnz_b, stats_avg["ms_light_symbolic"]),
-        "k3_light_numeric": (se * n_light_entries_a + se * nnz_b + se * (nnz_c - nnz_ch), stats_avg["ms_light_numeric"]),
-        "k4_expand": ((se * e + se * nnz_b + 24 * info.nnz_a_heavy + (4 * p.fanout[0] * info.nnz_a_heavy if l0 else 0)) if staged else 0,
-                      stats_avg["ms_expand"]),
-        "k5a_histogram": (hist + seg_tables if staged else 0, stats_avg["ms_histogram"]),
-        "k5b_multisplit": (split, stats_avg["ms_multisplit"]),
+    tbl = {}
+    # light rows: summed into the staging area and copied to C; counted first and then merged into C when all of them are
+    # merged; counted and then summed by the hash accumulator (which reads the products twice)
+    if info.rows_light:
+        merged = info.light_bin_rows[0] + info.rows_empty == info.n_rows
+        hashed = info.light_bin_rows[7] == info.rows_light
+        read_cols = 4 * n_light_entries_a + 8 * info.rows_light + 4 * nnz_b
+        read_all = se * n_light_entries_a + 8 * info.rows_light + se * nnz_b
+        if merged or hashed:
+            k = "k3_merge_rows" if merged else "k3_light_rows"
+            tbl[k + " (count)"] = (read_cols, stats_avg["ms_light_symbolic"])
+            tbl[k + " (into C)"] = (read_all + se * nnz_cl, stats_avg["ms_light_numeric"])
+        else:
+            tbl["k3_sort_rows, k3_merge_rows"] = (read_all + se * nnz_cl, stats_avg["ms_light_symbolic"])
+            tbl["k3_copy_rows"] = (2 * se * nnz_cl, stats_avg["ms_light_numeric"])
+    if rows_h and info.heavy_tasks:
+        # summed where the products are generated: B is read (by each kernel once, at least) and entries are written
+        tbl["k6_small_tasks"] = (se * nnz_b + se * nnz_small, stats_avg["ms_small_chunks"])
+        tbl["k6_mid_tasks"] = (se * nnz_b + se * nnz_mid, stats_avg["ms_mid_chunks"])
+        tbl["k6_big_tasks"] = (se * nnz_b + se * (nnz_ch - nnz_small - nnz_mid), stats_avg["ms_accumulate"])
+        tbl["k7_gather"] = (2 * se * nnz_ch, stats_avg["ms_gather"])
+    elif rows_h:
+        chunks = stats_avg["final_chunks"]
+        parents = [rows_h]
+        for l in range(L):
+            parents.append(parents[-1] * p.fanout[l])
+        # the expansion writes the first level's children itself (level0_direct): no pass over the staging buffer for
+        # that level, only per-segment run starts (read two child-boundary rows of B, write one row of prefixes)
+        l0 = 1 if (L > 0 and info.level0_direct) else 0
+        hist = sum(4 * e + 8 * (parents[l] + 1) + 4 * parents[l + 1] for l in range(l0, L))
+        seg_tables = (12 * p.fanout[0] * info.nnz_a_heavy + 4 * parents[1]) if l0 else 0
+        # a multisplit pass reads every column of the batch and moves (reads the value of, writes) only the products of
+        # chunks that have not left the hierarchy early
+        moved = stats_avg["split_products"]
+        split = (2 * se * moved + 4 * ((L - l0) * e - moved)
+                 + sum(8 * (parents[l] + 1) + 8 * parents[l + 1] for l in range(l0, L)))
+        tbl["k4_expand"] = (se * e + se * nnz_b + 24 * info.nnz_a_heavy + (4 * p.fanout[0] * info.nnz_a_heavy if l0 else 0),
+                            stats_avg["ms_expand"])
+        tbl["k5a_histogram"] = (hist + seg_tables, stats_avg["ms_histogram"])
+        tbl["k5b_multisplit"] = (split, stats_avg["ms_multisplit"])
         # chunks of few products are sorted by one warp each, mid-size ones take a small block each (its second pass
         # re-reads the chunk from L2: not counted), the dense-accumulator kernel owes the rest
-        "k6_small_chunks": (se * in_small + se * nnz_small + (12 * chunks if staged else 0), stats_avg["ms_small_chunks"]),
-        "k6_mid_chunks": (se * in_mid + se * nnz_mid, stats_avg["ms_mid_chunks"]),
-        "k6_accumulate": (se * in_big + se * (nnz_ch - nnz_small - nnz_mid) + (12 * chunks if staged else 0),
-                          stats_avg["ms_accumulate"]),
-        "k7_gather": (2 * se * nnz_ch + 24 * chunks, stats_avg["ms_gather"]),
-    }
+        tbl["k6_small_chunks"] = (se * e_small + se * nnz_small + 12 * chunks, stats_avg["ms_small_chunks"])
+        tbl["k6_mid_chunks"] = (se * e_mid + se * nnz_mid, stats_avg["ms_mid_chunks"])
+        tbl["k6_accumulate"] = (se * (e - e_small - e_mid) + se * (nnz_ch - nnz_small - nnz_mid) + 12 * chunks,
+                                stats_avg["ms_accumulate"])
+        tbl["k7_gather"] = (2 * se * nnz_ch + 24 * chunks, stats_avg["ms_gather"])
     return {k: {"bytes": int(b), "ms": float(ms), "gbs": (b / ms / 1e6 if ms > 0 else 0.0)} for k, (b, ms) in tbl.items()}
 
 
@@ -349,11 +364,17 @@ def main():
 
     def measure(A, B, dA, dB, opts, steps, warmup, sample_clocks):
         """`warmup` untimed and `steps` timed products (plan + execute each).  Returns a dict with the step time,
-        the plan's facts, the per-kernel table (algorithmic bytes, CUDA-event time) and the dominant kernel."""
+        the plan's facts, the per-kernel table (algorithmic bytes, CUDA-event time) and the dominant kernel.  The table's
+        times are from two more products with every kernel on one stream: beside another stream's kernels the events
+        around a kernel would measure its wait for the SMs too."""
         sv = A.val.dtype.itemsize
         step_parts = []
 
-        def step(timing: bool):
+        one_stream = gm.PlanOpts()
+        ctypes_copy(one_stream, opts)
+        one_stream.single_stream = 1
+
+        def step(timing: bool, opts=opts):
             t_a = time.perf_counter()
             plan = gm.spgemm_plan(dA, dB, SMEM_BYTES, opts)
             t_b = time.perf_counter()
@@ -379,22 +400,28 @@ def main():
         barrier()
         ev0.record()
         launches = 0
-        stats_sum: dict[str, float] = {}
+        ms_total = 0.0
         ms_steps = []  # host clock per step (execute returns after a stream synchronize): shows a hiccup if there is one
         for _ in range(steps):
             t_step = time.perf_counter()
             info, st, nnz = step(True)
             ms_steps.append(round((time.perf_counter() - t_step) * 1e3, 2))
             launches += int(info.launches + st.launches)
-            for name, _t in st._fields_:
-                if name != "reserved":
-                    stats_sum[name] = stats_sum.get(name, 0.0) + float(getattr(st, name))
+            ms_total += float(st.ms_total)
         ev1.record()
         barrier()
         clocks = sampler.stop() if sampler else None
         ms_step = max_over_ranks(ev0.elapsed_time(ev1), world, "cuda") / steps
         products = int(info.products_total)
-        stats_avg = {k: v / steps for k, v in stats_sum.items()}
+        n_parts = len(step_parts)
+        stats_sum: dict[str, float] = {}
+        for i in range(3):  # the first is a warm-up
+            _info, st, _nnz = step(True, one_stream)
+            for name, _t in st._fields_:
+                if name != "reserved" and i > 0:
+                    stats_sum[name] = stats_sum.get(name, 0.0) + float(getattr(st, name))
+        del step_parts[n_parts:]
+        stats_avg = {k: v / 2 for k, v in stats_sum.items()}
         # byte model: the row analysis (untimed plan) says which entries of A sit in light rows
         plan = gm.spgemm_plan(dA, dB, SMEM_BYTES, opts)
         ip_dev = plan.row_products().cpu().numpy()
@@ -405,19 +432,20 @@ def main():
         return {"ms_step": ms_step, "value": replicas_value(products, world, ms_step), "products": products,
                 "info": info, "kernels": kt, "dominant": dom, "launches": launches, "nnz": int(nnz), "clocks": clocks,
                 "early_exit_products": int(stats_avg["early_exit_products"]), "ms_steps": ms_steps, "step_parts": step_parts,
-                "ms_execute_device": stats_avg["ms_total"]}
+                "ms_execute_device": ms_total / steps, "ms_execute_device_one_stream": stats_avg["ms_total"]}
 
     peak, peak_kind = _peaks()
     m = measure(A, B, dA, dB, opts, args.steps, args.warmup, True)
     info, kt, dom, nnz, products, launches = m["info"], m["kernels"], m["dominant"], m["nnz"], m["products"], m["launches"]
     value, ms_step, clocks, tau = m["value"], m["ms_step"], m["clocks"], info.params.tau
 
-    # ---- roofline of the dominant kernel (times: CUDA events recorded by the library on the execute stream)
+    # ---- roofline of the dominant kernel (times: CUDA events recorded by the library, every kernel on the execute stream)
     n_b = max(int(info.n_batches), 1)
     n_split = max(info.params.n_levels - (1 if info.level0_direct else 0), 1)
     per_launch = {"k4_expand": n_b, "k5a_histogram": n_b * n_split,
                   "k5b_multisplit": n_b * n_split, "k6_accumulate": n_b,
-                  "k6_small_chunks": n_b, "k6_mid_chunks": n_b, "k7_gather": n_b}.get(dom, 1)
+                  "k6_small_chunks": n_b, "k6_mid_chunks": n_b, "k7_gather": n_b,
+                  "k6_small_tasks": n_b, "k6_mid_tasks": n_b, "k6_big_tasks": n_b}.get(dom, 1)
     roofline = {"kernel": dom, "bound": "hbm", "achieved": kt[dom]["gbs"], "peak": peak, "unit": "GB/s",
                 "frac": kt[dom]["gbs"] / peak, "peak_kind": f"of {peak_kind}",
                 "traffic": (kt[dom]["bytes"] / per_launch * TRAFFIC_RATIO[dom]) if dom in TRAFFIC_RATIO else None,
@@ -435,11 +463,12 @@ def main():
                    "products": products, "products_heavy": int(info.products_heavy), "nnz_c": int(nnz),
                    "rows_heavy": int(info.rows_heavy), "tau": int(tau), "chunk_width": int(info.params.chunk_width),
                    "levels": info.params.levels(), "batches": int(info.n_batches), "smem_bytes": SMEM_BYTES,
-                   "level0_direct": int(info.level0_direct),
+                   "level0_direct": int(info.level0_direct), "heavy_tasks": int(info.heavy_tasks),
                    "early_exit_products": m["early_exit_products"], "plan_opts": args.opt,
                    "step": "gm_spgemm_plan + gm_spgemm_execute (C freed after each step)"},
         "roofline": roofline, "kernels": kt, "clocks": clocks, "gpu_launches": launches,
         "ms_steps_host_clock": m["ms_steps"], "ms_execute_device": m["ms_execute_device"],
+        "ms_execute_device_one_stream": m["ms_execute_device_one_stream"],
         "ms_plan_execute_host_execute_device": m["step_parts"],
     }
 
@@ -447,8 +476,8 @@ def main():
         return {"bytes": k["bytes"], "ms": k["ms"], "gbs": k["gbs"], "frac": k["gbs"] / peak, "peak_kind": f"of {peak_kind}"}
 
     if rank == 0 and not args.no_extra and info.params.n_levels > 0 and info.rows_heavy > 0:
-        # The default plan of a one-level product lets the expansion place the products, so no multisplit pass runs
-        # in the timed steps above.  Same workload once more with the first level as the separate histogram and
+        # The default plan of a one-level product stages nothing, or lets the expansion place the products, so no multisplit
+        # pass runs in the timed steps above.  Same workload once more with the first level as the separate histogram and
         # multisplit passes over the staging buffer (Algorithm 5 as printed): the multisplit kernel's own number.
         o2 = gm.PlanOpts()
         ctypes_copy(o2, opts)

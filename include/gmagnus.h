@@ -1,8 +1,10 @@
 /*
  * gmagnus.h — C ABI of the B200 (sm_100a) SpGEMM library:  C = A * B  for CSR matrices with
- * irregular, power-law structure, following the gMAGNUS method (light rows: Gustavson with a
- * shared-memory hash accumulator; heavy rows: expansion of the intermediate products into a
- * staging buffer, hierarchical multisplit by column chunk, dense shared-memory accumulation).
+ * irregular, power-law structure, following the gMAGNUS method.  Light rows: Gustavson's method, a row's
+ * products merged by a thread or sorted by a warp (hashed in shared memory where a row has more than 1024,
+ * which takes a tau above the default, or where those have no room).  Heavy rows: cut into ranges of columns
+ * whose products are summed where they are generated, or expanded into a staging buffer, regrouped by a
+ * hierarchical multisplit by column chunk and accumulated chunk by chunk.
  *
  * Conventions
  *   - Every function returns an int status: GM_OK (0) or a negative GM_ERR_* code.  No exception
@@ -148,25 +150,28 @@ typedef struct gm_plan_info {
                               that was given, else three                                       */
 } gm_plan_info;
 
-/* Filled by the most recent gm_spgemm_execute on the plan.  Times are CUDA-event milliseconds on
- * the execute stream and are only recorded when the plan was made with GM_TIMING=1 in the
+/* Filled by the most recent gm_spgemm_execute on the plan.  Times are CUDA-event milliseconds around
+ * a part's kernels on the stream they run on (with two streams that includes what a kernel waits for the
+ * other stream's: set single_stream to compare parts) and are only recorded when the plan was made with GM_TIMING=1 in the
  * environment or through gm_plan_set_timing(plan, 1); otherwise they are 0. */
 typedef struct gm_exec_stats {
   int64_t c_nnz;
   int64_t c_nnz_heavy;         /* entries of C that belong to heavy rows                       */
   int64_t c_capacity;          /* entries the C arrays have room for                           */
-  int64_t staged_products;     /* products written to the staging buffer (all batches)         */
-  int64_t final_chunks;        /* (row, chunk) pairs handed to the accumulate kernel           */
+  int64_t staged_products;     /* products of the heavy rows (all batches): written to the staging buffer, or, with
+                                  gm_plan_info.heavy_tasks, summed without it                   */
+  int64_t final_chunks;        /* (row, chunk) pairs they fall into: what the accumulate kernels are handed, or what
+                                  the tasks were cut along                                      */
   int64_t launches;            /* kernels launched by this execute                             */
-  int64_t small_chunk_products; /* products in chunks handled by the one-warp-per-chunk kernel   */
-  int64_t small_chunk_entries;  /* entries of C those chunks produced                            */
+  int64_t small_chunk_products; /* products in chunks or tasks summed by one warp each           */
+  int64_t small_chunk_entries;  /* entries of C those produced                                   */
   float ms_light_symbolic, ms_light_numeric, ms_expand, ms_histogram, ms_multisplit,
       ms_accumulate, ms_gather, ms_scan, ms_total;
-  float ms_small_chunks;       /* the one-warp-per-chunk kernel; ms_accumulate is the dense-accumulator kernel alone */
-  float ms_mid_chunks;         /* the one-small-block-per-chunk kernel                                          */
+  float ms_small_chunks;       /* one warp per chunk or task; ms_accumulate is the dense-accumulator kernel alone */
+  float ms_mid_chunks;         /* one small block per chunk or task                                             */
   float reserved[3];
-  int64_t mid_chunk_products;  /* products in chunks handled by the one-small-block-per-chunk kernel             */
-  int64_t mid_chunk_entries;   /* entries of C those chunks produced                                             */
+  int64_t mid_chunk_products;  /* products in chunks or tasks summed by one small block each                     */
+  int64_t mid_chunk_entries;   /* entries of C those produced                                                    */
   int64_t early_exit_products; /* products of chunks that left the multisplit hierarchy before its last level    */
   int64_t early_exit_chunks;   /* ... and how many chunks did                                                     */
   int64_t split_products;      /* products moved by multisplit passes, summed over the levels                     */
@@ -218,8 +223,9 @@ int gm_spgemm_plan(const gm_csr* A, const gm_csr* B, size_t smem_bytes, gm_plan*
 int gm_spgemm_plan_ex(const gm_csr* A, const gm_csr* B, size_t smem_bytes,
                       const gm_plan_opts* opts, void* cuda_stream, gm_plan** plan_out);
 
-/* The rest of Algorithm 3: light rows by Gustavson's method with a shared-memory hash accumulator
- * (rows of few products: one sort or merge); heavy rows, batch by batch, either cut into ranges of columns whose
+/* The rest of Algorithm 3: light rows by Gustavson's method, every row's products merged by a thread, sorted
+ * by a warp, or (more than 1024, or no room to keep sums until C.row_ptr is known) added up in a hash table in
+ * shared memory; heavy rows, batch by batch, either cut into ranges of columns whose
  * products are summed where they are generated, without being staged (column spaces that one split covers, rows of
  * B long enough for it), or through the expansion (outer-product)
  * kernel (Algorithm 4), one histogram + multisplit (Algorithm 5) per level (by default the first
