@@ -364,13 +364,10 @@ struct gm_plan {
   cudaEvent_t ev_fork = nullptr, ev_light = nullptr;
 };
 
-#ifndef GM_MID_MIN_TASK_BLOCKS
-#define GM_MID_MIN_TASK_BLOCKS 5
-#endif
-#ifndef GM_MID_MIN_BLOCKS
-#define GM_MID_MIN_BLOCKS 7
-#endif
 namespace gm {
+
+// Blocks of the mid-size class that must fit an SM, with and without staged products.
+constexpr int kMidMinBlocks = 7, kMidMinTaskBlocks = 5;
 
 // Lets a kernel take all the dynamic shared memory there is.  (The limit belongs to the kernel and not to a launch: set to what
 // one launch needs, it failed the launch of another host thread whose plan has a larger budget.)
@@ -603,7 +600,7 @@ static bool plan_task_rules(gm_plan* p) {
   const int mid_default = static_cast<int>(std::max<i64>(256, std::min<i64>(p->sv == 4 ? 4096 : 2048, w / (p->info.products_heavy < (i64{1} << 24) ? 8 : 4))));
   int mid = o.mid_chunk_max < 0 ? 0 : (o.mid_chunk_max ? o.mid_chunk_max : mid_default);
   const size_t fixed = (p->sv == 4 ? sizeof(Pieces<float, kMidThreads * kMidPerThread>) : sizeof(Pieces<double, kMidThreads * kMidPerThread>)) + 2048;
-  while (mid > r.small_max && mid_task_smem_bytes(static_cast<int>(r.mid_width), p->sv, mid) + fixed > p->smem_bytes / GM_MID_MIN_TASK_BLOCKS) mid /= 2;
+  while (mid > r.small_max && mid_task_smem_bytes(static_cast<int>(r.mid_width), p->sv, mid) + fixed > p->smem_bytes / kMidMinTaskBlocks) mid /= 2;
   r.mid_max = std::max(mid, r.small_max);
   // A hub row's granule is cut when it would keep a block busy for longer than an eighth of its even share of the whole (but
   // not below 8192 products, where the pieces of the sub-ranges get short: R-MAT scale 12 took 312 us with a floor of 32768,
@@ -734,7 +731,7 @@ static int build_plan(gm_plan* p, cudaStream_t st) {
     p->small_max = o.small_chunk_max < 0 ? 0 : (o.small_chunk_max ? o.small_chunk_max : kAccSmallDefault);
     int mid = o.mid_chunk_max < 0 ? 0 : (o.mid_chunk_max ? o.mid_chunk_max : (p->sv == 4 ? 4096 : 2048));
     // several mid-chunk blocks must fit an SM next to each other for the class to pay
-    while (mid > p->small_max && mid_smem_bytes(prm.chunk_width, p->sv, mid) + 1024 > p->smem_bytes / GM_MID_MIN_BLOCKS) mid /= 2;
+    while (mid > p->small_max && mid_smem_bytes(prm.chunk_width, p->sv, mid) + 1024 > p->smem_bytes / kMidMinBlocks) mid /= 2;
     if (prm.chunk_width > 65536) mid = 0;  // the kernel keeps a chunk's columns as 16-bit offsets
     p->mid_max = std::max(mid, p->small_max);
     if (o.early_exit < -1 || o.early_exit > kAccSmallChunk) return fail(GM_ERR_INVALID_ARG, "early_exit out of range");
@@ -1511,7 +1508,7 @@ static int dev_error_to_status(int code) {
 
 template <typename V>
 static TaskInput<V> task_input(const gm_plan* p) {
-  return TaskInput<V>{p->A.col_idx, static_cast<const V*>(p->A.vals), p->B.row_ptr, p->B.col_idx, static_cast<const V*>(p->B.vals),
+  return TaskInput<V>{p->A.col_idx, static_cast<const V*>(p->A.vals), p->B.col_idx, static_cast<const V*>(p->B.vals),
                       p->piece_bound, p->task_rules.granules, p->task_rules.log2_g};
 }
 

@@ -44,7 +44,7 @@ struct TaskRules {
 constexpr int kMaxParts = 16;
 
 // bound[k * (granules + 1) + c] = position in B's arrays of the first entry of row k with column >= c << log2_g.
-// One warp per row of B: lane by lane over the boundaries, each a binary search inside the row.
+// A thread per boundary, each a binary search inside the row.
 // longest: (entries << 32) | row of the longest row of B.
 __global__ void __launch_bounds__(256) k_piece_bounds(const i64* __restrict__ b_row_ptr, const int32_t* __restrict__ b_col, i64 n_rows_b,
                                                       int granules, int log2_g, u32* __restrict__ bound, u64* __restrict__ longest) {
@@ -252,7 +252,6 @@ template <typename V>
 struct TaskInput {
   const int32_t* a_col;
   const V* a_val;
-  const i64* b_row_ptr;
   const int32_t* b_col;
   const V* b_val;
   const u32* bound;

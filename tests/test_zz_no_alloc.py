@@ -1,9 +1,9 @@
 """The entry point for callers that cannot allocate device memory (a component with a fixed memory
 budget, a latency-critical section, a host whose allocator belongs to another runtime):
-gm_row_products_noalloc computes the intermediate products per row with its scratch in a fixed array
-of the library image.  Checked here, through the C ABI, against the row analysis of gm_spgemm_plan
-(the existing entry point) and against the CPU oracle's count, bit for bit because the result is an
-integer count, on two calls in a row that share the scratch array.  This file sorts last so that a stop-at-first-failure run has
+gm_row_products_noalloc computes the intermediate products per row without scratch memory.  Checked
+here, through the C ABI, against the row analysis of gm_spgemm_plan (the existing entry point) and
+against the CPU oracle's count, bit for bit because the result is an integer count, on two calls in a
+row with nothing in between.  This file sorts last so that a stop-at-first-failure run has
 already been through every other test."""
 import numpy as np
 import pytest
@@ -26,7 +26,7 @@ def _reference(gm, dA, dB):
 def test_no_alloc_row_products_matches_plan_twice_in_a_row():
     import paper_2607_22866_b200 as gm
 
-    # second input is larger and rectangular, so stale scratch from the first call would show
+    # second input is larger and rectangular: anything left over from the first call would show
     A1 = gen.rmat(12, 16, seed=21, dtype=np.float32)
     A2, B2 = gen.zipf_rectangular_pair(1 << 13, 1 << 15, 1 << 17, seed=22, dtype=np.float32)
     assert A1.nnz <= gm.NOALLOC_MAX_NNZ_A and A2.nnz <= gm.NOALLOC_MAX_NNZ_A
@@ -45,7 +45,7 @@ def test_no_alloc_row_products_matches_plan_twice_in_a_row():
     for out, ref, (hA, hB) in zip(outs, refs, [(A1, A1), (A2, B2)]):
         assert torch.equal(out, ref)
         assert np.array_equal(out.cpu().numpy(), oracle.row_products(hA, hB))
-    # and once more in the other order: the scratch is reused, nothing needs clearing
+    # and once more in the other order
     for (dA, dB), out, ref in reversed(list(zip(cases, outs, refs))):
         out.fill_(-1)
         gm.row_products_noalloc(dA, dB, out)
@@ -53,7 +53,7 @@ def test_no_alloc_row_products_matches_plan_twice_in_a_row():
         assert torch.equal(out, ref)
 
 
-def test_no_alloc_rejects_inputs_beyond_its_fixed_scratch():
+def test_no_alloc_rejects_inputs_beyond_its_limit():
     import paper_2607_22866_b200 as gm
 
     A = gen.erdos_renyi_k(1 << 17, 9, seed=3, dtype=np.float32)   # 1,179,648 stored entries > 1,048,576
