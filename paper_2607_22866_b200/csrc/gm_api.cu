@@ -407,14 +407,18 @@ static void plan_free(gm_plan* p, void* q, cudaStream_t st) {
   }
 }
 
-// Bytes a plan sets aside for the light rows' staging area before it knows their products.
+// Bytes a plan sets aside for the light rows' staging area before it knows their products: an allocation less (a product call of
+// ER with 1000 rows takes 76 us, 84 without; with 10000 87.5 and 92), and nothing a device would miss.
 constexpr size_t kLightRoom = size_t{4} << 20;
 // C is allocated before its size is known, with room for every product, when that takes at most this much: the call then
-// does not wait in the middle for nnz(C), and the allocation overlaps the kernels.
+// does not wait in the middle for nnz(C), and the allocation overlaps the kernels.  Product calls with the wait and without, us:
+// ER of 1000 rows 88 / 76, of 10000 95 / 87.5, of 200000 (165 MB of room) 575 / 566; R-MAT scale 12 fp32 (33 MB) 223 / 215.5,
+// scale 13 with 15 edges a vertex (90 MB) 336 / 324.  More room would still gain, but is memory that a caller may not have.
 constexpr i64 kCRoomBytes = i64{64} << 20;
 // ... and what the caller then holds for nothing is at most this much, or as much again as C itself takes: with more C is
-// moved to arrays of its size.
-constexpr i64 kCSpareBytes = i64{4} << 20;
+// moved to arrays of its size, which costs some 20 us (block-dense fp32 of 2400 rows, 14 MB of C in 35 MB of room: 346 us moved,
+// 328 kept).
+constexpr i64 kCSpareBytes = i64{32} << 20;
 
 // Several device arrays in one allocation: the allocator hook of the Python binding costs a few microseconds a call.
 struct Arena {
@@ -859,7 +863,10 @@ static int build_plan(gm_plan* p, cudaStream_t st) {
     // Products are summed where they are generated, unless a first level is asked for or the pieces of B's rows get too short: a task looks every row of B up
     // in the boundary table, so that costs per (segment, granule) and not per product.  Products per (segment, granule) and time
     // per call, tasks against staged products: R-MAT scale 18 fp64 with 4 edges a vertex about 9, 4.2 against 5.4 ms; R-MAT scale 20
-    // fp32 20, 188 against 198 ms; R-MAT scale 21 fp64 3.7, 291 against 278 ms.
+    // fp32 20, 188 against 198 ms; R-MAT scale 21 fp64 3.7, 291 against 278 ms.  With rows of equal length (ER) 1.9 / 2.5: 3.25
+    // against 3.13 ms / 10.4 against 9.95; R-MAT scale 19 fp64 with 4 / 8 edges a vertex 5.1 / 9.0: 10.73 against 10.78 / 30.7 against
+    // 33.8.  Up to eight granules it is the pieces of a row that count little: ER of 65536 and 131072 columns, 1.0: 1.90 against 2.05 ms,
+    // 1.9: 1.51 against 1.87, 3.75: 1.46 against 1.65 and 2.47 against 2.74, and 7.5 with four granules 1.25 against 1.20.
     p->use_tasks = p->opts.level0_multisplit == 0 && !p->csc && !p->stream && (prm.n_levels == 0 || (prm.n_levels == 1 && p->direct)) && plan_task_rules(p) &&
                    (p->task_rules.granules <= 8 || info.products_heavy >= kMinPieceProducts * p->n_seg * p->task_rules.granules);
     info.heavy_tasks = p->use_tasks ? 1 : 0;
@@ -1039,6 +1046,8 @@ static int launch_merge(gm_plan* p, const int32_t* rows, i64 n_rows, const i64* 
                                          p->B.col_idx, static_cast<const V*>(p->B.vals), rows, n_rows, p->light_off,       \
                                          p->row_nnz, c_row_ptr, out_col, out_val);                                         \
   } while (0)
+  // (an instance costs registers for the lists it has room for: the 1024^2 grid fp64, five lists, takes 254 us a call with the
+  // instance for five, 279 with the one for eight)
   if (p->merge_lists <= 2) GM_MERGE(2);
   else if (p->merge_lists <= 4) GM_MERGE(4);
   else if (p->merge_lists <= 5) GM_MERGE(5);
