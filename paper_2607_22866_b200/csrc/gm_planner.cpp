@@ -75,11 +75,12 @@ int planner_params(int64_t c_cols, int dtype, size_t smem_bytes, const gm_plan_o
   if (required > (int64_t{1} << 30)) return GM_ERR_CAPACITY;
   out->chunks_required = static_cast<int32_t>(required);
 
-  // --- default tau.  The capacity is an upper limit.  A light row pays for a hash table and an n log^2 n sort
-  // in one block; a heavy row pays per chunk (a one-warp register sort for the small ones).  Measured on
-  // B200: with up to 32 chunks per row the heavy path is cheaper from about 512 products on, with more
-  // chunks per row from about 1024 (R-MAT 20: 445 ms at 4096, 414 ms at 512; R-MAT 21 in fp64, 128 chunks:
-  // 610 ms at 4096, 530 ms at 1024).
+  // --- default tau.  The capacity is an upper limit.  A light row is sorted by one warp up to 1024 products and
+  // hashed by a block above; a heavy row pays per task or chunk (a one-warp sort for the small ones).  Up to 1024
+  // it hardly matters, the hash accumulator is what costs.  Product calls at 128 / 256 / 512 / 1024 / 2048:
+  // R-MAT 12 fp32 215 / 215 / 214 / 235 / 379 us, 15 fp32 1144 / 1144 / 1151 / 1189 / 1737, 17 fp64
+  // 4045 / 4053 / 4015 / 3977 / 5079, 19 fp32 61.9 / 61.8 / 61.4 / 61.4 / 66.6 ms; the Zipf pair (512 chunks)
+  // 5645 / 5141 / 4819 / 4935 / 5894 us.
   int64_t tau = o.tau > 0 ? o.tau : std::min<int64_t>(cap, required <= 32 ? 512 : 1024);
   const int64_t top_cap = static_cast<int64_t>(pow2_ceil(static_cast<uint64_t>(std::max<int64_t>(tau, 16))));
   out->tau = tau;
