@@ -39,13 +39,13 @@ DEFAULT_CONFIG = 2  # R-MAT scale 20, edge factor 16, fp32: the largest fp32 pow
 
 
 # DRAM bytes per launch (ncu dram__bytes_read.sum + dram__bytes_write.sum) over the algorithmic bytes of the same
-# launch, from single-kernel, single-launch ncu captures of these kernels on the same product scaled down by 2**3
-# (R-MAT scale 17: one batch holds the whole product, 1.09 G products, about 9 GB staged).  Traffic grows in
+# launch, from single-kernel, single-launch ncu captures of these kernels on R-MAT products that one batch holds
+# (scale 17, 1.09 G products, about 9 GB staged; k7_gather scale 16, 115 M entries of C).  Traffic grows in
 # proportion to the products processed, so a full-size launch is its algorithmic figure times this ratio.  A kernel
 # that has changed since its capture must lose its entry (traffic is then reported as null).
-TRAFFIC_RATIO = {"k4_expand": 1.03, "k5a_histogram": 1.00, "k5b_multisplit": 1.00, "k7_gather": 1.00}
-TRAFFIC_SOURCE = ("single-kernel, single-launch ncu DRAM-counter captures on the same recipe 2**3 smaller (R-MAT scale 17, "
-                  "one batch holds the whole product), scaled by products")
+TRAFFIC_RATIO = {"k5a_histogram": 1.00, "k5b_multisplit": 1.00, "k7_gather": 0.97}
+TRAFFIC_SOURCE = ("single-kernel, single-launch ncu DRAM-counter captures on smaller R-MAT products (scale 17, k7_gather: scale 16 "
+                  "with 12 edges a vertex; one batch holds the whole product), scaled by products")
 
 
 def ctypes_copy(dst, src):
