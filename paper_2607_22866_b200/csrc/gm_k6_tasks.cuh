@@ -99,10 +99,24 @@ __device__ __forceinline__ void count_granules(const int32_t* __restrict__ a_col
   for (int c0 = 0; c0 < granules; c0 += 32) {
     const int c = c0 + (lane & (width - 1));
     u32 sum = 0;
+    if (add) {  // (a slice of a long row: many warps, one after the other)
 #pragma unroll 4
-    for (i64 j = s + sub; j < e; j += step) {
-      const u32* bp = bound + static_cast<i64>(a_col[j]) * (granules + 1) + c;
-      sum += bp[1] - bp[0];
+      for (i64 j = s + sub; j < e; j += step) {
+        const u32* bp = bound + static_cast<i64>(a_col[j]) * (granules + 1) + c;
+        sum += bp[1] - bp[0];
+      }
+    }
+    for (i64 j0 = s; !add && j0 < e; j0 += 32) {  // 32 entries' columns at once, so that the look-ups do not wait for one another
+      const int n = static_cast<int>(min(i64{32}, e - j0));
+      const int32_t mine = lane < n ? a_col[j0 + lane] : 0;
+#pragma unroll 8
+      for (int t = 0; t < n; t += step) {
+        const int32_t k = __shfl_sync(0xffffffffu, mine, t + sub);
+        if (t + sub < n) {
+          const u32* bp = bound + static_cast<i64>(k) * (granules + 1) + c;
+          sum += bp[1] - bp[0];
+        }
+      }
     }
     for (int o = width; o < 32; o <<= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
     if (sub == 0) {
@@ -126,22 +140,21 @@ __global__ void __launch_bounds__(256) k_granule_counts(const int32_t* __restric
     }
   }
 }
+// Block (x, y) takes rows x, x + gridDim.x, ... and of each the runs y, y + gridDim.y, ... of kCountRun entries, a slice per warp.  (With
+// all warps of the grid round-robin over all slices, every warp looked up every row's ends, one after the other: 730 us of R-MAT
+// scale 19.)
+constexpr int kCountRun = 8 * 256, kCountRuns = 16;
 __global__ void __launch_bounds__(256) k_granule_counts_long(const int32_t* __restrict__ x_heavy, const i64* __restrict__ a_row_ptr,
                                                              const int32_t* __restrict__ a_col, const u32* __restrict__ bound, int granules,
                                                              u32* __restrict__ counts, const int32_t* __restrict__ long_rows,
                                                              const u32* __restrict__ n_long) {
   const u32 n = *n_long;
-  const u32 w0 = blockIdx.x * 8 + (threadIdx.x >> 5), n_warps = gridDim.x * 8;
-  u32 before = 0;  // the warps go on round-robin from one row's slices to the next row's
-  for (u32 q = 0; q < n; ++q) {
+  for (u32 q = blockIdx.x; q < n; q += gridDim.x) {
     const i64 h = long_rows[q];
     const i64 row = x_heavy[h];
-    const i64 s = a_row_ptr[row], e = a_row_ptr[row + 1];
-    constexpr i64 kSlice = 256;
-    const u32 slices = static_cast<u32>((e - s + kSlice - 1) / kSlice);
-    for (u32 i = (w0 + n_warps - before % n_warps) % n_warps; i < slices; i += n_warps)
-      count_granules(a_col, s + i * kSlice, min(e, s + (i + 1) * kSlice), bound, granules, counts + h * granules, true);
-    before += slices;
+    const i64 e = a_row_ptr[row + 1];
+    for (i64 s = a_row_ptr[row] + static_cast<i64>(blockIdx.y) * kCountRun + (threadIdx.x >> 5) * 256; s < e; s += static_cast<i64>(gridDim.y) * kCountRun)
+      count_granules(a_col, s, min(e, s + 256), bound, granules, counts + h * granules, true);
   }
 }
 
@@ -194,20 +207,29 @@ struct TaskTables {
   i64 first, end;  // the batch's part of the tables
 };
 
-// Writes the tasks of heavy row h, the first of them at position id.
+// Class of a range (an index into TaskTables::counters).
+__device__ __forceinline__ int class_of(const TaskRules& r, int granules, u32 n, u32 parts) {
+  if (parts > 1) return 2;
+  if (n <= static_cast<u32>(r.small_max)) return 0;
+  if (n <= static_cast<u32>(r.mid_max) && static_cast<u32>(granules) << r.log2_g <= r.mid_width) return 1;
+  return n > static_cast<u32>(kHugeChunk) ? 2 : 3;
+}
+
+// Writes the tasks of heavy row h, the first of them at position id.  place(c): next position of class c.
+template <typename Place>
 __device__ __forceinline__ void emit_row(const u32* __restrict__ counts, const i64* __restrict__ heavy_base, i64 h, i64 elem0,
                                          const TaskRules& r, i64 id, const int32_t* __restrict__ x_heavy,
-                                         const i64* __restrict__ a_row_ptr, const u32* __restrict__ parts_tab, const TaskTables& tt) {
+                                         const i64* __restrict__ a_row_ptr, const u32* __restrict__ parts_tab, const TaskTables& tt, Place place) {
   const i64 row = x_heavy[h];
   HeavyTask t;
   t.a0 = a_row_ptr[row];
   t.n_a = static_cast<u32>(a_row_ptr[row + 1] - t.a0);
   i64 off = heavy_base[h] - elem0;
-  auto put = [&](int cls, bool front) {
+  auto put = [&](int cls) {
     const int b = static_cast<int>(id - tt.first);  // lists hold batch-relative ids
-    if (cls < 2) tt.list[cls][tt.first + atomicAdd(&tt.counters[cls], 1)] = b;
-    else if (front) tt.list[2][tt.first + atomicAdd(&tt.counters[2], 1)] = b;
-    else tt.list[2][tt.end - 1 - atomicAdd(&tt.counters[3], 1)] = b;
+    if (cls == 0 || cls == 1) tt.list[cls][tt.first + place(cls)] = b;
+    else if (cls == 2) tt.list[2][tt.first + place(2)] = b;
+    else tt.list[2][tt.end - 1 - place(3)] = b;
     tt.tasks[id] = t;
     tt.task_off[id] = t.off;
     ++id;
@@ -222,15 +244,14 @@ __device__ __forceinline__ void emit_row(const u32* __restrict__ counts, const i
         t.hi = cut[(i + 1) * (kMaxParts / parts)];
         t.off = off + (t.lo - lo);
         t.n = 0;
-        put(2, true);
+        put(2);
       }
     } else {
       t.lo = lo;
       t.hi = lo + width;
       t.off = off;
       t.n = n;
-      const int cls = n <= static_cast<u32>(r.small_max) ? 0 : (n <= static_cast<u32>(r.mid_max) && width <= r.mid_width ? 1 : 2);
-      put(cls, n > static_cast<u32>(kHugeChunk));
+      put(class_of(r, w, n, 1));
     }
     off += n;
   });
@@ -241,8 +262,33 @@ __global__ void __launch_bounds__(128) k_task_emit(const u32* __restrict__ count
                                                    i64 elem0, TaskRules r, const i64* __restrict__ row_task_off,
                                                    const int32_t* __restrict__ x_heavy, const i64* __restrict__ a_row_ptr,
                                                    const u32* __restrict__ parts_tab, TaskTables tt) {
+  // Places in the lists are drawn once per block and class.  With an atomic per task on four words of L2, which take turns, this kernel
+  // took 112 us for R-MAT scale 17 (now 27) and 1.5 ms for scale 19.
+  __shared__ u32 s_n[4], s_base[4];
   const i64 h = h0 + static_cast<i64>(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (h < h1) emit_row(counts, heavy_base, h, elem0, r, row_task_off[h], x_heavy, a_row_ptr, parts_tab, tt);
+  const bool mine = h < h1;
+  if (threadIdx.x < 4) s_n[threadIdx.x] = 0u;
+  __syncthreads();
+  if (mine) {
+    u32 n_of[4] = {0u, 0u, 0u, 0u};
+    cut_row(counts + h * r.granules, static_cast<u32>(heavy_base[h + 1] - heavy_base[h]), r, [&](int, int w, u32 n, u32 parts) {
+      const int c = class_of(r, w, n, parts);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) n_of[i] += i == c ? parts : 0u;
+    });
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      if (n_of[i]) atomicAdd(&s_n[i], n_of[i]);
+  }
+  __syncthreads();
+  if (threadIdx.x < 4) {
+    s_base[threadIdx.x] = s_n[threadIdx.x] ? static_cast<u32>(atomicAdd(&tt.counters[threadIdx.x], static_cast<int>(s_n[threadIdx.x]))) : 0u;
+    s_n[threadIdx.x] = 0u;
+  }
+  __syncthreads();
+  if (mine)
+    emit_row(counts, heavy_base, h, elem0, r, row_task_off[h], x_heavy, a_row_ptr, parts_tab, tt,
+             [&](int c) { return s_base[c] + atomicAdd(&s_n[c], 1u); });
 }
 
 // ---------------------------------------------------------------------------------------------------------------------
@@ -1019,8 +1065,14 @@ __global__ void __launch_bounds__(kFinishThreads) k_plan_small(const u32* counts
     row_tasks[h] = cut_row(counts + h * r.granules, static_cast<u32>(heavy_base[h + 1] - heavy_base[h]), r, [](int, int, u32, u32) {});
   __syncthreads();
   finish_scan(row_tasks, n_heavy, n_heavy, row_task_off, tmp);
+  __shared__ u32 s_n[4];
+  if (threadIdx.x < 4) s_n[threadIdx.x] = 0u;
+  __syncthreads();
   for (i64 h = threadIdx.x; h < n_heavy; h += kFinishThreads)
-    emit_row(counts, heavy_base, h, 0, r, row_task_off[h], x_heavy, a_row_ptr, parts_tab, tt);
+    emit_row(counts, heavy_base, h, 0, r, row_task_off[h], x_heavy, a_row_ptr, parts_tab, tt,
+             [&](int c) { return atomicAdd(&s_n[c], 1u); });
+  __syncthreads();
+  if (threadIdx.x < 4) tt.counters[threadIdx.x] = static_cast<int>(s_n[threadIdx.x]);
 }
 
 }  // namespace gm
