@@ -1261,7 +1261,7 @@ static int launch_gather(gm_plan* p, const Batch& b, const HeavyBatchState<V>& h
   const bool alt = hs.tags && hs.xt.alt_bits;
   auto kern = alt ? (tile == kGatherTile ? k7_gather<V, kGatherTile, true> : tile == 4096 ? k7_gather<V, 4096, true> : k7_gather<V, 2048, true>)
                   : (tile == kGatherTile ? k7_gather<V, kGatherTile> : tile == 4096 ? k7_gather<V, 4096> : k7_gather<V, 2048>);
-  kern<<<grid, kGatherThreads, 0, st>>>(hs.fin_col, hs.fin_val, hs.chunk_off, p->chunk_nnz_off, p->chunk_base, hs.n_chunks,
+  kern<<<std::min(grid, static_cast<unsigned>(p->num_sms * kGatherBlocksPerSm)), kGatherThreads, 0, st>>>(hs.fin_col, hs.fin_val, hs.chunk_off, p->chunk_nnz_off, p->chunk_base, hs.n_chunks,
                                         p->tile_meta, c_col, c_val, c_capacity, p->err, alt ? hs.alt_col : nullptr,
                                         alt ? hs.alt_val : nullptr, alt ? hs.tags : nullptr, alt ? hs.xt.alt_bits : 0);
   p->stats.launches += 3;
@@ -1623,7 +1623,7 @@ static int task_batch_gather(gm_plan* p, size_t bi, bool bases, const i64* c_row
     k_tile_bounds<<<grid_for(grid, 256, p->num_sms), 256, 0, st>>>(p->chunk_nnz_off, n, 0, 0, kGatherTile, p->tile_meta, p->chunk_nnz_off + n);
     p->stats.launches += 2;
   }
-  k7_gather<V, kGatherTile><<<grid, kGatherThreads, 0, st>>>(
+  k7_gather<V, kGatherTile><<<std::min(grid, static_cast<unsigned>(p->num_sms * kGatherBlocksPerSm)), kGatherThreads, 0, st>>>(
       p->stage_col[0], static_cast<const V*>(p->stage_val[0]), p->task_off + t0, p->chunk_nnz_off, p->chunk_base, n, p->tile_meta, c_col,
       c_val, c_capacity, p->err, nullptr, nullptr, nullptr, 0);
   p->stats.launches += 1;
