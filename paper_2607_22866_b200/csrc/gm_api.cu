@@ -273,6 +273,10 @@ struct gm_plan {
   bool light_relist = false;       // the area is gone, the rows have to be listed for the hash accumulator first
   int merge_lists = 0;             // most entries of A in a merged row
   bool merge_only = false;         // every row of A is merged or empty
+  bool row_sums = false;           // no prefix sum over the rows (see RowSums)
+  gm::u32* sums[2]{};              // this execute's and the next one's
+  int sums_at = 0;
+  bool sums_dirty = false;         // an execute failed on the way
   gm::LightBins bins{};            // hash rows by entry count, for their numeric pass
   int bin_slots[gm::kMaxLightBins]{};
   gm::HostSlot* slot = nullptr;
@@ -415,6 +419,9 @@ constexpr size_t kLightRoom = size_t{4} << 20;
 // ER of 1000 rows 88 / 76, of 10000 95 / 87.5, of 200000 (165 MB of room) 575 / 566; R-MAT scale 12 fp32 (33 MB) 223 / 215.5,
 // scale 13 with 15 edges a vertex (90 MB) 336 / 324.  More room would still gain, but is memory that a caller may not have.
 constexpr i64 kCRoomBytes = i64{64} << 20;
+// ... and this much where a prefix sum over the rows is left out with the wait (see RowSums; product calls, us, with the wait and the
+// prefix sum / without: the 1024^2 grid fp64, 314 MB of room for 163 MB of C, 250 / 243; ER of 200000 rows of 12 fp32, 230 MB, 575 / 560).
+constexpr i64 kCRoomBytesPlaced = i64{512} << 20;
 // ... and what the caller then holds for nothing is at most this much, or as much again as C itself takes: with more C is
 // moved to arrays of its size, which costs some 20 us (block-dense fp32 of 2400 rows, 14 MB of C in 35 MB of room: 346 us moved,
 // 328 kept).
@@ -478,18 +485,22 @@ __global__ void k_validate_csr(const i64* __restrict__ row_ptr, const int32_t* _
   }
 }
 
+static size_t row_sum_words(i64 n_rows) { return (static_cast<size_t>(n_rows) / kSumRows + 64) & ~size_t{63}; }
+
 // What the row analysis wants zeroed, at the front of an arena.
 struct K1Zeroed {
   K1Totals* totals = nullptr;
   HeavyTile* tiles = nullptr;
   i64* ip = nullptr;
   u32* parts = nullptr;
+  u32* sums[2]{};  // row_sum_words each, one after the other
   size_t bytes = 0;
   void add_to(Arena& ar, i64 n_rows) {
     ar.add(&totals, 1);
     ar.add(&tiles, static_cast<size_t>((n_rows + kHeavyRows - 1) / kHeavyRows) + 1);
     ar.add(&ip, static_cast<size_t>(n_rows) + 1);
     ar.add(&parts, static_cast<size_t>(n_rows) + 1);
+    for (auto& q : sums) ar.add(&q, row_sum_words(n_rows));
     bytes = ar.bytes;
   }
 };
@@ -537,6 +548,7 @@ static int analyse_rows(gm_plan* p, const K1Zeroed& z, cudaStream_t st) {
 static int light_rows_by_hash(gm_plan* p, cudaStream_t st) {
   const i64 nA = p->A.n_rows;
   p->light_relist = true;
+  p->row_sums = false;
   plan_free(p, p->light_stage, st);
   p->light_stage = nullptr;
   p->light_col = nullptr;
@@ -799,6 +811,7 @@ static int build_plan(gm_plan* p, cudaStream_t st) {
   GM_TRY(analyse_rows(p, z, st));  // ---- first host sync: totals
   const i64 nH = info.rows_heavy;
   p->n_seg = info.nnz_a_heavy;
+  for (int i = 0; i < 2; ++i) p->sums[i] = z.sums[i];
 
   // ---- light rows: staging area (not when all rows are merged), bins of the hash rows
   bool hash_all = false;
@@ -827,6 +840,8 @@ static int build_plan(gm_plan* p, cudaStream_t st) {
       ar.add(&p->num_fill, 8);
       GM_TRY(ar.commit(p, st));
     }
+    p->row_sums = nH == 0 && !hash_rows && info.rows_empty < nA && nA <= kSumRowsMax &&
+                  info.c_nnz_upper * static_cast<i64>(4 + p->sv) <= kCRoomBytesPlaced;
   }
 
   // ---- heavy rows
@@ -1031,9 +1046,13 @@ static int launch_hash(gm_plan* p, int cap, int slots, const int32_t* rows, i64 
 #undef GM_LIGHT
 }
 
+static RowSums row_sums_of(const gm_plan* p) {
+  return p->row_sums ? RowSums{p->sums[p->sums_at], p->sums[p->sums_at ^ 1]} : RowSums{nullptr, nullptr};
+}
+
 // One thread per row: count, write to C, or write to the staging area.
 template <typename V, int MODE>
-static int launch_merge(gm_plan* p, const int32_t* rows, i64 n_rows, const i64* c_row_ptr, int32_t* out_col, V* out_val,
+static int launch_merge(gm_plan* p, const int32_t* rows, i64 n_rows, i64* c_row_ptr, int32_t* out_col, V* out_val,
                         cudaStream_t st) {
   const unsigned grid = static_cast<unsigned>((n_rows + kMergeThreads - 1) / kMergeThreads);
   // Entries for C are collected in shared memory, but the rows of B that neighbouring rows share want to stay in L1: with
@@ -1041,10 +1060,12 @@ static int launch_merge(gm_plan* p, const int32_t* rows, i64 n_rows, const i64* 
 #define GM_MERGE(NL)                                                                                                       \
   do {                                                                                                                     \
     auto kern = k3_merge_rows<V, NL, MODE>;                                                                                \
-    if (MODE == kMergeToC) GM_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 60));        \
+    if (MODE == kMergeToC || MODE == kMergePlace)                                                                          \
+      GM_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 60));                             \
     kern<<<grid, kMergeThreads, 0, st>>>(p->A.row_ptr, p->A.col_idx, static_cast<const V*>(p->A.vals), p->B.row_ptr,       \
                                          p->B.col_idx, static_cast<const V*>(p->B.vals), rows, n_rows, p->light_off,       \
-                                         p->row_nnz, c_row_ptr, out_col, out_val);                                         \
+                                         p->row_nnz, c_row_ptr, out_col, out_val, row_sums_of(p),                          \
+                                         reinterpret_cast<i64*>(&p->slot->c_total));                                       \
   } while (0)
   // (an instance costs registers for the lists it has room for: the 1024^2 grid fp64, five lists, takes 254 us a call with the
   // instance for five, 279 with the one for eight)
@@ -1063,7 +1084,7 @@ static int launch_sort_one(gm_plan* p, const SortLists& lists, i64 n, cudaStream
   const unsigned grid = grid_for(n, kSortWarpsOf<KMAX>, p->num_sms, KMAX > 4 ? 16 : 24);
   k3_sort_rows<V, Key, KMAX><<<grid, kSortWarpsOf<KMAX> * 32, 0, st>>>(
       p->A.row_ptr, p->A.col_idx, static_cast<const V*>(p->A.vals), p->B.row_ptr, p->B.col_idx,
-      static_cast<const V*>(p->B.vals), lists, p->light_off, p->row_nnz, p->light_col, static_cast<V*>(p->light_val));
+      static_cast<const V*>(p->B.vals), lists, p->light_off, p->row_nnz, p->light_col, static_cast<V*>(p->light_val), row_sums_of(p).now);
   ++p->stats.launches;
   GM_CUDA(cudaGetLastError());
   return GM_OK;
@@ -1117,8 +1138,9 @@ static int light_front(gm_plan* p, cudaStream_t st) {
 
 // Light rows [r0, r1) into C, once C.row_ptr covers them.
 template <typename V>
-static int light_back(gm_plan* p, i64 r0, i64 r1, const i64* c_row_ptr, int32_t* c_col, V* c_val, i64 capacity, cudaStream_t st) {
+static int light_back(gm_plan* p, i64 r0, i64 r1, i64* c_row_ptr, int32_t* c_col, V* c_val, i64 capacity, cudaStream_t st) {
   if (p->info.rows_light <= 0 || r1 <= r0) return GM_OK;
+  if (p->merge_only && p->row_sums) return launch_merge<V, kMergePlace>(p, nullptr, p->A.n_rows, c_row_ptr, c_col, c_val, st);
   if (p->merge_only) return launch_merge<V, kMergeToC>(p, nullptr, p->A.n_rows, c_row_ptr, c_col, c_val, st);
   if (p->staged_light > 0) {
     i64 n_staged = 0;
@@ -1127,9 +1149,17 @@ static int light_back(gm_plan* p, i64 r0, i64 r1, const i64* c_row_ptr, int32_t*
 #define GM_COPY(LPR)                                                                                                     \
   k3_copy_rows<V, LPR><<<static_cast<unsigned>(((r1 - r0) * LPR + 255) / 256), 256, 0, st>>>(                             \
       p->light_col, static_cast<const V*>(p->light_val), p->light_off, r0, r1, c_row_ptr, c_col, c_val, capacity, p->err)
-    if (avg <= 16) GM_COPY(8);
+#define GM_PLACE(LPR)                                                                                                             \
+  k3_place_rows<V, LPR><<<static_cast<unsigned>((p->A.n_rows + kPlaceRows<LPR> - 1) / kPlaceRows<LPR>), 256, 0, st>>>(             \
+      p->light_col, static_cast<const V*>(p->light_val), p->light_off, p->A.n_rows, p->row_nnz, row_sums_of(p), c_row_ptr, c_col, \
+      c_val, capacity, reinterpret_cast<i64*>(&p->slot->c_total), p->err)
+    if (p->row_sums) {  // (all rows: there are no batches)
+      if (avg <= 16) GM_PLACE(8);
+      else GM_PLACE(32);
+    } else if (avg <= 16) GM_COPY(8);
     else GM_COPY(32);
 #undef GM_COPY
+#undef GM_PLACE
     ++p->stats.launches;
     GM_CUDA(cudaGetLastError());
   }
@@ -1659,6 +1689,10 @@ static int execute_t(gm_plan* p, cudaStream_t st, gm_csr* C) {
   HostSlot* const slot = p->slot;
   slot->err[0] = 0;  // (nothing of this plan is in flight: every return of an execute has waited for its streams)
   slot->c_total = 0;
+  if (p->row_sums && p->sums_dirty) {
+    GM_CUDA(cudaMemsetAsync(p->sums[0], 0, 2 * row_sum_words(nA) * sizeof(u32), st));
+  }
+  p->sums_dirty = true;  // until the call is through
 
   // ---- result row_ptr
   i64* c_row_ptr = static_cast<i64*>(dev_alloc(static_cast<size_t>(nA + 1) * sizeof(i64), st));
@@ -1736,14 +1770,19 @@ static int execute_t(gm_plan* p, cudaStream_t st, gm_csr* C) {
       p->stats.launches += 1;
       p->stats.final_chunks += info.rows_heavy * info.params.chunks_required;
       p->stats.staged_products += info.products_heavy;
-    } else {
+    } else if (!p->row_sums) {
       p->stats.launches += exclusive_scan<int32_t, i64>(p->row_nnz, c_row_ptr, nA, p->scan_tmp, nullptr, nullptr, nullptr, st,
                                                         reinterpret_cast<i64*>(&slot->c_total));
     }
     tm.end(st);
-    if (info.c_nnz_upper * static_cast<i64>(4 + sizeof(V)) <= kCRoomBytes && alloc_c(info.c_nnz_upper, &c_col, &c_val, st)) {
+    if ((p->row_sums || info.c_nnz_upper * static_cast<i64>(4 + sizeof(V)) <= kCRoomBytes) && alloc_c(info.c_nnz_upper, &c_col, &c_val, st)) {
       capacity = info.c_nnz_upper;
     } else {
+      if (p->row_sums) {  // refused: C takes what it needs, from now on
+        p->row_sums = false;
+        p->stats.launches += exclusive_scan<int32_t, i64>(p->row_nnz, c_row_ptr, nA, p->scan_tmp, nullptr, nullptr, nullptr, st,
+                                                          reinterpret_cast<i64*>(&slot->c_total));
+      }
       if (cudaStreamSynchronize(st) != cudaSuccess) {
         cleanup();
         return fail(GM_ERR_CUDA, std::string("symbolic phase failed: ") + cudaGetErrorString(cudaGetLastError()));
@@ -1912,6 +1951,8 @@ static int execute_t(gm_plan* p, cudaStream_t st, gm_csr* C) {
     p->stats.ms_scan = ph[PhaseTimes::kScan];
     cudaEventElapsedTime(&p->stats.ms_total, ev_total0, ev_total1);
   }
+  p->sums_at ^= 1;
+  p->sums_dirty = false;
   C->n_rows = nA;
   C->n_cols = B.n_cols;
   C->nnz = total;

@@ -28,7 +28,34 @@ namespace gm {
 constexpr int kMergeThreads = 128;
 constexpr int kMergeStageEntries = 2048;  // entries of C one block collects in shared memory before it writes them out
 
-enum MergeMode { kMergeCount = 0, kMergeToC = 1, kMergeToStage = 2 };
+// kMergePlace: kMergeToC for a block that finds its rows' place in C itself.
+enum MergeMode { kMergeCount = 0, kMergeToC = 1, kMergeToStage = 2, kMergePlace = 3 };
+
+// Without heavy rows (and up to kSumRowsMax rows) there is no prefix sum over the rows: whoever counts a row's entries adds them to
+// the sum of its group of kSumRows rows, and a block that writes rows to C adds up the groups before its own.  Two launches and
+// a pass less (us a call, with the prefix sum / without: 5-point grids of 1024^2 points fp64 250 / 243, of 300^2 86 / 78; ER, 4096 rows of
+// 8 73 / 69, 100000 rows of 4 113 / 103, an execute of 30011 rows of 12 fp64 111 / 107 to 112).
+// The sums of the next execute are cleared by this one, which the next has waited for.
+constexpr int kSumRows = 256;
+constexpr i64 kSumRowsMax = i64{1} << 20;
+struct RowSums {
+  u32* now;   // nullptr: offsets come from a prefix sum
+  u32* next;
+};
+// Entries of C before row r0, a multiple of 16 (at least, and of the rows a block has).  All T threads of the block; s_tmp: 33 values.
+template <int T>
+__device__ __forceinline__ i64 entries_before(const RowSums& rs, const int32_t* __restrict__ row_nnz, i64 r0, i64* s_tmp) {
+  const i64 group = r0 / kSumRows;
+  i64 n = 0;
+  for (i64 g = threadIdx.x; g < group; g += T) n += rs.now[g];
+  for (i64 r = group * kSumRows + threadIdx.x; r < r0; r += T) n += row_nnz[r];
+  i64 total;
+  block_exclusive_scan(n, s_tmp, &total);
+  return total;
+}
+__device__ __forceinline__ void clear_next_sums(const RowSums& rs, i64 n_rows) {
+  for (i64 g = static_cast<i64>(blockIdx.x) * blockDim.x + threadIdx.x; g * kSumRows < n_rows; g += static_cast<i64>(gridDim.x) * blockDim.x) rs.next[g] = 0u;
+}
 
 // One row.  emit(i, column, sum) for the row's i-th entry; returns the number of entries.
 template <typename V, int NL, bool NUMERIC, typename Emit>
@@ -88,20 +115,38 @@ __global__ void __launch_bounds__(kMergeThreads) k3_merge_rows(
     const i64* __restrict__ a_row_ptr, const int32_t* __restrict__ a_col, const V* __restrict__ a_val,
     const i64* __restrict__ b_row_ptr, const int32_t* __restrict__ b_col, const V* __restrict__ b_val,
     const int32_t* __restrict__ rows, i64 n_rows, const i64* __restrict__ light_off, int32_t* __restrict__ row_nnz,
-    const i64* __restrict__ c_row_ptr, int32_t* __restrict__ out_col, V* __restrict__ out_val) {
+    i64* __restrict__ c_row_ptr, int32_t* __restrict__ out_col, V* __restrict__ out_val, RowSums rs, i64* __restrict__ host_total) {
   const i64 i = static_cast<i64>(blockIdx.x) * kMergeThreads + threadIdx.x;
-  if constexpr (MODE == kMergeToC) {
+  const u32 lanes = __ballot_sync(0xffffffffu, i < n_rows);
+  if constexpr (MODE == kMergeToC || MODE == kMergePlace) {
     // the block's rows are consecutive, and so are their entries in C: collected in shared memory, written in one run
     // (a thread writing its own entries would touch one sector per lane and store)
     __shared__ int32_t s_col[kMergeStageEntries];
     __shared__ V s_val[kMergeStageEntries];
     const i64 r0 = static_cast<i64>(blockIdx.x) * kMergeThreads;
     const i64 r1 = min(n_rows, r0 + kMergeThreads);
-    const i64 c0 = c_row_ptr[r0];
-    const i64 n_out = c_row_ptr[r1] - c0;
+    i64 c0, n_out;
+    int at = 0;
+    if constexpr (MODE == kMergePlace) {
+      __shared__ i64 s_tmp[33];
+      __shared__ int s_scan[33];
+      int n_all;
+      at = block_exclusive_scan(i < n_rows ? row_nnz[i] : 0, s_scan, &n_all);
+      c0 = entries_before<kMergeThreads>(rs, row_nnz, r0, s_tmp);
+      n_out = n_all;
+      if (i < n_rows) c_row_ptr[i] = c0 + at;
+      if (i == n_rows - 1) {
+        c_row_ptr[n_rows] = c0 + n_out;
+        *host_total = c0 + n_out;  // (read after a synchronisation)
+      }
+      clear_next_sums(rs, n_rows);
+    } else {
+      c0 = c_row_ptr[r0];
+      n_out = c_row_ptr[r1] - c0;
+      if (i < n_rows) at = static_cast<int>(c_row_ptr[i] - c0);
+    }
     if (n_out <= kMergeStageEntries) {
       if (i < n_rows) {
-        const int at = static_cast<int>(c_row_ptr[i] - c0);
         merge_row<V, NL, true>(a_row_ptr[i], a_row_ptr[i + 1], a_col, a_val, b_row_ptr, b_col, b_val, [&](int q, int32_t c, V v) {
           s_col[at + q] = c;
           s_val[at + q] = v;
@@ -113,10 +158,9 @@ __global__ void __launch_bounds__(kMergeThreads) k3_merge_rows(
         out_val[c0 + q] = s_val[q];
       }
     } else if (i < n_rows) {
-      const i64 at = c_row_ptr[i];
       merge_row<V, NL, true>(a_row_ptr[i], a_row_ptr[i + 1], a_col, a_val, b_row_ptr, b_col, b_val, [&](int q, int32_t c, V v) {
-        out_col[at + q] = c;
-        out_val[at + q] = v;
+        out_col[c0 + at + q] = c;
+        out_val[c0 + at + q] = v;
       });
     }
   } else if (i < n_rows) {
@@ -130,6 +174,14 @@ __global__ void __launch_bounds__(kMergeThreads) k3_merge_rows(
           }
         });
     row_nnz[row] = n;
+    if (rs.now) {
+      if constexpr (MODE == kMergeCount) {  // a warp's rows are in one group
+        const u32 sum = __reduce_add_sync(lanes, static_cast<u32>(n));
+        if ((threadIdx.x & 31) == 0) atomicAdd(&rs.now[row / kSumRows], sum);
+      } else {
+        atomicAdd(&rs.now[row / kSumRows], static_cast<u32>(n));
+      }
+    }
   }
 }
 
@@ -222,7 +274,8 @@ __device__ __forceinline__ void sort_row(i64 row, const i64* __restrict__ a_row_
                                          const V* __restrict__ a_val, const i64* __restrict__ b_row_ptr,
                                          const int32_t* __restrict__ b_col, const V* __restrict__ b_val,
                                          const i64* __restrict__ light_off, int32_t* __restrict__ row_nnz,
-                                         int32_t* __restrict__ out_col, V* __restrict__ out_val, SortSmem<V, Key, KMAX>& sm) {
+                                         int32_t* __restrict__ out_col, V* __restrict__ out_val, u32* __restrict__ sums,
+                                         SortSmem<V, Key, KMAX>& sm) {
   constexpr int kPosBits = kSortPosBits<K>;
   const int lane = threadIdx.x & 31;
   const i64 at = light_off[row];
@@ -236,7 +289,10 @@ __device__ __forceinline__ void sort_row(i64 row, const i64* __restrict__ a_row_
   __syncwarp();
   warp_sort_keys<Key, K>(key, lane);
   const int m = warp_sum_runs<V, Key, K, kPosBits>(key, n, sm.key, sm.val, 0u, out_col + at, out_val + at);
-  if (lane == 0) row_nnz[row] = m;
+  if (lane == 0) {
+    row_nnz[row] = m;
+    if (sums) atomicAdd(&sums[row / kSumRows], static_cast<u32>(m));
+  }
   __syncwarp();  // the warp's shared memory is reused by its next row
 }
 
@@ -245,7 +301,8 @@ template <typename V, typename Key, int KMAX>
 __global__ void __launch_bounds__(kSortWarpsOf<KMAX> * 32, KMAX > 4 ? 8 : 12) k3_sort_rows(
     const i64* __restrict__ a_row_ptr, const int32_t* __restrict__ a_col, const V* __restrict__ a_val,
     const i64* __restrict__ b_row_ptr, const int32_t* __restrict__ b_col, const V* __restrict__ b_val, SortLists lists,
-    const i64* __restrict__ light_off, int32_t* __restrict__ row_nnz, int32_t* __restrict__ out_col, V* __restrict__ out_val) {
+    const i64* __restrict__ light_off, int32_t* __restrict__ row_nnz, int32_t* __restrict__ out_col, V* __restrict__ out_val,
+    u32* __restrict__ sums) {
   constexpr int kSortWarps = kSortWarpsOf<KMAX>;
   __shared__ SortSmem<V, Key, KMAX> s_sm[kSortWarps];
   SortSmem<V, Key, KMAX>& sm = s_sm[threadIdx.x >> 5];
@@ -257,7 +314,7 @@ __global__ void __launch_bounds__(kSortWarpsOf<KMAX> * 32, KMAX > 4 ? 8 : 12) k3
     /* the warps go on round-robin from one class to the next */                                                              \
     for (i64 q = ((w0 - before) % n_warps + n_warps) % n_warps; q < lists.n[I]; q += n_warps)                                  \
       sort_row<V, Key, K, KMAX>(lists.rows[I][q], a_row_ptr, a_col, a_val, b_row_ptr, b_col, b_val, light_off, row_nnz, out_col, \
-                                out_val, sm);                                                                                 \
+                                out_val, sums, sm);                                                                               \
     before += lists.n[I];                                                                                                     \
   }
   if constexpr (KMAX > 16) {
@@ -297,6 +354,54 @@ __global__ void __launch_bounds__(256) k3_copy_rows(const int32_t* __restrict__ 
   for (int q = l; q < n; q += LPR) {
     c_col[dst + q] = s_col[src + q];
     c_val[dst + q] = s_val[src + q];
+  }
+}
+
+template <int LPR> constexpr int kPlaceRows = 256 / LPR * 2;  // rows of a block
+// The same for all rows of a product without heavy rows; a block finds the place of its rows itself.
+template <typename V, int LPR>
+__global__ void __launch_bounds__(256) k3_place_rows(const int32_t* __restrict__ s_col, const V* __restrict__ s_val,
+                                                     const i64* __restrict__ light_off, i64 n_rows, const int32_t* __restrict__ row_nnz,
+                                                     RowSums rs, i64* __restrict__ c_row_ptr, int32_t* __restrict__ c_col,
+                                                     V* __restrict__ c_val, i64 c_capacity, i64* __restrict__ host_total,
+                                                     int* __restrict__ err) {
+  constexpr int R = kPlaceRows<LPR>;
+  static_assert(kSumRows % R == 0 && R <= 256, "a block's rows are in one group");
+  __shared__ i64 s_tmp[33];
+  __shared__ i64 s_at[R + 1];
+  const i64 r0 = static_cast<i64>(blockIdx.x) * R;
+  const int n = threadIdx.x < R && r0 + threadIdx.x < n_rows ? row_nnz[r0 + threadIdx.x] : 0;
+  const i64 before = entries_before<256>(rs, row_nnz, r0, s_tmp);
+  __syncthreads();
+  i64 total;
+  const i64 at = before + block_exclusive_scan(static_cast<i64>(n), s_tmp, &total);
+  if (threadIdx.x < R) {
+    s_at[threadIdx.x] = at;
+    if (r0 + threadIdx.x < n_rows) c_row_ptr[r0 + threadIdx.x] = at;
+    if (r0 + threadIdx.x == n_rows - 1) {
+      c_row_ptr[n_rows] = at + n;
+      *host_total = at + n;  // (read after a synchronisation)
+    }
+  }
+  if (threadIdx.x == 0) s_at[R] = before + total;
+  clear_next_sums(rs, n_rows);
+  __syncthreads();
+  const int l = threadIdx.x % LPR;
+#pragma unroll 1
+  for (int i = threadIdx.x / LPR; i < R; i += 256 / LPR) {
+    const i64 dst = s_at[i];
+    const int m = static_cast<int>(s_at[i + 1] - dst);
+    if (m == 0) continue;
+    const i64 src = light_off[r0 + i];
+    if (dst + m > c_capacity) {
+      if (l == 0) dev_set_error(err, kDevCapacity);
+      continue;
+    }
+#pragma unroll 4
+    for (int q = l; q < m; q += LPR) {
+      c_col[dst + q] = s_col[src + q];
+      c_val[dst + q] = s_val[src + q];
+    }
   }
 }
 

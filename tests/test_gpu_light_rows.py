@@ -7,7 +7,7 @@ import torch
 import gen
 import oracle
 from helpers import random_csr
-from parity import check_product
+from parity import check_product, compare_rows
 
 pytestmark = pytest.mark.gpu
 
@@ -97,3 +97,28 @@ def test_row_products_of_full_rows(n_rows, n_cols):
     out = torch.full((n_rows,), -1, dtype=torch.int64, device="cuda")
     gm.row_products_noalloc(A, B, out)
     assert bool((out == n_cols).all())
+
+
+@pytest.mark.parametrize("dtype", [np.float32, np.float64])
+@pytest.mark.parametrize("n", [1, 15, 16, 17, 255, 256, 257, 5000, (1 << 16) + 300, (1 << 20) + 1])
+@pytest.mark.parametrize("longest", [4, 40])
+def test_light_rows_find_their_place_by_themselves(n, longest, dtype):
+    # no heavy rows: groups of 256 rows and one more, rows without entries at either end, a kept plan executed again, and one row
+    # more than may do without a prefix sum
+    import paper_2607_22866_b200 as gm
+    rng = np.random.default_rng(n)
+    m = 3000
+    B = _csr([rng.choice(m, int(k), replace=False) for k in rng.integers(0, 6, m)], m, rng, dtype)
+    k = rng.integers(0, longest, n)
+    k[rng.random(n) < 0.3] = 0
+    k[n // 2] = longest
+    starts = rng.integers(0, m - longest, n)
+    rp = np.zeros(n + 1, np.int64)
+    np.cumsum(k, out=rp[1:])
+    col = np.repeat(starts - rp[:-1], k) + np.arange(rp[-1])
+    A = gen.CSR(n, m, rp, col.astype(np.int32), rng.uniform(-1, 1, rp[-1]).astype(dtype))
+    ref = oracle.spgemm(A, B)
+    plan = gm.spgemm_plan(gm.DeviceCSR.from_host(A), gm.DeviceCSR.from_host(B))
+    assert plan.info().rows_heavy == 0
+    for _ in range(3):
+        compare_rows(gm.spgemm_execute(plan), ref, dtype)
