@@ -244,12 +244,12 @@ def kernel_table(info, stats_avg, sv, nnz_b, n_light_entries_a):
             tbl[k + " (into C)"] = (read_all + se * nnz_cl, stats_avg["ms_light_numeric"])
         else:
             tbl["k3_sort_rows, k3_merge_rows"] = (read_all + se * nnz_cl, stats_avg["ms_light_symbolic"])
-            tbl["k3_copy_rows"] = (2 * se * nnz_cl, stats_avg["ms_light_numeric"])
+            tbl["k3_copy_rows" if rows_h or info.n_rows > 1 << 20 else "k3_place_rows"] = (2 * se * nnz_cl, stats_avg["ms_light_numeric"])
     if rows_h and info.heavy_tasks:
         # summed where the products are generated: B is read (by each kernel once, at least) and entries are written
         tbl["k6_small_tasks"] = (se * nnz_b + se * nnz_small, stats_avg["ms_small_chunks"])
         tbl["k6_mid_tasks"] = (se * nnz_b + se * nnz_mid, stats_avg["ms_mid_chunks"])
-        tbl["k6_big_tasks"] = (se * nnz_b + se * (nnz_ch - nnz_small - nnz_mid), stats_avg["ms_accumulate"])
+        tbl["k6_panels, k6_big_tasks" if stats_avg["panel_rows"] else "k6_big_tasks"] = (se * nnz_b + se * (nnz_ch - nnz_small - nnz_mid), stats_avg["ms_accumulate"])
         tbl["k7_gather"] = (2 * se * nnz_ch, stats_avg["ms_gather"])
     elif rows_h:
         chunks = stats_avg["final_chunks"]

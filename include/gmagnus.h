@@ -169,7 +169,9 @@ typedef struct gm_exec_stats {
       ms_accumulate, ms_gather, ms_scan, ms_total;
   float ms_small_chunks;       /* one warp per chunk or task; ms_accumulate is the dense-accumulator kernel alone */
   float ms_mid_chunks;         /* one small block per chunk or task                                             */
-  float reserved[3];
+  float panel_rows;            /* heavy rows summed several at a time, as a small dense product (neighbouring rows of A with
+                                  much the same columns; their kernel's time is part of ms_accumulate)            */
+  float reserved[2];
   int64_t mid_chunk_products;  /* products in chunks or tasks summed by one small block each                     */
   int64_t mid_chunk_entries;   /* entries of C those produced                                                    */
   int64_t early_exit_products; /* products of chunks that left the multisplit hierarchy before its last level    */

@@ -77,7 +77,7 @@ class ExecStats(ctypes.Structure):
                 ("ms_expand", ctypes.c_float), ("ms_histogram", ctypes.c_float), ("ms_multisplit", ctypes.c_float),
                 ("ms_accumulate", ctypes.c_float), ("ms_gather", ctypes.c_float), ("ms_scan", ctypes.c_float),
                 ("ms_total", ctypes.c_float), ("ms_small_chunks", ctypes.c_float), ("ms_mid_chunks", ctypes.c_float),
-                ("reserved", ctypes.c_float * 3), ("mid_chunk_products", ctypes.c_int64), ("mid_chunk_entries", ctypes.c_int64),
+                ("panel_rows", ctypes.c_float), ("reserved", ctypes.c_float * 2), ("mid_chunk_products", ctypes.c_int64), ("mid_chunk_entries", ctypes.c_int64),
                 ("early_exit_products", ctypes.c_int64), ("early_exit_chunks", ctypes.c_int64),
                 ("split_products", ctypes.c_int64)]
 

@@ -21,6 +21,7 @@
 #include "gm_k4_csc.cuh"
 #include "gm_k5_multisplit.cuh"
 #include "gm_k6_accumulate.cuh"
+#include "gm_k6_panels.cuh"
 #include "gm_k6_tasks.cuh"
 #include "gm_k7_gather.cuh"
 #include "gm_planner.h"
@@ -328,7 +329,8 @@ struct gm_plan {
   int64_t* scan_tmp = nullptr;
   int64_t* c_total = nullptr;      // [0] running nnz(C) (device carry), [1] heavy entries, [2] products and [3] entries of
                                    // small chunks, [4] products and [5] entries of mid-size chunks, [6] products and
-                                   // [7] chunks that left the hierarchy early, [8] products the levels did not move
+                                   // [7] chunks that left the hierarchy early, [8] products the levels did not move, [9] rows
+                                   // in panels
   int* err = nullptr;              // in the host slot: kernels write it through the mapping
   // heavy workspace
   int32_t* stage_col[2]{};
@@ -360,7 +362,10 @@ struct gm_plan {
   int64_t* task_off = nullptr;     // place of a task in the staging area
   int32_t* task_list[3]{};         // small, mid, big
   int* task_counters = nullptr;    // 8 per batch
-  int* task_tickets = nullptr;     // 4 per batch
+  int* task_tickets = nullptr;     // 4 per batch: big, mid, panels
+  bool use_panels = false;         // neighbouring heavy rows with much the same columns are summed together (gm_k6_panels.cuh)
+  gm::PanelTables panels{};
+  std::vector<int64_t> batch_starts;
   gm::PhaseTimes times;
   HostSink* sink = nullptr;        // set by gm_spgemm_host for the duration of one execute
   bool c_is_passing = false;       // C is copied out and freed at once: what it takes more than its entries does not matter
@@ -626,6 +631,18 @@ static bool plan_task_rules(gm_plan* p) {
   return true;
 }
 
+// Panels are looked for where heavy rows have many entries (R-MAT graphs have 25 to 40, and hardly two rows alike) and where there are
+// products enough to pay for the lists.  Block-dense products, us a call, tasks / panels: 2.8 M products fp64 150 / 195, 23 M fp32
+// 292 / 319, 166 M fp64 (kept plan) 895 / 510, 1.3 G fp64 5690 / 1630, 2.7 G fp32 8560 / 2440.
+constexpr i64 kPanelMinEntries = 48, kPanelMinHeavy = i64{1} << 25;
+static int panel_max_u(const gm_plan* p) { return p->sv == 4 ? kPanelColumns<float> : kPanelColumns<double>; }
+static bool plan_panel_rules(const gm_plan* p) {
+  const i64 n_groups = ((p->B.n_cols - 1) >> panel_group_bits(p->sv)) + 1;
+  const size_t smem = p->sv == 4 ? sizeof(PanelSmem<float>) : sizeof(PanelSmem<double>);
+  return p->info.products_heavy >= kPanelMinHeavy && p->n_seg >= kPanelMinEntries * p->info.rows_heavy && p->B.n_rows <= kPanelMaxRowsB && n_groups <= kPanelMaxGroups &&
+         std::max(smem, panel_build_smem(p->B.n_rows, n_groups)) + 1024 <= p->smem_bytes;
+}
+
 // Tasks of the heavy rows: piece boundaries of B, products per row and granule, ranges, lists.
 static int plan_tasks(gm_plan* p, cudaStream_t st) {
   const gm_csr& A = p->A;
@@ -636,6 +653,11 @@ static int plan_tasks(gm_plan* p, cudaStream_t st) {
   u32* n_long = nullptr;
   int32_t* long_rows = nullptr;
   i64* tmp = nullptr;
+  unsigned char* similar = nullptr;
+  u32* piece_count = nullptr;
+  i64* piece_tmp = nullptr;
+  i64* starts = nullptr;
+  PanelTables& pt = p->panels;
   // Small products: the tables take their upper bound (a granule of n products gives fewer than 2 n / split_above
   // sub-ranges), so that nothing waits for the number of tasks.
   const i64 bound = nH * r.granules + 2 * (p->info.products_heavy / r.split_above) + 64;
@@ -656,6 +678,10 @@ static int plan_tasks(gm_plan* p, cudaStream_t st) {
     ar.add(&p->longest_row, 1);
     ar.add(&n_long, 1);
     ar.add(&p->task_counters, 8 * n_batches);
+    if (p->use_panels) {
+      ar.add(&pt.counts, 2);
+      ar.add(&starts, n_batches);
+    }
     const size_t zeroed = ar.bytes;
     ar.add(&p->c_total, 16);  // (next to the tickets: one clear for both, see execute_t)
     ar.add(&p->task_tickets, 4 * n_batches);
@@ -671,7 +697,44 @@ static int plan_tasks(gm_plan* p, cudaStream_t st) {
     if (p->finish) add_tables(ar, bound, bound);
     GM_TRY(ar.commit(p, st));
     GM_CUDA(cudaMemsetAsync(p->longest_row, 0, zeroed, st));
+    if (p->use_panels) {
+      Arena par;
+      const size_t n = static_cast<size_t>(nH), seg = static_cast<size_t>(p->n_seg);
+      par.add(&pt.list, n / kPanelMinRows + 1);
+      par.add(&pt.of_row, n);
+      par.add(&pt.a_u, seg);
+      par.add(&pt.u_mask, seg);
+      par.add(&pt.visits, seg * kPanelVisitsPerEntry);
+      par.add(&pt.groups, seg / kPanelEntriesPerGroup + 1);
+      par.add(&pt.group_rows, (seg / kPanelEntriesPerGroup + 1) * kPanelRows);
+      par.add(&pt.units, seg / kPanelEntriesPerGroup + 1);
+      par.add(&similar, n);
+      par.add(&pt.piece_ptr, static_cast<size_t>(B.n_rows) + 1);
+      par.add(&piece_count, static_cast<size_t>(B.n_rows));
+      pt.max_pieces = B.nnz / kPanelEntriesPerPiece + 1;
+      par.add(&pt.pieces, static_cast<size_t>(pt.max_pieces));
+      par.add(&piece_tmp, static_cast<size_t>(scan_tmp_elems(B.n_rows)));
+      if (par.commit(p, st) != GM_OK) p->use_panels = false;  // no room: the rows are tasks like the others
+    }
   }
+  if (p->use_panels) {
+    if (n_batches > 1) {
+      for (const Batch& b : p->batches) p->batch_starts.push_back(b.h0);
+      GM_CUDA(cudaMemcpyAsync(starts, p->batch_starts.data(), n_batches * sizeof(i64), cudaMemcpyHostToDevice, st));
+    }
+    const int group_bits = panel_group_bits(p->sv), n_groups = static_cast<int>(((B.n_cols - 1) >> group_bits) + 1);
+    const unsigned row_grid = grid_for(B.n_rows, 8, p->num_sms, 16);
+    k_piece_count<<<row_grid, 256, 0, st>>>(B.row_ptr, B.col_idx, B.n_rows, group_bits, piece_count);
+    p->info.launches += 5 + exclusive_scan<u32, i64>(piece_count, pt.piece_ptr, B.n_rows, piece_tmp, nullptr, nullptr, nullptr, st);
+    k_piece_fill<<<row_grid, 256, 0, st>>>(B.row_ptr, B.col_idx, B.n_rows, group_bits, pt);
+    k_panel_similar<<<static_cast<unsigned>((nH + 7) / 8), 256, 0, st>>>(p->x_heavy, nH, A.row_ptr, A.col_idx, similar);
+    k_panel_cut<<<static_cast<unsigned>((nH + 1023) / 1024), 1024, 0, st>>>(similar, nH, starts, static_cast<int>(n_batches), pt);
+    GM_TRY(allow_smem<k_panel_build>(p));
+    k_panel_build<<<static_cast<unsigned>(std::min<i64>(nH / kPanelMinRows + 1, static_cast<i64>(p->num_sms) * 3)), kPanelBuildThreads,
+                    panel_build_smem(B.n_rows, n_groups), st>>>(pt, p->x_heavy, p->heavy_base, p->heavy_nz_off, A.row_ptr, A.col_idx, B.n_rows,
+                                                                n_groups, panel_max_u(p), nH >= kPanelRows * 256 ? 2 * kPanelWarps : kPanelWarps);
+  }
+  const unsigned char* const in_panel = p->use_panels ? pt.of_row : nullptr;
   k_piece_bounds<<<grid_for(B.n_rows * (r.granules + 1), 256, p->num_sms, 32), 256, 0, st>>>(B.row_ptr, B.col_idx, B.n_rows, r.granules,
                                                                                            r.log2_g, p->piece_bound, p->longest_row);
   k_granule_parts<<<static_cast<unsigned>(r.granules), 32, 0, st>>>(B.col_idx, p->piece_bound, p->longest_row, r.granules, r.log2_g,
@@ -679,7 +742,7 @@ static int plan_tasks(gm_plan* p, cudaStream_t st) {
   p->info.launches += 2;
   if (r.granules > 1) {
     k_granule_counts<<<grid_for(nH, 8, p->num_sms, 8), 256, 0, st>>>(p->x_heavy, nH, A.row_ptr, A.col_idx, p->piece_bound, r.granules,
-                                                                   p->granule_counts, long_rows, n_long);
+                                                                   p->granule_counts, long_rows, n_long, in_panel);
     k_granule_counts_long<<<dim3(static_cast<unsigned>(p->num_sms), kCountRuns), 256, 0, st>>>(p->x_heavy, A.row_ptr, A.col_idx, p->piece_bound, r.granules,
                                                                                p->granule_counts, long_rows, n_long);
     p->info.launches += 2;
@@ -689,12 +752,12 @@ static int plan_tasks(gm_plan* p, cudaStream_t st) {
     p->task_begin[1] = bound;
     const TaskTables tt{p->tasks, p->task_off, {p->task_list[0], p->task_list[1], p->task_list[2]}, p->task_counters, 0, bound};
     k_plan_small<<<1, kFinishThreads, 0, st>>>(p->granule_counts, p->heavy_base, nH, r, p->row_tasks, p->row_task_off, p->x_heavy, A.row_ptr,
-                                              p->part_cols, tt);
+                                              p->part_cols, tt, in_panel);
     ++p->info.launches;
     GM_CUDA(cudaGetLastError());
     return GM_OK;
   }
-  k_task_count<<<static_cast<unsigned>((nH + 127) / 128), 128, 0, st>>>(p->granule_counts, p->heavy_base, nH, r, p->row_tasks);
+  k_task_count<<<static_cast<unsigned>((nH + 127) / 128), 128, 0, st>>>(p->granule_counts, p->heavy_base, nH, r, p->row_tasks, in_panel);
   p->info.launches += 1 + exclusive_scan<u32, i64>(p->row_tasks, p->row_task_off, nH, tmp, nullptr, nullptr, nullptr, st,
                                                   reinterpret_cast<i64*>(&p->slot->n_tasks));
   for (size_t i = 1; i < n_batches; ++i)
@@ -713,7 +776,7 @@ static int plan_tasks(gm_plan* p, cudaStream_t st) {
     const TaskTables tt{p->tasks, p->task_off, {p->task_list[0], p->task_list[1], p->task_list[2]}, p->task_counters + 8 * i,
                         p->task_begin[i], p->task_begin[i + 1]};
     k_task_emit<<<static_cast<unsigned>((b.h1 - b.h0 + 127) / 128), 128, 0, st>>>(p->granule_counts, p->heavy_base, b.h0, b.h1, b.elem0, r,
-                                                                                p->row_task_off, p->x_heavy, A.row_ptr, p->part_cols, tt);
+                                                                                p->row_task_off, p->x_heavy, A.row_ptr, p->part_cols, tt, in_panel);
     ++p->info.launches;
   }
   GM_CUDA(cudaGetLastError());
@@ -933,6 +996,7 @@ static int build_plan(gm_plan* p, cudaStream_t st) {
       p->stage_val[i] = v;
     }
     if (p->use_tasks) {
+      p->use_panels = plan_panel_rules(p);
       p->pending = true;  // (the lists' kernels may still run when the call returns: see gm_spgemm_execute)
       GM_TRY(plan_tasks(p, st));
       return GM_OK;
@@ -1578,6 +1642,15 @@ static int task_batch_sums(gm_plan* p, size_t bi, cudaStream_t st) {
   PhaseTimes& tm = p->times;
   if constexpr (BIG) {
     tm.begin(PhaseTimes::kAccNum, st);
+    if (p->use_panels) {
+      constexpr auto kern = k6_panels<V>;
+      GM_TRY(allow_smem<kern>(p));
+      kern<<<static_cast<unsigned>(p->num_sms * 2), kPanelThreads, sizeof(PanelSmem<V>), st>>>(
+          p->A.row_ptr, static_cast<const V*>(p->A.vals), static_cast<const V*>(p->B.vals), p->panels, p->x_heavy, p->heavy_base,
+          p->heavy_nz_off, b.h0, b.h1, b.elem0, p->row_task_off, tickets + 2, out_col, out_val, p->chunk_nnz,
+          reinterpret_cast<u64*>(p->c_total + 9));
+      ++p->stats.launches;
+    }
     const size_t smem = big_task_smem_bytes<V>(p->acc_width, p->acc_threads);
     const unsigned grid = static_cast<unsigned>(std::min<i64>(n, static_cast<i64>(p->num_sms) * p->acc_blocks));
 #define GM_BIG(BT, BLOCKS)                                                                                                        \
@@ -1890,7 +1963,7 @@ static int execute_t(gm_plan* p, cudaStream_t st, gm_csr* C) {
   if (tm.enabled) cudaEventRecord(ev_total1, st);
   // [0] nnz(C) so far (several batches), [1] heavy entries; products and entries of small chunks; of mid-size chunks;
   // products and chunks that left the hierarchy early; products the multisplit levels left in place
-  if (n_batches > 0 && !finished) cudaMemcpyAsync(slot->tail, p->c_total, 9 * sizeof(i64), cudaMemcpyDeviceToHost, st);
+  if (n_batches > 0 && !finished) cudaMemcpyAsync(slot->tail, p->c_total, kTailWords * sizeof(i64), cudaMemcpyDeviceToHost, st);
   const cudaError_t e2 = cudaStreamSynchronize(st);
   if (e2 != cudaSuccess) {
     cleanup();
@@ -1934,6 +2007,7 @@ static int execute_t(gm_plan* p, cudaStream_t st, gm_csr* C) {
     p->stats.early_exit_products = t[6];
     p->stats.early_exit_chunks = t[7];
     p->stats.split_products -= t[8];
+    p->stats.panel_rows = static_cast<float>(t[9]);
   }
   p->stats.c_capacity = capacity;
   if (tm.enabled) {

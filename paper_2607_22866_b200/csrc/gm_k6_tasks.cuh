@@ -127,9 +127,11 @@ __device__ __forceinline__ void count_granules(const int32_t* __restrict__ a_col
 }
 __global__ void __launch_bounds__(256) k_granule_counts(const int32_t* __restrict__ x_heavy, i64 n_heavy, const i64* __restrict__ a_row_ptr,
                                                         const int32_t* __restrict__ a_col, const u32* __restrict__ bound, int granules,
-                                                        u32* __restrict__ counts, int32_t* __restrict__ long_rows, u32* __restrict__ n_long) {
+                                                        u32* __restrict__ counts, int32_t* __restrict__ long_rows, u32* __restrict__ n_long,
+                                                        const unsigned char* __restrict__ in_panel) {
   const i64 n_warps = static_cast<i64>(gridDim.x) * 8;
   for (i64 h = static_cast<i64>(blockIdx.x) * 8 + (threadIdx.x >> 5); h < n_heavy; h += n_warps) {
+    if (in_panel && in_panel[h]) continue;
     const i64 row = x_heavy[h];
     const i64 s = a_row_ptr[row], e = a_row_ptr[row + 1];
     if (e - s > kCountLong) {
@@ -191,10 +193,11 @@ __device__ __forceinline__ u32 cut_row(const u32* __restrict__ counts, u32 produ
 }
 
 __global__ void __launch_bounds__(128) k_task_count(const u32* __restrict__ counts, const i64* __restrict__ heavy_base, i64 n_heavy,
-                                                    TaskRules r, u32* __restrict__ row_tasks) {
+                                                    TaskRules r, u32* __restrict__ row_tasks, const unsigned char* __restrict__ in_panel) {
   const i64 h = static_cast<i64>(blockIdx.x) * blockDim.x + threadIdx.x;
   if (h >= n_heavy) return;
-  row_tasks[h] = cut_row(counts + h * r.granules, static_cast<u32>(heavy_base[h + 1] - heavy_base[h]), r, [](int, int, u32, u32) {});
+  if (in_panel && in_panel[h]) row_tasks[h] = 1;
+  else row_tasks[h] = cut_row(counts + h * r.granules, static_cast<u32>(heavy_base[h + 1] - heavy_base[h]), r, [](int, int, u32, u32) {});
 }
 
 // Where the tasks of a batch go.  lists: [0] small, [1] mid, [2] big (the huge ones from the front of the batch's part of the
@@ -219,7 +222,8 @@ __device__ __forceinline__ int class_of(const TaskRules& r, int granules, u32 n,
 template <typename Place>
 __device__ __forceinline__ void emit_row(const u32* __restrict__ counts, const i64* __restrict__ heavy_base, i64 h, i64 elem0,
                                          const TaskRules& r, i64 id, const int32_t* __restrict__ x_heavy,
-                                         const i64* __restrict__ a_row_ptr, const u32* __restrict__ parts_tab, const TaskTables& tt, Place place) {
+                                         const i64* __restrict__ a_row_ptr, const u32* __restrict__ parts_tab, const TaskTables& tt,
+                                         const unsigned char* __restrict__ in_panel, Place place) {
   const i64 row = x_heavy[h];
   HeavyTask t;
   t.a0 = a_row_ptr[row];
@@ -229,11 +233,19 @@ __device__ __forceinline__ void emit_row(const u32* __restrict__ counts, const i
     const int b = static_cast<int>(id - tt.first);  // lists hold batch-relative ids
     if (cls == 0 || cls == 1) tt.list[cls][tt.first + place(cls)] = b;
     else if (cls == 2) tt.list[2][tt.first + place(2)] = b;
-    else tt.list[2][tt.end - 1 - place(3)] = b;
+    else if (cls == 3) tt.list[2][tt.end - 1 - place(3)] = b;
     tt.tasks[id] = t;
     tt.task_off[id] = t.off;
     ++id;
   };
+  if (in_panel && in_panel[h]) {
+    t.lo = 0;
+    t.hi = static_cast<u32>(r.granules) << r.log2_g;
+    t.off = off;
+    t.n = static_cast<u32>(heavy_base[h + 1] - heavy_base[h]);
+    put(-1);  // (a panel's row is in no list)
+    return;
+  }
   cut_row(counts + h * r.granules, static_cast<u32>(heavy_base[h + 1] - heavy_base[h]), r, [&](int g, int w, u32 n, u32 parts) {
     const u32 lo = static_cast<u32>(g) << r.log2_g;
     const u32 width = static_cast<u32>(w) << r.log2_g;
@@ -261,7 +273,8 @@ __device__ __forceinline__ void emit_row(const u32* __restrict__ counts, const i
 __global__ void __launch_bounds__(128) k_task_emit(const u32* __restrict__ counts, const i64* __restrict__ heavy_base, i64 h0, i64 h1,
                                                    i64 elem0, TaskRules r, const i64* __restrict__ row_task_off,
                                                    const int32_t* __restrict__ x_heavy, const i64* __restrict__ a_row_ptr,
-                                                   const u32* __restrict__ parts_tab, TaskTables tt) {
+                                                   const u32* __restrict__ parts_tab, TaskTables tt,
+                                                   const unsigned char* __restrict__ in_panel) {
   // Places in the lists are drawn once per block and class.  With an atomic per task on four words of L2, which take turns, this kernel
   // took 112 us for R-MAT scale 17 (now 27) and 1.5 ms for scale 19.
   __shared__ u32 s_n[4], s_base[4];
@@ -269,7 +282,7 @@ __global__ void __launch_bounds__(128) k_task_emit(const u32* __restrict__ count
   const bool mine = h < h1;
   if (threadIdx.x < 4) s_n[threadIdx.x] = 0u;
   __syncthreads();
-  if (mine) {
+  if (mine && !(in_panel && in_panel[h])) {
     u32 n_of[4] = {0u, 0u, 0u, 0u};
     cut_row(counts + h * r.granules, static_cast<u32>(heavy_base[h + 1] - heavy_base[h]), r, [&](int, int w, u32 n, u32 parts) {
       const int c = class_of(r, w, n, parts);
@@ -287,7 +300,7 @@ __global__ void __launch_bounds__(128) k_task_emit(const u32* __restrict__ count
   }
   __syncthreads();
   if (mine)
-    emit_row(counts, heavy_base, h, elem0, r, row_task_off[h], x_heavy, a_row_ptr, parts_tab, tt,
+    emit_row(counts, heavy_base, h, elem0, r, row_task_off[h], x_heavy, a_row_ptr, parts_tab, tt, in_panel,
              [&](int c) { return s_base[c] + atomicAdd(&s_n[c], 1u); });
 }
 
@@ -1006,6 +1019,7 @@ __global__ void k_task_bases(const i64* __restrict__ nnz_off, const i64* __restr
 // entries, entries per heavy row, C.rowPtr, position in C of every task's first entry, the gather's tile records, and the
 // totals for the host.  (Five launches and a copy otherwise, each of which costs more than its work: 55 us from the last
 // sum to the end of the call for R-MAT scales 10 to 12, of 130 to 260.)
+constexpr int kTailWords = 10;  // totals the host reads at the end of an execute (see gm_plan::c_total)
 constexpr i64 kFinishMax = 16384;  // tasks, and rows of A: above, one block takes as long as the launches
 constexpr int kFinishThreads = 1024;
 // out[0 .. n) = exclusive prefix sums of in (values from position n_valid on count as zero); returns the total (every thread).
@@ -1050,7 +1064,7 @@ __global__ void __launch_bounds__(kFinishThreads) k_finish_small(const u32* task
     for (i64 t = a; t < b; ++t) base[t] = nnz_off[t] + shift;
   }
   for (i64 t = threadIdx.x; t * tile < heavy; t += kFinishThreads) meta[t] = tile_bounds(nnz_off, n_tasks, 0, heavy, tile, t);
-  if (threadIdx.x < 9) host_totals[threadIdx.x] = threadIdx.x == 1 ? heavy : totals[threadIdx.x];
+  if (threadIdx.x < kTailWords) host_totals[threadIdx.x] = threadIdx.x == 1 ? heavy : totals[threadIdx.x];
   if (threadIdx.x == 0) *host_total = all;  // (the host reads after a synchronisation)
 }
 
@@ -1059,17 +1073,18 @@ __global__ void __launch_bounds__(kFinishThreads) k_finish_small(const u32* task
 // (Zipf-like, 4096 rows: 319 us with a count, a wait and an allocation in between, 284 with this.)
 __global__ void __launch_bounds__(kFinishThreads) k_plan_small(const u32* counts, const i64* heavy_base, i64 n_heavy, TaskRules r,
                                                                u32* row_tasks, i64* row_task_off, const int32_t* x_heavy,
-                                                               const i64* a_row_ptr, const u32* parts_tab, TaskTables tt) {
+                                                               const i64* a_row_ptr, const u32* parts_tab, TaskTables tt,
+                                                               const unsigned char* in_panel) {
   __shared__ i64 tmp[33];
   for (i64 h = threadIdx.x; h < n_heavy; h += kFinishThreads)
-    row_tasks[h] = cut_row(counts + h * r.granules, static_cast<u32>(heavy_base[h + 1] - heavy_base[h]), r, [](int, int, u32, u32) {});
+    row_tasks[h] = in_panel && in_panel[h] ? 1 : cut_row(counts + h * r.granules, static_cast<u32>(heavy_base[h + 1] - heavy_base[h]), r, [](int, int, u32, u32) {});
   __syncthreads();
   finish_scan(row_tasks, n_heavy, n_heavy, row_task_off, tmp);
   __shared__ u32 s_n[4];
   if (threadIdx.x < 4) s_n[threadIdx.x] = 0u;
   __syncthreads();
   for (i64 h = threadIdx.x; h < n_heavy; h += kFinishThreads)
-    emit_row(counts, heavy_base, h, 0, r, row_task_off[h], x_heavy, a_row_ptr, parts_tab, tt,
+    emit_row(counts, heavy_base, h, 0, r, row_task_off[h], x_heavy, a_row_ptr, parts_tab, tt, in_panel,
              [&](int c) { return atomicAdd(&s_n[c], 1u); });
   __syncthreads();
   if (threadIdx.x < 4) tt.counters[threadIdx.x] = static_cast<int>(s_n[threadIdx.x]);

@@ -34,7 +34,7 @@ constexpr int kGatherTileMin = 2048;
 // The number of tiles is only known on the device, and the products are an upper bound that can be forty times the entries:
 // at most this many blocks per SM go over the tiles.  (A block-dense product, forty products per entry, 262140 tiles and 64481 of which
 // most are empty: this kernel 287 + 61 us with a block each, 166 + 47 so.)
-constexpr int kGatherBlocksPerSm = 32;
+constexpr int kGatherBlocksPerSm = 128;
 inline int gather_tile(i64 n_chunks, i64 n_elems) {
   int t = kGatherTile;
   while (t > kGatherTileMin && n_chunks * t > n_elems * (kGatherChunkCap * 3 / 4)) t /= 2;

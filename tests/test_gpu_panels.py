@@ -1,0 +1,148 @@
+"""Neighbouring heavy rows with much the same columns, summed together: sizes of panels, of their column sets and of the
+groups of columns they reach, against the oracle with its tolerance (tau * sum|a*b|)."""
+import numpy as np
+import pytest
+import torch
+
+import gen
+import oracle
+import paper_2607_22866_b200 as gm
+from parity import check_product, compare_rows, run_gpu
+from test_gpu_scratch_and_errors import allocator  # noqa: F401 (fixture)
+
+pytestmark = pytest.mark.gpu
+
+
+def _csr(row_lists, n_cols, rng, dtype):
+    rp = np.zeros(len(row_lists) + 1, np.int64)
+    np.cumsum([len(r) for r in row_lists], out=rp[1:])
+    col = np.concatenate([np.sort(np.asarray(r, np.int32)) for r in row_lists] + [np.zeros(0, np.int32)]).astype(np.int32)
+    return gen.CSR(len(row_lists), n_cols, rp, col, rng.uniform(-1, 1, col.size).astype(dtype))
+
+
+def _blocks(rng, sizes, per_row, fill, n_cols, dtype):
+    """Consecutive row blocks of the given sizes; the rows of one draw their columns from the same per_row columns."""
+    rows = []
+    for n in sizes:
+        pool = rng.choice(n_cols, per_row, replace=False)
+        rows += [pool[rng.random(per_row) < fill] for _ in range(n)]
+    return _csr(rows, n_cols, rng, dtype)
+
+
+def _spans(rng, n_rows, n_cols, n_spans, width, fill, dtype):
+    """Rows made of a few runs of neighbouring columns, which begin at one of some twenty places."""
+    rows = []
+    places = np.append(rng.integers(0, max(1, n_cols - width), 20), max(0, n_cols - width))
+    for _ in range(n_rows):
+        at = rng.choice(places, n_spans)
+        c = np.unique(np.concatenate([a + np.nonzero(rng.random(width) < fill)[0] for a in at]))
+        rows.append(c[c < n_cols])
+    return _csr(rows, n_cols, rng, dtype)
+
+
+@pytest.mark.parametrize("dtype", [np.float32, np.float64])
+@pytest.mark.parametrize("n_mid,n_cols", [(300, 130), (700, 4001), (3000, 70001)])
+def test_panels_of_every_size(dtype, n_mid, n_cols):
+    # row blocks below and above what a panel holds, next to rows of their own; column sets that end in the middle of a round
+    rng = np.random.default_rng(n_cols)
+    sizes = [1, 2, 3, 4, 5, 7, 8, 9, 15, 16, 17, 31, 32, 33, 40, 63, 64, 65, 1, 100] * 9
+    A = _blocks(rng, sizes, 113, 0.8, n_mid, dtype)
+    B = _spans(rng, n_mid, n_cols, 2, 90, 0.7, dtype)
+    C, info, stats = check_product(A, B, tau=64)
+    assert info.heavy_tasks == 1 and stats.panel_rows > 0.7 * info.rows_heavy
+    # several batches: panels end where a batch does
+    big = int(info.products_max_row) * 91 + 5
+    C2, info2, stats2 = check_product(A, B, tau=64, stage_elems=big)
+    assert info2.n_batches > 3 and stats2.panel_rows > 0
+
+
+@pytest.mark.parametrize("dtype,most", [(np.float32, 704), (np.float64, 384)])
+@pytest.mark.parametrize("more", [None, 0, 1])
+@pytest.mark.parametrize("rows", [3000, 16500])
+def test_column_sets_at_their_limits(dtype, most, more, rows):
+    # as many columns as a panel may have and one more (then the rows are tasks); units of a few groups and of whole panels
+    rng = np.random.default_rng(most)
+    n = 60 if more is None else most + more
+    A = _blocks(rng, [32] * (rows // 32) + [rows % 32], n, 1.0, n, dtype)
+    B = _spans(rng, n, 900, 2, 40, 0.6, dtype) if rows > 16384 else _spans(rng, n, 4000, 3, 100, 0.9, dtype)
+    C, info, stats = check_product(A, B, tau=300)
+    assert stats.panel_rows == (0 if more == 1 else rows)
+
+
+def test_rows_of_b_without_entries_and_scattered_ones():
+    # U holds rows of B that are empty, short and long; scattered rows of B leave the panel to the tasks
+    rng = np.random.default_rng(5)
+    A = _blocks(rng, [32] * 60, 120, 0.9, 400, np.float32)
+    B = _spans(rng, 400, 5000, 3, 100, 0.9, np.float32)
+    rp, keep = B.row_ptr, rng.random(400) < 0.7
+    B = _csr([B.col[rp[i]:rp[i + 1]] if keep[i] else [] for i in range(400)], 5000, rng, np.float32)
+    C, info, stats = check_product(A, B, tau=100)
+    assert stats.panel_rows == info.rows_heavy
+    D = _csr([rng.choice(60000, 190, replace=False) for _ in range(400)], 60000, rng, np.float32)
+    C, info, stats = check_product(A, D, tau=100)
+    assert stats.panel_rows == 0 and info.heavy_tasks == 1
+
+
+@pytest.mark.parametrize("dtype", [np.float32, np.float64])
+def test_infinities_nans_and_zeros_stay_where_they_are(dtype):
+    # an infinity or a NaN must not reach entries that no stored product of it belongs to; zeros of either sign are entries
+    rng = np.random.default_rng(9)
+    A = _blocks(rng, [32] * 90, 100, 0.85, 200, dtype)
+    B = _spans(rng, 200, 700, 2, 120, 0.8, dtype)
+    for M, n in ((A, 400), (B, 25)):
+        at = rng.choice(M.val.size, n, replace=False)
+        M.val[at] = rng.choice([np.inf, -np.inf, np.nan, 0.0, -0.0], n)
+    C, info, stats = run_gpu(A, B, tau=64)
+    assert stats.panel_rows == info.rows_heavy == A.n_rows
+    a, b = np.zeros((A.n_rows, 200)), np.zeros((200, 700))
+    has_a, has_b = np.zeros(a.shape, bool), np.zeros(b.shape, bool)
+    for M, d, h in ((A, a, has_a), (B, b, has_b)):
+        r = np.repeat(np.arange(M.n_rows), np.diff(M.row_ptr))
+        d[r, M.col], h[r, M.col] = M.val, True
+    want, bound = np.zeros((A.n_rows, 700)), np.zeros((A.n_rows, 700))
+    with np.errstate(invalid="ignore"):
+        for i in range(A.n_rows):
+            k = np.nonzero(has_a[i])[0]
+            p = np.where(has_b[k], a[i, k, None] * b[k], 0.0)
+            want[i], bound[i] = p.sum(0), np.abs(p).sum(0)
+    has = (has_a.astype(np.float32) @ has_b.astype(np.float32)) > 0
+    rp, col, val = C.row_ptr.cpu().numpy(), C.col.cpu().numpy(), C.val.cpu().numpy()
+    r = np.repeat(np.arange(A.n_rows), np.diff(rp))
+    assert np.array_equal(np.flatnonzero(has), r * 700 + col)
+    w, t = want[r, col], bound[r, col]
+    fin = np.isfinite(w)
+    assert fin.any() and not fin.all()
+    assert np.array_equal(np.isnan(val), np.isnan(w)) and np.array_equal(val[~fin & ~np.isnan(w)], w[~fin & ~np.isnan(w)].astype(dtype))
+    tol = 1e-5 if dtype == np.float32 else 1e-12
+    assert np.all(np.abs(val[fin] - w[fin]) <= tol * t[fin])
+    assert not np.any(np.signbit(val[val == 0]))
+
+
+def test_a_kept_plan_with_new_values():
+    rng = np.random.default_rng(2)
+    A = _blocks(rng, [20] * 300, 90, 0.8, 500, np.float32)
+    B = _spans(rng, 500, 2000, 2, 60, 0.8, np.float32)
+    dA, dB = gm.DeviceCSR.from_host(A), gm.DeviceCSR.from_host(B)
+    plan = gm.spgemm_plan(dA, dB)
+    first = gm.spgemm_execute(plan)
+    v0 = first.val.clone()
+    dA.val.mul_(2.0)
+    second = gm.spgemm_execute(plan)
+    assert plan.stats().panel_rows == A.n_rows
+    assert torch.equal(first.col, second.col) and torch.equal(second.val, v0 * 2)
+
+
+def test_no_room_for_the_panels_lists(allocator):
+    # their memory is refused: the rows are tasks like the others
+    rng = np.random.default_rng(3)
+    A = _blocks(rng, [30] * 200, 90, 0.8, 500, np.float32)
+    B = _spans(rng, 500, 2000, 2, 70, 0.8, np.float32)
+    dA, dB = gm.DeviceCSR.from_host(A), gm.DeviceCSR.from_host(B)
+    ref = oracle.spgemm(A, B)
+    for refused in (False, True):
+        if refused:
+            allocator.refuse = staticmethod(lambda n: 30 * A.nnz < n < 70 * A.nnz)
+        plan = gm.spgemm_plan(dA, dB)
+        allocator.refuse = staticmethod(lambda n: False)
+        compare_rows(gm.spgemm_execute(plan), ref, np.float32)
+        assert plan.stats().panel_rows == (0 if refused else A.n_rows)
