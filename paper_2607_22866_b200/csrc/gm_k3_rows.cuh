@@ -280,15 +280,23 @@ __device__ __forceinline__ void sort_row(i64 row, const i64* __restrict__ a_row_
   const int lane = threadIdx.x & 31;
   const i64 at = light_off[row];
   const int n = gather_row<V, Key, K, KMAX>(a_row_ptr[row], a_row_ptr[row + 1], a_col, a_val, b_row_ptr, b_col, b_val, sm);
-  Key key[K];
+  int m = 0;
+  auto sort = [&](auto width) {
+    constexpr int W = decltype(width)::value;
+    Key key[W];
 #pragma unroll
-  for (int r = 0; r < K; ++r) {
-    const int q = r * 32 + lane;
-    key[r] = q < n ? sm.key[q] : ~Key(0);  // padding sorts to the end
-  }
-  __syncwarp();
-  warp_sort_keys<Key, K>(key, lane);
-  const int m = warp_sum_runs<V, Key, K, kPosBits>(key, n, sm.key, sm.val, 0u, out_col + at, out_val + at);
+    for (int r = 0; r < W; ++r) {
+      const int q = r * 32 + lane;
+      key[r] = q < n ? sm.key[q] : ~Key(0);  // padding sorts to the end
+    }
+    __syncwarp();
+    warp_sort_keys<Key, W>(key, lane);
+    m = warp_sum_runs<V, Key, W, kPosBits>(key, n, sm.key, sm.val, 0u, out_col + at, out_val + at);
+  };
+  if (K == 8 && n <= 160) sort(std::integral_constant<int, 5>{});
+  else if (K == 8 && n <= 192) sort(std::integral_constant<int, 6>{});
+  else if (K == 4 && n <= 96) sort(std::integral_constant<int, 3>{});
+  else sort(std::integral_constant<int, K>{});
   if (lane == 0) {
     row_nnz[row] = m;
     if (sums) atomicAdd(&sums[row / kSumRows], static_cast<u32>(m));
