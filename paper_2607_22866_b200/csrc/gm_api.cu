@@ -490,7 +490,8 @@ __global__ void k_validate_csr(const i64* __restrict__ row_ptr, const int32_t* _
   }
 }
 
-static size_t row_sum_words(i64 n_rows) { return (static_cast<size_t>(n_rows) / kSumRows + 64) & ~size_t{63}; }
+static i64 row_sum_groups(i64 n_rows) { return (n_rows + kSumRows - 1) / kSumRows; }
+static size_t row_sum_words(i64 n_rows) { return (static_cast<size_t>(row_sum_groups(n_rows) * (kSumGroups + 1) / kSumGroups) + 65) & ~size_t{63}; }
 
 // What the row analysis wants zeroed, at the front of an arena.
 struct K1Zeroed {
@@ -633,8 +634,8 @@ static bool plan_task_rules(gm_plan* p) {
 
 // Panels are looked for where heavy rows have many entries (R-MAT graphs have 25 to 40, and hardly two rows alike) and where there are
 // products enough to pay for the lists.  Block-dense products, us a call, tasks / panels: 2.8 M products fp64 150 / 195, 23 M fp32
-// 292 / 319, 166 M fp64 (kept plan) 895 / 510, 1.3 G fp64 5690 / 1630, 2.7 G fp32 8560 / 2440.
-constexpr i64 kPanelMinEntries = 48, kPanelMinHeavy = i64{1} << 25;
+// 292 / 319, 43 M fp32 336 / 342, 166 M fp64 (kept plan) 895 / 510, 1.3 G fp64 5690 / 1630, 2.7 G fp32 8560 / 2440.
+constexpr i64 kPanelMinEntries = 48, kPanelMinHeavy = i64{1} << 26;
 static int panel_max_u(const gm_plan* p) { return p->sv == 4 ? kPanelColumns<float> : kPanelColumns<double>; }
 static bool plan_panel_rules(const gm_plan* p) {
   const i64 n_groups = ((p->B.n_cols - 1) >> panel_group_bits(p->sv)) + 1;
@@ -1111,7 +1112,7 @@ static int launch_hash(gm_plan* p, int cap, int slots, const int32_t* rows, i64 
 }
 
 static RowSums row_sums_of(const gm_plan* p) {
-  return p->row_sums ? RowSums{p->sums[p->sums_at], p->sums[p->sums_at ^ 1]} : RowSums{nullptr, nullptr};
+  return p->row_sums ? RowSums{p->sums[p->sums_at], p->sums[p->sums_at ^ 1], row_sum_groups(p->A.n_rows)} : RowSums{nullptr, nullptr, 0};
 }
 
 // One thread per row: count, write to C, or write to the staging area.
@@ -1148,7 +1149,7 @@ static int launch_sort_one(gm_plan* p, const SortLists& lists, i64 n, cudaStream
   const unsigned grid = grid_for(n, kSortWarpsOf<KMAX>, p->num_sms, KMAX > 4 ? 16 : 24);
   k3_sort_rows<V, Key, KMAX><<<grid, kSortWarpsOf<KMAX> * 32, 0, st>>>(
       p->A.row_ptr, p->A.col_idx, static_cast<const V*>(p->A.vals), p->B.row_ptr, p->B.col_idx,
-      static_cast<const V*>(p->B.vals), lists, p->light_off, p->row_nnz, p->light_col, static_cast<V*>(p->light_val), row_sums_of(p).now);
+      static_cast<const V*>(p->B.vals), lists, p->light_off, p->row_nnz, p->light_col, static_cast<V*>(p->light_val), row_sums_of(p));
   ++p->stats.launches;
   GM_CUDA(cudaGetLastError());
   return GM_OK;

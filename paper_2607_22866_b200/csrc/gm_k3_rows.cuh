@@ -36,25 +36,38 @@ enum MergeMode { kMergeCount = 0, kMergeToC = 1, kMergeToStage = 2, kMergePlace 
 // a pass less (us a call, with the prefix sum / without: 5-point grids of 1024^2 points fp64 250 / 243, of 300^2 86 / 78; ER, 4096 rows of
 // 8 73 / 69, 100000 rows of 4 113 / 103, an execute of 30011 rows of 12 fp64 111 / 107 to 112).
 // The sums of the next execute are cleared by this one, which the next has waited for.
-constexpr int kSumRows = 256;
+// Above 256 groups, 64 of them together have a sum of their own, so that a block loads a few values per thread, all at once.  (Fewer
+// rows add to few of those, one after the other: ER, 5000 rows of 5 fp64, 39 us an execute with them, 36 without.)
+constexpr int kSumRows = 256, kSumGroups = 64;
+constexpr i64 kSumDirect = 256;
 constexpr i64 kSumRowsMax = i64{1} << 20;
 struct RowSums {
   u32* now;   // nullptr: offsets come from a prefix sum
   u32* next;
+  i64 n_groups;  // the sums of groups of groups lie behind those of the groups
 };
+__device__ __forceinline__ void add_entries(const RowSums& rs, i64 row, u32 n) {
+  atomicAdd(&rs.now[row / kSumRows], n);
+  if (rs.n_groups > kSumDirect) atomicAdd(&rs.now[rs.n_groups + row / (kSumRows * kSumGroups)], n);
+}
 // Entries of C before row r0, a multiple of 16 (at least, and of the rows a block has).  All T threads of the block; s_tmp: 33 values.
 template <int T>
 __device__ __forceinline__ i64 entries_before(const RowSums& rs, const int32_t* __restrict__ row_nnz, i64 r0, i64* s_tmp) {
-  const i64 group = r0 / kSumRows;
-  i64 n = 0;
-  for (i64 g = threadIdx.x; g < group; g += T) n += rs.now[g];
-  for (i64 r = group * kSumRows + threadIdx.x; r < r0; r += T) n += row_nnz[r];
+  static_assert(kSumRowsMax / (kSumRows * kSumGroups) <= T && kSumGroups <= T && kSumDirect <= 2 * T && kSumRows <= 2 * T, "a value of each kind per thread");
+  const i64 group = r0 / kSumRows, super = rs.n_groups > kSumDirect ? group / kSumGroups : 0;
+  const int t = threadIdx.x;
+  const i64 g = super * kSumGroups + t, r = group * kSumRows + t;
+  const u32 a = t < super ? rs.now[rs.n_groups + t] : 0u, b = g < group ? rs.now[g] : 0u;
+  const u32 b2 = g + T < group ? rs.now[g + T] : 0u;  // (T = 128: up to 256 groups without supers)
+  const int c = r < r0 ? row_nnz[r] : 0, d = r + T < r0 ? row_nnz[r + T] : 0;
+  const i64 n = static_cast<i64>(a) + b + b2 + c + d;
   i64 total;
   block_exclusive_scan(n, s_tmp, &total);
   return total;
 }
 __device__ __forceinline__ void clear_next_sums(const RowSums& rs, i64 n_rows) {
-  for (i64 g = static_cast<i64>(blockIdx.x) * blockDim.x + threadIdx.x; g * kSumRows < n_rows; g += static_cast<i64>(gridDim.x) * blockDim.x) rs.next[g] = 0u;
+  const i64 n = rs.n_groups + (n_rows + kSumRows * kSumGroups - 1) / (kSumRows * kSumGroups);
+  for (i64 g = static_cast<i64>(blockIdx.x) * blockDim.x + threadIdx.x; g < n; g += static_cast<i64>(gridDim.x) * blockDim.x) rs.next[g] = 0u;
 }
 
 // One row.  emit(i, column, sum) for the row's i-th entry; returns the number of entries.
@@ -177,9 +190,9 @@ __global__ void __launch_bounds__(kMergeThreads) k3_merge_rows(
     if (rs.now) {
       if constexpr (MODE == kMergeCount) {  // a warp's rows are in one group
         const u32 sum = __reduce_add_sync(lanes, static_cast<u32>(n));
-        if ((threadIdx.x & 31) == 0) atomicAdd(&rs.now[row / kSumRows], sum);
+        if ((threadIdx.x & 31) == 0) add_entries(rs, row, sum);
       } else {
-        atomicAdd(&rs.now[row / kSumRows], static_cast<u32>(n));
+        add_entries(rs, row, static_cast<u32>(n));
       }
     }
   }
@@ -274,7 +287,7 @@ __device__ __forceinline__ void sort_row(i64 row, const i64* __restrict__ a_row_
                                          const V* __restrict__ a_val, const i64* __restrict__ b_row_ptr,
                                          const int32_t* __restrict__ b_col, const V* __restrict__ b_val,
                                          const i64* __restrict__ light_off, int32_t* __restrict__ row_nnz,
-                                         int32_t* __restrict__ out_col, V* __restrict__ out_val, u32* __restrict__ sums,
+                                         int32_t* __restrict__ out_col, V* __restrict__ out_val, const RowSums& rs,
                                          SortSmem<V, Key, KMAX>& sm) {
   constexpr int kPosBits = kSortPosBits<K>;
   const int lane = threadIdx.x & 31;
@@ -299,7 +312,7 @@ __device__ __forceinline__ void sort_row(i64 row, const i64* __restrict__ a_row_
   else sort(std::integral_constant<int, K>{});
   if (lane == 0) {
     row_nnz[row] = m;
-    if (sums) atomicAdd(&sums[row / kSumRows], static_cast<u32>(m));
+    if (rs.now) add_entries(rs, row, static_cast<u32>(m));
   }
   __syncwarp();  // the warp's shared memory is reused by its next row
 }
@@ -310,7 +323,7 @@ __global__ void __launch_bounds__(kSortWarpsOf<KMAX> * 32, KMAX > 4 ? 8 : 12) k3
     const i64* __restrict__ a_row_ptr, const int32_t* __restrict__ a_col, const V* __restrict__ a_val,
     const i64* __restrict__ b_row_ptr, const int32_t* __restrict__ b_col, const V* __restrict__ b_val, SortLists lists,
     const i64* __restrict__ light_off, int32_t* __restrict__ row_nnz, int32_t* __restrict__ out_col, V* __restrict__ out_val,
-    u32* __restrict__ sums) {
+    RowSums rs) {
   constexpr int kSortWarps = kSortWarpsOf<KMAX>;
   __shared__ SortSmem<V, Key, KMAX> s_sm[kSortWarps];
   SortSmem<V, Key, KMAX>& sm = s_sm[threadIdx.x >> 5];
@@ -322,7 +335,7 @@ __global__ void __launch_bounds__(kSortWarpsOf<KMAX> * 32, KMAX > 4 ? 8 : 12) k3
     /* the warps go on round-robin from one class to the next */                                                              \
     for (i64 q = ((w0 - before) % n_warps + n_warps) % n_warps; q < lists.n[I]; q += n_warps)                                  \
       sort_row<V, Key, K, KMAX>(lists.rows[I][q], a_row_ptr, a_col, a_val, b_row_ptr, b_col, b_val, light_off, row_nnz, out_col, \
-                                out_val, sums, sm);                                                                               \
+                                out_val, rs, sm);                                                                               \
     before += lists.n[I];                                                                                                     \
   }
   if constexpr (KMAX > 16) {
