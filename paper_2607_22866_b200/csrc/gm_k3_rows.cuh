@@ -16,6 +16,8 @@
 // C.row_ptr is known (one pass over the products, and the entries are written twice), or, when every row of the matrix
 // is merged, they are counted first and then written to their place in C: a second merge is cheaper than the copy.
 #pragma once
+#include <type_traits>
+
 #include "gm_common.cuh"
 #include "gm_k1_analysis.cuh"
 #include "gm_sort.cuh"

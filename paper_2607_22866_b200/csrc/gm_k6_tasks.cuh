@@ -390,7 +390,7 @@ struct RoundSize {
 };
 
 // The products of a round that fall to warp `warp` of `n_warps`: a contiguous, equal share, 32 at a time and U times that in
-// flight: load(u, position in B, a) for the valid lanes of U windows, then use(u, valid) for each.  `load` only requests;
+// flight: load(u, position in B, a) for the valid lanes of U windows, then use(u, valid, number of the product in the round) for each.  `load` only requests;
 // arithmetic on what it loads would wait there, window after window.
 // Every lane finds its piece from the ones that start inside the windows, all U windows at once: the chain from one round of U
 // windows to the next is one look at the piece starts and a population count.  (Window after window, with a way of its own for
@@ -431,7 +431,7 @@ __device__ __forceinline__ void walk_products(const Pieces<V, CAP>& pc, const Ro
     }
 #pragma unroll
     for (int u = 0; u < U; ++u)
-      if (f + u * 32 < f1) use(u, f + u * 32 + lane < f1);
+      if (f + u * 32 < f1) use(u, f + u * 32 + lane < f1, f + u * 32 + lane);
   }
 }
 
@@ -657,8 +657,9 @@ struct TaskFeed {
 // mid tasks: symbolic pass, ranks, numeric pass
 // ---------------------------------------------------------------------------------------------------------------------
 // Per block: bitmap of the task's columns | rank of every word's first entry | compact values | compact columns.  Pass 1
-// marks the columns, a prefix sum over the words ranks them, pass 2 adds every product to the slot of its column's rank and
-// notes the column; the write-out is one coalesced copy.
+// marks the columns (and keeps the products, if they fit the half of the arrays that the entries do not take), a prefix sum over the
+// words ranks them, pass 2 adds every product to the slot of its column's rank and notes the column; the write-out is one coalesced
+// copy.
 constexpr int kMidPerThread = 2;    // rows of B per thread and round
 // Windows of 32 products a warp has in flight (fp64: with four the registers spill, 1.35 against 1.19 ms for the big tasks
 // of R-MAT scale 17, 1.89 against 1.67 for the mid ones).
@@ -715,6 +716,14 @@ __global__ void __launch_bounds__(kMidThreads, 6) k6_mid_tasks(
     u32 c[U];
     V v[U], av[U];
     RoundSize rs = build_pieces<V, T, PER>(regs, pc, s_sum);
+    // Products that fill at most half of the compact arrays wait in the other half for pass 2, which then neither walks the pieces nor
+    // loads anything: this kernel 5.82 -> 5.47 ms for R-MAT scale 18 fp32, the call 59.1 -> 57.4 for scale 19.  (Larger arrays, for all of
+    // the class, leave four blocks an SM: 63.8; tasks cut so that more of them fit: 57.7.)
+    const int half = entries / 2;
+    const bool keep = task.n <= static_cast<u32>(half);
+    V* const kept_val = oval + half;
+    unsigned short* const kept_col = ocol + half;
+    int before = 0;  // products of the rounds before
 
     // ---- pass 1 (symbolic): mark the columns
     auto mark = [&](u32 c) {
@@ -725,9 +734,26 @@ __global__ void __launch_bounds__(kMidThreads, 6) k6_mid_tasks(
     for (int r = 0;;) {
       const bool more = ++r < n_rounds;
       if (more) load_rows<V, T, PER>(in, task, r, regs);
-      walk_products<V, CAP, U>(
-          pc, rs, warp, kWarps, [&](int u, u32 src, V) { c[u] = static_cast<u32>(in.b_col[src]); },
-          [&](int u, bool valid) { if (valid) mark(c[u] - lo); });
+      if (keep)
+        walk_products<V, CAP, U>(
+            pc, rs, warp, kWarps,
+            [&](int u, u32 src, V a) {
+              c[u] = static_cast<u32>(in.b_col[src]);
+              v[u] = in.b_val[src];
+              av[u] = a;
+            },
+            [&](int u, bool valid, int f) {
+              if (valid) {
+                mark(c[u] - lo);
+                kept_col[before + f] = static_cast<unsigned short>(c[u] - lo);
+                kept_val[before + f] = av[u] * v[u];
+              }
+            });
+      else
+        walk_products<V, CAP, U>(
+            pc, rs, warp, kWarps, [&](int u, u32 src, V) { c[u] = static_cast<u32>(in.b_col[src]); },
+            [&](int u, bool valid, int) { if (valid) mark(c[u] - lo); });
+      before += rs.products;
       if (!more) break;
       load_pieces<V, PER>(in, task, regs);
       __syncthreads();
@@ -779,7 +805,13 @@ __global__ void __launch_bounds__(kMidThreads, 6) k6_mid_tasks(
       atomicAdd(&oval[r], v);
       ocol[r] = static_cast<unsigned short>(c);  // (every product of the column writes the same value)
     };
-    for (int r = 0; r < n_rounds; ++r) {
+    if (keep) {
+      for (int i = tid; i < static_cast<int>(task.n); i += T) {
+        put(kept_col[i], kept_val[i]);
+        kept_val[i] = V(0);  // (the slots of a larger task)
+      }
+    }
+    for (int r = 0; !keep && r < n_rounds; ++r) {
       if (n_rounds > 1) {
         if (r > 0) __syncthreads();  // (the first time the pieces of the last round are no longer read either)
         load_rows<V, T, PER>(in, task, r, regs);
@@ -793,7 +825,7 @@ __global__ void __launch_bounds__(kMidThreads, 6) k6_mid_tasks(
             v[u] = in.b_val[src];
             av[u] = a;
           },
-          [&](int u, bool valid) { if (valid) put(c[u] - lo, av[u] * v[u]); });
+          [&](int u, bool valid, int) { if (valid) put(c[u] - lo, av[u] * v[u]); });
     }
     // the next task's first rows of B are requested before this task is written out
     if (next_id >= 0) load_rows<V, T, PER>(in, next, 0, regs);
@@ -918,7 +950,7 @@ __global__ void __launch_bounds__(BT, BLOCKS) k6_big_tasks(
             v[u] = in.b_val[src];
             av[u] = a;
           },
-          [&](int u, bool valid) { if (valid) add(c[u], product(av[u], v[u])); });
+          [&](int u, bool valid, int) { if (valid) add(c[u], product(av[u], v[u])); });
       if (!more) break;
       load_pieces<V, PER>(in, task, regs);
       __syncthreads();
