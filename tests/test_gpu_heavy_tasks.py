@@ -155,3 +155,18 @@ def test_tables_per_row_of_b_stay_small(n_rows_b, tasks):
     assert info.rows_heavy == 4 and info.heavy_tasks == tasks
     assert info.workspace_bytes < 3 << 29
     compare_rows(C, oracle.spgemm(gen.CSR(4, 1000, A.row_ptr, A.col, A.val), B), np.float32)
+
+
+@pytest.mark.parametrize("dtype", [np.float32, np.float64])
+@pytest.mark.parametrize("mid", [0, 600, 2048, 4096])
+def test_products_kept_between_the_passes(dtype, mid):
+    # tasks around half of the products that a mid-size block holds (kept for the second pass), over several rounds of rows of B;
+    # a large one after a small one finds its slots empty
+    rng = np.random.default_rng(mid)
+    n_cols, m = 30000, 4600
+    B = _csr([rng.choice(n_cols, 8 if i < 4300 else 1, replace=False) for i in range(m)], n_cols, rng, dtype)
+    sizes = [300, 301, 511, 512, 513, 1023, 1024, 1025, 1500, 2047, 2048, 2049, 3000, 4095, 4096, 4097] * 6
+    rows = [np.concatenate([rng.choice(4300, n // 8, replace=False), 4300 + rng.choice(300, n % 8, replace=False)]) for n in sizes]
+    A = _csr(rows, m, rng, dtype)
+    C, info, stats = check_product(A, B, tau=256, mid_chunk_max=mid)
+    assert info.heavy_tasks == 1 and stats.mid_chunk_products > 0
