@@ -108,13 +108,14 @@ struct K1Tile {
   __device__ __forceinline__ i64 before(int q) const { return base[q / (T / (kK1Threads / 32))] + static_cast<i64>(pre[q]); }
 };
 
-// Rows at the first items of the tiles from `tile` on, a warp each (the last one's end with them).  Ends with a barrier.
+// Rows at the first items of n tiles from `tile` on, and behind the last, a warp each.  Ends with a barrier.
 template <int T>
-__device__ __forceinline__ void k1_find_rows(const i64* __restrict__ a_row_ptr, i64 n_rows, i64 nnz_a, i64 tile, i64* s_row) {
+__device__ __forceinline__ void k1_find_rows(const i64* __restrict__ a_row_ptr, i64 n_rows, i64 nnz_a, i64 tile, int n, i64* s_row) {
   const int warp = threadIdx.x >> 5;
-  const i64 d = min((tile + warp) * T, n_rows + nnz_a);
-  const i64 r = find_row(a_row_ptr, n_rows, d);
-  if ((threadIdx.x & 31) == 0) s_row[warp] = r;
+  if (warp <= n) {
+    const i64 r = find_row(a_row_ptr, n_rows, min((tile + warp) * T, n_rows + nnz_a));
+    if ((threadIdx.x & 31) == 0) s_row[warp] = r;
+  }
   __syncthreads();
 }
 constexpr int kK1Ahead = kK1Threads / 32 - 1;  // tiles whose rows are looked up together
@@ -206,7 +207,7 @@ __global__ void __launch_bounds__(kK1Threads) k1_rows(
     if (tid < kRowClasses) s_cnt[tid] = 0;
     if (tid == 32) s_room_n = 0;
     const int ahead = static_cast<int>((tile - tile0) % kK1Ahead);
-    if (ahead == 0) k1_find_rows<T>(a_row_ptr, n_rows, nnz_a, tile, s_row);
+    if (ahead == 0) k1_find_rows<T>(a_row_ptr, n_rows, nnz_a, tile, static_cast<int>(min(i64{kK1Ahead}, tile1 - tile)), s_row);
     k1_load_tile<T, P>(s, a_row_ptr, a_col, n_rows, nnz_a, b_row_ptr, tile, s_row[ahead], s_row[ahead + 1]);
     for (int i0 = 0; i0 <= s.n_rows; i0 += kK1Threads) {
       // ---- one thread per row: class, room, totals
@@ -356,12 +357,7 @@ __global__ void __launch_bounds__(kK1Threads) k1_row_products_only(const i64* __
                                                                    i64* __restrict__ ip) {
   __shared__ K1Tile<T, P> s;
   __shared__ i64 s_row[2];
-  const int warp = threadIdx.x >> 5;
-  if (warp < 2) {
-    const i64 r = find_row(a_row_ptr, n_rows, min((static_cast<i64>(blockIdx.x) + warp) * T, n_rows + nnz_a));
-    if ((threadIdx.x & 31) == 0) s_row[warp] = r;
-  }
-  __syncthreads();
+  k1_find_rows<T>(a_row_ptr, n_rows, nnz_a, blockIdx.x, 1, s_row);
   k1_load_tile<T, P>(s, a_row_ptr, a_col, n_rows, nnz_a, b_row_ptr, blockIdx.x, s_row[0], s_row[1]);
   for (int i = threadIdx.x; i <= s.n_rows; i += kK1Threads) {
     const i64 row = s.r0 + i;
