@@ -518,8 +518,9 @@ static int analyse_rows(gm_plan* p, const K1Zeroed& z, cudaStream_t st) {
   if (A.n_rows > 0) {
     GM_CUDA(cudaMemsetAsync(z.totals, 0, z.bytes, st));
     const int T = k1_tile_items(A.n_rows, A.nnz, p->num_sms);
-    const unsigned grid = static_cast<unsigned>(std::min<i64>((A.n_rows + A.nnz + T - 1) / T, static_cast<i64>(p->num_sms) * 6));
     const bool wide = p->B.n_cols > (i64{1} << 24);
+    // (blocks that fit the SMs together: 33 KB of shared memory each, 41 with 64-bit prefix sums)
+    const unsigned grid = static_cast<unsigned>(std::min<i64>((A.n_rows + A.nnz + T - 1) / T, static_cast<i64>(p->num_sms) * (wide ? 5 : 6)));
     auto kern = T == kK1Small ? (wide ? k1_rows<kK1Small, i64> : k1_rows<kK1Small, u32>)
                               : (wide ? k1_rows<kK1Large, i64> : k1_rows<kK1Large, u32>);
     kern<<<grid, kK1Threads, 0, st>>>(A.row_ptr, A.col_idx, A.n_rows, A.nnz, p->B.row_ptr, p->rules, z.ip, z.parts, p->heavy_flag,

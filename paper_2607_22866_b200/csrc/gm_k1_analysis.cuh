@@ -108,17 +108,19 @@ struct K1Tile {
   __device__ __forceinline__ i64 before(int q) const { return base[q / (T / (kK1Threads / 32))] + static_cast<i64>(pre[q]); }
 };
 
-// Rows at the first items of n tiles from `tile` on, and behind the last, a warp each.  Ends with a barrier.
+// Rows at the first items of tiles `tile`, `tile` + stride, ... (kK1Ahead of them, as far as there are any) and behind their last, a warp
+// each: s_row[2 k] and s_row[2 k + 1].  Ends with a barrier.
+constexpr int kK1Ahead = kK1Threads / 64;  // tiles whose rows are looked up together
 template <int T>
-__device__ __forceinline__ void k1_find_rows(const i64* __restrict__ a_row_ptr, i64 n_rows, i64 nnz_a, i64 tile, int n, i64* s_row) {
+__device__ __forceinline__ void k1_find_rows(const i64* __restrict__ a_row_ptr, i64 n_rows, i64 nnz_a, i64 tile, i64 stride, i64 n_tiles, i64* s_row) {
   const int warp = threadIdx.x >> 5;
-  if (warp <= n) {
-    const i64 r = find_row(a_row_ptr, n_rows, min((tile + warp) * T, n_rows + nnz_a));
+  const i64 t = tile + (warp >> 1) * stride;
+  if (t < n_tiles) {
+    const i64 r = find_row(a_row_ptr, n_rows, min((t + (warp & 1)) * T, n_rows + nnz_a));
     if ((threadIdx.x & 31) == 0) s_row[warp] = r;
   }
   __syncthreads();
 }
-constexpr int kK1Ahead = kK1Threads / 32 - 1;  // tiles whose rows are looked up together
 
 // Loads the rows of a tile that begins in row r0 and ends in row r1, and the prefix sums of its entries' products.  Ends with a barrier.
 template <int T, typename P>
@@ -199,16 +201,17 @@ __global__ void __launch_bounds__(kK1Threads) k1_rows(
   u32 nh = 0, ne = 0;
   const i64 n_tiles = (n_rows + nnz_a + T - 1) / T;
   // (a few blocks per SM, each with many tiles: the totals sit in one line of L2, and a set of atomics per tile was most
-  // of this kernel's time.  A block's tiles are neighbours, and its eight warps look up the rows at eight tiles' beginnings together:
-  // with two warps that did so for every tile while the others waited, the 1024^2 grid took 55 us, now 52, ER of 200000 rows of 12 65, now 59.)
-  __shared__ i64 s_row[kK1Ahead + 1];
-  const i64 per_block = (n_tiles + gridDim.x - 1) / gridDim.x, tile0 = blockIdx.x * per_block, tile1 = min(n_tiles, tile0 + per_block);
-  for (i64 tile = tile0; tile < tile1; ++tile) {
+  // of this kernel's time.  The blocks go round-robin over the tiles: with a run of neighbouring tiles for each, 1400 tiles kept 700 of 888
+  // blocks busy, and the Zipf pair of 2^20 rows took 315 us here instead of 277.  The eight warps look up the rows of a block's next four
+  // tiles together: with two warps that did so for every tile while the others waited, that pair took 290 us, the 1024^2 grid 55
+  // instead of 50, ER of 200000 rows of 12 56 instead of 54.)
+  __shared__ i64 s_row[2 * kK1Ahead];
+  int ahead = 0;
+  for (i64 tile = blockIdx.x; tile < n_tiles; tile += gridDim.x, ahead = (ahead + 1) % kK1Ahead) {
     if (tid < kRowClasses) s_cnt[tid] = 0;
     if (tid == 32) s_room_n = 0;
-    const int ahead = static_cast<int>((tile - tile0) % kK1Ahead);
-    if (ahead == 0) k1_find_rows<T>(a_row_ptr, n_rows, nnz_a, tile, static_cast<int>(min(i64{kK1Ahead}, tile1 - tile)), s_row);
-    k1_load_tile<T, P>(s, a_row_ptr, a_col, n_rows, nnz_a, b_row_ptr, tile, s_row[ahead], s_row[ahead + 1]);
+    if (ahead == 0) k1_find_rows<T>(a_row_ptr, n_rows, nnz_a, tile, gridDim.x, n_tiles, s_row);
+    k1_load_tile<T, P>(s, a_row_ptr, a_col, n_rows, nnz_a, b_row_ptr, tile, s_row[2 * ahead], s_row[2 * ahead + 1]);
     for (int i0 = 0; i0 <= s.n_rows; i0 += kK1Threads) {
       // ---- one thread per row: class, room, totals
       const int i = i0 + tid;
@@ -356,8 +359,8 @@ __global__ void __launch_bounds__(kK1Threads) k1_row_products_only(const i64* __
                                                                    i64 n_rows, i64 nnz_a, const i64* __restrict__ b_row_ptr,
                                                                    i64* __restrict__ ip) {
   __shared__ K1Tile<T, P> s;
-  __shared__ i64 s_row[2];
-  k1_find_rows<T>(a_row_ptr, n_rows, nnz_a, blockIdx.x, 1, s_row);
+  __shared__ i64 s_row[2];  // (a block has one tile)
+  k1_find_rows<T>(a_row_ptr, n_rows, nnz_a, blockIdx.x, gridDim.x, gridDim.x, s_row);
   k1_load_tile<T, P>(s, a_row_ptr, a_col, n_rows, nnz_a, b_row_ptr, blockIdx.x, s_row[0], s_row[1]);
   for (int i = threadIdx.x; i <= s.n_rows; i += kK1Threads) {
     const i64 row = s.r0 + i;

@@ -122,3 +122,30 @@ def test_light_rows_find_their_place_by_themselves(n, longest, dtype):
     assert plan.info().rows_heavy == 0
     for _ in range(3):
         compare_rows(gm.spgemm_execute(plan), ref, dtype)
+
+
+@pytest.mark.parametrize("n_cols", [1 << 24, (1 << 24) + 1])  # 32-bit prefix sums, and the first width with 64-bit ones
+def test_row_analysis_with_many_tiles_to_a_block(n_cols):
+    # some ten tiles for every block, so that its warps look up the rows of four tiles at a time, thrice; hub rows over several tiles
+    import paper_2607_22866_b200 as gm
+    rng = np.random.default_rng(6)
+    n, m = 9_000_000, 4000
+    k = rng.integers(0, 3, n)
+    k[[0, n // 3, n - 1]] = m
+    k[n // 2:n // 2 + 50000] = 0
+    rp = np.zeros(n + 1, np.int64)
+    np.cumsum(k, out=rp[1:])
+    col = (np.arange(rp[-1]) - np.repeat(rp[:-1], k) + np.repeat(np.where(k == m, 0, rng.integers(0, m - 3, n)), k)).astype(np.int32)
+    length = rng.integers(0, 30, m)
+    b_rp = np.zeros(m + 1, np.int64)
+    np.cumsum(length, out=b_rp[1:])
+    A = gm.DeviceCSR(n, m, torch.from_numpy(rp).cuda(), torch.from_numpy(col).cuda(), torch.ones(col.size, device="cuda"))
+    B = gm.DeviceCSR(m, n_cols, torch.from_numpy(b_rp).cuda(), torch.from_numpy((np.arange(b_rp[-1]) - np.repeat(b_rp[:-1], length)).astype(np.int32)).cuda(),
+                     torch.ones(int(b_rp[-1]), device="cuda"))
+    before = np.zeros(col.size + 1, np.int64)
+    np.cumsum(length[col], out=before[1:])
+    ref = before[rp[1:]] - before[rp[:-1]]
+    plan = gm.spgemm_plan(A, B)
+    assert np.array_equal(plan.row_products().cpu().numpy(), ref)
+    info = plan.info()
+    assert info.products_total == ref.sum() and info.products_max_row == ref.max() and info.rows_empty == int((ref == 0).sum()) and info.rows_heavy == 3
