@@ -1355,9 +1355,12 @@ static int launch_gather(gm_plan* p, const Batch& b, const HeavyBatchState<V>& h
   k_tile_bounds<<<grid_for(grid, 256, p->num_sms), 256, 0, st>>>(p->chunk_nnz_off, hs.n_chunks, 0, 0, tile, p->tile_meta,
                                                                p->chunk_nnz_off + hs.n_chunks);
   const bool alt = hs.tags && hs.xt.alt_bits;
-  auto kern = alt ? (tile == kGatherTile ? k7_gather<V, kGatherTile, true> : tile == 4096 ? k7_gather<V, 4096, true> : k7_gather<V, 2048, true>)
-                  : (tile == kGatherTile ? k7_gather<V, kGatherTile> : tile == 4096 ? k7_gather<V, 4096> : k7_gather<V, 2048>);
-  kern<<<std::min(grid, static_cast<unsigned>(p->num_sms * kGatherBlocksPerSm)), kGatherThreads, 0, st>>>(hs.fin_col, hs.fin_val, hs.chunk_off, p->chunk_nnz_off, p->chunk_base, hs.n_chunks,
+  const unsigned most = static_cast<unsigned>(p->num_sms * kGatherBlocksPerSm);
+#define GM_GATHER(ALT, LOOP) \
+  (tile == kGatherTile ? k7_gather<V, kGatherTile, ALT, LOOP> : tile == 4096 ? k7_gather<V, 4096, ALT, LOOP> : k7_gather<V, 2048, ALT, LOOP>)
+  auto kern = grid > most ? (alt ? GM_GATHER(true, true) : GM_GATHER(false, true)) : (alt ? GM_GATHER(true, false) : GM_GATHER(false, false));
+#undef GM_GATHER
+  kern<<<std::min(grid, most), kGatherThreads, 0, st>>>(hs.fin_col, hs.fin_val, hs.chunk_off, p->chunk_nnz_off, p->chunk_base, hs.n_chunks,
                                         p->tile_meta, c_col, c_val, c_capacity, p->err, alt ? hs.alt_col : nullptr,
                                         alt ? hs.alt_val : nullptr, alt ? hs.tags : nullptr, alt ? hs.xt.alt_bits : 0);
   p->stats.launches += 3;

@@ -34,13 +34,15 @@ constexpr int kGatherTileMin = 2048;
 // The number of tiles is only known on the device, and the products are an upper bound that can be forty times the entries:
 // at most this many blocks per SM go over the tiles.  (A block-dense product, forty products per entry, 262140 tiles and 64481 of which
 // most are empty: this kernel 287 + 61 us with a block each, 166 + 47 so.)
+// A grid that has a block for every tile takes the kernel without the loop: the Zipf pair's chunks of both buffers 548 us with, 526 without
+// (tasks, without a second buffer: no difference, 168.5 us of R-MAT scale 15, 706 of scale 17 fp64).
 constexpr int kGatherBlocksPerSm = 128;
 inline int gather_tile(i64 n_chunks, i64 n_elems) {
   int t = kGatherTile;
   while (t > kGatherTileMin && n_chunks * t > n_elems * (kGatherChunkCap * 3 / 4)) t /= 2;
   return t;
 }
-template <typename V, int TILE, bool ALT = false>
+template <typename V, int TILE, bool ALT = false, bool LOOP = true>
 __global__ void __launch_bounds__(kGatherThreads) k7_gather(
     const int32_t* __restrict__ s_col_in, const V* __restrict__ s_val_in,  // staging buffer (compacted chunks)
     const i64* __restrict__ chunk_off, const i64* __restrict__ chunk_nnz_off, const i64* __restrict__ chunk_base,
@@ -166,6 +168,7 @@ __global__ void __launch_bounds__(kGatherThreads) k7_gather(
         }
       }
     }
+    if constexpr (!LOOP) return;
     __syncthreads();  // the tables are the next tile's
   }
 }

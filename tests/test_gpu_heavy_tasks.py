@@ -170,3 +170,17 @@ def test_products_kept_between_the_passes(dtype, mid):
     A = _csr(rows, m, rng, dtype)
     C, info, stats = check_product(A, B, tau=256, mid_chunk_max=mid)
     assert info.heavy_tasks == 1 and stats.mid_chunk_products > 0
+
+
+@pytest.mark.parametrize("opts", [dict(), dict(level0_multisplit=1), dict(level0_multisplit=1, chunk_width=32, max_fanout=4)])
+def test_gather_goes_over_more_tiles_than_it_has_blocks(opts):
+    # 160 products to an entry of C: 19531 tiles of products, 148 SMs of 128 blocks each; in one staging buffer and in two
+    n, m = 1000, 400
+    rng = np.random.default_rng(7)
+    A = _csr([np.arange(m)] * n, m, rng, np.float32)
+    B = _csr([np.arange(m)] * m, m, rng, np.float32)
+    C, info, stats = run_gpu(A, B, **opts)
+    assert info.rows_heavy == n and info.n_batches == 1 and info.products_heavy > 148 * 128 * 8192
+    assert C.nnz == n * m and np.array_equal(C.col.cpu().numpy(), np.tile(np.arange(m), n))
+    a, b = A.val.reshape(n, m).astype(np.float64), B.val.reshape(m, m).astype(np.float64)
+    assert np.all(np.abs(C.val.cpu().numpy().reshape(n, m) - a @ b) <= 1e-5 * (np.abs(a) @ np.abs(b)))
