@@ -422,11 +422,10 @@ constexpr size_t kLightRoom = size_t{4} << 20;
 // C is allocated before its size is known, with room for every product, when that takes at most this much: the call then
 // does not wait in the middle for nnz(C), and the allocation overlaps the kernels.  Product calls with the wait and without, us:
 // ER of 1000 rows 88 / 76, of 10000 95 / 87.5, of 200000 (165 MB of room) 575 / 566; R-MAT scale 12 fp32 (33 MB) 223 / 215.5,
-// scale 13 with 15 edges a vertex (90 MB) 336 / 324.  More room would still gain, but is memory that a caller may not have.
+// scale 13 with 15 edges a vertex (90 MB) 336 / 324.  More room would still gain (some 12 us: the 1024^2 grid fp64 245 / 232), but is memory
+// that a caller may not have (314 MB of room for that grid's 163 MB), and where C has to move out of it again the call loses: rows of 15
+// and 21 neighbouring columns, 60000 and 20000 rows fp64, 100000 fp32, 294 / 312, 226 / 237, 800 / 820, with up to 336 MB more at the peak.
 constexpr i64 kCRoomBytes = i64{64} << 20;
-// ... and this much where a prefix sum over the rows is left out with the wait (see RowSums; product calls, us, with the wait and the
-// prefix sum / without: the 1024^2 grid fp64, 314 MB of room for 163 MB of C, 250 / 243; ER of 200000 rows of 12 fp32, 230 MB, 575 / 560).
-constexpr i64 kCRoomBytesPlaced = i64{512} << 20;
 // ... and what the caller then holds for nothing is at most this much, or as much again as C itself takes: with more C is
 // moved to arrays of its size, which costs some 20 us (block-dense fp32 of 2400 rows, 14 MB of C in 35 MB of room: 346 us moved,
 // 328 kept).
@@ -905,8 +904,7 @@ static int build_plan(gm_plan* p, cudaStream_t st) {
       ar.add(&p->num_fill, 8);
       GM_TRY(ar.commit(p, st));
     }
-    p->row_sums = nH == 0 && !hash_rows && info.rows_empty < nA && nA <= kSumRowsMax &&
-                  info.c_nnz_upper * static_cast<i64>(4 + p->sv) <= kCRoomBytesPlaced;
+    p->row_sums = nH == 0 && !hash_rows && info.rows_empty < nA && nA <= kSumRowsMax;
   }
 
   // ---- heavy rows
@@ -1853,13 +1851,12 @@ static int execute_t(gm_plan* p, cudaStream_t st, gm_csr* C) {
                                                         reinterpret_cast<i64*>(&slot->c_total));
     }
     tm.end(st);
-    if ((p->row_sums || info.c_nnz_upper * static_cast<i64>(4 + sizeof(V)) <= kCRoomBytes) && alloc_c(info.c_nnz_upper, &c_col, &c_val, st)) {
+    if (info.c_nnz_upper * static_cast<i64>(4 + sizeof(V)) <= kCRoomBytes && alloc_c(info.c_nnz_upper, &c_col, &c_val, st)) {
       capacity = info.c_nnz_upper;
     } else {
-      if (p->row_sums) {  // refused: C takes what it needs, from now on
-        p->row_sums = false;
-        p->stats.launches += exclusive_scan<int32_t, i64>(p->row_nnz, c_row_ptr, nA, p->scan_tmp, nullptr, nullptr, nullptr, st,
-                                                          reinterpret_cast<i64*>(&slot->c_total));
+      if (p->row_sums) {
+        k3_total<<<1, 256, 0, st>>>(row_sums_of(p), nA, reinterpret_cast<i64*>(&slot->c_total));
+        p->stats.launches += 1;
       }
       if (cudaStreamSynchronize(st) != cudaSuccess) {
         cleanup();

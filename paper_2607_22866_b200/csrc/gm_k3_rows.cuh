@@ -42,6 +42,9 @@ enum MergeMode { kMergeCount = 0, kMergeToC = 1, kMergeToStage = 2, kMergePlace 
 // rows add to few of those, one after the other: ER, 5000 rows of 5 fp64, 39 us an execute with them, 36 without.)
 constexpr int kSumRows = 256, kSumGroups = 64;
 constexpr i64 kSumDirect = 256;
+// Also where C's room waits for the total (see kCRoomBytes; with the prefix sum / without: the 1024^2 grid fp64 258 / 245, of 700^2
+// 159 / 158, an execute of ER of 400000 rows of 10 fp32 639 / 633, product of 10^6 rows of 12 2340 / 2348).  Above 2^20 rows it is even or a
+// loss: with 2^21 allowed the 1448^2 grid fp32 334 / 340, fp64 399 / 405, ER of 1.5 M rows of 6 2137 / 2126.
 constexpr i64 kSumRowsMax = i64{1} << 20;
 struct RowSums {
   u32* now;   // nullptr: offsets come from a prefix sum
@@ -70,6 +73,16 @@ __device__ __forceinline__ i64 entries_before(const RowSums& rs, const int32_t* 
 __device__ __forceinline__ void clear_next_sums(const RowSums& rs, i64 n_rows) {
   const i64 n = rs.n_groups + (n_rows + kSumRows * kSumGroups - 1) / (kSumRows * kSumGroups);
   for (i64 g = static_cast<i64>(blockIdx.x) * blockDim.x + threadIdx.x; g < n; g += static_cast<i64>(gridDim.x) * blockDim.x) rs.next[g] = 0u;
+}
+// Entries of C in all, for a host that waits for them before it allocates C.  One block of 256 threads.
+__global__ void __launch_bounds__(256) k3_total(RowSums rs, i64 n_rows, i64* __restrict__ host_total) {
+  static_assert(kSumDirect <= 256 && kSumRowsMax / (kSumRows * kSumGroups) <= 256, "a value per thread");
+  __shared__ i64 s_tmp[33];
+  const bool direct = rs.n_groups <= kSumDirect;
+  const i64 n = direct ? rs.n_groups : (n_rows + kSumRows * kSumGroups - 1) / (kSumRows * kSumGroups);
+  i64 total;
+  block_exclusive_scan(threadIdx.x < n ? static_cast<i64>(rs.now[(direct ? 0 : rs.n_groups) + threadIdx.x]) : i64{0}, s_tmp, &total);
+  if (threadIdx.x == 0) *host_total = total;  // (read after a synchronisation)
 }
 
 // One row.  emit(i, column, sum) for the row's i-th entry; returns the number of entries.

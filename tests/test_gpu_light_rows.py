@@ -8,6 +8,7 @@ import gen
 import oracle
 from helpers import random_csr
 from parity import check_product, compare_rows
+from test_gpu_scratch_and_errors import allocator  # noqa: F401 (fixture)
 
 pytestmark = pytest.mark.gpu
 
@@ -149,3 +150,53 @@ def test_row_analysis_with_many_tiles_to_a_block(n_cols):
     assert np.array_equal(plan.row_products().cpu().numpy(), ref)
     info = plan.info()
     assert info.products_total == ref.sum() and info.products_max_row == ref.max() and info.rows_empty == int((ref == 0).sum()) and info.rows_heavy == 3
+
+
+@pytest.mark.parametrize("dtype", [np.float32, np.float64])
+@pytest.mark.parametrize("rows", ["merged", "sorted"])
+def test_c_takes_what_its_entries_take(rows, dtype):
+    # no heavy rows, several products per entry of C, 64 to 512 MB for all of them: nothing is held for those, at no time
+    import paper_2607_22866_b200 as gm
+    if rows == "merged":
+        A = gen.laplacian_2d(700, dtype=dtype)
+    else:
+        n, w = 40000, 19
+        i = np.arange(n)[:, None] + np.arange(w) - w // 2
+        A = _csr([r[(r >= 0) & (r < n)] for r in i], n, np.random.default_rng(1), dtype)
+    dA = gm.DeviceCSR.from_host(A)
+    ref = oracle.spgemm(A, A)
+    plan = gm.spgemm_plan(dA, dA)
+    entry = 4 + np.dtype(dtype).itemsize
+    assert plan.info().rows_heavy == 0 and 64 << 20 < plan.info().c_nnz_upper * entry < 512 << 20
+    for _ in range(2):
+        torch.cuda.synchronize()
+        torch.cuda.reset_peak_memory_stats()
+        before = torch.cuda.memory_allocated()
+        C = gm.spgemm_execute(plan)
+        peak = torch.cuda.max_memory_allocated() - before
+        compare_rows(C, ref, dtype)
+        assert peak <= ref.nnz * entry + (A.n_rows + 1) * 8 + (4 << 20)
+        del C
+
+
+@pytest.mark.parametrize("n", [3000, (1 << 16) + 300])  # sorted rows; merged rows
+def test_light_rows_after_a_refusal(allocator, n):
+    # the room for every product is refused: C takes what it needs.  C is refused: the next execute starts from cleared sums.
+    import paper_2607_22866_b200 as gm
+    A = gen.erdos_renyi_k(n, 4, seed=n, dtype=np.float32)
+    dA = gm.DeviceCSR.from_host(A)
+    ref = oracle.spgemm(A, A)
+    plan = gm.spgemm_plan(dA, dA)
+    upper = plan.info().c_nnz_upper
+    assert plan.info().rows_heavy == 0 and ref.nnz < upper
+    for refuse, ok in ((lambda b: b >= upper * 4, True), (lambda b: b < n * 8 or b > (n + 1) * 8, False), (lambda b: False, True),
+                       (lambda b: b >= upper * 4, True), (lambda b: False, True)):
+        allocator.refuse = staticmethod(refuse)
+        if ok:
+            C = gm.spgemm_execute(plan)
+            allocator.refuse = staticmethod(lambda b: False)
+            compare_rows(C, ref, np.float32)
+        else:
+            with pytest.raises(gm.GmError) as ei:
+                gm.spgemm_execute(plan)
+            assert ei.value.status == -5
