@@ -744,7 +744,7 @@ static int plan_tasks(gm_plan* p, cudaStream_t st) {
   if (r.granules > 1) {
     k_granule_counts<<<grid_for(nH, 8, p->num_sms, 8), 256, 0, st>>>(p->x_heavy, nH, A.row_ptr, A.col_idx, p->piece_bound, r.granules,
                                                                    p->granule_counts, long_rows, n_long, in_panel);
-    k_granule_counts_long<<<dim3(static_cast<unsigned>(p->num_sms), kCountRuns), 256, 0, st>>>(p->x_heavy, A.row_ptr, A.col_idx, p->piece_bound, r.granules,
+    k_granule_counts_long<<<static_cast<unsigned>(p->num_sms * kCountRuns), 256, 0, st>>>(p->x_heavy, A.row_ptr, A.col_idx, p->piece_bound, r.granules,
                                                                                p->granule_counts, long_rows, n_long);
     p->info.launches += 2;
   }

@@ -142,20 +142,24 @@ __global__ void __launch_bounds__(256) k_granule_counts(const int32_t* __restric
     }
   }
 }
-// Block (x, y) takes rows x, x + gridDim.x, ... and of each the runs y, y + gridDim.y, ... of kCountRun entries, a slice per warp.  (With
-// all warps of the grid round-robin over all slices, every warp looked up every row's ends, one after the other: 730 us of R-MAT
-// scale 19.)
+// The blocks form groups, one row at a time to a group, and the blocks of a group take the row's runs of kCountRun entries in turn, a
+// slice per warp: kCountRuns blocks to a group, or as many more as few rows leave.  (With all warps of the grid round-robin over all
+// slices, every warp looked up every row's ends, one after the other: 730 us of R-MAT scale 19.  With kCountRuns blocks however few the
+// rows: one row of 10^6 entries 750 us, two of 300000 250.)
 constexpr int kCountRun = 8 * 256, kCountRuns = 16;
 __global__ void __launch_bounds__(256) k_granule_counts_long(const int32_t* __restrict__ x_heavy, const i64* __restrict__ a_row_ptr,
                                                              const int32_t* __restrict__ a_col, const u32* __restrict__ bound, int granules,
                                                              u32* __restrict__ counts, const int32_t* __restrict__ long_rows,
                                                              const u32* __restrict__ n_long) {
   const u32 n = *n_long;
-  for (u32 q = blockIdx.x; q < n; q += gridDim.x) {
+  if (n == 0) return;
+  const u32 groups = min(n, gridDim.x / kCountRuns), blocks = gridDim.x / groups, run = blockIdx.x % blocks;
+  if (blockIdx.x / blocks >= groups) return;  // (left over)
+  for (u32 q = blockIdx.x / blocks; q < n; q += groups) {
     const i64 h = long_rows[q];
     const i64 row = x_heavy[h];
     const i64 e = a_row_ptr[row + 1];
-    for (i64 s = a_row_ptr[row] + static_cast<i64>(blockIdx.y) * kCountRun + (threadIdx.x >> 5) * 256; s < e; s += static_cast<i64>(gridDim.y) * kCountRun)
+    for (i64 s = a_row_ptr[row] + static_cast<i64>(run) * kCountRun + (threadIdx.x >> 5) * 256; s < e; s += static_cast<i64>(blocks) * kCountRun)
       count_granules(a_col, s, min(e, s + 256), bound, granules, counts + h * granules, true);
   }
 }

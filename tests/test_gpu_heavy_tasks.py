@@ -184,3 +184,15 @@ def test_gather_goes_over_more_tiles_than_it_has_blocks(opts):
     assert C.nnz == n * m and np.array_equal(C.col.cpu().numpy(), np.tile(np.arange(m), n))
     a, b = A.val.reshape(n, m).astype(np.float64), B.val.reshape(m, m).astype(np.float64)
     assert np.all(np.abs(C.val.cpu().numpy().reshape(n, m) - a @ b) <= 1e-5 * (np.abs(a) @ np.abs(b)))
+
+
+@pytest.mark.parametrize("n_long", [1, 2, 147, 148, 149, 300])
+def test_counting_long_rows_with_all_blocks(n_long):
+    # rows of A above 1024 entries share the blocks that count them: one row has all of them, from 149 on a group of blocks has several
+    rng = np.random.default_rng(n_long)
+    m, n_cols = 6000, 30000
+    B = _csr([_row(rng, n_cols, int(k), 3000) for k in rng.integers(4, 24, m)], n_cols, rng, np.float32)
+    longest = [m, 1025, 2048, 2049, 1024] if n_long < 10 else [1025, 1300, 1026, 2049]
+    A = _csr([rng.choice(m, longest[i % len(longest)], replace=False) for i in range(n_long)] + [rng.choice(m, 200, replace=False)] * 3, m, rng, np.float32)
+    C, info, stats = check_product(A, B, tau=512, chunk_width=8192)
+    assert info.heavy_tasks == 1 and info.rows_heavy == n_long + 3 and info.params.chunks_required > 1
