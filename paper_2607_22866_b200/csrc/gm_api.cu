@@ -184,6 +184,7 @@ struct HostSlot {
   i64 c_total;           // nnz(C)
   i64 n_tasks;           // tasks of the heavy rows
   i64 tail[16];          // copy of gm_plan::c_total
+  u64 panels[gm::kPanelCounts];  // copy of PanelTables::counts
 };
 constexpr int kHostSlotBytes = 512;
 static_assert(sizeof(HostSlot) <= kHostSlotBytes, "one slot");
@@ -365,6 +366,7 @@ struct gm_plan {
   int* task_tickets = nullptr;     // 4 per batch: big, mid, panels
   bool use_panels = false;         // neighbouring heavy rows with much the same columns are summed together (gm_k6_panels.cuh)
   gm::PanelTables panels{};
+  void* panel_mem = nullptr;       // their lists
   std::vector<int64_t> batch_starts;
   gm::PhaseTimes times;
   HostSink* sink = nullptr;        // set by gm_spgemm_host for the duration of one execute
@@ -436,15 +438,20 @@ struct Arena {
   struct Item { void** slot; size_t offset; };
   std::vector<Item> items;
   size_t bytes = 0;
+  void* base = nullptr;
   template <typename T>
   void add(T** slot, size_t n) {
     items.push_back({reinterpret_cast<void**>(slot), bytes});
     bytes += (n * sizeof(T) + 255) & ~size_t{255};
   }
+  void place(void* at) {  // (memory that is there already)
+    base = at;
+    for (const Item& it : items) *it.slot = static_cast<unsigned char*>(at) + it.offset;
+  }
   int commit(gm_plan* p, cudaStream_t st) {
-    unsigned char* base = nullptr;
-    GM_TRY(plan_alloc(p, &base, bytes, st));
-    for (const Item& it : items) *it.slot = base + it.offset;
+    unsigned char* q = nullptr;
+    GM_TRY(plan_alloc(p, &q, bytes, st));
+    place(q);
     return GM_OK;
   }
 };
@@ -636,12 +643,64 @@ static bool plan_task_rules(gm_plan* p) {
 // products enough to pay for the lists.  Block-dense products, us a call, tasks / panels: 2.8 M products fp64 150 / 195, 23 M fp32
 // 292 / 319, 43 M fp32 336 / 342, 166 M fp64 (kept plan) 895 / 510, 1.3 G fp64 5690 / 1630, 2.7 G fp32 8560 / 2440.
 constexpr i64 kPanelMinEntries = 48, kPanelMinHeavy = i64{1} << 26;
+constexpr size_t kPanelMemoryShare = 32;  // the lists take at most this part of the device's memory
 static int panel_max_u(const gm_plan* p) { return p->sv == 4 ? kPanelColumns<float> : kPanelColumns<double>; }
+static i64 panel_groups(const gm_plan* p) { return ((p->B.n_cols - 1) >> panel_group_bits(p->sv)) + 1; }
 static bool plan_panel_rules(const gm_plan* p) {
-  const i64 n_groups = ((p->B.n_cols - 1) >> panel_group_bits(p->sv)) + 1;
   const size_t smem = p->sv == 4 ? sizeof(PanelSmem<float>) : sizeof(PanelSmem<double>);
-  return p->info.products_heavy >= kPanelMinHeavy && p->n_seg >= kPanelMinEntries * p->info.rows_heavy && p->B.n_rows <= kPanelMaxRowsB && n_groups <= kPanelMaxGroups &&
-         std::max(smem, panel_build_smem(p->B.n_rows, n_groups)) + 1024 <= p->smem_bytes;
+  return p->info.products_heavy >= kPanelMinHeavy && p->n_seg >= kPanelMinEntries * p->info.rows_heavy && p->B.n_rows <= kPanelMaxRowsB &&
+         panel_groups(p) <= kPanelMaxGroups && std::max(smem, panel_build_smem(p->B.n_rows, panel_groups(p))) + 1024 <= p->smem_bytes;
+}
+
+// No panels after all: the lists are given back (nothing that is queued uses them), the rows are tasks like the others.
+static void drop_panels(gm_plan* p, cudaStream_t st) {
+  p->use_panels = false;
+  plan_free(p, p->panel_mem, st);
+  p->panel_mem = nullptr;
+}
+
+// The lists of the panels, sized by what was found (in the host slot).  Nothing is allocated where that does not pay: for ER of 20000
+// rows of 60 fp32, no two rows alike, lists for all heavy rows took 38 us of 915 and 62 MB.
+static int build_panels(gm_plan* p, cudaStream_t st) {
+  const gm_csr& A = p->A;
+  const gm_csr& B = p->B;
+  const i64 nH = p->info.rows_heavy;
+  PanelTables& pt = p->panels;
+  const u64* const found = p->slot->panels;
+  const size_t entries = static_cast<size_t>(found[kPanelEntries]), groups = entries / kPanelEntriesPerGroup + 1;
+  u32* piece_count = nullptr;
+  i64* piece_tmp = nullptr;
+  Arena ar, scratch;
+  ar.add(&pt.a_u, entries);
+  ar.add(&pt.u_mask, entries);
+  ar.add(&pt.groups, groups);
+  ar.add(&pt.group_rows, groups * kPanelRows);
+  ar.add(&pt.units, groups);
+  ar.add(&pt.piece_ptr, static_cast<size_t>(B.n_rows) + 1);
+  pt.max_pieces = B.nnz / kPanelEntriesPerPiece + 1;
+  ar.add(&pt.pieces, static_cast<size_t>(pt.max_pieces));
+  // (what only the prefix sum over the pieces needs lies where the visits will be)
+  scratch.add(&piece_count, static_cast<size_t>(B.n_rows));
+  scratch.add(&piece_tmp, static_cast<size_t>(scan_tmp_elems(B.n_rows)));
+  ar.add(&pt.visits, std::max(entries * kPanelVisitsPerEntry, scratch.bytes / sizeof(PanelVisit) + 1));
+  DeviceFacts facts;
+  GM_TRY(device_facts(&facts));
+  if (static_cast<i64>(found[kPanelProducts]) < kPanelMinHeavy || ar.bytes > facts.total_mem / kPanelMemoryShare || ar.commit(p, st) != GM_OK) {
+    p->use_panels = false;  // too few, or no room
+    return GM_OK;
+  }
+  p->panel_mem = ar.base;
+  scratch.place(pt.visits);
+  const int group_bits = panel_group_bits(p->sv), n_groups = static_cast<int>(panel_groups(p));
+  const unsigned row_grid = grid_for(B.n_rows, 8, p->num_sms, 16);
+  k_piece_count<<<row_grid, 256, 0, st>>>(B.row_ptr, B.col_idx, B.n_rows, group_bits, piece_count);
+  p->info.launches += 3 + exclusive_scan<u32, i64>(piece_count, pt.piece_ptr, B.n_rows, piece_tmp, nullptr, nullptr, nullptr, st);
+  k_piece_fill<<<row_grid, 256, 0, st>>>(B.row_ptr, B.col_idx, B.n_rows, group_bits, pt);
+  GM_TRY(allow_smem<k_panel_build>(p));
+  k_panel_build<<<static_cast<unsigned>(std::min<i64>(static_cast<i64>(found[kPanelsFound]), static_cast<i64>(p->num_sms) * 3)), kPanelBuildThreads,
+                  panel_build_smem(B.n_rows, n_groups), st>>>(pt, p->x_heavy, p->heavy_base, p->heavy_nz_off, A.row_ptr, A.col_idx, B.n_rows,
+                                                              n_groups, panel_max_u(p), nH >= kPanelRows * 256 ? 2 * kPanelWarps : kPanelWarps);
+  return GM_OK;
 }
 
 // Tasks of the heavy rows: piece boundaries of B, products per row and granule, ranges, lists.
@@ -655,8 +714,6 @@ static int plan_tasks(gm_plan* p, cudaStream_t st) {
   int32_t* long_rows = nullptr;
   i64* tmp = nullptr;
   unsigned char* similar = nullptr;
-  u32* piece_count = nullptr;
-  i64* piece_tmp = nullptr;
   i64* starts = nullptr;
   PanelTables& pt = p->panels;
   // Small products: the tables take their upper bound (a granule of n products gives fewer than 2 n / split_above
@@ -680,10 +737,15 @@ static int plan_tasks(gm_plan* p, cudaStream_t st) {
     ar.add(&n_long, 1);
     ar.add(&p->task_counters, 8 * n_batches);
     if (p->use_panels) {
-      ar.add(&pt.counts, 2);
+      ar.add(&pt.counts, kPanelCounts);
       ar.add(&starts, n_batches);
     }
     const size_t zeroed = ar.bytes;
+    if (p->use_panels) {
+      ar.add(&pt.list, static_cast<size_t>(nH) / kPanelMinRows + 1);
+      ar.add(&pt.of_row, static_cast<size_t>(nH));
+      ar.add(&similar, static_cast<size_t>(nH));
+    }
     ar.add(&p->c_total, 16);  // (next to the tickets: one clear for both, see execute_t)
     ar.add(&p->task_tickets, 4 * n_batches);
     ar.add(&p->piece_bound, static_cast<size_t>(B.n_rows) * static_cast<size_t>(r.granules + 1));
@@ -698,49 +760,30 @@ static int plan_tasks(gm_plan* p, cudaStream_t st) {
     if (p->finish) add_tables(ar, bound, bound);
     GM_TRY(ar.commit(p, st));
     GM_CUDA(cudaMemsetAsync(p->longest_row, 0, zeroed, st));
-    if (p->use_panels) {
-      Arena par;
-      const size_t n = static_cast<size_t>(nH), seg = static_cast<size_t>(p->n_seg);
-      par.add(&pt.list, n / kPanelMinRows + 1);
-      par.add(&pt.of_row, n);
-      par.add(&pt.a_u, seg);
-      par.add(&pt.u_mask, seg);
-      par.add(&pt.visits, seg * kPanelVisitsPerEntry);
-      par.add(&pt.groups, seg / kPanelEntriesPerGroup + 1);
-      par.add(&pt.group_rows, (seg / kPanelEntriesPerGroup + 1) * kPanelRows);
-      par.add(&pt.units, seg / kPanelEntriesPerGroup + 1);
-      par.add(&similar, n);
-      par.add(&pt.piece_ptr, static_cast<size_t>(B.n_rows) + 1);
-      par.add(&piece_count, static_cast<size_t>(B.n_rows));
-      pt.max_pieces = B.nnz / kPanelEntriesPerPiece + 1;
-      par.add(&pt.pieces, static_cast<size_t>(pt.max_pieces));
-      par.add(&piece_tmp, static_cast<size_t>(scan_tmp_elems(B.n_rows)));
-      if (par.commit(p, st) != GM_OK) p->use_panels = false;  // no room: the rows are tasks like the others
-    }
   }
   if (p->use_panels) {
     if (n_batches > 1) {
+      p->batch_starts.clear();
       for (const Batch& b : p->batches) p->batch_starts.push_back(b.h0);
       GM_CUDA(cudaMemcpyAsync(starts, p->batch_starts.data(), n_batches * sizeof(i64), cudaMemcpyHostToDevice, st));
     }
-    const int group_bits = panel_group_bits(p->sv), n_groups = static_cast<int>(((B.n_cols - 1) >> group_bits) + 1);
-    const unsigned row_grid = grid_for(B.n_rows, 8, p->num_sms, 16);
-    k_piece_count<<<row_grid, 256, 0, st>>>(B.row_ptr, B.col_idx, B.n_rows, group_bits, piece_count);
-    p->info.launches += 5 + exclusive_scan<u32, i64>(piece_count, pt.piece_ptr, B.n_rows, piece_tmp, nullptr, nullptr, nullptr, st);
-    k_piece_fill<<<row_grid, 256, 0, st>>>(B.row_ptr, B.col_idx, B.n_rows, group_bits, pt);
     k_panel_similar<<<static_cast<unsigned>((nH + 7) / 8), 256, 0, st>>>(p->x_heavy, nH, A.row_ptr, A.col_idx, similar);
-    k_panel_cut<<<static_cast<unsigned>((nH + 1023) / 1024), 1024, 0, st>>>(similar, nH, starts, static_cast<int>(n_batches), pt);
-    GM_TRY(allow_smem<k_panel_build>(p));
-    k_panel_build<<<static_cast<unsigned>(std::min<i64>(nH / kPanelMinRows + 1, static_cast<i64>(p->num_sms) * 3)), kPanelBuildThreads,
-                    panel_build_smem(B.n_rows, n_groups), st>>>(pt, p->x_heavy, p->heavy_base, p->heavy_nz_off, A.row_ptr, A.col_idx, B.n_rows,
-                                                                n_groups, panel_max_u(p), nH >= kPanelRows * 256 ? 2 * kPanelWarps : kPanelWarps);
+    k_panel_cut<<<static_cast<unsigned>((nH + 1023) / 1024), 1024, 0, st>>>(similar, nH, starts, static_cast<int>(n_batches), p->heavy_base,
+                                                                          p->heavy_nz_off, pt, p->slot->panels);
+    p->info.launches += 2;
+    if (!p->ev_light) GM_CUDA(cudaEventCreateWithFlags(&p->ev_light, cudaEventDisableTiming));
+    GM_CUDA(cudaEventRecord(p->ev_light, st));
   }
-  const unsigned char* const in_panel = p->use_panels ? pt.of_row : nullptr;
   k_piece_bounds<<<grid_for(B.n_rows * (r.granules + 1), 256, p->num_sms, 32), 256, 0, st>>>(B.row_ptr, B.col_idx, B.n_rows, r.granules,
                                                                                            r.log2_g, p->piece_bound, p->longest_row);
   k_granule_parts<<<static_cast<unsigned>(r.granules), 32, 0, st>>>(B.col_idx, p->piece_bound, p->longest_row, r.granules, r.log2_g,
                                                                   p->part_cols);
   p->info.launches += 2;
+  if (p->use_panels) {
+    GM_CUDA(cudaEventSynchronize(p->ev_light));  // (while the two kernels before this run)
+    GM_TRY(build_panels(p, st));
+  }
+  const unsigned char* in_panel = p->use_panels ? p->panels.of_row : nullptr;
   if (r.granules > 1) {
     k_granule_counts<<<grid_for(nH, 8, p->num_sms, 8), 256, 0, st>>>(p->x_heavy, nH, A.row_ptr, A.col_idx, p->piece_bound, r.granules,
                                                                    p->granule_counts, long_rows, n_long, in_panel);
@@ -758,13 +801,18 @@ static int plan_tasks(gm_plan* p, cudaStream_t st) {
     GM_CUDA(cudaGetLastError());
     return GM_OK;
   }
-  k_task_count<<<static_cast<unsigned>((nH + 127) / 128), 128, 0, st>>>(p->granule_counts, p->heavy_base, nH, r, p->row_tasks, in_panel);
+  k_task_count<<<static_cast<unsigned>((nH + 127) / 128), 128, 0, st>>>(p->granule_counts, p->heavy_base, nH, r, p->row_tasks, in_panel,
+                                                                       p->use_panels ? pt.counts : nullptr, p->slot->panels);
   p->info.launches += 1 + exclusive_scan<u32, i64>(p->row_tasks, p->row_task_off, nH, tmp, nullptr, nullptr, nullptr, st,
                                                   reinterpret_cast<i64*>(&p->slot->n_tasks));
   for (size_t i = 1; i < n_batches; ++i)
     GM_CUDA(cudaMemcpyAsync(&p->task_begin[i], p->row_task_off + p->batches[i].h0, sizeof(i64), cudaMemcpyDeviceToHost, st));
   GM_CUDA(cudaStreamSynchronize(st));
   p->task_begin[n_batches] = p->slot->n_tasks;
+  if (p->use_panels && p->slot->panels[kPanelUnits] == 0) {  // none pays (a small product finds that out in its first execute)
+    drop_panels(p, st);
+    in_panel = nullptr;
+  }
   i64 max_tasks = 0;
   for (size_t i = 0; i < n_batches; ++i) max_tasks = std::max(max_tasks, p->task_begin[i + 1] - p->task_begin[i]);
   {
@@ -2010,6 +2058,7 @@ static int execute_t(gm_plan* p, cudaStream_t st, gm_csr* C) {
     p->stats.early_exit_chunks = t[7];
     p->stats.split_products -= t[8];
     p->stats.panel_rows = static_cast<float>(t[9]);
+    if (p->use_panels && t[9] == 0) drop_panels(p, st);
   }
   p->stats.c_capacity = capacity;
   if (tm.enabled) {

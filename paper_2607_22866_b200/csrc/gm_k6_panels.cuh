@@ -42,6 +42,7 @@ constexpr int kPanelEntriesPerPiece = 4, kPanelVisitsPerEntry = 3, kPanelEntries
 
 struct Panel {
   u32 h, rows, n_u, n_groups;  // first heavy row, rows, columns of U, groups reached (n_u = 0: not a panel)
+  i64 e;                       // entries of A in the panels before
 };
 struct __align__(16) GroupPiece {  // the entries of a row of B in one group
   u32 start;      // position of the first in B's arrays
@@ -62,11 +63,10 @@ struct PanelTables {
   GroupPiece* pieces;
   i64 max_pieces;
   Panel* list;
-  u32* counts;            // [0] panels, [1] units
+  u64* counts;            // kPanelCounts: see below
   unsigned char* of_row;  // per heavy row: 1 = in a panel
   PanelUnit* units;
-  // of a panel whose first entry of A is the e-th of the heavy rows: from e (a_u, u_mask), e * kPanelVisitsPerEntry (visits) and
-  // e / kPanelEntriesPerGroup (groups) on
+  // of a panel: from its e (a_u, u_mask), e * kPanelVisitsPerEntry (visits) and e / kPanelEntriesPerGroup (groups) on
   unsigned short* a_u;    // the entry's column in U
   u32* u_mask;
   PanelVisit* visits;
@@ -150,7 +150,8 @@ __global__ void __launch_bounds__(256) k_panel_similar(const int32_t* __restrict
 
 // A block per 1024 heavy rows (runs end there, and where a batch begins).  starts: first rows of the batches.
 __global__ void __launch_bounds__(1024) k_panel_cut(const unsigned char* __restrict__ similar, i64 n_heavy, const i64* __restrict__ starts,
-                                                    int n_batches, PanelTables pt) {
+                                                    int n_batches, const i64* __restrict__ heavy_base, const i64* __restrict__ heavy_nz_off,
+                                                    PanelTables pt, u64* __restrict__ host_counts) {
   __shared__ int s_first[1024], s_end[1024];
   const int tid = threadIdx.x;
   const i64 h = static_cast<i64>(blockIdx.x) * 1024 + tid;
@@ -172,13 +173,24 @@ __global__ void __launch_bounds__(1024) k_panel_cut(const unsigned char* __restr
     s_end[tid] = min(s_end[tid], b);
     __syncthreads();
   }
-  if (h >= n_heavy) return;
-  pt.of_row[h] = 0;
-  const int begin = s_first[tid], end = min(tid + 1 < 1024 ? s_end[tid + 1] : n, n);
-  const int len = end - begin, pieces = (len + kPanelRows - 1) / kPanelRows, per = (len + pieces - 1) / pieces;
-  if ((tid - begin) % per) return;
-  const int rows = min(per, end - tid);
-  if (rows >= kPanelMinRows) pt.list[atomicAdd(&pt.counts[0], 1u)] = Panel{static_cast<u32>(h), static_cast<u32>(rows), 0u, 0u};
+  if (h < n_heavy) {
+    pt.of_row[h] = 0;
+    const int begin = s_first[tid], end = min(tid + 1 < 1024 ? s_end[tid + 1] : n, n);
+    const int len = end - begin, pieces = (len + kPanelRows - 1) / kPanelRows, per = (len + pieces - 1) / pieces;
+    const int rows = (tid - begin) % per ? 0 : min(per, end - tid);
+    if (rows >= kPanelMinRows) {
+      const u64 at = atomicAdd(&pt.counts[kPanelsFound], 1ull);
+      const u64 e = atomicAdd(&pt.counts[kPanelEntries], static_cast<u64>(heavy_nz_off[h + rows] - heavy_nz_off[h]));
+      atomicAdd(&pt.counts[kPanelProducts], static_cast<u64>(heavy_base[h + rows] - heavy_base[h]));
+      pt.list[at] = Panel{static_cast<u32>(h), static_cast<u32>(rows), 0u, 0u, static_cast<i64>(e)};
+    }
+  }
+  __threadfence();
+  __syncthreads();
+  if (tid == 0 && atomicAdd(&pt.counts[kPanelBlocks], 1ull) == gridDim.x - 1) {  // the last block: the counts to the host
+    __threadfence();
+    for (int i = 0; i < kPanelCounts; ++i) host_counts[i] = static_cast<const volatile u64*>(pt.counts)[i];  // (read after an event)
+  }
 }
 
 constexpr int kPanelBuildThreads = 512;
@@ -208,7 +220,7 @@ __global__ void __launch_bounds__(kPanelBuildThreads) k_panel_build(
   u32* const g_count = bits + n_words_max;
   unsigned short* const before = reinterpret_cast<unsigned short*>(g_count + n_groups);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const u32 n_panels = pt.piece_ptr[n_rows_b] > pt.max_pieces ? 0u : pt.counts[0];
+  const u32 n_panels = pt.piece_ptr[n_rows_b] > pt.max_pieces ? 0u : static_cast<u32>(pt.counts[kPanelsFound]);
   for (u32 q = blockIdx.x; q < n_panels; q += gridDim.x) {
     const Panel p = pt.list[q];
     const int R = static_cast<int>(p.rows);
@@ -253,7 +265,7 @@ __global__ void __launch_bounds__(kPanelBuildThreads) k_panel_build(
     }
     if (n_u > max_u) continue;  // (block-uniform, as all that follow)
     for (int r = warp; r < R; r += kWarps) {
-      const i64 at = heavy_nz_off[p.h + r];
+      const i64 at = p.e + (heavy_nz_off[p.h + r] - heavy_nz_off[p.h]);
 #pragma unroll 4
       for (int j = lane; j < sm.n[r]; j += 32) {
         const int c = a_col[sm.row[r] + j];
@@ -278,7 +290,7 @@ __global__ void __launch_bounds__(kPanelBuildThreads) k_panel_build(
     }
     int n_visits;
     block_exclusive_scan(mine, sm.tmp, &n_visits);
-    const i64 entry0 = heavy_nz_off[p.h], entries = heavy_nz_off[p.h + R] - entry0;
+    const i64 entry0 = p.e, entries = heavy_nz_off[p.h + R] - heavy_nz_off[p.h];
     const i64 products = heavy_base[p.h + R] - heavy_base[p.h];
     if (products < static_cast<i64>(n_visits) * kPanelMinProducts || n_visits > entries * kPanelVisitsPerEntry) continue;
     __syncthreads();
@@ -358,7 +370,7 @@ __global__ void __launch_bounds__(kPanelBuildThreads) k_panel_build(
       pt.list[q].n_u = static_cast<u32>(n_u);
       pt.list[q].n_groups = static_cast<u32>(n_g);
       const int n = (n_g + unit_groups - 1) / unit_groups;
-      const u32 at = atomicAdd(&pt.counts[1], static_cast<u32>(n));
+      const u64 at = atomicAdd(&pt.counts[kPanelUnits], static_cast<u64>(n));
       for (int i = 0; i < n; ++i)
         pt.units[at + i] = PanelUnit{q, static_cast<u32>(i * unit_groups), static_cast<u32>(min(unit_groups, n_g - i * unit_groups))};
     }
@@ -402,7 +414,7 @@ __global__ void __launch_bounds__(kPanelThreads, 2) k6_panels(
   PanelSmem<V>& sm = *reinterpret_cast<PanelSmem<V>*>(smem_panel_raw);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int rg = lane >> 3, cg = lane & 7;  // the lane's rows rg * 8 .. + 7
-  const int n_units = static_cast<int>(pt.counts[1]);
+  const int n_units = static_cast<int>(pt.counts[kPanelUnits]);
   V(*const part)[G] = sm.part[warp];
   for (;;) {
     __syncthreads();
@@ -413,7 +425,7 @@ __global__ void __launch_bounds__(kPanelThreads, 2) k6_panels(
     const Panel p = pt.list[unit.panel];
     if (p.h < h0 || p.h >= h1) continue;
     const int n_u = static_cast<int>(p.n_u), R = static_cast<int>(p.rows);
-    const i64 entry0 = heavy_nz_off[p.h], group0 = (entry0 + kPanelEntriesPerGroup - 1) / kPanelEntriesPerGroup;
+    const i64 entry0 = p.e, group0 = (entry0 + kPanelEntriesPerGroup - 1) / kPanelEntriesPerGroup;
     // ---- the panel's part of A
     for (int i = tid; i < n_u * S / VEC; i += kPanelThreads) reinterpret_cast<int4*>(sm.dense)[i] = make_int4(0, 0, 0, 0);
     for (int u = tid; u < n_u; u += kPanelThreads) sm.u_mask[u] = pt.u_mask[entry0 + u];
@@ -421,8 +433,8 @@ __global__ void __launch_bounds__(kPanelThreads, 2) k6_panels(
     __syncthreads();
     bool a_bad = false;
     for (int r = warp; r < R; r += kPanelWarps) {
-      const i64 from = a_row_ptr[x_heavy[p.h + r]], at = heavy_nz_off[p.h + r];
-      const int n = static_cast<int>(heavy_nz_off[p.h + r + 1] - at);
+      const i64 from = a_row_ptr[x_heavy[p.h + r]], before = heavy_nz_off[p.h + r], at = entry0 + (before - heavy_nz_off[p.h]);
+      const int n = static_cast<int>(heavy_nz_off[p.h + r + 1] - before);
 #pragma unroll 4
       for (int j = lane; j < n; j += 32) {
         const V v = a_val[from + j];

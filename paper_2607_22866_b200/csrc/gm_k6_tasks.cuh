@@ -43,6 +43,9 @@ struct TaskRules {
 };
 constexpr int kMaxParts = 16;
 
+// Counts about panels (see gm_k6_panels.cuh).  Entries, products: of all that were found; blocks: of k_panel_cut that are through.
+enum PanelCount { kPanelsFound = 0, kPanelUnits, kPanelEntries, kPanelProducts, kPanelBlocks, kPanelCounts };
+
 // bound[k * (granules + 1) + c] = position in B's arrays of the first entry of row k with column >= c << log2_g.
 // A thread per boundary, each a binary search inside the row.
 // longest: (entries << 32) | row of the longest row of B.
@@ -197,8 +200,10 @@ __device__ __forceinline__ u32 cut_row(const u32* __restrict__ counts, u32 produ
 }
 
 __global__ void __launch_bounds__(128) k_task_count(const u32* __restrict__ counts, const i64* __restrict__ heavy_base, i64 n_heavy,
-                                                    TaskRules r, u32* __restrict__ row_tasks, const unsigned char* __restrict__ in_panel) {
+                                                    TaskRules r, u32* __restrict__ row_tasks, const unsigned char* __restrict__ in_panel,
+                                                    const u64* __restrict__ panels, u64* __restrict__ host_panels) {
   const i64 h = static_cast<i64>(blockIdx.x) * blockDim.x + threadIdx.x;
+  if (panels && h < kPanelCounts) host_panels[h] = panels[h];  // (read after a synchronisation)
   if (h >= n_heavy) return;
   if (in_panel && in_panel[h]) row_tasks[h] = 1;
   else row_tasks[h] = cut_row(counts + h * r.granules, static_cast<u32>(heavy_base[h + 1] - heavy_base[h]), r, [](int, int, u32, u32) {});

@@ -7,7 +7,7 @@ import torch
 import gen
 import oracle
 import paper_2607_22866_b200 as gm
-from parity import check_product, compare_rows, run_gpu
+from parity import check_product, compare_rows, make_opts, run_gpu
 from test_gpu_scratch_and_errors import allocator  # noqa: F401 (fixture)
 
 pytestmark = pytest.mark.gpu
@@ -147,3 +147,46 @@ def test_no_room_for_the_panels_lists(allocator):
         allocator.refuse = staticmethod(lambda n: False)
         compare_rows(gm.spgemm_execute(plan), ref, np.float32)
         assert plan.stats().panel_rows == 0 if refused else plan.stats().panel_rows > 0.9 * A.n_rows
+
+
+def _held(allocator, plan, *results):
+    """What the plan has from the allocator: all but the results."""
+    mine = {t.data_ptr() for C in results for t in (C.row_ptr, C.col, C.val)}
+    return sum(n for p, n in allocator.held.items() if p not in mine)
+
+
+@pytest.mark.parametrize("n_rows", [8000, 20000])  # tasks listed by one block, and by many
+def test_rows_that_are_not_alike_take_no_lists(allocator, n_rows):
+    # the same rows in another order, no two neighbours alike: planned as if there were no panels
+    rng = np.random.default_rng(n_rows)
+    A = _blocks(rng, [20] * (n_rows // 20), 150, 0.8, 4000, np.float32)
+    B = _spans(rng, 4000, 3000, 2, 50, 0.9, np.float32)
+    rows = np.split(A.col, A.row_ptr[1:-1])
+    shuffled = _csr([rows[i] for i in rng.permutation(n_rows)], 4000, rng, np.float32)
+    dB, held = gm.DeviceCSR.from_host(B), []
+    for M in (A, shuffled):
+        allocator.held.clear()
+        plan = gm.spgemm_plan(gm.DeviceCSR.from_host(M), dB)
+        torch.cuda.synchronize()
+        assert plan.info().products_heavy >= 1 << 26
+        held.append(_held(allocator, plan))
+        C = gm.spgemm_execute(plan)
+        assert plan.stats().panel_rows > 0.9 * n_rows if M is A else plan.stats().panel_rows == 0
+        if M is shuffled:
+            compare_rows(C, oracle.spgemm(M, B), np.float32)
+    assert held[1] < held[0] - 40 * A.nnz
+
+
+@pytest.mark.parametrize("n_rows", [8000, 20000])
+def test_lists_of_no_panel_are_given_back(allocator, n_rows):
+    # rows alike, but with more columns than a panel may have: nothing of the lists is left after the first product
+    rng = np.random.default_rng(n_rows)
+    A = _blocks(rng, [32] * (n_rows // 32), 705, 1.0, 705, np.float32)
+    B = _spans(rng, 705, 3000, 1, 30, 0.6, np.float32)
+    plan = gm.spgemm_plan(gm.DeviceCSR.from_host(A), gm.DeviceCSR.from_host(B))
+    C = gm.spgemm_execute(plan)
+    before = plan.info().workspace_bytes
+    assert plan.stats().panel_rows == 0 and plan.info().products_heavy >= 1 << 26
+    stage = plan.info().stage_elems * 8
+    assert _held(allocator, plan, C) == before < stage + 30 * A.nnz + (8 << 20)
+    compare_rows(gm.spgemm_execute(plan), oracle.spgemm(A, B), np.float32)
