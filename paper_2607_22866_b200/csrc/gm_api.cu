@@ -359,6 +359,8 @@ struct gm_plan {
   gm::u32* row_tasks = nullptr;    // nH
   int64_t* row_task_off = nullptr; // nH + 1
   std::vector<int64_t> task_begin; // per batch (and the end): first task
+  void* task_mem[2]{};             // the tables of the tasks
+  bool task_replan = false;        // they are gone: the tasks have to be listed again
   gm::HeavyTask* tasks = nullptr;
   int64_t* task_off = nullptr;     // place of a task in the staging area
   int32_t* task_list[3]{};         // small, mid, big
@@ -759,6 +761,7 @@ static int plan_tasks(gm_plan* p, cudaStream_t st) {
     }
     if (p->finish) add_tables(ar, bound, bound);
     GM_TRY(ar.commit(p, st));
+    p->task_mem[0] = ar.base;
     GM_CUDA(cudaMemsetAsync(p->longest_row, 0, zeroed, st));
   }
   if (p->use_panels) {
@@ -819,6 +822,7 @@ static int plan_tasks(gm_plan* p, cudaStream_t st) {
     Arena ar;
     add_tables(ar, p->slot->n_tasks, max_tasks);
     GM_TRY(ar.commit(p, st));
+    p->task_mem[1] = ar.base;
   }
   for (size_t i = 0; i < n_batches; ++i) {
     const Batch& b = p->batches[i];
@@ -829,6 +833,19 @@ static int plan_tasks(gm_plan* p, cudaStream_t st) {
     ++p->info.launches;
   }
   GM_CUDA(cudaGetLastError());
+  return GM_OK;
+}
+
+// Lists the heavy rows' tasks again, without panels, whose lists are given back: for products whose C is refused beside them.
+static int tasks_without_panels(gm_plan* p, cudaStream_t st) {
+  p->task_replan = true;
+  drop_panels(p, st);
+  for (auto& q : p->task_mem) {
+    plan_free(p, q, st);
+    q = nullptr;
+  }
+  GM_TRY(plan_tasks(p, st));
+  p->task_replan = false;
   return GM_OK;
 }
 
@@ -2155,10 +2172,15 @@ int gm_spgemm_execute(gm_plan* plan, void* cuda_stream, gm_csr* C_out) {
   }
   auto run = [&]() { return plan->A.dtype == GM_F32 ? execute_t<float>(plan, st, C_out) : execute_t<double>(plan, st, C_out); };
   if (plan->light_relist) GM_TRY(light_rows_by_hash(plan, st));  // (an execute before this one had no room for the lists)
+  if (plan->task_replan) GM_TRY(tasks_without_panels(plan, st));
   int rc = run();
   plan->pending = false;  // (whatever the result, the execute has waited for its stream)
-  if (plan->light_stage && (rc == GM_ERR_OOM || (rc == GM_ERR_CAPACITY && plan->opts.c_capacity <= 0))) {
-    // C does not fit beside the light rows' staging area: once more without it
+  auto no_room = [&]() { return rc == GM_ERR_OOM || (rc == GM_ERR_CAPACITY && plan->opts.c_capacity <= 0); };
+  if (plan->use_panels && no_room()) {  // C does not fit beside the panels' lists: once more without them
+    GM_TRY(tasks_without_panels(plan, st));
+    rc = run();
+  }
+  if (plan->light_stage && no_room()) {  // ... nor beside the light rows' staging area
     GM_TRY(light_rows_by_hash(plan, st));
     rc = run();
   }

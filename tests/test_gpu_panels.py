@@ -190,3 +190,39 @@ def test_lists_of_no_panel_are_given_back(allocator, n_rows):
     stage = plan.info().stage_elems * 8
     assert _held(allocator, plan, C) == before < stage + 30 * A.nnz + (8 << 20)
     compare_rows(gm.spgemm_execute(plan), oracle.spgemm(A, B), np.float32)
+
+
+@pytest.mark.parametrize("batches", [False, True])
+@pytest.mark.parametrize("n_rows", [8000, 20000])
+def test_c_is_refused_beside_the_lists(allocator, n_rows, batches):
+    # there is room for C or for the panels' lists: the lists go, and the rows are tasks from then on; not even that much room: an error,
+    # and the plan goes on when there is room again
+    rng = np.random.default_rng(n_rows)
+    A = _blocks(rng, [20] * (n_rows // 20), 150, 0.8, 4000, np.float32)
+    B = _spans(rng, 4000, 3000, 2, 50, 0.9, np.float32)
+    ref = oracle.spgemm(A, B)
+    c_bytes = ref.nnz * 8 + (n_rows + 1) * 8
+    opts = make_opts(stage_elems=1 << 25, c_capacity=ref.nnz) if batches else None
+    plan = gm.spgemm_plan(gm.DeviceCSR.from_host(A), gm.DeviceCSR.from_host(B), opts=opts)
+    torch.cuda.synchronize()
+    assert (plan.info().n_batches > 1) == batches
+
+    def check():
+        C = gm.spgemm_execute(plan)
+        compare_rows(C, ref, np.float32)
+        for t in (C.row_ptr, C.col, C.val):
+            allocator.held.pop(t.data_ptr())
+
+    check()
+    assert plan.stats().panel_rows > 0.9 * n_rows
+    for room in (c_bytes - 30 * A.nnz, 0, c_bytes, None):
+        most = sum(allocator.held.values()) + room if room is not None else 1 << 40
+        allocator.refuse = staticmethod(lambda n: sum(allocator.held.values()) + n > most)
+        if room == 0:
+            with pytest.raises(gm.GmError) as ei:
+                gm.spgemm_execute(plan)
+            assert ei.value.status == -5
+        else:
+            check()
+            assert plan.stats().panel_rows == 0
+    allocator.refuse = staticmethod(lambda n: False)
