@@ -87,18 +87,24 @@ __global__ void __launch_bounds__(256) k_piece_count(const i64* __restrict__ b_r
     if (lane == 0) count[k] = n;
   }
 }
+// Panels take the order of their rows from the matrices' contract and look whether it holds, since the tasks, with columns that fit one
+// granule, give the right sums without it: there are no panels where a row of B is not strictly ascending, and a row of A that is
+// not leaves its panel to the tasks.
 __global__ void __launch_bounds__(256) k_piece_fill(const i64* __restrict__ b_row_ptr, const int32_t* __restrict__ b_col, i64 n_rows_b,
                                                     int group_bits, PanelTables pt) {
   if (pt.piece_ptr[n_rows_b] > pt.max_pieces) return;
   const int lane = threadIdx.x & 31;
+  bool bad = false;
   for (i64 k = static_cast<i64>(blockIdx.x) * 8 + (threadIdx.x >> 5); k < n_rows_b; k += static_cast<i64>(gridDim.x) * 8) {
     const i64 s = b_row_ptr[k], e = b_row_ptr[k + 1];
     GroupPiece* const out = pt.pieces + pt.piece_ptr[k];
     int n = 0;
     for (i64 i0 = s; i0 < e; i0 += 32) {
       const i64 i = i0 + lane;
-      const int g = i < e ? b_col[i] >> group_bits : -1;
-      const bool head = i < e && (i == s || (b_col[i - 1] >> group_bits) != g);
+      const int32_t c = i < e ? b_col[i] : INT_MAX, before = i < e && i > s ? b_col[i - 1] : -1;
+      const int g = c >> group_bits;
+      const bool head = i < e && (i == s || (before >> group_bits) != g);
+      bad |= c <= before;
       const u32 heads = __ballot_sync(0xffffffffu, head);
       if (head) {
         const int at = n + __popc(heads & lanemask_lt());
@@ -118,6 +124,7 @@ __global__ void __launch_bounds__(256) k_piece_fill(const i64* __restrict__ b_ro
     }
     __syncwarp();
   }
+  if (bad) pt.counts[kPanelUnordered] = 1ull;
 }
 
 // A warp per heavy row: similar[h] = 1 if about half of the row's columns are in heavy row h - 1, and neither is much longer.
@@ -201,8 +208,10 @@ struct PanelBuildSmem {
   unsigned short group[kPanelMaxReach];
   unsigned short n_rows[kPanelMaxReach][kPanelRows];  // entries of a row in a group
   i64 row[kPanelRows];
+  i64 off[kPanelRows + 1];             // a row's first entry in the lists
   int n[kPanelRows];
   int lo, hi, tmp[33];
+  i64 tmp64[33];
 };
 // columns of A: bitmap and ranks; groups of C: visits, then cursors
 inline size_t panel_build_smem(i64 n_rows_b, i64 n_groups) {
@@ -220,13 +229,14 @@ __global__ void __launch_bounds__(kPanelBuildThreads) k_panel_build(
   u32* const g_count = bits + n_words_max;
   unsigned short* const before = reinterpret_cast<unsigned short*>(g_count + n_groups);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const u32 n_panels = pt.piece_ptr[n_rows_b] > pt.max_pieces ? 0u : static_cast<u32>(pt.counts[kPanelsFound]);
+  const u32 n_panels = pt.piece_ptr[n_rows_b] > pt.max_pieces || pt.counts[kPanelUnordered] ? 0u : static_cast<u32>(pt.counts[kPanelsFound]);
   for (u32 q = blockIdx.x; q < n_panels; q += gridDim.x) {
     const Panel p = pt.list[q];
     const int R = static_cast<int>(p.rows);
     __syncthreads();
     if (tid == 0) { sm.lo = INT_MAX; sm.hi = 0; }
     __syncthreads();
+    if (tid >= 64 && tid <= 64 + R) sm.off[tid - 64] = p.e + (heavy_nz_off[p.h + tid - 64] - heavy_nz_off[p.h]);
     if (tid < R) {
       const i64 row = x_heavy[p.h + tid];
       const i64 s = a_row_ptr[row];
@@ -238,21 +248,23 @@ __global__ void __launch_bounds__(kPanelBuildThreads) k_panel_build(
     }
     __syncthreads();
     // ---- U: the columns as a bitmap, their ranks, the rows that hold them
-    const int w0 = sm.lo, n_words = sm.hi - sm.lo + 1;
+    const int w0 = sm.lo, n_words = max(sm.hi - sm.lo, 0) + 1;
     for (int w = tid; w < n_words; w += T) bits[w] = 0u;
     for (int i = tid; i < kPanelMaxU; i += T) sm.mask[i] = 0u;
     for (int g = tid; g < n_groups; g += T) g_count[g] = 0u;
     __syncthreads();
+    bool bad = false;  // not ascending: a column outside the range of the rows' ends
     for (int r = warp; r < R; r += kWarps) {
 #pragma unroll 4
       for (int j = lane; j < sm.n[r]; j += 32) {
         const int c = a_col[sm.row[r] + j];
         const u32 bit = 1u << (c & 31);
-        u32* const w = &bits[(c >> 5) - w0];
-        if (!(*w & bit)) atomicOr(w, bit);
+        const u32 at = static_cast<u32>((c >> 5) - w0), w = min(at, static_cast<u32>(n_words - 1));
+        bad |= at != w;
+        if (!(bits[w] & bit)) atomicOr(&bits[w], bit);
       }
     }
-    __syncthreads();
+    if (__syncthreads_or(bad)) continue;  // (block-uniform, as all that follow)
     int n_u = 0;
     for (int i0 = 0; i0 < n_words; i0 += T) {
       const int w = i0 + tid;
@@ -263,9 +275,9 @@ __global__ void __launch_bounds__(kPanelBuildThreads) k_panel_build(
       n_u += total;
       __syncthreads();
     }
-    if (n_u > max_u) continue;  // (block-uniform, as all that follow)
+    if (n_u > max_u) continue;
     for (int r = warp; r < R; r += kWarps) {
-      const i64 at = p.e + (heavy_nz_off[p.h + r] - heavy_nz_off[p.h]);
+      const i64 at = sm.off[r];
 #pragma unroll 4
       for (int j = lane; j < sm.n[r]; j += 32) {
         const int c = a_col[sm.row[r] + j];
@@ -281,18 +293,19 @@ __global__ void __launch_bounds__(kPanelBuildThreads) k_panel_build(
     }
     __syncthreads();
     // ---- visits per group
-    int mine = 0;
+    i64 mine = 0;  // (visits << 32) | entries in the masks, fewer than in the rows where a row has a column twice
     for (int u = tid; u < n_u; u += T) {
       const i64 s = pt.piece_ptr[sm.u_col[u]], e = pt.piece_ptr[sm.u_col[u] + 1];
 #pragma unroll 4
       for (i64 i = s; i < e; ++i) atomicAdd(&g_count[pt.pieces[i].group], 1u);
-      mine += static_cast<int>(e - s);
+      mine += ((e - s) << 32) + __popc(sm.mask[u]);
     }
-    int n_visits;
-    block_exclusive_scan(mine, sm.tmp, &n_visits);
-    const i64 entry0 = p.e, entries = heavy_nz_off[p.h + R] - heavy_nz_off[p.h];
+    i64 sums;
+    block_exclusive_scan(mine, sm.tmp64, &sums);
+    const i64 n_visits = sums >> 32;
+    const i64 entry0 = sm.off[0], entries = sm.off[R] - entry0;
     const i64 products = heavy_base[p.h + R] - heavy_base[p.h];
-    if (products < static_cast<i64>(n_visits) * kPanelMinProducts || n_visits > entries * kPanelVisitsPerEntry) continue;
+    if ((sums & 0xffffffff) != entries || products < n_visits * kPanelMinProducts || n_visits > entries * kPanelVisitsPerEntry) continue;
     __syncthreads();
     int n_g = 0, run = 0;
     for (int i0 = 0; i0 < n_groups; i0 += T) {

@@ -43,8 +43,9 @@ struct TaskRules {
 };
 constexpr int kMaxParts = 16;
 
-// Counts about panels (see gm_k6_panels.cuh).  Entries, products: of all that were found; blocks: of k_panel_cut that are through.
-enum PanelCount { kPanelsFound = 0, kPanelUnits, kPanelEntries, kPanelProducts, kPanelBlocks, kPanelCounts };
+// Counts about panels (see gm_k6_panels.cuh).  Entries, products: of all that were found; blocks: of k_panel_cut that are through;
+// unordered: a row of B does not ascend.
+enum PanelCount { kPanelsFound = 0, kPanelUnits, kPanelEntries, kPanelProducts, kPanelBlocks, kPanelUnordered, kPanelCounts };
 
 // bound[k * (granules + 1) + c] = position in B's arrays of the first entry of row k with column >= c << log2_g.
 // A thread per boundary, each a binary search inside the row.

@@ -226,3 +226,37 @@ def test_c_is_refused_beside_the_lists(allocator, n_rows, batches):
             check()
             assert plan.stats().panel_rows == 0
     allocator.refuse = staticmethod(lambda n: False)
+
+
+@pytest.mark.parametrize("dtype", [np.float32, np.float64])
+@pytest.mark.parametrize("what", ["A swapped", "A twice", "A ends inside", "B shuffled", "B twice"])
+def test_rows_that_do_not_ascend_are_left_to_the_tasks(what, dtype):
+    # against the contract, but the sums by tasks give the right product here (one granule of columns), and so they go on
+    rng = np.random.default_rng(len(what))
+    A = _blocks(rng, [25] * 480, 100, 0.85, 600, dtype)
+    B = _spans(rng, 600, 900, 2, 60, 0.8, dtype)
+    M, some = (A, [r for r in range(A.n_rows) if r // 25 % 3 == 0]) if what[0] == "A" else (B, range(0, 600, 7))
+    col = M.col.copy()
+    for r in some:
+        s, e = M.row_ptr[r], M.row_ptr[r + 1]
+        if what.endswith("shuffled"):
+            col[s:e] = rng.permutation(col[s:e])
+        elif what.endswith("swapped"):
+            col[s + 40:s + 42] = col[s + 40:s + 42][::-1].copy()
+        elif what.endswith("twice"):
+            col[s + 5] = col[s + 4]
+        else:  # the last column first: the row's ends leave out nearly all the others
+            col[s:e] = np.roll(col[s:e], 1)
+    a, b = np.zeros((A.n_rows, 600)), np.zeros((600, 900))
+    X = gen.CSR(M.n_rows, M.n_cols, M.row_ptr, col, M.val)
+    for S, d in ((X if M is A else A, a), (X if M is B else B, b)):
+        np.add.at(d, (np.repeat(np.arange(S.n_rows), np.diff(S.row_ptr)), S.col), S.val.astype(np.float64))
+    C, info, stats = run_gpu(X if M is A else A, X if M is B else B, tau=64)
+    assert info.heavy_tasks == 1 and (stats.panel_rows == 0 if M is B else 0.6 * A.n_rows < stats.panel_rows <= A.n_rows)
+    assert stats.panel_rows > 0.9 * A.n_rows if what == "A swapped" else stats.panel_rows < 0.7 * A.n_rows
+    rp, cc, val = C.row_ptr.cpu().numpy(), C.col.cpu().numpy(), C.val.cpu().numpy()
+    got = np.zeros((A.n_rows, 900))
+    got[np.repeat(np.arange(A.n_rows), np.diff(rp)), cc] = val
+    assert rp[-1] == np.count_nonzero((a != 0).astype(np.float32) @ (b != 0).astype(np.float32))
+    tol = 1e-5 if dtype == np.float32 else 1e-12
+    assert np.all(np.abs(got - a @ b) <= tol * (np.abs(a) @ np.abs(b)))
