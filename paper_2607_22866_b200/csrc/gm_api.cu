@@ -1689,6 +1689,12 @@ static int validate_tasks(gm_plan* p, cudaStream_t st) {
   k_validate_tasks<V><<<grid_for(p->info.rows_heavy, 1, p->num_sms, 8), 256, 0, st>>>(task_input<V>(p), p->tasks, p->row_task_off, p->heavy_base,
                                                                                     p->info.rows_heavy, p->B.n_cols, p->err);
   ++p->stats.launches;
+  if (p->use_panels) {
+    k_validate_panels<<<static_cast<unsigned>(p->num_sms * 4), 256, 0, st>>>(p->panels, p->x_heavy, p->info.rows_heavy, p->heavy_base, p->heavy_nz_off,
+                                                                            p->A.row_ptr, p->A.col_idx, p->B.row_ptr, p->B.col_idx, p->B.n_rows,
+                                                                            p->B.n_cols, panel_group_bits(p->sv), p->err);
+    ++p->stats.launches;
+  }
   GM_CUDA(cudaGetLastError());
   GM_CUDA(cudaStreamSynchronize(st));
   return dev_error_to_status(*static_cast<volatile int*>(&p->slot->err[0]));

@@ -390,6 +390,97 @@ __global__ void __launch_bounds__(kPanelBuildThreads) k_panel_build(
   }
 }
 
+// Debug mode: the lists of every panel (a block each) hold its products and no others, in the columns and at the places that they say:
+// entries of A find the column of U that selects their row of B; the visits are pieces of those rows, with the entries that their masks
+// say, in the group that lists them; they add up to the products; the entries of a row fit its part of the staging area.
+__global__ void __launch_bounds__(256) k_validate_panels(PanelTables pt, const int32_t* __restrict__ x_heavy, i64 n_heavy,
+                                                         const i64* __restrict__ heavy_base, const i64* __restrict__ heavy_nz_off,
+                                                         const i64* __restrict__ a_row_ptr, const int32_t* __restrict__ a_col,
+                                                         const i64* __restrict__ b_row_ptr, const int32_t* __restrict__ b_col, i64 n_rows_b,
+                                                         i64 n_cols, int group_bits, int* __restrict__ err) {
+  __shared__ int s_col[kPanelMaxU];
+  __shared__ u32 s_mask[kPanelMaxU];
+  __shared__ i64 s_sum[33];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  for (i64 q = blockIdx.x; q < static_cast<i64>(pt.counts[kPanelsFound]); q += gridDim.x) {
+    const Panel p = pt.list[q];
+    if (p.n_u == 0) continue;
+    if (p.n_u > kPanelMaxU || p.n_groups >= kPanelMaxReach || p.rows > kPanelRows || static_cast<i64>(p.h) + p.rows > n_heavy) {
+      if (tid == 0) dev_set_error(err, kDevBadChunk);
+      continue;
+    }
+    const int R = static_cast<int>(p.rows);
+    const i64 entries = heavy_nz_off[p.h + R] - heavy_nz_off[p.h], group0 = (p.e + kPanelEntriesPerGroup - 1) / kPanelEntriesPerGroup;
+    bool bad = false;
+    i64 bits = 0;
+    for (int u = tid; u < static_cast<int>(p.n_u); u += 256) {
+      s_col[u] = -1;
+      s_mask[u] = pt.u_mask[p.e + u];
+      bits += __popc(s_mask[u]);
+    }
+    __syncthreads();
+    for (int r = warp; r < R; r += 8) {
+      const i64 row = x_heavy[p.h + r], from = a_row_ptr[row], at = p.e + (heavy_nz_off[p.h + r] - heavy_nz_off[p.h]);
+      for (i64 j = lane; j < a_row_ptr[row + 1] - from; j += 32) {
+        const int k = a_col[from + j];
+        const u32 u = pt.a_u[at + j];
+        if (u >= p.n_u || k < 0 || k >= n_rows_b) {
+          bad = true;
+          continue;
+        }
+        const int was = atomicCAS(&s_col[u], -1, k);
+        bad |= (was != -1 && was != k) || !(s_mask[u] >> r & 1u);
+      }
+    }
+    i64 n;
+    block_exclusive_scan(bits, s_sum, &n);
+    bad |= n != entries;
+    __syncthreads();
+    i64 products = 0;
+    for (int k = warp; k < static_cast<int>(p.n_groups); k += 8) {
+      const PanelGroup g = pt.groups[group0 + k];
+      if (static_cast<i64>(g.first) + g.n > entries * kPanelVisitsPerEntry) {
+        bad = true;
+        continue;
+      }
+      for (u32 i = lane; i < g.n; i += 32) {
+        const PanelVisit v = pt.visits[p.e * kPanelVisitsPerEntry + g.first + i];
+        const int row = v.u < p.n_u ? s_col[v.u] : -1;
+        if (row < 0 || v.piece < pt.piece_ptr[row] || v.piece >= pt.piece_ptr[row + 1]) {
+          bad = true;
+          continue;
+        }
+        const GroupPiece piece = pt.pieces[v.piece];
+        const int m = __popcll(piece.mask);
+        bad |= piece.group != g.group;
+        if (piece.start < b_row_ptr[row] || static_cast<i64>(piece.start) + m > b_row_ptr[row + 1]) {
+          bad = true;
+          continue;
+        }
+        u64 left = piece.mask;
+        for (int t = 0; t < m; ++t, left &= left - 1) {
+          const i64 c = b_col[piece.start + t];
+          bad |= c >= n_cols || c != (static_cast<i64>(g.group) << group_bits) + __ffsll(static_cast<long long>(left)) - 1;
+        }
+        products += static_cast<i64>(m) * __popc(s_mask[v.u]);
+      }
+    }
+    block_exclusive_scan(products, s_sum, &n);
+    bad |= n != heavy_base[p.h + R] - heavy_base[p.h];
+    if (tid < R) {
+      u32 before = 0;
+      for (u32 k = 0; k <= p.n_groups; ++k) {
+        const u32 m = pt.group_rows[(group0 + k) * kPanelRows + tid];
+        bad |= m < before || m - before > 1u << group_bits;
+        before = m;
+      }
+      bad |= before > heavy_base[p.h + tid + 1] - heavy_base[p.h + tid];
+    }
+    if (bad) dev_set_error(err, kDevBadChunk);
+    __syncthreads();  // (the arrays are the next panel's)
+  }
+}
+
 // ---------------------------------------------------------------------------------------------------------------------
 // the product of a panel
 // ---------------------------------------------------------------------------------------------------------------------

@@ -260,3 +260,29 @@ def test_rows_that_do_not_ascend_are_left_to_the_tasks(what, dtype):
     assert rp[-1] == np.count_nonzero((a != 0).astype(np.float32) @ (b != 0).astype(np.float32))
     tol = 1e-5 if dtype == np.float32 else 1e-12
     assert np.all(np.abs(got - a @ b) <= tol * (np.abs(a) @ np.abs(b)))
+
+
+@pytest.mark.parametrize("dtype", [np.float32, np.float64])
+@pytest.mark.parametrize("stage", [0, 1 << 25])
+def test_debug_mode_checks_the_products_of_panels(dtype, stage):
+    # columns of B, and of A, that have changed since the plan; all of them in range, products per row as they were
+    rng = np.random.default_rng(8)
+    A = _blocks(rng, [31] * 500, 96, 0.85, 600, dtype)
+    B = _spans(rng, 600, 900, 2, 60, 0.8, dtype)
+    dA, dB = gm.DeviceCSR.from_host(A), gm.DeviceCSR.from_host(B)
+    plan = gm.spgemm_plan(dA, dB, opts=make_opts(tau=64, validate_inputs=1, stage_elems=stage))
+    assert plan.info().heavy_tasks == 1 and (plan.info().n_batches > 1) == (stage > 0)
+    ref = oracle.spgemm(A, B)
+    for _ in range(2):
+        compare_rows(gm.spgemm_execute(plan), ref, dtype)
+        assert plan.stats().panel_rows > 0.9 * A.n_rows
+    one = dB.col.clone()
+    one[B.row_ptr[300]:B.row_ptr[301]] = one[B.row_ptr[300]:B.row_ptr[301]].flip(0)
+    for col, bad in ((dB.col, torch.clamp(dB.col + 1, max=899)), (dB.col, one), (dA.col, 599 - dA.col)):
+        good = col.clone()
+        col.copy_(bad)
+        with pytest.raises(gm.GmError) as ei:
+            gm.spgemm_execute(plan)
+        assert ei.value.status == -10
+        col.copy_(good)
+    compare_rows(gm.spgemm_execute(plan), ref, dtype)
