@@ -645,9 +645,14 @@ static bool plan_task_rules(gm_plan* p) {
 // products enough to pay for the lists.  Block-dense products, us a call, tasks / panels: 2.8 M products fp64 150 / 195, 23 M fp32
 // 292 / 319, 43 M fp32 336 / 342, 166 M fp64 (kept plan) 895 / 510, 1.3 G fp64 5690 / 1630, 2.7 G fp32 8560 / 2440.
 constexpr i64 kPanelMinEntries = 48, kPanelMinHeavy = i64{1} << 26;
+// They are built where what they are expected to save, in products, pays for them (some 50 us and 20 ps an entry of A).
+constexpr i64 kPanelMinGain = i64{1} << 25, kPanelGainPerEntry = 16;
 constexpr size_t kPanelMemoryShare = 32;  // the lists take at most this part of the device's memory
 static int panel_max_u(const gm_plan* p) { return p->sv == 4 ? kPanelColumns<float> : kPanelColumns<double>; }
 static i64 panel_groups(const gm_plan* p) { return ((p->B.n_cols - 1) >> panel_group_bits(p->sv)) + 1; }
+// Groups of a unit: two for every warp where the panels keep the device busy all the same.  (Block-dense fp32, us with one / two, block rows
+// of 40: 3300 heavy rows 358 / 358, 7300 551 / 546, 11200 742 / 712, 16800 917 / 872; fp64 7300 648 / 630, 14000 918 / 868.)
+static int panel_unit_groups(i64 n_heavy) { return n_heavy >= kPanelRows * 256 ? 2 * kPanelWarps : kPanelWarps; }
 static bool plan_panel_rules(const gm_plan* p) {
   const size_t smem = p->sv == 4 ? sizeof(PanelSmem<float>) : sizeof(PanelSmem<double>);
   return p->info.products_heavy >= kPanelMinHeavy && p->n_seg >= kPanelMinEntries * p->info.rows_heavy && p->B.n_rows <= kPanelMaxRowsB &&
@@ -687,7 +692,7 @@ static int build_panels(gm_plan* p, cudaStream_t st) {
   ar.add(&pt.visits, std::max(entries * kPanelVisitsPerEntry, scratch.bytes / sizeof(PanelVisit) + 1));
   DeviceFacts facts;
   GM_TRY(device_facts(&facts));
-  if (static_cast<i64>(found[kPanelProducts]) < kPanelMinHeavy || ar.bytes > facts.total_mem / kPanelMemoryShare || ar.commit(p, st) != GM_OK) {
+  if (static_cast<i64>(found[kPanelGain]) < kPanelMinGain + kPanelGainPerEntry * static_cast<i64>(entries) || ar.bytes > facts.total_mem / kPanelMemoryShare || ar.commit(p, st) != GM_OK) {
     p->use_panels = false;  // too few, or no room
     return GM_OK;
   }
@@ -701,7 +706,7 @@ static int build_panels(gm_plan* p, cudaStream_t st) {
   GM_TRY(allow_smem<k_panel_build>(p));
   k_panel_build<<<static_cast<unsigned>(std::min<i64>(static_cast<i64>(found[kPanelsFound]), static_cast<i64>(p->num_sms) * 3)), kPanelBuildThreads,
                   panel_build_smem(B.n_rows, n_groups), st>>>(pt, p->x_heavy, p->heavy_base, p->heavy_nz_off, A.row_ptr, A.col_idx, B.n_rows,
-                                                              n_groups, panel_max_u(p), nH >= kPanelRows * 256 ? 2 * kPanelWarps : kPanelWarps);
+                                                              n_groups, panel_max_u(p), panel_unit_groups(nH));
   return GM_OK;
 }
 
@@ -770,9 +775,11 @@ static int plan_tasks(gm_plan* p, cudaStream_t st) {
       for (const Batch& b : p->batches) p->batch_starts.push_back(b.h0);
       GM_CUDA(cudaMemcpyAsync(starts, p->batch_starts.data(), n_batches * sizeof(i64), cudaMemcpyHostToDevice, st));
     }
-    k_panel_similar<<<static_cast<unsigned>((nH + 7) / 8), 256, 0, st>>>(p->x_heavy, nH, A.row_ptr, A.col_idx, similar);
+    k_panel_similar<<<static_cast<unsigned>((nH + 7) / 8), 256, 0, st>>>(p->x_heavy, nH, A.row_ptr, A.col_idx, B.row_ptr, B.col_idx,
+                                                                       panel_group_bits(p->sv), pt.counts, similar);
     k_panel_cut<<<static_cast<unsigned>((nH + 1023) / 1024), 1024, 0, st>>>(similar, nH, starts, static_cast<int>(n_batches), p->heavy_base,
-                                                                          p->heavy_nz_off, pt, p->slot->panels);
+                                                                          p->heavy_nz_off, static_cast<int>(panel_groups(p)), panel_unit_groups(nH),
+                                                                          p->sv == 4 ? kPanelCost<float> : kPanelCost<double>, pt, p->slot->panels);
     p->info.launches += 2;
     if (!p->ev_light) GM_CUDA(cudaEventCreateWithFlags(&p->ev_light, cudaEventDisableTiming));
     GM_CUDA(cudaEventRecord(p->ev_light, st));

@@ -34,10 +34,21 @@ template <typename V> constexpr int kPanelColumns = sizeof(V) == 4 ? kPanelMaxU 
 // Columns of a group: what a warp multiplies at a time.
 template <typename V> constexpr int kPanelGroup = 256 / sizeof(V);
 inline int panel_group_bits(int val_bytes) { return val_bytes == 4 ? 6 : 5; }
-// Products per visit from which on a panel is the faster way: a visit takes about 95 instructions of a warp, a product of the dense
-// accumulator four.
+// What panels cost, counted in products of the dense accumulator, which has `piece` of them to add for every entry of A.  A unit takes a
+// block some 15 us, and a warp 0.3 us for each visit of its groups, whether two rows are in it or thirty-two.  (fp32: 1.7 ps a product and
+// 115 a piece against 0.07 us a unit and 1.05 ns a visit of all eight warps, with 296 blocks at a time; fp64 2.9 ps and 100 against 0.07 and 1.1.)
+// 16000 rows in groups of R alike, 80 to 95 entries each, rows of B with k entries in n columns, us a call by tasks / by panels, fp32:
+//   R 2, k 150, n 200    712 / 1523    R 4, k 200, n 300  833 / 966    R 8, k 150, n 500    699 / 670    R 32, k 150, n 2000  883 / 826
+//   R 3, k 100, n 300    606 / 1211    R 4, k 200, n 230  832 / 907    R 16, k 150, n 1500  810 / 928    R 32, k 150, n 1500  812 / 679
+//   R 4, k 200, n 400    842 / 1035    R 8, k 150, n 700  736 / 942    R 16, k 150, n 800   745 / 687    (panels from R 8, n 500 on but R 16, n 1500)
+// fp64: R 4, k 200, n 300 and 230  1031 / 1288, 1016 / 922; R 8, n 400, k 100 and 150  711 / 842, 853 / 843 (panels for the second of both).
+struct PanelCost {
+  float piece, unit, visit;
+};
+template <typename V> constexpr PanelCost kPanelCost = sizeof(V) == 4 ? PanelCost{66.f, 41000.f, 610.f} : PanelCost{35.f, 24500.f, 380.f};
+// Once there are lists, panels with fewer products per visit than this stay with the tasks.
 constexpr u32 kPanelMinProducts = 40;
-// Room for pieces of rows of B, per entry of B, and for visits and groups, per entry of A in heavy rows: what takes more does not pay either.
+// Room for pieces of rows of B, per entry of B, and for visits and groups, per entry of A in panels; what takes more is left to the tasks.
 constexpr int kPanelEntriesPerPiece = 4, kPanelVisitsPerEntry = 3, kPanelEntriesPerGroup = 8;
 
 struct Panel {
@@ -128,16 +139,21 @@ __global__ void __launch_bounds__(256) k_piece_fill(const i64* __restrict__ b_ro
 }
 
 // A warp per heavy row: similar[h] = 1 if about half of the row's columns are in heavy row h - 1, and neither is much longer.
+// Some of those rows, spread out, are looked at closer: how many columns they share, and how many pieces a row of B that they use has.
+constexpr i64 kPanelSampleAll = 1024;  // heavy rows up to which all are, and about one in 32 above
 __global__ void __launch_bounds__(256) k_panel_similar(const int32_t* __restrict__ x_heavy, i64 n_heavy, const i64* __restrict__ a_row_ptr,
-                                                       const int32_t* __restrict__ a_col, unsigned char* __restrict__ similar) {
+                                                       const int32_t* __restrict__ a_col, const i64* __restrict__ b_row_ptr,
+                                                       const int32_t* __restrict__ b_col, int group_bits, u64* __restrict__ counts,
+                                                       unsigned char* __restrict__ similar) {
   const i64 h = static_cast<i64>(blockIdx.x) * 8 + (threadIdx.x >> 5);
   if (h >= n_heavy) return;
   const int lane = threadIdx.x & 31;
   bool hit = false;
-  i64 n = 0, n0 = 0;
+  i64 n = 0, n0 = 0, s = 0;
   if (h > 0) {
     const i64 row = x_heavy[h], prev = x_heavy[h - 1];
-    const i64 s = a_row_ptr[row], s0 = a_row_ptr[prev];
+    s = a_row_ptr[row];
+    const i64 s0 = a_row_ptr[prev];
     n = a_row_ptr[row + 1] - s;
     n0 = a_row_ptr[prev + 1] - s0;
     const i64 j = n <= 32 ? lane : n * lane / 32;
@@ -152,13 +168,29 @@ __global__ void __launch_bounds__(256) k_panel_similar(const int32_t* __restrict
     }
   }
   const int hits = __popc(__ballot_sync(0xffffffffu, hit));
-  if (lane == 0) similar[h] = hits > 0 && hits * 9 >= static_cast<int>(min(n, i64{32})) * 4 && 2 * min(n, n0) >= max(n, n0);
+  const int tried = static_cast<int>(min(n, i64{32}));
+  const bool alike = hits > 0 && hits * 9 >= tried * 4 && 2 * min(n, n0) >= max(n, n0);
+  if (lane == 0) similar[h] = alike;
+  const u32 mix = static_cast<u32>(h) * 2654435761u;
+  if (!alike || (n_heavy > kPanelSampleAll && mix >> 27 != 0)) return;
+  const int32_t k = a_col[s + (mix >> 3) % n];
+  const i64 b0 = b_row_ptr[k], b1 = b_row_ptr[k + 1];
+  u32 pieces = 0;
+  for (i64 i = b0 + lane; i < b1; i += 32) pieces += i == b0 || (b_col[i] >> group_bits) != (b_col[i - 1] >> group_bits);
+  pieces = __reduce_add_sync(0xffffffffu, pieces);
+  if (lane == 0) {
+    atomicAdd(&counts[kPanelTried], static_cast<u64>(tried));
+    atomicAdd(&counts[kPanelHits], static_cast<u64>(hits));
+    atomicAdd(&counts[kPanelSampled], 1ull);
+    atomicAdd(&counts[kPanelPieces], static_cast<u64>(pieces));
+    atomicAdd(&counts[kPanelSampleLen], static_cast<u64>(b1 - b0));
+  }
 }
 
 // A block per 1024 heavy rows (runs end there, and where a batch begins).  starts: first rows of the batches.
 __global__ void __launch_bounds__(1024) k_panel_cut(const unsigned char* __restrict__ similar, i64 n_heavy, const i64* __restrict__ starts,
                                                     int n_batches, const i64* __restrict__ heavy_base, const i64* __restrict__ heavy_nz_off,
-                                                    PanelTables pt, u64* __restrict__ host_counts) {
+                                                    int n_groups, int unit_groups, PanelCost cost, PanelTables pt, u64* __restrict__ host_counts) {
   __shared__ int s_first[1024], s_end[1024];
   const int tid = threadIdx.x;
   const i64 h = static_cast<i64>(blockIdx.x) * 1024 + tid;
@@ -187,8 +219,19 @@ __global__ void __launch_bounds__(1024) k_panel_cut(const unsigned char* __restr
     const int rows = (tid - begin) % per ? 0 : min(per, end - tid);
     if (rows >= kPanelMinRows) {
       const u64 at = atomicAdd(&pt.counts[kPanelsFound], 1ull);
-      const u64 e = atomicAdd(&pt.counts[kPanelEntries], static_cast<u64>(heavy_nz_off[h + rows] - heavy_nz_off[h]));
-      atomicAdd(&pt.counts[kPanelProducts], static_cast<u64>(heavy_base[h + rows] - heavy_base[h]));
+      const i64 entries = heavy_nz_off[h + rows] - heavy_nz_off[h];
+      const u64 e = atomicAdd(&pt.counts[kPanelEntries], static_cast<u64>(entries));
+      // what the panel is expected to gain: its columns by what neighbouring rows share, its visits by the pieces of some rows of B
+      const float pieces = static_cast<float>(pt.counts[kPanelPieces]) / fmaxf(1.f, static_cast<float>(pt.counts[kPanelSampled]));
+      const float share = static_cast<float>(pt.counts[kPanelHits]) / fmaxf(1.f, static_cast<float>(pt.counts[kPanelTried]));
+      const float visits = static_cast<float>(entries) / static_cast<float>(rows) / fmaxf(share, 0.25f) * pieces;
+      // (with 10 % more than there is room for, which is counted when the lists are built)
+      const bool room = pieces * (kPanelEntriesPerPiece * 0.9f) <= static_cast<float>(pt.counts[kPanelSampleLen]) / fmaxf(1.f, static_cast<float>(pt.counts[kPanelSampled])) &&
+                        visits * 0.9f <= static_cast<float>(entries) * kPanelVisitsPerEntry;
+      const float by_tasks = static_cast<float>(heavy_base[h + rows] - heavy_base[h]) + cost.piece * static_cast<float>(entries);
+      const float by_panel = cost.unit * ceilf(pieces / static_cast<float>(unit_groups)) + cost.visit * visits / static_cast<float>(min(n_groups, kPanelWarps));
+      const float gain = room ? by_tasks - by_panel : fminf(by_tasks - by_panel, 0.f);
+      atomicAdd(&pt.counts[kPanelGain], static_cast<u64>(static_cast<i64>(gain)));  // (of either sign)
       pt.list[at] = Panel{static_cast<u32>(h), static_cast<u32>(rows), 0u, 0u, static_cast<i64>(e)};
     }
   }

@@ -43,9 +43,10 @@ struct TaskRules {
 };
 constexpr int kMaxParts = 16;
 
-// Counts about panels (see gm_k6_panels.cuh).  Entries, products: of all that were found; blocks: of k_panel_cut that are through;
-// unordered: a row of B does not ascend.
-enum PanelCount { kPanelsFound = 0, kPanelUnits, kPanelEntries, kPanelProducts, kPanelBlocks, kPanelUnordered, kPanelCounts };
+// Counts about panels (see gm_k6_panels.cuh).  Entries of A in all that were found; blocks of k_panel_cut that are through; unordered: a
+// row of B does not ascend.  Of the rows that k_panel_similar looked at closer: columns tried and found in the row before, rows of B, their
+// pieces and entries.  Gain: what the panels are expected to save, in products.
+enum PanelCount { kPanelsFound = 0, kPanelUnits, kPanelEntries, kPanelBlocks, kPanelUnordered, kPanelTried, kPanelHits, kPanelSampled, kPanelPieces, kPanelSampleLen, kPanelGain, kPanelCounts };
 
 // bound[k * (granules + 1) + c] = position in B's arrays of the first entry of row k with column >= c << log2_g.
 // A thread per boundary, each a binary search inside the row.

@@ -286,3 +286,30 @@ def test_debug_mode_checks_the_products_of_panels(dtype, stage):
         assert ei.value.status == -10
         col.copy_(good)
     compare_rows(gm.spgemm_execute(plan), ref, dtype)
+
+
+def _scattered(rng, R, n_rows, per_row, fill, n_mid, n_cols, k, dtype):
+    """Groups of R rows alike, times rows of k columns anywhere."""
+    A = _blocks(rng, [R] * (n_rows // R), per_row, fill, n_mid, dtype)
+    return A, _csr([rng.choice(n_cols, k, replace=False) for _ in range(n_mid)], n_cols, rng, dtype)
+
+
+@pytest.mark.parametrize("dtype,R,k,n_cols,panels", [
+    (np.float32, 2, 150, 200, False), (np.float32, 3, 100, 300, False), (np.float32, 4, 200, 400, False), (np.float32, 8, 150, 700, False),
+    (np.float32, 8, 150, 400, True), (np.float32, 16, 150, 600, True), (np.float32, 32, 150, 1500, True),
+    (np.float64, 4, 200, 300, False), (np.float64, 8, 100, 400, False), (np.float64, 8, 200, 400, True), (np.float64, 32, 200, 1500, True)])
+def test_panels_where_they_are_the_faster_way(dtype, R, k, n_cols, panels):
+    # few rows alike, or short pieces of rows of B: a panel takes longer than its rows one by one (up to twice the call)
+    A, B = _scattered(np.random.default_rng(R * n_cols), R, 16000, 100, 0.9 if R < 8 else 0.8, 2000, n_cols, k, dtype)
+    C, info, stats = run_gpu(A, B)
+    assert info.heavy_tasks == 1 and info.products_heavy >= 1 << 26
+    assert stats.panel_rows > 0.9 * A.n_rows if panels else stats.panel_rows == 0
+    ref = oracle.spgemm(A, B)
+    compare_rows(C, ref, dtype)
+
+
+@pytest.mark.parametrize("n_rows,R", [(1024, 32), (1025, 41), (2000, 40)])  # all rows looked at, or one in 32
+def test_few_heavy_rows_alike(n_rows, R):
+    A, B = _scattered(np.random.default_rng(n_rows), R, n_rows, 300, 0.9, 1000, 400, 380, np.float32)
+    C, info, stats = check_product(A, B)
+    assert info.rows_heavy == n_rows and stats.panel_rows >= n_rows - 1  # (a run ends after 1024 rows)
