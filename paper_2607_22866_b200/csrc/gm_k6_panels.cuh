@@ -9,7 +9,7 @@
 //            k_piece_count, k_piece_fill  the pieces of every row of B per group of neighbouring columns
 //            k_panel_build    U with a mask of the rows that hold each column; per group of columns of C the pieces of rows of B
 //                             that reach it (visits), and where the group's entries of every row go; kept if it pays
-//   execute  k6_panels        a warp per group, eight groups of a panel to a block
+//   execute  k6_panels        a warp per group, a unit of eight or sixteen groups of a panel to a block
 // A panel's row is one task (see gm_k6_tasks.cuh) that is in no list: its entries go to the row's place in the staging area.
 //
 // What bounds it: nothing near its limit; block-dense fp32, 1.3 G products in 0.53 ms, issue slots 42 % with sixteen warps per SM (two blocks
@@ -535,6 +535,7 @@ __global__ void __launch_bounds__(256) k_validate_panels(PanelTables pt, const i
 // What is not there counts as zero, which is right as long as all is finite: with an infinity or a NaN in the panel's A or in a
 // round of visits the products are formed entry by entry instead.
 constexpr int kPanelDepth = 4;
+static_assert(kPanelDepth == 4 && 32 % kPanelDepth == 0, "entries leave four rows at a time through the visits' rows; a warp's 32 visits are whole rounds");
 template <typename V>
 struct PanelSmem {
   static constexpr int kStride = kPanelRows + 16 / sizeof(V);  // (columns of A are filled row by row: not all in one bank)

@@ -200,3 +200,20 @@ def test_light_rows_after_a_refusal(allocator, n):
             with pytest.raises(gm.GmError) as ei:
                 gm.spgemm_execute(plan)
             assert ei.value.status == -5
+
+
+@pytest.mark.parametrize("dtype", [np.float32, np.float64])
+@pytest.mark.parametrize("n_cols", [700, 1 << 21, (1 << 27) + 1])  # 32-bit and 64-bit sort keys
+def test_sorted_rows_around_the_widths_between_powers_of_two(dtype, n_cols):
+    # 3, 5 and 6 keys a lane: rows of up to 96, 160 and 192 products, and one more or less; columns repeat
+    rng = np.random.default_rng(n_cols % 1000)
+    pool = np.unique(np.concatenate([[0, n_cols - 1], rng.choice(n_cols, 600, replace=False) if n_cols < 1000 else rng.integers(0, n_cols, 600)]))
+    sizes = [64, 65, 66, 94, 95, 96, 97, 98, 129, 145, 158, 159, 160, 161, 162, 190, 191, 192, 193, 194]
+    B = _csr([rng.choice(pool, 1 << r, replace=False) for r in range(8)], n_cols, rng, dtype)
+    A = _csr([[r for r in range(8) if n >> r & 1] for n in sizes] * 7, 8, rng, dtype)
+    C, info, stats = check_product(A, B)  # rows placed by the sums of their groups
+    assert info.rows_heavy == 0 and info.rows_light == A.n_rows
+    rows = [[r for r in range(8) if n >> r & 1] for n in sizes] + [[8]]
+    B2 = _csr([B.col[B.row_ptr[r]:B.row_ptr[r + 1]] for r in range(8)] + [pool], n_cols, rng, dtype)
+    C, info, stats = check_product(_csr(rows, 9, rng, dtype), B2, tau=256)  # next to a heavy row
+    assert info.rows_heavy == 1

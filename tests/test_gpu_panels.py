@@ -313,3 +313,17 @@ def test_few_heavy_rows_alike(n_rows, R):
     A, B = _scattered(np.random.default_rng(n_rows), R, n_rows, 300, 0.9, 1000, 400, 380, np.float32)
     C, info, stats = check_product(A, B)
     assert info.rows_heavy == n_rows and stats.panel_rows >= n_rows - 1  # (a run ends after 1024 rows)
+
+
+@pytest.mark.parametrize("dtype,width", [(np.float32, 64), (np.float64, 32)])
+@pytest.mark.parametrize("groups", [509, 510, 511, 512, 513])
+def test_groups_that_a_panel_may_reach(dtype, width, groups):
+    # every panel reaches all groups of columns: up to 511 (the last one's sums lie behind it), and more, which stays with the tasks
+    rng = np.random.default_rng(groups)
+    n_mid, n_cols = 200, groups * width
+    at = [int(i * (groups - 4) / (n_mid - 1)) * width for i in range(n_mid)]
+    B = _csr([a + np.nonzero(rng.random(4 * width) < 0.9)[0] for a in at], n_cols, rng, dtype)
+    assert np.unique(B.col // width).size == groups
+    A = _blocks(rng, [32] * 70, n_mid, 1.0, n_mid, dtype) if dtype == np.float32 else _blocks(rng, [32] * 110, n_mid, 1.0, n_mid, dtype)
+    C, info, stats = check_product(A, B)
+    assert info.heavy_tasks == 1 and stats.panel_rows == (A.n_rows if groups <= 511 else 0)
