@@ -244,7 +244,8 @@ def kernel_table(info, stats_avg, sv, nnz_b, n_light_entries_a):
             tbl[k + " (into C)"] = (read_all + se * nnz_cl, stats_avg["ms_light_numeric"])
         else:
             tbl["k3_sort_rows, k3_merge_rows"] = (read_all + se * nnz_cl, stats_avg["ms_light_symbolic"])
-            tbl["k3_copy_rows" if rows_h or info.n_rows > 1 << 20 else "k3_place_rows"] = (2 * se * nnz_cl, stats_avg["ms_light_numeric"])
+            # (without heavy and hashed rows, and up to 2^20 rows, the copy finds the rows' place itself)
+            tbl["k3_copy_rows" if rows_h or info.light_bin_rows[7] or info.n_rows > 1 << 20 else "k3_place_rows"] = (2 * se * nnz_cl, stats_avg["ms_light_numeric"])
     if rows_h and info.heavy_tasks:
         # summed where the products are generated: B is read (by each kernel once, at least) and entries are written
         tbl["k6_small_tasks"] = (se * nnz_b + se * nnz_small, stats_avg["ms_small_chunks"])

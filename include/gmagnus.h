@@ -3,8 +3,9 @@
  * irregular, power-law structure, following the gMAGNUS method.  Light rows: Gustavson's method, a row's
  * products merged by a thread or sorted by a warp (hashed in shared memory where a row has more than 1024,
  * which takes a tau above the default, or where those have no room).  Heavy rows: cut into ranges of columns
- * whose products are summed where they are generated, or expanded into a staging buffer, regrouped by a
- * hierarchical multisplit by column chunk and accumulated chunk by chunk.
+ * whose products are summed where they are generated (neighbouring rows with much the same columns several at
+ * a time, as a small dense product), or expanded into a staging buffer, regrouped by a hierarchical multisplit
+ * by column chunk and accumulated chunk by chunk.
  *
  * Conventions
  *   - Every function returns an int status: GM_OK (0) or a negative GM_ERR_* code.  No exception
@@ -167,10 +168,11 @@ typedef struct gm_exec_stats {
   int64_t small_chunk_entries;  /* entries of C those produced                                   */
   float ms_light_symbolic, ms_light_numeric, ms_expand, ms_histogram, ms_multisplit,
       ms_accumulate, ms_gather, ms_scan, ms_total;
-  float ms_small_chunks;       /* one warp per chunk or task; ms_accumulate is the dense-accumulator kernel alone */
+  float ms_small_chunks;       /* one warp per chunk or task; ms_accumulate is the dense-accumulator kernel and that of
+                                  the rows summed several at a time                                               */
   float ms_mid_chunks;         /* one small block per chunk or task                                             */
   float panel_rows;            /* heavy rows summed several at a time, as a small dense product (neighbouring rows of A with
-                                  much the same columns; their kernel's time is part of ms_accumulate)            */
+                                  much the same columns); a whole number, exact up to 2^24                        */
   float reserved[2];
   int64_t mid_chunk_products;  /* products in chunks or tasks summed by one small block each                     */
   int64_t mid_chunk_entries;   /* entries of C those produced                                                    */

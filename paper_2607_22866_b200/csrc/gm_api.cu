@@ -641,8 +641,9 @@ static bool plan_task_rules(gm_plan* p) {
   return true;
 }
 
-// Panels are looked for where heavy rows have many entries (R-MAT graphs have 25 to 40, and hardly two rows alike) and where there are
-// products enough to pay for the lists.  Block-dense products, us a call, tasks / panels: 2.8 M products fp64 150 / 195, 23 M fp32
+// Panels are looked for where heavy rows have many entries (R-MAT graphs have 25 to 40, and hardly two rows alike; with 8 instead of 48
+// R-MAT scale 17 fp64 took 3880 us instead of 3857, ER of 100000 rows of 30 1962 instead of 1927) and where there are products enough to pay
+// for the lists.  Block-dense products, us a call, tasks / panels: 2.8 M products fp64 150 / 195, 23 M fp32
 // 292 / 319, 43 M fp32 336 / 342, 166 M fp64 (kept plan) 895 / 510, 1.3 G fp64 5690 / 1630, 2.7 G fp32 8560 / 2440.
 constexpr i64 kPanelMinEntries = 48, kPanelMinHeavy = i64{1} << 26;
 // They are built where what they are expected to save, in products, pays for them (some 50 us and 20 ps an entry of A).

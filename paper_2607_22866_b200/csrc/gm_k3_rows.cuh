@@ -15,6 +15,8 @@
 // Rows either go to the staging area of the light rows at light_off[row], from where k3_copy_rows moves them once
 // C.row_ptr is known (one pass over the products, and the entries are written twice), or, when every row of the matrix
 // is merged, they are counted first and then written to their place in C: a second merge is cheaper than the copy.
+// Without heavy and hashed rows nobody makes C.row_ptr first: k3_place_rows, or the second merge, finds its rows' place in C
+// from sums over groups of rows, and writes C.row_ptr too (see RowSums).
 #pragma once
 #include <type_traits>
 
