@@ -694,7 +694,7 @@ static int build_panels(gm_plan* p, cudaStream_t st) {
   DeviceFacts facts;
   GM_TRY(device_facts(&facts));
   if (static_cast<i64>(found[kPanelGain]) < kPanelMinGain + kPanelGainPerEntry * static_cast<i64>(entries) || ar.bytes > facts.total_mem / kPanelMemoryShare || ar.commit(p, st) != GM_OK) {
-    p->use_panels = false;  // too few, or no room
+    p->use_panels = false;  // they do not pay, or there is no room
     return GM_OK;
   }
   p->panel_mem = ar.base;

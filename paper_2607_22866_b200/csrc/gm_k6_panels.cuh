@@ -15,7 +15,7 @@
 // What bounds it: nothing near its limit; block-dense fp32, 1.3 G products in 0.53 ms, issue slots 42 % with sixteen warps per SM (two blocks
 // of 128 registers a thread), which wait for the next visits' entries and, at the end of a panel, for one another.  A product costs five
 // warp instructions per 32, against 135 by the dense accumulator, whose kernel took 5.7 + 1.4 ms of the call's 8.5 for 2.7 G products;
-// now 0.87 + 0.25 ms, the lists 0.30 ms, the call 2.4.
+// now 1.03 ms, the lists 0.30 ms, the call 2.35.
 #pragma once
 #include "gm_common.cuh"
 #include "gm_k6_tasks.cuh"

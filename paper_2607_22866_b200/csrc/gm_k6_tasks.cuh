@@ -150,7 +150,7 @@ __global__ void __launch_bounds__(256) k_granule_counts(const int32_t* __restric
 // The blocks form groups, one row at a time to a group, and the blocks of a group take the row's runs of kCountRun entries in turn, a
 // slice per warp: kCountRuns blocks to a group, or as many more as few rows leave.  (With all warps of the grid round-robin over all
 // slices, every warp looked up every row's ends, one after the other: 730 us of R-MAT scale 19.  With kCountRuns blocks however few the
-// rows: one row of 10^6 entries 750 us, two of 300000 250.)
+// rows: one row of 10^6 entries 750 us, two of 300000 255, now 34 and 35.)
 constexpr int kCountRun = 8 * 256, kCountRuns = 16;
 __global__ void __launch_bounds__(256) k_granule_counts_long(const int32_t* __restrict__ x_heavy, const i64* __restrict__ a_row_ptr,
                                                              const int32_t* __restrict__ a_col, const u32* __restrict__ bound, int granules,
