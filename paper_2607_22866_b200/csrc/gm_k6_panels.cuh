@@ -225,8 +225,8 @@ __global__ void __launch_bounds__(1024) k_panel_cut(const unsigned char* __restr
       const float pieces = static_cast<float>(pt.counts[kPanelPieces]) / fmaxf(1.f, static_cast<float>(pt.counts[kPanelSampled]));
       const float share = static_cast<float>(pt.counts[kPanelHits]) / fmaxf(1.f, static_cast<float>(pt.counts[kPanelTried]));
       const float visits = static_cast<float>(entries) / static_cast<float>(rows) / fmaxf(share, 0.25f) * pieces;
-      // (with 10 % more than there is room for, which is counted when the lists are built)
-      const bool room = pieces * (kPanelEntriesPerPiece * 0.9f) <= static_cast<float>(pt.counts[kPanelSampleLen]) / fmaxf(1.f, static_cast<float>(pt.counts[kPanelSampled])) &&
+      // (with 10 % more than there is room for, which is counted when the lists are built; nothing where no row was looked at closer)
+      const bool room = pt.counts[kPanelSampled] != 0 && pieces * (kPanelEntriesPerPiece * 0.9f) <= static_cast<float>(pt.counts[kPanelSampleLen]) / fmaxf(1.f, static_cast<float>(pt.counts[kPanelSampled])) &&
                         visits * 0.9f <= static_cast<float>(entries) * kPanelVisitsPerEntry;
       const float by_tasks = static_cast<float>(heavy_base[h + rows] - heavy_base[h]) + cost.piece * static_cast<float>(entries);
       const float by_panel = cost.unit * ceilf(pieces / static_cast<float>(unit_groups)) + cost.visit * visits / static_cast<float>(min(n_groups, kPanelWarps));
